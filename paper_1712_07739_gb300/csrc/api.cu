@@ -9,8 +9,7 @@
 int fmm_kernel_attrs(gbfmm_ctx *ctx);  // fmm.cu
 void mlp_free(gbfmm_ctx *ctx);         // mlp.cu
 int mixed_alloc(gbfmm_ctx *ctx);       // fmm.cu
-int near_alloc(gbfmm_ctx *ctx, int64_t n_targets);  // near.cu
-int near_sym_alloc(gbfmm_ctx *ctx);                 // near.cu
+int near_alloc(gbfmm_ctx *ctx);        // near.cu
 int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t);
 
 int set_err(gbfmm_ctx *c, int code, const std::string &msg) {
@@ -32,8 +31,6 @@ static void free_tree(gbfmm_ctx *ctx) {
     release(ctx->d_pos);
     release(ctx->d_pleaf);
     release(ctx->d_sig);
-    release(ctx->d_P);
-    release(ctx->d_Pf);
     release(ctx->d_y0);
     release(ctx->d_q0);
     release(ctx->d_leaf_of);
@@ -51,7 +48,6 @@ static void free_tree(gbfmm_ctx *ctx) {
     release(ctx->d_tmp_d);
     release(ctx->d_part);
     release(ctx->d_bad);
-    release(ctx->d_yrel);
     {
         auto &RF = ctx->rf;
         release(RF.child_of);
@@ -65,7 +61,7 @@ static void free_tree(gbfmm_ctx *ctx) {
         release(RF.Sc7);
         RF.cap_N = RF.cap_leaves = RF.cap_ref = RF.cap_cells = 0;
     }
-    ctx->mx_cap_N = ctx->mx_cap_cells = 0;
+    ctx->mx_cap_cells = 0;
     ctx->cap_N = ctx->cap_segs = ctx->cap_cells = ctx->cap_leaves = 0;
     ctx->built = false;
 }
@@ -75,16 +71,15 @@ static void free_tree(gbfmm_ctx *ctx) {
 static int ensure_tree_buffers(gbfmm_ctx *ctx) {
     const int64_t N = ctx->N, ns = ctx->n_segs, nc = ctx->n_cells, nl = ctx->n_leaves;
     const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
-    const bool fp64 = ctx->opt.precision == GBFMM_FP64;
     const bool w64 = ctx->opt.precision != GBFMM_MIXED;  // FP64 multipole and local values
     {
-        GrowBuf b[12] = {{(void **)&ctx->d_y, N * 3 * sizeof(double)},  {(void **)&ctx->d_q, N * 9 * sizeof(double)},
+        GrowBuf b[11] = {{(void **)&ctx->d_y, N * 3 * sizeof(double)},  {(void **)&ctx->d_q, N * 9 * sizeof(double)},
                          {(void **)&ctx->d_sid, N * sizeof(int64_t)},   {(void **)&ctx->d_slen, N * sizeof(double)},
                          {(void **)&ctx->d_pos, N * sizeof(int)},       {(void **)&ctx->d_pleaf, N * sizeof(int)},
                          {(void **)&ctx->d_sig, N * 6 * sizeof(double)}, {(void **)&ctx->d_y0, N * 3 * sizeof(double)},
                          {(void **)&ctx->d_q0, N * 9 * sizeof(double)}, {(void **)&ctx->d_leaf_of, N * sizeof(int)},
-                         {(void **)&ctx->d_perm, N * sizeof(int)},      {(void **)&ctx->d_P, N * 108 * sizeof(double)}};
-        if (int rc = grow_dev(ctx, ctx->cap_N, N, b, fp64 ? 12 : 11, "points")) return rc;
+                         {(void **)&ctx->d_perm, N * sizeof(int)}};
+        if (int rc = grow_dev(ctx, ctx->cap_N, N, b, 11, "points")) return rc;
     }
     if (int rc = grow_dev(ctx, ctx->cap_segs, ns, {{(void **)&ctx->d_len0, ns * sizeof(double)}}, "segments"))
         return rc;
@@ -208,7 +203,7 @@ extern "C" void fmm_destroy(gbfmm_ctx *ctx) {
         ctx->tc.Thi = ctx->tc.Tlo = nullptr;
     }
     void *ps[] = {ctx->d_box, ctx->d_mat, ctx->d_Asym, ctx->d_Asym_f, ctx->d_Klat,
-                  ctx->d_t_pos, ctx->d_t_x, ctx->d_t_sig, ctx->d_t_tmp};
+                  ctx->d_t_pos, ctx->d_t_leaf, ctx->d_t_x, ctx->d_t_sig, ctx->d_t_tmp};
     for (void *p : ps)
         if (p) cudaFree(p);
     m2l_tc_free(ctx);
@@ -216,8 +211,7 @@ extern "C" void fmm_destroy(gbfmm_ctx *ctx) {
     mlp_free(ctx);
     {
         NearWork &W = ctx->nw;
-        void *ps2[] = {W.items, W.sorted, W.keys, W.cnt, W.key_of, W.off, W.misc, W.pitems, W.psorted, W.pkeys,
-                       W.pmisc, W.part};
+        void *ps2[] = {W.rec, W.trec, W.plan, W.lp, W.pitems, W.rows, W.pcnt};
         for (void *q : ps2)
             if (q) cudaFree(q);
     }
@@ -266,9 +260,7 @@ extern "C" int fmm_build_tree(gbfmm_ctx *ctx, int64_t n_nodes, const double *nod
         rc = mixed_alloc(ctx);
         if (rc) return rc;
     } else {
-        // work list and partial sums of the FP64 symmetric near field (unit-circle h)
-        rc = near_alloc(ctx, ctx->N);
-        if (!rc) rc = near_sym_alloc(ctx);
+        rc = near_alloc(ctx);  // records, work plan and partial sums of the near field
         if (rc) return rc;
     }
     ctx->built = true;
@@ -286,13 +278,13 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     v(c->L), v(c->N), v(c->n_segs), v(c->n_nodes), v(c->n_cells), v(c->n_leaves), v(c->t_cap);
     v(c->node_xyz), v(c->seg_nodes), v(c->burgers), v(c->stream);
     const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Asym_f, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
-                          c->d_slen, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_P,
-                          c->d_Pf, c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_yrel, c->d_t_pos, c->d_t_start,
+                          c->d_slen, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf,
+                          c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_t_pos, c->d_t_start,
                           c->d_t_x, c->d_t_sig, c->tc.Thi, c->tc.Tlo, c->tc.Whi, c->tc.Wlo, c->tc.d_status,
                           c->tc.d_flags, c->tc.d_pos, c->tc.d_list, c->tc.d_seg, c->tc.d_wmax, c->mlp.theta, c->mlp.theta_h,
-                          c->mlp.scale, c->mlp.d_binmask, c->nw.items, c->nw.sorted, c->nw.keys, c->nw.cnt,
-                          c->nw.key_of, c->nw.off, c->nw.misc, c->nw.pitems, c->nw.psorted,
-                          c->nw.pkeys, c->nw.pmisc, c->nw.part, c->tc.Uh, c->tc.Ul, c->tc.Rh, c->tc.Rl,
+                          c->mlp.scale, c->mlp.d_binmask, c->mlp.poly,
+                          c->nw.rec, c->nw.trec, c->nw.plan,
+                          c->nw.lp, c->nw.pitems, c->nw.rows, c->nw.pcnt, c->tc.Uh, c->tc.Ul, c->tc.Rh, c->tc.Rl,
                           c->tc.Xh, c->tc.Xl, c->tc.d_scal, c->tc.d_bits, c->tc.Wc, c->tc.Sc, c->tc.blas_ws,
                           c->rf.child_of, c->rf.ref_start, c->rf.ref_leaf, c->rf.child_start, c->rf.pfine,
                           c->rf.W7, c->rf.S7, c->rf.Wc7, c->rf.Sc7, c->tc.d_pcnt, c->tc.d_pairs, c->tc.Gh,
@@ -300,7 +292,7 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     mix(ptrs, sizeof(ptrs));
     v(c->mat.mode), v(c->mat.Q), v(c->mat.cubic), v(c->tc.n_work), v(c->tc.split), v(c->tc.tf32);
     mix(c->tc.wofs, sizeof(c->tc.wofs));
-    v(c->tc.n_slots), v(c->tc.n_seg), v(c->nw.cap), v(c->nw.cap_leaves), v(c->mlp.trained);
+    v(c->tc.n_slots), v(c->tc.n_seg), v(c->mlp.trained);
     v(c->tc.r1), v(c->tc.r2), v(c->rf.cap_ref), v(c->rf.n_ref_host), v(c->tc.blas);
     return h;
 }

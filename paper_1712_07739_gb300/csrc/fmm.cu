@@ -1,5 +1,4 @@
 // The Lagrange FMM pass (Sec. 4, Algorithm 2), FP64 path:
-//   precontract  P_j[ab][k] = sum_wr Asym[ab][wr][k] q_j[wr]   (per source)
 //   P2M  W_m = sum_{y_j in leaf} L_p(ybar_m, y_j) q_j          (Eq. "far-field", source side)
 //   M2M  W_m' = sum_children sum_m L_p(ybar_m', ybar_m) W_m    (parent basis at the child nodes)
 //   M2L  s(xbar_l) = sum_{A in I(B)} sum_m K(xbar_l - ybar_m) W_m   (Eq. "m2l")
@@ -25,25 +24,6 @@ __device__ __forceinline__ void cell_xyz(int64_t lin, int n, int &x, int &y, int
     x = int(lin % n);
     y = int((lin / n) % n);
     z = int(lin / (int64_t(n) * n));
-}
-
-// ---------------------------------------------------------------- precontract
-template <typename R>
-__global__ void k_precontract(int64_t N, const double *__restrict__ q, const double *__restrict__ Asym,
-                              R *__restrict__ P) {
-    __shared__ double As[6 * 9 * 18];
-    for (int i = threadIdx.x; i < 6 * 9 * 18; i += blockDim.x) As[i] = Asym[i];
-    __syncthreads();
-    int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (j >= N) return;
-    double qq[9];
-    for (int i = 0; i < 9; ++i) qq[i] = q[9 * j + i];
-    for (int ab = 0; ab < 6; ++ab)
-        for (int k = 0; k < 18; ++k) {
-            double s = 0.0;
-            for (int wr = 0; wr < 9; ++wr) s += As[(ab * 9 + wr) * 18 + k] * qq[wr];
-            P[108 * j + ab * 18 + k] = R(s);
-        }
 }
 
 // ---------------------------------------------------------------- occupancy
@@ -498,119 +478,6 @@ __global__ void k_m2l_f64(int p, int L, int lat_n, const TreeBox *__restrict__ b
     }
 }
 
-// ---------------------------------------------------------------- L2P + P2P (FP64)
-// One block per leaf holding targets.  Far part: interpolate the leaf's
-// local values at the target; near part: direct sum over the source points
-// of the 27 neighbouring leaves (Eq. "stress3"), skipping the target's own
-// segment.
-template <int MODE>
-__global__ void k_leaf_eval_f64(int p, int nodes, int L, const TreeBox *__restrict__ box, const DevMaterial *__restrict__ mat,
-                                const int *__restrict__ tstart, const double *__restrict__ xt,
-                                const int64_t *__restrict__ tsid, const int *__restrict__ sstart,
-                                const double *__restrict__ ys, const double *__restrict__ P,
-                                const int64_t *__restrict__ ssid, const double *__restrict__ S,
-                                double *__restrict__ sig) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    double *sm = reinterpret_cast<double *>(sm_raw);
-    constexpr int CH = 64;
-    const int P3 = p * p * p;
-    const int64_t leaf = blockIdx.x;
-    const int t0 = tstart[leaf], t1 = tstart[leaf + 1];
-    if (t0 == t1) return;
-    const int nl = 1 << (L - 1);
-    int cx, cy, cz;
-    cell_xyz(leaf, nl, cx, cy, cz);
-    const bool far = L >= 3;
-    double *sS = sm;                     // [P3][6]
-    double *sy = sm + P3 * 6;            // [CH][3]
-    double *sP = sy + CH * 3;            // [CH][108]
-    int64_t *ssd = (int64_t *)(sP + CH * 108);  // [CH]
-    if (far) {
-        const double *Sl = S + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 6;
-        for (int i = threadIdx.x; i < P3 * 6; i += blockDim.x) sS[i] = Sl[i];
-    }
-    const double h = box->H / nl, ih = double(nl) / box->H;
-    const double c0[3] = {box->origin[0] + cx * h, box->origin[1] + cy * h, box->origin[2] + cz * h};
-    DevMaterial m = *mat;
-    for (int r0 = t0; r0 < t1; r0 += blockDim.x) {
-        const int t = r0 + threadIdx.x;
-        const bool valid = t < t1;
-        double x[3] = {0, 0, 0}, acc[6] = {0, 0, 0, 0, 0, 0};
-        int64_t myseg = -1;
-        __syncthreads();
-        if (valid) {
-            for (int d = 0; d < 3; ++d) x[d] = xt[3 * int64_t(t) + d];
-            myseg = tsid ? tsid[t] : -1;
-            if (far) {
-                double bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP];
-                lagrange_1d<double>(p, (x[0] - c0[0]) * ih, bx, nodes);
-                lagrange_1d<double>(p, (x[1] - c0[1]) * ih, by, nodes);
-                lagrange_1d<double>(p, (x[2] - c0[2]) * ih, bz, nodes);
-                for (int l = 0; l < P3; ++l) {
-                    double w = bx[l % p] * by[(l / p) % p] * bz[l / (p * p)];
-                    for (int ab = 0; ab < 6; ++ab) acc[ab] += w * sS[l * 6 + ab];
-                }
-            }
-        }
-        for (int nb = 0; nb < 27; ++nb) {
-            const int ax = cx + nb % 3 - 1, ay = cy + (nb / 3) % 3 - 1, az = cz + nb / 9 - 1;
-            if (ax < 0 || ay < 0 || az < 0 || ax >= nl || ay >= nl || az >= nl) continue;
-            const int64_t A = (int64_t(az) * nl + ay) * nl + ax;
-            const int s0 = sstart[A], s1 = sstart[A + 1];
-            for (int j0 = s0; j0 < s1; j0 += CH) {
-                const int nj = min(CH, s1 - j0);
-                __syncthreads();
-                for (int i = threadIdx.x; i < nj * 3; i += blockDim.x) sy[i] = ys[3 * int64_t(j0) + i];
-                for (int i = threadIdx.x; i < nj * 108; i += blockDim.x) sP[i] = P[108 * int64_t(j0) + i];
-                for (int i = threadIdx.x; i < nj; i += blockDim.x) ssd[i] = ssid[j0 + i];
-                __syncthreads();
-                if (!valid) continue;
-                for (int j = 0; j < nj; ++j) {
-                    if (ssd[j] == myseg) continue;
-                    double d[3] = {x[0] - sy[3 * j], x[1] - sy[3 * j + 1], x[2] - sy[3 * j + 2]};
-                    double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                    if (r2 == 0.0) continue;
-                    double ir = rsqrt(r2);
-                    double T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
-                    double hs[18];
-                    if (MODE == GBFMM_H_ISO)
-                        h_iso_sym<double>(m.hc, m.ha, T, hs);
-                    else if (m.cubic)
-                        h_circle_cubic<double>(m.c12, m.c44, m.cd, m.Q, T, hs);
-                    else
-                        h_circle_sym<double, double>(mat->C, m.Q, T, hs);
-                    const double ir2 = ir * ir;
-                    const double *Pj = sP + 108 * j;
-                    for (int ab = 0; ab < 6; ++ab) {
-                        double s = 0.0;
-                        for (int k = 0; k < 18; ++k) s += Pj[ab * 18 + k] * hs[k];
-                        acc[ab] += s * ir2;
-                    }
-                }
-            }
-        }
-        if (valid)
-            for (int ab = 0; ab < 6; ++ab) sig[6 * int64_t(t) + ab] = acc[ab];
-    }
-}
-
-// ---------------------------------------------------------------- mixed-precision leaf pass
-// Source points relative to their leaf centre, in FP32, plus the length of
-// their segment: yrel[i] = (y_i - c_leaf(i), |S|).
-__global__ void k_prep_mixed(int64_t N, int L, const TreeBox *__restrict__ box, const double *__restrict__ y,
-                             const int *__restrict__ pleaf, const double *__restrict__ slen,
-                             float4 *__restrict__ yrel) {
-    int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i >= N) return;
-    const int nl = 1 << (L - 1);
-    int cx, cy, cz;
-    cell_xyz(pleaf[i], nl, cx, cy, cz);
-    const double h = box->H / nl;
-    yrel[i] = make_float4(float(y[3 * i] - (box->origin[0] + (cx + 0.5) * h)),
-                          float(y[3 * i + 1] - (box->origin[1] + (cy + 0.5) * h)),
-                          float(y[3 * i + 2] - (box->origin[2] + (cz + 0.5) * h)), float(slen[i]));
-}
-
 // ---------------------------------------------------------------- forces
 struct ForceParams {
     double xi[GB_MAXG], w[GB_MAXG];
@@ -834,22 +701,22 @@ void timer_mark(gbfmm_ctx *ctx) {
     cudaEventRecord(ctx->timer.ev[ctx->timer.n++], ctx->stream);
 }
 
-int near_run_sym64(gbfmm_ctx *ctx, double *sig);  // near.cu
+int near_prepare(gbfmm_ctx *ctx);                                             // near.cu
+int near_alloc(gbfmm_ctx *ctx);                                               // near.cu
+int near_run(gbfmm_ctx *ctx, bool free_targets, int64_t n_t, double *sig);   // near.cu
 
 // Runs the pass.  free_targets: targets are the sorted free points of
 // targets_sort (no segment exclusion), else the sorted Gauss points.
 int fmm_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     cudaStream_t st = ctx->stream;
     const int p = ctx->opt.p, L = ctx->L, P3 = p * p * p;
-    const int64_t N = ctx->N, nl = ctx->n_leaves;
+    const int64_t nl = ctx->n_leaves;
     int *occ = ctx->d_tmp_i;                 // [n_cells] sources per cell
     int *tocc = free_targets ? occ + ctx->n_cells : occ;
-    const int *tstart = free_targets ? ctx->d_t_start : ctx->d_leaf_start;
     Transfer tr = make_transfer(p, ctx->opt.nodes);
 
     timer_mark(ctx);
-    ++ctx->launches;
-    k_precontract<double><<<nblk(N, 128), 128, 0, st>>>(N, ctx->d_q, ctx->d_Asym, ctx->d_P);
+    if (int rc = near_prepare(ctx)) return rc;
     compute_occ(ctx, ctx->d_leaf_start, occ);
     if (free_targets) compute_occ(ctx, ctx->d_t_start, tocc);
     CK(cudaGetLastError());
@@ -883,27 +750,8 @@ int fmm_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
         CK(cudaGetLastError());
     }
     timer_mark(ctx);
-    if (!free_targets && ctx->mat.mode == GBFMM_H_CIRCLE) {
-        // nodal forces with the unit-circle h: one h per unordered point pair (h is odd)
-        if (int rc = near_run_sym64(ctx, ctx->d_sig)) return rc;
-    } else {
-        const size_t smem = (size_t(P3) * 6 + 64 * 3 + 64 * 108) * sizeof(double) + 64 * sizeof(int64_t);
-        const double *xt = free_targets ? ctx->d_t_x : ctx->d_y;
-        const int64_t *tsid = free_targets ? nullptr : ctx->d_sid;
-        double *sig = free_targets ? ctx->d_t_sig : ctx->d_sig;
-        ++ctx->launches;
-        if (ctx->mat.mode == GBFMM_H_ISO)
-            k_leaf_eval_f64<GBFMM_H_ISO><<<unsigned(nl), 128, smem, st>>>(
-                p, ctx->opt.nodes, L, ctx->d_box, ctx->d_mat, tstart, xt, tsid, ctx->d_leaf_start, ctx->d_y, ctx->d_P, ctx->d_sid,
-                ctx->d_S, sig);
-        else
-            k_leaf_eval_f64<GBFMM_H_CIRCLE><<<unsigned(nl), 128, smem, st>>>(
-                p, ctx->opt.nodes, L, ctx->d_box, ctx->d_mat, tstart, xt, tsid, ctx->d_leaf_start, ctx->d_y, ctx->d_P, ctx->d_sid,
-                ctx->d_S, sig);
-        CK(cudaGetLastError());
-    }
+    if (int rc = near_run(ctx, free_targets, n_t, free_targets ? ctx->d_t_sig : ctx->d_sig)) return rc;
     timer_mark(ctx);
-    (void)n_t;
     return GBFMM_OK;
 }
 
@@ -936,45 +784,26 @@ int mixed_kernel_attrs(gbfmm_ctx *ctx);
 int fmm_kernel_attrs(gbfmm_ctx *ctx) {
     if (int rc = mixed_kernel_attrs(ctx)) return rc;
     const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
-    const size_t smem = (size_t(P3) * 6 + 64 * 3 + 64 * 108) * sizeof(double) + 64 * sizeof(int64_t);
-    CK(cudaFuncSetAttribute(k_leaf_eval_f64<GBFMM_H_ISO>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    CK(cudaFuncSetAttribute(k_leaf_eval_f64<GBFMM_H_CIRCLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     CK(cudaFuncSetAttribute(k_m2m<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(2 * P3 * 9 * sizeof(double))));
     CK(cudaFuncSetAttribute(k_l2l<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(2 * P3 * 6 * sizeof(double))));
     CK(cudaFuncSetAttribute(k_m2l_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, int(P3 * 9 * sizeof(double))));
     return GBFMM_OK;
 }
 
-int near_prepare(gbfmm_ctx *ctx);  // near.cu
-int near_alloc(gbfmm_ctx *ctx, int64_t n_targets);  // near.cu
-int near_sym_alloc(gbfmm_ctx *ctx);                 // near.cu
-int near_run(gbfmm_ctx *ctx, const int *tstart, const double *xt, const int64_t *tsid, double *sig);
-
 int mixed_alloc(gbfmm_ctx *ctx) {
-    const int64_t N = ctx->N, nc = ctx->n_cells;
+    const int64_t nc = ctx->n_cells;
     const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
-    if (int rc = grow_dev(ctx, ctx->mx_cap_N, N,
-                          {{(void **)&ctx->d_Pf, N * 108 * sizeof(float)}, {(void **)&ctx->d_yrel, N * sizeof(float4)}},
-                          "mixed-pass points"))
-        return rc;
     if (int rc = grow_dev(ctx, ctx->mx_cap_cells, nc,
                           {{(void **)&ctx->d_Wf, nc * P3 * 9 * sizeof(float)},
                            {(void **)&ctx->d_Sf, nc * P3 * 6 * sizeof(float)}},
                           "mixed-pass cells"))
         return rc;
-    if (int rc = near_alloc(ctx, N)) return rc;
-    if (int rc = near_sym_alloc(ctx)) return rc;
+    if (int rc = near_alloc(ctx)) return rc;
     if (!ctx->tc.ready_ops) {
         int rc = m2l_tc_setup(ctx);
         if (rc) return rc;
     }
     return m2l_tc_prepare(ctx);
-}
-
-// leaf-level local values FP64 -> FP32 (GBFMM_MIXED_F64T, for the near kernels that read FP32)
-__global__ void k_leaf_s_to_f32(int64_t n, const double *__restrict__ S, float *__restrict__ Sf) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-        Sf[i] = float(S[i]);
 }
 
 int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
@@ -985,10 +814,9 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     cudaStream_t st = ctx->stream;
     const bool t64 = ctx->opt.precision == GBFMM_MIXED_F64T;  // FP64 P2M, M2M, L2L, L2P
     const int p = ctx->opt.p, L = ctx->L, P3 = p * p * p;
-    const int64_t N = ctx->N, nl = ctx->n_leaves;
+    const int64_t nl = ctx->n_leaves;
     int *occ = ctx->d_tmp_i;
     int *tocc = free_targets ? occ + ctx->n_cells : occ;
-    const int *tstart = free_targets ? ctx->d_t_start : ctx->d_leaf_start;
     Transfer tr = make_transfer(p, ctx->opt.nodes);
     // adaptive tree: the children of split leaves take part in nodal-force passes (free
     // targets keep the uniform tree, whose near field covers whole leaves)
@@ -998,8 +826,6 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     const int *n_ref = RF.ref_start ? RF.ref_start + nl : nullptr;
     timer_mark(ctx);
     if (int rc = near_prepare(ctx)) return rc;
-    ++ctx->launches;
-    k_prep_mixed<<<nblk(N, 256), 256, 0, st>>>(N, L, ctx->d_box, ctx->d_y, ctx->d_pleaf, ctx->d_slen, ctx->d_yrel);
     compute_occ(ctx, ctx->d_leaf_start, occ);
     if (free_targets) compute_occ(ctx, ctx->d_t_start, tocc);
     CK(cudaGetLastError());
@@ -1054,22 +880,9 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
             p, L, tr, n_ref, RF.ref_leaf, RF.child_start, ctx->d_Sf, RF.S7);
         CK(cudaGetLastError());
     }
-    if (t64 && L >= 3) {
-        // FP32 copy of the leaf level for the near kernels that read FP32 local values
-        const int64_t n = nl * P3 * 6;
-        ++ctx->launches;
-        k_leaf_s_to_f32<<<unsigned(std::min<int64_t>((n + 255) / 256, 4096)), 256, 0, st>>>(
-            n, ctx->d_S + cell_base(L - 1) * P3 * 6, ctx->d_Sf + cell_base(L - 1) * P3 * 6);
-    }
     timer_mark(ctx);
-    {
-        const double *xt = free_targets ? ctx->d_t_x : ctx->d_y;
-        const int64_t *tsid = free_targets ? nullptr : ctx->d_sid;
-        double *sig = free_targets ? ctx->d_t_sig : ctx->d_sig;
-        if (int rc = near_run(ctx, tstart, xt, tsid, sig)) return rc;
-    }
+    if (int rc = near_run(ctx, free_targets, n_t, free_targets ? ctx->d_t_sig : ctx->d_sig)) return rc;
     timer_mark(ctx);
-    (void)n_t;
     return GBFMM_OK;
 }
 

@@ -27,6 +27,7 @@ struct DevMaterial {
     double hc;    // iso: 1 / (16 pi mu (1 - nu))
     double ha;    // iso: 3 - 4 nu
     double C[81]; // C_ijkl
+    double V[36]; // the Voigt stiffness it came from
     int cubic;    // 1: cubic with axes along x, y, z (c12, c44, cd below are set)
     double c12, c44, cd;  // C12, C44, C11 - C12 - 2 C44
 };
@@ -47,22 +48,22 @@ struct MlpState {
     float *loss = nullptr;
     void *bufs = nullptr;              // batch activations
     uint32_t *d_binmask = nullptr;     // [48] angular bins where the plain evaluator is used
+    float *poly = nullptr;             // [1280][108] the network as polynomials, one per angular bin (near field)
+    bool poly_ok = false;              // poly belongs to the current network
     double fallback_frac = 1.0;        // fraction of bins flagged by the last calibration
     bool trained = false;
     int64_t step = 0;
 };
 
-// work list of the near kernels (near.cu)
+// buffers of the near field (near.cu)
 struct NearWork {
-    int2 *items = nullptr, *sorted = nullptr;
-    int *keys = nullptr, *cnt = nullptr, *key_of = nullptr, *off = nullptr, *misc = nullptr;
-    int64_t cap = 0, cap_leaves = 0;
-    // symmetric near field (nodal forces, unit-circle h): leaf-pair items and
-    // per-direction partial stresses [28][N][6]
-    int2 *pitems = nullptr, *psorted = nullptr;
-    int *pkeys = nullptr, *pmisc = nullptr;
-    double *part = nullptr;
-    int64_t pcap = 0, part_cap = 0;
+    // point records of the sources and of free targets, per-leaf plan and list
+    // offsets, items, counters, and the rows of partial sums
+    void *rec = nullptr, *trec = nullptr, *plan = nullptr, *pitems = nullptr;
+    int *lp = nullptr;
+    unsigned long long *pcnt = nullptr;
+    double *rows = nullptr;
+    int64_t rec_cap = 0, trec_cap = 0, plan_cap = 0, item_cap = 0, row_cap = 0;
 };
 
 struct Timer {
@@ -146,21 +147,19 @@ struct gbfmm_ctx {
     } rf;
 
     // per-eval buffers
-    double *d_P = nullptr;     // [N][108] precontracted source tensors (FP64)
-    float *d_Pf = nullptr;     // [N][108] FP32 copy for the mixed path
     double *d_W = nullptr;     // [n_cells][p^3][9] multipole weights
     double *d_S = nullptr;     // [n_cells][p^3][6] local values
     float *d_Wf = nullptr;
     float *d_Sf = nullptr;
     double *d_sig = nullptr;   // [N][6] stress at sorted points
-    float4 *d_yrel = nullptr;  // [N] mixed: leaf-relative FP32 position, segment length
-    int64_t mx_cap_N = 0, mx_cap_cells = 0;
+    int64_t mx_cap_cells = 0;
 
     // free-target evaluation
     int64_t t_cap = 0;                 // targets the buffers below hold (0 after a failed allocation)
     int64_t t_cap_leaves = 0;          // leaves the target scratch was sized for
     int *d_t_pos = nullptr;     // target -> sorted slot
     int *d_t_start = nullptr;   // [n_leaves + 1]
+    int *d_t_leaf = nullptr;    // their leaves
     double *d_t_x = nullptr;    // sorted targets
     double *d_t_sig = nullptr;  // sorted results
     int *d_t_tmp = nullptr;

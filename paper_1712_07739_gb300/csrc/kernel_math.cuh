@@ -187,230 +187,9 @@ __device__ __forceinline__ void h_circle_cubic(R c12, R c44, R D, int Q, const R
     for (int i = 0; i < 18; ++i) hs[i] = acc[i] * f;
 }
 
-// FP32 form of h_circle_cubic for the near-field loop: scalar registers only,
-// the points (cos, sin)(pi k / Q) of the half circle from a table.
-__device__ __forceinline__ void h_cubic_f32(float cp, float c44, float D, int Q, const float2 *__restrict__ tab,
-                                            const float T[3], float hs[18]) {
-    const float T0 = T[0], T1 = T[1], T2 = T[2];
-    int k0 = 0;
-    if (fabsf(T1) < fabsf(T0)) k0 = 1;
-    if (fabsf(T2) < fabsf(k0 == 0 ? T0 : T1)) k0 = 2;
-    float a0 = k0 == 0 ? 1.f : 0.f, a1 = k0 == 1 ? 1.f : 0.f, a2 = k0 == 2 ? 1.f : 0.f;
-    const float dd = a0 * T0 + a1 * T1 + a2 * T2;
-    a0 -= dd * T0;
-    a1 -= dd * T1;
-    a2 -= dd * T2;
-    const float nr = rsqrtf(a0 * a0 + a1 * a1 + a2 * a2);
-    const float e10 = a0 * nr, e11 = a1 * nr, e12 = a2 * nr;
-    const float e20 = T1 * e12 - T2 * e11, e21 = T2 * e10 - T0 * e12, e22 = T0 * e11 - T1 * e10;
-    const float cpD = cp + D, cpD2 = 2.f * (cp + D);
-    // With C = adj(zz), (zz)^-1 = C / det and F = C S C / det^2, so the point's
-    // factors fold into z (z / det^2) and the (zz)^-1 sum (C / det); the
-    // T-term of the integrand is summed over the points first,
-    // sum_k T_q (zz)^-1_vp = T_q sum_k (zz)^-1_vp.
-    float acc[18], msum[6];
-#pragma unroll
-    for (int i = 0; i < 18; ++i) acc[i] = 0.f;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) msum[i] = 0.f;
-    for (int k = 0; k < Q; ++k) {
-        const float2 t = tab[k];
-        const float z0 = t.x * e10 + t.y * e20, z1 = t.x * e11 + t.y * e21, z2 = t.x * e12 + t.y * e22;
-        const float m00 = fmaf(cpD, z0 * z0, c44), m11 = fmaf(cpD, z1 * z1, c44), m22 = fmaf(cpD, z2 * z2, c44);
-        const float m01 = cp * z0 * z1, m02 = cp * z0 * z2, m12 = cp * z1 * z2;
-        const float i00 = m11 * m22 - m12 * m12, i01 = m02 * m12 - m01 * m22, i02 = m01 * m12 - m02 * m11;
-        const float i11 = m00 * m22 - m02 * m02, i12 = m01 * m02 - m00 * m12, i22 = m00 * m11 - m01 * m01;
-        float idet;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(idet) : "f"(m00 * i00 + m01 * i01 + m02 * i02));
-        const float s00 = cpD2 * z0 * T0, s11 = cpD2 * z1 * T1, s22 = cpD2 * z2 * T2;
-        const float s01 = cp * (z0 * T1 + z1 * T0), s02 = cp * (z0 * T2 + z2 * T0), s12 = cp * (z1 * T2 + z2 * T1);
-        // U = C S, F = U C (symmetric), both without the 1 / det factors
-        const float u00 = i00 * s00 + i01 * s01 + i02 * s02, u01 = i00 * s01 + i01 * s11 + i02 * s12,
-                    u02 = i00 * s02 + i01 * s12 + i02 * s22;
-        const float u10 = i01 * s00 + i11 * s01 + i12 * s02, u11 = i01 * s01 + i11 * s11 + i12 * s12,
-                    u12 = i01 * s02 + i11 * s12 + i12 * s22;
-        const float u20 = i02 * s00 + i12 * s01 + i22 * s02, u21 = i02 * s01 + i12 * s11 + i22 * s12,
-                    u22 = i02 * s02 + i12 * s12 + i22 * s22;
-        const float F00 = u00 * i00 + u01 * i01 + u02 * i02, F01 = u00 * i01 + u01 * i11 + u02 * i12,
-                    F02 = u00 * i02 + u01 * i12 + u02 * i22;
-        const float F11 = u10 * i01 + u11 * i11 + u12 * i12, F12 = u10 * i02 + u11 * i12 + u12 * i22,
-                    F22 = u20 * i02 + u21 * i12 + u22 * i22;
-        const float w = idet * idet;
-        const float y0 = z0 * w, y1 = z1 * w, y2 = z2 * w;
-        // pairs (00) (11) (22) (12) (02) (01), each with q = 0, 1, 2
-        const float Mp[6] = {i00, i11, i22, i12, i02, i01};
-        const float Fp[6] = {F00, F11, F22, F12, F02, F01};
-#pragma unroll
-        for (int pr = 0; pr < 6; ++pr) {
-            acc[3 * pr + 0] = fmaf(y0, Fp[pr], acc[3 * pr + 0]);
-            acc[3 * pr + 1] = fmaf(y1, Fp[pr], acc[3 * pr + 1]);
-            acc[3 * pr + 2] = fmaf(y2, Fp[pr], acc[3 * pr + 2]);
-            msum[pr] = fmaf(Mp[pr], idet, msum[pr]);
-        }
-    }
-    const float f = 1.f / (4.f * 3.14159265358979f * float(Q));
-#pragma unroll
-    for (int pr = 0; pr < 6; ++pr) {
-        hs[3 * pr + 0] = (acc[3 * pr + 0] - T0 * msum[pr]) * f;
-        hs[3 * pr + 1] = (acc[3 * pr + 1] - T1 * msum[pr]) * f;
-        hs[3 * pr + 2] = (acc[3 * pr + 2] - T2 * msum[pr]) * f;
-    }
-}
-
-// Same rule with two circle points per step in packed FP32x2 arithmetic
-// (one instruction for the two points' products); Q even.
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+// packed FP32x2 arithmetic (one instruction for two values)
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-// a b - c d
-__device__ __forceinline__ float2 fms2(float2 a, float2 b, float2 c, float2 d) { return fma2(a, b, mul2(neg2(c), d)); }
-
-__device__ __forceinline__ void h_cubic_f32x2(float cp, float c44, float D, int Q, const float4 *__restrict__ tab2,
-                                              const float T[3], float hs[18]) {
-    const float T0 = T[0], T1 = T[1], T2 = T[2];
-    int k0 = 0;
-    if (fabsf(T1) < fabsf(T0)) k0 = 1;
-    if (fabsf(T2) < fabsf(k0 == 0 ? T0 : T1)) k0 = 2;
-    float a0 = k0 == 0 ? 1.f : 0.f, a1 = k0 == 1 ? 1.f : 0.f, a2 = k0 == 2 ? 1.f : 0.f;
-    const float dd = a0 * T0 + a1 * T1 + a2 * T2;
-    a0 -= dd * T0;
-    a1 -= dd * T1;
-    a2 -= dd * T2;
-    const float nr = rsqrtf(a0 * a0 + a1 * a1 + a2 * a2);
-    const float e10 = a0 * nr, e11 = a1 * nr, e12 = a2 * nr;
-    const float e20 = T1 * e12 - T2 * e11, e21 = T2 * e10 - T0 * e12, e22 = T0 * e11 - T1 * e10;
-    const float2 cpD = f2(cp + D), cp2 = f2(cp), c442 = f2(c44);
-    // zT products folded with their constants: s_ii = z_i (2 (cp + D) T_i), s_ij = z_i (cp T_j) + z_j (cp T_i)
-    const float2 dT0 = f2(2.f * (cp + D) * T0), dT1 = f2(2.f * (cp + D) * T1), dT2 = f2(2.f * (cp + D) * T2);
-    const float2 cT0 = f2(cp * T0), cT1 = f2(cp * T1), cT2 = f2(cp * T2);
-    float2 acc[18], msum[6];
-#pragma unroll
-    for (int i = 0; i < 18; ++i) acc[i] = f2(0.f);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) msum[i] = f2(0.f);
-    for (int k = 0; k < Q / 2; ++k) {
-        const float4 t = tab2[k];  // (cos, sin) of points 2k and 2k + 1
-        const float2 c = make_float2(t.x, t.z), sn = make_float2(t.y, t.w);
-        const float2 z0 = fma2(c, f2(e10), mul2(sn, f2(e20)));
-        const float2 z1 = fma2(c, f2(e11), mul2(sn, f2(e21)));
-        const float2 z2 = fma2(c, f2(e12), mul2(sn, f2(e22)));
-        const float2 m00 = fma2(cpD, mul2(z0, z0), c442), m11 = fma2(cpD, mul2(z1, z1), c442),
-                     m22 = fma2(cpD, mul2(z2, z2), c442);
-        const float2 cz0 = mul2(cp2, z0), cz1 = mul2(cp2, z1);
-        const float2 m01 = mul2(cz0, z1), m02 = mul2(cz0, z2), m12 = mul2(cz1, z2);
-        const float2 i00 = fms2(m11, m22, m12, m12), i01 = fms2(m02, m12, m01, m22), i02 = fms2(m01, m12, m02, m11);
-        const float2 i11 = fms2(m00, m22, m02, m02), i12 = fms2(m01, m02, m00, m12), i22 = fms2(m00, m11, m01, m01);
-        const float2 det = fma2(m00, i00, fma2(m01, i01, mul2(m02, i02)));
-        float2 idet;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(idet.x) : "f"(det.x));
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(idet.y) : "f"(det.y));
-        const float2 s00 = mul2(z0, dT0), s11 = mul2(z1, dT1), s22 = mul2(z2, dT2);
-        const float2 s01 = fma2(z0, cT1, mul2(z1, cT0)), s02 = fma2(z0, cT2, mul2(z2, cT0)),
-                     s12 = fma2(z1, cT2, mul2(z2, cT1));
-        // U = C S, F = U C (symmetric), without the 1 / det factors
-        const float2 u00 = fma2(i00, s00, fma2(i01, s01, mul2(i02, s02)));
-        const float2 u01 = fma2(i00, s01, fma2(i01, s11, mul2(i02, s12)));
-        const float2 u02 = fma2(i00, s02, fma2(i01, s12, mul2(i02, s22)));
-        const float2 u10 = fma2(i01, s00, fma2(i11, s01, mul2(i12, s02)));
-        const float2 u11 = fma2(i01, s01, fma2(i11, s11, mul2(i12, s12)));
-        const float2 u12 = fma2(i01, s02, fma2(i11, s12, mul2(i12, s22)));
-        const float2 u20 = fma2(i02, s00, fma2(i12, s01, mul2(i22, s02)));
-        const float2 u21 = fma2(i02, s01, fma2(i12, s11, mul2(i22, s12)));
-        const float2 u22 = fma2(i02, s02, fma2(i12, s12, mul2(i22, s22)));
-        const float2 F00 = fma2(u00, i00, fma2(u01, i01, mul2(u02, i02)));
-        const float2 F01 = fma2(u00, i01, fma2(u01, i11, mul2(u02, i12)));
-        const float2 F02 = fma2(u00, i02, fma2(u01, i12, mul2(u02, i22)));
-        const float2 F11 = fma2(u10, i01, fma2(u11, i11, mul2(u12, i12)));
-        const float2 F12 = fma2(u10, i02, fma2(u11, i12, mul2(u12, i22)));
-        const float2 F22 = fma2(u20, i02, fma2(u21, i12, mul2(u22, i22)));
-        const float2 w = mul2(idet, idet);
-        const float2 y0 = mul2(z0, w), y1 = mul2(z1, w), y2 = mul2(z2, w);
-        const float2 Mp[6] = {i00, i11, i22, i12, i02, i01};
-        const float2 Fp[6] = {F00, F11, F22, F12, F02, F01};
-#pragma unroll
-        for (int pr = 0; pr < 6; ++pr) {
-            acc[3 * pr + 0] = fma2(y0, Fp[pr], acc[3 * pr + 0]);
-            acc[3 * pr + 1] = fma2(y1, Fp[pr], acc[3 * pr + 1]);
-            acc[3 * pr + 2] = fma2(y2, Fp[pr], acc[3 * pr + 2]);
-            msum[pr] = fma2(Mp[pr], idet, msum[pr]);
-        }
-    }
-    const float f = 1.f / (4.f * 3.14159265358979f * float(Q));
-#pragma unroll
-    for (int pr = 0; pr < 6; ++pr) {
-        const float ms = msum[pr].x + msum[pr].y;
-        hs[3 * pr + 0] = (acc[3 * pr + 0].x + acc[3 * pr + 0].y - T0 * ms) * f;
-        hs[3 * pr + 1] = (acc[3 * pr + 1].x + acc[3 * pr + 1].y - T1 * ms) * f;
-        hs[3 * pr + 2] = (acc[3 * pr + 2].x + acc[3 * pr + 2].y - T2 * ms) * f;
-    }
-}
-
-// The cubic rule of h_cubic_f32 in any precision (the FP64 pass's symmetric
-// near field): points from a table, the adjugate C of (zz) with
-// (zz)^-1 = C / det and F = C S C / det^2, so each point costs one reciprocal.
-template <typename R>
-__device__ __forceinline__ void h_cubic_tab(R cp, R c44, R D, int Q, const R *__restrict__ tab_c,
-                                            const R *__restrict__ tab_s, const R T[3], R hs[18]) {
-    const R T0 = T[0], T1 = T[1], T2 = T[2];
-    int k0 = 0;
-    if (fabs(T1) < fabs(T0)) k0 = 1;
-    if (fabs(T2) < fabs(k0 == 0 ? T0 : T1)) k0 = 2;
-    R a0 = k0 == 0 ? R(1) : R(0), a1 = k0 == 1 ? R(1) : R(0), a2 = k0 == 2 ? R(1) : R(0);
-    const R dd = a0 * T0 + a1 * T1 + a2 * T2;
-    a0 -= dd * T0;
-    a1 -= dd * T1;
-    a2 -= dd * T2;
-    const R nr = R(1) / sqrt(a0 * a0 + a1 * a1 + a2 * a2);
-    const R e10 = a0 * nr, e11 = a1 * nr, e12 = a2 * nr;
-    const R e20 = T1 * e12 - T2 * e11, e21 = T2 * e10 - T0 * e12, e22 = T0 * e11 - T1 * e10;
-    const R cpD = cp + D, cpD2 = R(2) * (cp + D);
-    R acc[18], msum[6];
-#pragma unroll
-    for (int i = 0; i < 18; ++i) acc[i] = R(0);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) msum[i] = R(0);
-    for (int k = 0; k < Q; ++k) {
-        const R c = tab_c[k], sn = tab_s[k];
-        const R z0 = c * e10 + sn * e20, z1 = c * e11 + sn * e21, z2 = c * e12 + sn * e22;
-        const R m00 = cpD * z0 * z0 + c44, m11 = cpD * z1 * z1 + c44, m22 = cpD * z2 * z2 + c44;
-        const R m01 = cp * z0 * z1, m02 = cp * z0 * z2, m12 = cp * z1 * z2;
-        const R i00 = m11 * m22 - m12 * m12, i01 = m02 * m12 - m01 * m22, i02 = m01 * m12 - m02 * m11;
-        const R i11 = m00 * m22 - m02 * m02, i12 = m01 * m02 - m00 * m12, i22 = m00 * m11 - m01 * m01;
-        const R idet = R(1) / (m00 * i00 + m01 * i01 + m02 * i02);
-        const R s00 = cpD2 * z0 * T0, s11 = cpD2 * z1 * T1, s22 = cpD2 * z2 * T2;
-        const R s01 = cp * (z0 * T1 + z1 * T0), s02 = cp * (z0 * T2 + z2 * T0), s12 = cp * (z1 * T2 + z2 * T1);
-        const R u00 = i00 * s00 + i01 * s01 + i02 * s02, u01 = i00 * s01 + i01 * s11 + i02 * s12,
-                u02 = i00 * s02 + i01 * s12 + i02 * s22;
-        const R u10 = i01 * s00 + i11 * s01 + i12 * s02, u11 = i01 * s01 + i11 * s11 + i12 * s12,
-                u12 = i01 * s02 + i11 * s12 + i12 * s22;
-        const R u20 = i02 * s00 + i12 * s01 + i22 * s02, u21 = i02 * s01 + i12 * s11 + i22 * s12,
-                u22 = i02 * s02 + i12 * s12 + i22 * s22;
-        const R F00 = u00 * i00 + u01 * i01 + u02 * i02, F01 = u00 * i01 + u01 * i11 + u02 * i12,
-                F02 = u00 * i02 + u01 * i12 + u02 * i22;
-        const R F11 = u10 * i01 + u11 * i11 + u12 * i12, F12 = u10 * i02 + u11 * i12 + u12 * i22,
-                F22 = u20 * i02 + u21 * i12 + u22 * i22;
-        const R w = idet * idet;
-        const R y0 = z0 * w, y1 = z1 * w, y2 = z2 * w;
-        const R Mp[6] = {i00, i11, i22, i12, i02, i01};
-        const R Fp[6] = {F00, F11, F22, F12, F02, F01};
-#pragma unroll
-        for (int pr = 0; pr < 6; ++pr) {
-            acc[3 * pr + 0] += y0 * Fp[pr];
-            acc[3 * pr + 1] += y1 * Fp[pr];
-            acc[3 * pr + 2] += y2 * Fp[pr];
-            msum[pr] += Mp[pr] * idet;
-        }
-    }
-    const R f = R(1.0 / (4.0 * 3.14159265358979323846 * double(Q)));
-#pragma unroll
-    for (int pr = 0; pr < 6; ++pr) {
-        hs[3 * pr + 0] = (acc[3 * pr + 0] - T0 * msum[pr]) * f;
-        hs[3 * pr + 1] = (acc[3 * pr + 1] - T1 * msum[pr]) * f;
-        hs[3 * pr + 2] = (acc[3 * pr + 2] - T2 * msum[pr]) * f;
-    }
-}
 
 // Lagrange basis ell_a(t) = prod_{b != a} (t - t_b) / (t_a - t_b) on the p
 // nodes of [0, 1]: nodes = GBFMM_NODES_EQUISPACED, t_a = a / (p - 1) (Sec. 4.1

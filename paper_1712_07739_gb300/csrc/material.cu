@@ -219,6 +219,7 @@ extern "C" int fmm_set_material(gbfmm_ctx *ctx, const double *V) {
     if (!positive_definite(V)) return set_err(ctx, GBFMM_ERR_DEGENERATE, "fmm_set_material: stiffness not positive definite");
     DevMaterial m{};
     voigt_to_full(V, m.C);
+    std::memcpy(m.V, V, sizeof(m.V));
     {
         // cubic with axes along x, y, z: C11 = C22 = C33, C12 = C13 = C23, C44 = C55 = C66, rest 0
         const double c11 = V[0], c12 = V[1], c44 = V[21];

@@ -1,30 +1,47 @@
-// Near field (the direct sum over neighbouring leaves in Algorithm 2) and L2P of the mixed-
-// precision pass: one warp per target leaf.
+// Near field of Algorithm 2 (the direct sum over neighbouring leaves) and L2P.
 //
-// For a source point j the kernel contraction of Sec. 2 Eq. "stress3",
-// s_ab += sum_wr K_abwr(x - y_j) q_j,wr, is folded once per source into
-// P_j[ab][k] = sum_wr Asym[ab][wr][k] q_j,wr, so a pair costs
-// s_ab += sum_k P_j[ab][k] h_k(T) / R^2 (k over the 18 distinct h
-// components).  Since q_j = (omega_g / 2) b (x S), P_j is the segment's
-// tensor scaled by the point's Gauss weight.
+// Nodal forces (targets = sources): h is odd, so one h serves both directions of a point
+// pair.  The sources of a leaf A are the points of the 14 leaves A + o, o in the upper half
+// of the 3 x 3 x 3 neighbourhood (A itself first), as one list; a pair (target i of A, list
+// entry j) with j > i adds to the strain at i and, with the sign reversed, to the one at j.
+// Free targets meet the list of all 27 leaves in one direction.
 //
-// Isotropic medium: h is the odd cubic polynomial of Sec. 2 Eq. "k_iso"
-// differentiated, h_vpq = c [-a d_vp T_q + d_vq T_p + d_pq T_v - 3 T_v T_p T_q],
-// so sum_k P[ab][k] h_k(T) / R^2 = (lin_ab . d) / R^3 + (cub_ab . d^(3)) / R^5
-// with d = x - y, 3 linear and 10 cubic-monomial coefficients per ab
-// (78 per source, an exact rewrite).  Other media keep the 108 entries of P
-// and evaluate h by the unit-circle rule in FP32.
+// Work items are (leaf, target tile, list section).  A warp takes one item at a time: 32
+// list entries are staged in shared memory, the item's targets go in chunks of tg lanes (a
+// power of two), and lane (ti, tj) meets the tg entries of group tj one after the other in an
+// order rotated by ti, so the 32 lanes of a step hold 32 different entries and add the
+// reverse sums to shared memory without exchanging anything.  A list of all 14 leaves keeps
+// the steps full where single leaf pairs would not (a leaf of the 1,000,000-segment walls
+// holds 34 points on average); the tiles are cut so that no warp gets more than a bounded
+// number of pairs, since clustered networks put a thousand points in one leaf (with one warp
+// per leaf pair a 3,001-segment network took 560 ms in FP64 for 4 ms of arithmetic).
 //
-// Precision: positions enter as FP32 offsets from their own leaf centre, so
-// a separation carries the rounding of leaf-sized numbers, not of the box
-// size; pairs closer than near_fp64 x (source segment length) take their
-// separation from the FP64 positions and are summed apart in extended
-// precision (FP64 in the one-sided kernels, two-float in the symmetric one).
+// The learned h (GBFMM_H_MLP) runs in the same kernel: pairs whose direction lies in an angular
+// bin the calibration accepted, and farther apart than mlp_min_dist segment lengths, take the
+// network in its tabulated form, the others the plain rule.  Pairs are queued by kind and
+// worked off 32 at a time, since lanes of mixed kinds would pay for both.
+//
+// Sums: an item writes one row of six doubles (strain) for every target and, in the
+// symmetric form, for every list entry of its section; k_near_combine adds a point's rows in
+// a fixed order, applies the stiffness and adds the far field (L2P).  Nothing depends on which
+// warp takes which item or on where the rows lie, so results repeat exactly.
+//
+// Bound: instruction issue and the FMA pipe (250,000-segment walls, cubic, Q = 16: issue slots 75 %
+// and FMA pipe 66 % busy, ~1,170 warp instructions per 32 pairs for both directions, DRAM 27
+// GB/s).  Time of the near field with L2P, one h by the pointwise rule, 108-entry source tensors and
+// one warp per leaf pair before: those walls 43 -> 21 ps a pair; 50,003 segments of loops
+// (Q = 32) 35.1 -> 9.9 ms; 6,101 segments in a turned crystal ~120 -> 5 ms; FP64, 3,001 segments
+// 620 -> 9 ms; 2,000 isotropic segments 125 -> 5 ms.
+//
+// Precision of the FP32 form: positions are FP32 pairs (value + remainder) relative to the
+// leaf centre, so every separation is correct to its own rounding, also of close pairs; h and
+// the contraction run in FP32; every sum over pairs is a two-float sum (~48 bits).
+#include <algorithm>
 #include <cmath>
 
 #include "internal.cuh"
 #include "kernel_math.cuh"
-#include "mlp_warp.cuh"
+#include "unit_circle.cuh"
 
 namespace {
 
@@ -36,311 +53,252 @@ __device__ __forceinline__ void cell_xyz3(int64_t lin, int n, int &x, int &y, in
     z = int(lin / (int64_t(n) * n));
 }
 
-// cubic monomials d_i d_j d_k, i <= j <= k
-__host__ __device__ constexpr int mono_index(int i, int j, int k) {
-    // sorted triple -> 0..9 in the order 000 001 002 011 012 022 111 112 122 222
-    return (i == 0) ? ((j == 0) ? k : (j == 1 ? 2 + k : 5)) : ((i == 1) ? (j == 1 ? 5 + k : 8) : 9);
-}
+// h models of the near kernels: closed form; moment form of a cubic medium; any medium, point by
+// point (FP32) or in moment form (FP64, and FP32 beside the learned h, whose error covers its rounding)
+constexpr int HM_ISO = 0, HM_CUBIC = 1, HM_POINTS = 2, HM_GENERAL = 3;
 
-template <typename R>
-__device__ __forceinline__ void monomials(const R d[3], R m[10]) {
-    const R a00 = d[0] * d[0], a01 = d[0] * d[1], a02 = d[0] * d[2];
-    const R a11 = d[1] * d[1], a12 = d[1] * d[2], a22 = d[2] * d[2];
-    m[0] = a00 * d[0];
-    m[1] = a00 * d[1];
-    m[2] = a00 * d[2];
-    m[3] = a11 * d[0];
-    m[4] = a01 * d[2];
-    m[5] = a22 * d[0];
-    m[6] = a11 * d[1];
-    m[7] = a11 * d[2];
-    m[8] = a22 * d[1];
-    m[9] = a22 * d[2];
-    (void)a02;
-    (void)a12;
-}
+// ---------------------------------------------------------------- point records
+// FP32: four float4 per point, (y hi, |S|^2) (y lo, segment) (b', 0) (S, 0), y relative to the
+// leaf centre; FP64: five double2, (y0, y1) (y2, segment) (b0', b1') (b2', S0) (S1, S2), y
+// absolute.  b' = omega / 2 times the Burgers vector times the factor of h.  Structure of arrays
+// (row r of point i at r n + i), so a staging warp reads whole lines: 64 (80) bytes a point
+// where a 6 x 18 tensor takes 432 (864).
+struct GaussWeights {
+    double w[GB_MAXG];
+    int n;
+};
 
-// Per-source coefficient tensors of the isotropic polynomial form, 80 per
-// point (78 used, padded for 16-byte rows): 3 linear and 10 cubic-monomial
-// coefficients per stress component, from P = sum_wr A q formed in FP32
-// (nine terms per entry; the near field reads FP32 coefficients, and FP64
-// arithmetic runs at a small fraction of the FP32 rate on this part).
-__global__ void k_src_coef80(int64_t N, const double *__restrict__ q, const double *__restrict__ Asym, float hc,
-                             float ha, float *__restrict__ c32) {
-    __shared__ float As[6 * 9 * 18];
-    for (int i = threadIdx.x; i < 6 * 9 * 18; i += blockDim.x) As[i] = float(Asym[i]);
-    __syncthreads();
-    const int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (j >= N) return;
-    float qq[9];
-    for (int i = 0; i < 9; ++i) qq[i] = float(q[9 * j + i]);
-    constexpr int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
-    for (int ab = 0; ab < 6; ++ab) {
-        float P[18];
-        for (int k = 0; k < 18; ++k) {
-            float s = 0.f;
-            for (int wr = 0; wr < 9; ++wr) s = fmaf(As[(ab * 9 + wr) * 18 + k], qq[wr], s);
-            P[k] = s;
-        }
-        float lin[3] = {0, 0, 0}, cub[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int pr = 0; pr < 6; ++pr) {
-            const int v = PV[pr], p = PP[pr];
-            for (int qd = 0; qd < 3; ++qd) {
-                const float w = P[3 * pr + qd];
-                if (v == p) lin[qd] += -ha * hc * w;
-                if (v == qd) lin[p] += hc * w;
-                if (p == qd) lin[v] += hc * w;
-                int a = v, b = p, c = qd, t;
-                if (a > b) { t = a; a = b; b = t; }
-                if (b > c) { t = b; b = c; c = t; }
-                if (a > b) { t = a; a = b; b = t; }
-                cub[mono_index(a, b, c)] += -3.f * hc * w;
-            }
-        }
-        for (int i = 0; i < 3; ++i) c32[j * 80 + ab * 13 + i] = lin[i];
-        for (int i = 0; i < 10; ++i) c32[j * 80 + ab * 13 + 3 + i] = cub[i];
-    }
-    for (int i = 78; i < 80; ++i) c32[j * 80 + i] = 0.f;
-}
-
-// The 108-entry tensors P for 64 points per block: q staged in shared memory,
-// consecutive threads compute and store consecutive entries (coalesced rows).
-constexpr int kCoefPts = 64;
-__global__ void __launch_bounds__(256) k_src_coef108(int64_t N, const double *__restrict__ q,
-                                                     const double *__restrict__ Asym, float *__restrict__ c32) {
-    __shared__ float As[6 * 9 * 18];
-    __shared__ float sq[kCoefPts][9];
-    for (int i = threadIdx.x; i < 6 * 9 * 18; i += blockDim.x) As[i] = float(Asym[i]);
-    const int64_t j0 = blockIdx.x * int64_t(kCoefPts);
-    const int np = int(min(int64_t(kCoefPts), N - j0));
-    for (int i = threadIdx.x; i < np * 9; i += blockDim.x) (&sq[0][0])[i] = float(q[9 * j0 + i]);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < np * 108; idx += blockDim.x) {
-        const int jl = idx / 108, e = idx - jl * 108, ab = e / 18, k = e - ab * 18;
-        float acc = 0.f;
-#pragma unroll
-        for (int wr = 0; wr < 9; ++wr) acc = fmaf(As[(ab * 9 + wr) * 18 + k], sq[jl][wr], acc);
-        c32[j0 * 108 + idx] = acc;
-    }
-}
-
-template <typename R>
-__device__ __forceinline__ void pair_iso(const R d[3], R ir, const R *c, R acc[6]) {
-    const R ir2 = ir * ir, ir3 = ir * ir2, ir5 = ir3 * ir2;
-    R m[10];
-    monomials<R>(d, m);
-#pragma unroll
-    for (int ab = 0; ab < 6; ++ab) {
-        const R *cc = c + ab * 13;
-        const R l = cc[0] * d[0] + cc[1] * d[1] + cc[2] * d[2];
-        R u = R(0);
-#pragma unroll
-        for (int i = 0; i < 10; ++i) u += cc[3 + i] * m[i];
-        acc[ab] += ir3 * l + ir5 * u;
-    }
-}
-
-// h models of the near kernel
-constexpr int HM_ISO = 0, HM_CUBIC = 1, HM_GENERIC = 2;
-
-template <int HM, typename R, typename CT>
-__device__ __forceinline__ void pair_generic(const R d[3], R ir, const R *c, const CT *C, int Q, R c12, R c44, R cd,
-                                             R acc[6], const float2 *tab = nullptr) {
-    R T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
-    R hs[18];
-    if (HM == HM_CUBIC) {
-        if constexpr (sizeof(R) == 4)
-            h_cubic_f32(c12 + c44, c44, cd, Q, tab, T, hs);
-        else
-            h_circle_cubic<R>(c12, c44, cd, Q, T, hs);
-    } else {
-        h_circle_sym<R, CT>(C, Q, T, hs);
-    }
-    const R ir2 = ir * ir;
-#pragma unroll
-    for (int ab = 0; ab < 6; ++ab) {
-        R s = R(0);
-#pragma unroll
-        for (int k = 0; k < 18; ++k) s += c[ab * 18 + k] * hs[k];
-        acc[ab] += s * ir2;
-    }
-}
-
-constexpr int WARPS = 4;
-
-// NCS: per-source coefficient stride (80 isotropic, 108 otherwise); SCH
-// sources are staged per warp chunk (static shared memory stays < 48 KB)
-template <int HM, int NCS, int SCH>
-__global__ void __launch_bounds__(WARPS * 32) k_near_mixed(
-    int p, int nodes, int L, int64_t nl, float near2, const TreeBox *__restrict__ box, const DevMaterial *__restrict__ mat,
-    const int *__restrict__ tstart, const double *__restrict__ xt, const int64_t *__restrict__ tsid,
-    const int *__restrict__ sstart, const float4 *__restrict__ yrel, const double *__restrict__ ys,
-    const float *__restrict__ c32, const int64_t *__restrict__ ssid,
-    const float *__restrict__ S, double *__restrict__ sig, const int2 *__restrict__ items,
-    const int *__restrict__ n_items) {
-    __shared__ __align__(16) float sP[WARPS][SCH * NCS];
-    __shared__ float4 sy[WARPS][SCH];
-    __shared__ int ssd[WARPS][SCH];
-    __shared__ float sC[81];
-    __shared__ float2 sTab[128];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    if (HM == HM_GENERIC)
-        for (int i = threadIdx.x; i < 81; i += blockDim.x) sC[i] = float(mat->C[i]);
-    if (HM == HM_CUBIC)
-        for (int i = threadIdx.x; i < mat->Q && i < 128; i += blockDim.x) {
-            float sn, cs;
-            sincospif(float(i) / float(mat->Q), &sn, &cs);
-            sTab[i] = make_float2(cs, sn);
-        }
-    __syncthreads();
-    // one work item per warp: up to 32 targets of one leaf, heaviest first
-    const int64_t item = blockIdx.x * int64_t(WARPS) + warp;
-    if (item >= *n_items) return;
-    const int2 wi = items[item];
-    const int64_t leaf = wi.x;
-    const int t0 = wi.y, t1 = min(wi.y + 32, tstart[leaf + 1]);
-    const int P3 = p * p * p;
-    const int nlv = 1 << (L - 1);
+__device__ __forceinline__ void leaf_centre(const TreeBox *box, int nl, int64_t leaf, double c[3]) {
     int cx, cy, cz;
-    cell_xyz3(leaf, nlv, cx, cy, cz);
-    const bool far = L >= 3;
-    const double h = box->H / nlv, ih = double(nlv) / box->H;
-    const double c0[3] = {box->origin[0] + cx * h, box->origin[1] + cy * h, box->origin[2] + cz * h};
-    const int Q = mat->Q;
-    const float c12f = float(mat->c12), c44f = float(mat->c44), cdf = float(mat->cd);
-    const float *Sl = S + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 6;
-    float *wP = sP[warp];
-    float4 *wy = sy[warp];
-    int *wsd = ssd[warp];
-    for (int r0 = t0; r0 < t1; r0 += 32) {
-        // tg targets in this pass, 32 / tg lanes per target splitting the sources
-        const int nrem = min(32, t1 - r0);
-        int tg = 1;
-        while (tg < nrem) tg <<= 1;
-        const int ls = 32 / tg, tl = lane % tg, ph = lane / tg;
-        const int t = r0 + tl;
-        const bool valid = tl < nrem;
-        double x[3] = {0, 0, 0};
-        float xr[3] = {0.f, 0.f, 0.f};
-        float acc[6] = {0, 0, 0, 0, 0, 0};
-        double acc64[6] = {0, 0, 0, 0, 0, 0};
-        int myseg = -1;
-        if (valid) {
-            for (int d = 0; d < 3; ++d) {
-                x[d] = xt[3 * int64_t(t) + d];
-                xr[d] = float(x[d] - (c0[d] + 0.5 * h));
-            }
-            myseg = tsid ? int(tsid[t]) : -1;
-        }
-        if (far && ph == 0) {
-            float bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP];
-            lagrange_1d<float>(p, float((x[0] - c0[0]) * ih), bx, nodes);
-            lagrange_1d<float>(p, float((x[1] - c0[1]) * ih), by, nodes);
-            lagrange_1d<float>(p, float((x[2] - c0[2]) * ih), bz, nodes);
-            for (int lz = 0; lz < p; ++lz)
-                for (int ly = 0; ly < p; ++ly) {
-                    const float wyz = by[ly] * bz[lz];
-                    for (int lx = 0; lx < p; ++lx) {
-                        const float w = bx[lx] * wyz;
-                        const float *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
-                        for (int ab = 0; ab < 6; ++ab) acc[ab] += w * __ldg(s6 + ab);
-                    }
-                }
-        }
-        for (int nb = 0; nb < 27; ++nb) {
-            const int dxn = nb % 3 - 1, dyn = (nb / 3) % 3 - 1, dzn = nb / 9 - 1;
-            const int ax = cx + dxn, ay = cy + dyn, az = cz + dzn;
-            if (ax < 0 || ay < 0 || az < 0 || ax >= nlv || ay >= nlv || az >= nlv) continue;
-            const int64_t A = (int64_t(az) * nlv + ay) * nlv + ax;
-            const int s0 = sstart[A], s1 = sstart[A + 1];
-            const float xs[3] = {xr[0] - float(dxn * h), xr[1] - float(dyn * h), xr[2] - float(dzn * h)};
-            for (int j0 = s0; j0 < s1; j0 += SCH) {
-                const int nj = min(SCH, s1 - j0);
-                __syncwarp();
-                if (lane < nj) {
-                    wy[lane] = yrel[j0 + lane];
-                    wsd[lane] = int(ssid[j0 + lane]);
-                }
-                {
-                    const float4 *src = reinterpret_cast<const float4 *>(c32 + int64_t(NCS) * j0);
-                    float4 *dst = reinterpret_cast<float4 *>(wP);
-                    const int nv = nj * NCS / 4;
-                    for (int i = lane; i < nv; i += 32) dst[i] = __ldg(src + i);
-                }
-                __syncwarp();
-                if (!valid) continue;
-                for (int j = ph; j < nj; j += ls) {
-                    if (wsd[j] == myseg) continue;
-                    const float4 yj = wy[j];
-                    float d[3] = {xs[0] - yj.x, xs[1] - yj.y, xs[2] - yj.z};
-                    const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                    // A close pair takes its separation from the FP64 positions (the
-                    // FP32 difference would cancel) and goes to its own FP64
-                    // accumulator; the kernel itself is evaluated in FP32 on that
-                    // separation, whose relative error is then ~1e-7.
-                    const bool close = r2 < near2 * yj.w * yj.w;
-                    float ir;
-                    if (close) {
-                        const int64_t jj = j0 + j;
-                        const double dd0 = x[0] - ys[3 * jj], dd1 = x[1] - ys[3 * jj + 1], dd2 = x[2] - ys[3 * jj + 2];
-                        const double rr = dd0 * dd0 + dd1 * dd1 + dd2 * dd2;
-                        if (rr == 0.0) continue;
-                        d[0] = float(dd0);
-                        d[1] = float(dd1);
-                        d[2] = float(dd2);
-                        ir = float(rsqrt(rr));
-                    } else {
-                        ir = rsqrtf(r2);
-                    }
-                    float part[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    if (HM == HM_ISO)
-                        pair_iso<float>(d, ir, wP + 80 * j, part);
-                    else
-                        pair_generic<HM, float, float>(d, ir, wP + 108 * j, sC, Q, c12f, c44f, cdf, part, sTab);
-                    if (close) {
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) acc64[ab] += double(part[ab]);
-                    } else {
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) acc[ab] += part[ab];
-                    }
-                }
-            }
-        }
-        // fold the lanes that shared a target (fixed order: deterministic)
-        for (int off = tg; off < 32; off <<= 1)
-            for (int ab = 0; ab < 6; ++ab) {
-                acc[ab] += __shfl_xor_sync(0xffffffffu, acc[ab], off);
-                acc64[ab] += __shfl_xor_sync(0xffffffffu, acc64[ab], off);
-            }
-        if (valid && ph == 0)
-            for (int ab = 0; ab < 6; ++ab) sig[6 * int64_t(t) + ab] = double(acc[ab]) + acc64[ab];
+    cell_xyz3(leaf, nl, cx, cy, cz);
+    const double h = box->H / nl;
+    c[0] = box->origin[0] + (cx + 0.5) * h;
+    c[1] = box->origin[1] + (cy + 0.5) * h;
+    c[2] = box->origin[2] + (cz + 0.5) * h;
+}
+
+__device__ __forceinline__ void split_position(const double *y, const double c[3], float hi[3], float lo[3]) {
+    for (int d = 0; d < 3; ++d) {
+        const double v = y[d] - c[d];
+        hi[d] = float(v);
+        lo[d] = float(v - double(hi[d]));
     }
 }
 
-// ---------------------------------------------------------------- symmetric near field
-// Nodal forces (targets = sources): h is odd, h(-T) = -h(T), so one
-// evaluation of h for the point pair (i, j) serves both directions,
-//     s_i += P_j h(T_ij) / R^2   and   s_j -= P_i h(T_ij) / R^2.
-// Work items are leaf pairs (A, B) with B = A + o over the 14 offsets o of
-// the upper half of the 3 x 3 x 3 neighbourhood (o = 0 included: pairs j > i
-// of one leaf).  Contributions are written to partial slots, one per point
-// and neighbour direction (27 directions + the reverse half of the own
-// leaf), each written by exactly one warp in a fixed order; the combine kernel
-// adds the far field (L2P) and the slots in a fixed order.  Close pairs
-// (closer than near_fp64 x the longer of the two segments) take their
-// separation from the FP64 positions, where the cancellation is, and are
-// summed apart from the other pairs in two-float (hi + lo) sums.
-// One warp per block (a block's shared-memory slice is freed as soon as its leaf pair is
-// done) and 12 resident blocks per SM (152 registers): at 1M segments, Q = 16, the near
-// field took 195 ms against 204 ms with four warps per block at the same 12 warps per SM
-// (there the slowest warp of a block held the other three slices).
-constexpr int SYM_WARPS = 1, SYM_SCH = 8, SYM_MINB = 12;
-constexpr int kSlots = 28;
+template <typename R>
+__global__ void k_near_records(int64_t N, int L, const TreeBox *__restrict__ box, const double *__restrict__ y,
+                               const int *__restrict__ perm, const int *__restrict__ pleaf,
+                               const double *__restrict__ nodes, const int64_t *__restrict__ segs,
+                               const double *__restrict__ burgers, GaussWeights gw, double fac, void *__restrict__ rec) {
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i >= N) return;
+    const int k = perm[i];
+    const int64_t s = k / gw.n;
+    const int64_t n0 = segs[2 * s], n1 = segs[2 * s + 1];
+    const double f = 0.5 * gw.w[k - int(s) * gw.n] * fac;
+    double S[3], b[3];
+    for (int d = 0; d < 3; ++d) {
+        S[d] = nodes[3 * n1 + d] - nodes[3 * n0 + d];
+        b[d] = f * burgers[3 * s + d];
+    }
+    if constexpr (sizeof(R) == 4) {
+        float4 *r = static_cast<float4 *>(rec);
+        double c[3];
+        leaf_centre(box, 1 << (L - 1), pleaf[i], c);
+        float hi[3], lo[3];
+        split_position(y + 3 * i, c, hi, lo);
+        r[i] = make_float4(hi[0], hi[1], hi[2], float(S[0] * S[0] + S[1] * S[1] + S[2] * S[2]));
+        r[N + i] = make_float4(lo[0], lo[1], lo[2], __int_as_float(int(s)));
+        r[2 * N + i] = make_float4(float(b[0]), float(b[1]), float(b[2]), 0.f);
+        r[3 * N + i] = make_float4(float(S[0]), float(S[1]), float(S[2]), 0.f);
+    } else {
+        double2 *r = static_cast<double2 *>(rec);
+        r[i] = make_double2(y[3 * i], y[3 * i + 1]);
+        r[N + i] = make_double2(y[3 * i + 2], __longlong_as_double(s));
+        r[2 * N + i] = make_double2(b[0], b[1]);
+        r[3 * N + i] = make_double2(b[2], S[0]);
+        r[4 * N + i] = make_double2(S[1], S[2]);
+    }
+}
 
-// Two-float sums for the close pairs: the value is hi + lo, and each addition
-// keeps its exact rounding error (Knuth's two-sum, six FP32 operations), so
-// the sum of FP32 terms carries ~48 mantissa bits without FP64 arithmetic
+// free targets, sorted by leaf: the position rows alone, segment -1
+template <typename R>
+__global__ void k_near_targets(int64_t n, int L, const TreeBox *__restrict__ box, const double *__restrict__ x,
+                               const int *__restrict__ leaf_of, void *__restrict__ rec) {
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (i >= n) return;
+    if constexpr (sizeof(R) == 4) {
+        float4 *r = static_cast<float4 *>(rec);
+        double c[3];
+        leaf_centre(box, 1 << (L - 1), leaf_of[i], c);
+        float hi[3], lo[3];
+        split_position(x + 3 * i, c, hi, lo);
+        r[i] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        r[n + i] = make_float4(lo[0], lo[1], lo[2], __int_as_float(-1));
+    } else {
+        double2 *r = static_cast<double2 *>(rec);
+        r[i] = make_double2(x[3 * i], x[3 * i + 1]);
+        r[n + i] = make_double2(x[3 * i + 2], __longlong_as_double(-1));
+    }
+}
+
+// ---------------------------------------------------------------- work plan
+// Per leaf with targets: where its rows start, the length of its source list, and its tiles:
+// ca target tiles of ta targets (a split leaf of the adaptive tree: ca groups of children), cb
+// list sections of sb entries.  Rows: [cb][targets] forward, then [ca][list] reverse.
+struct NearPlan {
+    long long base;
+    int ns, ta, ca, sb, cb, pad;
+};
+struct NearItem {
+    int leaf, a, b, pad;
+};
+
+constexpr int kPlanSizes = 8;  // candidates of pairs per item: 512 4^k, the last without bound
+// counters: [0] pairs, [1 + k] rows, [1 + kPlanSizes + k] items of candidate k, then the
+// allocation cursors of rows and items and the items taken
+constexpr int kCntRows = 1 + 2 * kPlanSizes, kCntItems = kCntRows + 1, kCntNext = kCntItems + 1, kCnt = kCntNext + 1;
+
+__device__ __forceinline__ int64_t plan_size(int k) {
+    return k == kPlanSizes - 1 ? (int64_t(1) << 62) : int64_t(512) << (2 * k);
+}
+
+// tiles of a leaf with nt targets and ns list entries at w pairs per item.  List sections first
+// (a section costs nt rows, a target tile ns, and ns is about 14 nt), at least 32 entries long;
+// then target tiles of a multiple of 8.  A split leaf's tiles are groups of children.
+__device__ __forceinline__ void plan_tiles(int nt, int ns, bool split, int64_t w, int &ta, int &ca, int &sb, int &cb) {
+    const int64_t pairs = int64_t(nt) * ns;
+    ta = nt, ca = 1, sb = ns, cb = 1;
+    if (ns == 0) return;
+    if (split) {
+        while (ca < 8 && pairs / ca > w) ca *= 2;
+        ta = 8 / ca;
+        const int64_t c = min((pairs / ca + w - 1) / w, int64_t((ns + 31) / 32));
+        if (c > 1) {
+            sb = int(((ns + c - 1) / c + 31) / 32 * 32);
+            cb = (ns + sb - 1) / sb;
+        }
+        return;
+    }
+    if (pairs <= w) return;
+    const int64_t c = min((pairs + w - 1) / w, int64_t((ns + 31) / 32));
+    sb = int(((ns + c - 1) / c + 31) / 32 * 32);
+    cb = (ns + sb - 1) / sb;
+    const int64_t each = int64_t(nt) * min(sb, ns);
+    if (each > w) {
+        const int64_t t = min((each + w - 1) / w, int64_t((nt + 7) / 8));
+        ta = int(((nt + t - 1) / t + 7) / 8 * 8);
+        ca = (nt + ta - 1) / ta;
+    }
+}
+
+// leaf A + o of direction nb (0..26), -1 outside the grid
+__device__ __forceinline__ int64_t neighbour(int x, int y, int z, int nb, int nl) {
+    const int bx = x + nb % 3 - 1, by = y + (nb / 3) % 3 - 1, bz = z + nb / 9 - 1;
+    if (bx < 0 || by < 0 || bz < 0 || bx >= nl || by >= nl || bz >= nl) return -1;
+    return (int64_t(bz) * nl + by) * nl + bx;
+}
+
+// pairs of the pass and, for every candidate size, its rows and items (exact integer sums)
+template <bool SYM>
+__global__ void __launch_bounds__(256) k_near_totals(int64_t nl, int L, const int *__restrict__ tstart,
+                                                     const int *__restrict__ sstart, const int *__restrict__ ref_start,
+                                                     unsigned long long *__restrict__ cnt) {
+    constexpr int D0 = SYM ? 13 : 0;
+    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    long long v[1 + 2 * kPlanSizes];
+    for (int i = 0; i < 1 + 2 * kPlanSizes; ++i) v[i] = 0;
+    if (l < nl) {
+        const int nt = tstart[l + 1] - tstart[l];
+        if (nt > 0) {
+            const int nlv = 1 << (L - 1);
+            int x, y, z, ns = 0;
+            cell_xyz3(l, nlv, x, y, z);
+            for (int nb = D0; nb < 27; ++nb) {
+                const int64_t B = neighbour(x, y, z, nb, nlv);
+                if (B >= 0) ns += sstart[B + 1] - sstart[B];
+            }
+            const bool split = ref_start && ref_start[l + 1] > ref_start[l];
+            v[0] = (long long)nt * ns;
+            for (int k = 0; k < kPlanSizes; ++k) {
+                int ta, ca, sb, cb;
+                plan_tiles(nt, ns, split, plan_size(k), ta, ca, sb, cb);
+                v[1 + k] = (long long)cb * nt + (SYM ? (long long)ca * ns : 0);
+                v[1 + kPlanSizes + k] = (long long)ca * cb;
+            }
+        }
+    }
+    __shared__ long long sm[8];
+    for (int i = 0; i < 1 + 2 * kPlanSizes; ++i) {
+        long long s = v[i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) sm[threadIdx.x / 32] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long t = 0;
+            for (int w = 0; w < int(blockDim.x) / 32; ++w) t += sm[w];
+            if (t) atomicAdd(&cnt[i], (unsigned long long)t);
+        }
+    }
+}
+
+// The size is the smallest candidate whose rows and items fit the buffers and that leaves a
+// resident warp about eight items (a warp's last item is then a small part of its time), but
+// not above 32,768 pairs where the buffers allow (about 1 ms of a warp): every quantity
+// depends on the network and the options alone, so results do not depend on a buffer's history.
+template <bool SYM>
+__global__ void __launch_bounds__(256) k_near_plan(int64_t nl, int L, int warps, long long cap_rows, long long cap_items,
+                                                   const int *__restrict__ tstart, const int *__restrict__ sstart,
+                                                   const int *__restrict__ ref_start,
+                                                   unsigned long long *__restrict__ cnt, NearPlan *__restrict__ plan,
+                                                   int *__restrict__ lp, NearItem *__restrict__ items) {
+    constexpr int D0 = SYM ? 13 : 0, ND = 27 - D0;
+    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int lane = threadIdx.x % 32;
+    int nt = 0, ns = 0, ta = 1, ca = 0, sb = 1, cb = 0;
+    if (l < nl) nt = tstart[l + 1] - tstart[l];
+    if (nt > 0) {
+        const int nlv = 1 << (L - 1);
+        int x, y, z;
+        cell_xyz3(l, nlv, x, y, z);
+        for (int d = 0; d < ND; ++d) {
+            const int64_t B = neighbour(x, y, z, D0 + d, nlv);
+            lp[ND * l + d] = ns;
+            if (B >= 0) ns += sstart[B + 1] - sstart[B];
+        }
+        int64_t want = int64_t(cnt[0] / (8ull * (unsigned long long)warps));
+        want = min(want, int64_t(32768));
+        int k = 0;
+        while (k < kPlanSizes - 1 && (plan_size(k) < want || (long long)cnt[1 + k] > cap_rows ||
+                                      (long long)cnt[1 + kPlanSizes + k] > cap_items))
+            ++k;
+        plan_tiles(nt, ns, ref_start && ref_start[l + 1] > ref_start[l], plan_size(k), ta, ca, sb, cb);
+    }
+    // one allocation per warp
+    long long rows = (long long)cb * nt + (SYM ? (long long)ca * ns : 0), n_it = (long long)ca * cb;
+    long long r0 = rows, i0 = n_it;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long a = __shfl_up_sync(0xffffffffu, r0, o), b = __shfl_up_sync(0xffffffffu, i0, o);
+        if (lane >= o) r0 += a, i0 += b;
+    }
+    long long rb = 0, ib = 0;
+    if (lane == 31) {
+        if (r0) rb = (long long)atomicAdd(&cnt[kCntRows], (unsigned long long)r0);
+        if (i0) ib = (long long)atomicAdd(&cnt[kCntItems], (unsigned long long)i0);
+    }
+    rb = __shfl_sync(0xffffffffu, rb, 31) + r0 - rows;
+    ib = __shfl_sync(0xffffffffu, ib, 31) + i0 - n_it;
+    if (nt > 0) {
+        plan[l] = NearPlan{rb, ns, ta, ca, sb, cb, 0};
+        for (int a = 0; a < ca; ++a)
+            for (int b = 0; b < cb; ++b) items[ib++] = NearItem{int(l), a, b, 0};
+    }
+}
+
+// ---------------------------------------------------------------- pair kernel
+// Two-float sums: the value is hi + lo, and each addition keeps its exact rounding error
+// (Knuth's two-sum), so a sum of FP32 terms carries ~48 mantissa bits without FP64 arithmetic
 // (FP64 runs at a small fraction of the FP32 rate on this part).
 __device__ __forceinline__ void tsum(float &hi, float &lo, float b) {
     const float s = hi + b;
@@ -355,1072 +313,816 @@ __device__ __forceinline__ void tsum2(float &hi, float &lo, float bhi, float blo
     hi = s;
 }
 
-template <int HM>
-__global__ void __launch_bounds__(SYM_WARPS * 32, SYM_MINB) k_near_sym(
-    int L, float near2, const TreeBox *__restrict__ box, const DevMaterial *__restrict__ mat,
-    const int *__restrict__ sstart, const float4 *__restrict__ yrel, const double *__restrict__ ys,
-    const float *__restrict__ c32, const int64_t *__restrict__ ssid, double *__restrict__ part, int64_t N,
-    const int2 *__restrict__ items, const int *__restrict__ n_items, const int *__restrict__ ref_start,
-    const int *__restrict__ child_start) {
-    extern __shared__ __align__(16) float sm_sym[];
-    float *wPA = sm_sym + (threadIdx.x / 32) * (32 * 108 + SYM_SCH * 108);  // [32][108]: lanes' own tensors
-    float *wPB = wPA + 32 * 108;                                            // [SCH][108] staged sources
-    __shared__ float4 syB[SYM_WARPS][SYM_SCH];
-    __shared__ int sdB[SYM_WARPS][SYM_SCH];
-    __shared__ float saccB[SYM_WARPS][SYM_SCH][6];
-    __shared__ float2 saccCB[SYM_WARPS][SYM_SCH][6];  // close pairs: two-float (hi, lo)
-    __shared__ double sxB[SYM_WARPS][SYM_SCH][3];      // FP64 positions of the staged sources
-    __shared__ float sC[81];
-    __shared__ __align__(16) float2 sTab[128];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    if (HM == HM_GENERIC)
-        for (int i = threadIdx.x; i < 81; i += blockDim.x) sC[i] = float(mat->C[i]);
-    if (HM == HM_CUBIC)
-        for (int i = threadIdx.x; i < mat->Q && i < 128; i += blockDim.x) {
-            float sn, cs;
-            sincospif(float(i) / float(mat->Q), &sn, &cs);
-            sTab[i] = make_float2(cs, sn);
-        }
-    __syncthreads();
-    const bool packed = (mat->Q & 1) == 0;  // two circle points per packed step
-    const int64_t item = blockIdx.x * int64_t(SYM_WARPS) + warp;
-    if (item >= *n_items) return;
-    const int2 wi = items[item];
-    const int64_t Aleaf = wi.x;
-    const int d = wi.y;  // 0..13: neighbour index 13 + d
-    const int nlv = 1 << (L - 1);
-    int ax, ay, az;
-    cell_xyz3(Aleaf, nlv, ax, ay, az);
-    const int nb = 13 + d;
-    const int ox = nb % 3 - 1, oy = (nb / 3) % 3 - 1, oz = nb / 9 - 1;
-    const int64_t Bleaf = (int64_t(az + oz) * nlv + (ay + oy)) * nlv + (ax + ox);
-    const bool self = d == 0;
-    const int sA0 = sstart[Aleaf], sA1 = sstart[Aleaf + 1];
-    const int sB0 = sstart[Bleaf], sB1 = sstart[Bleaf + 1];
-    const int slot_f = nb, slot_r = self ? 27 : 26 - nb;
-    const double h = box->H / nlv;
-    // B's leaf-relative positions, seen from A's leaf centre
-    const float bsh[3] = {float(ox * h), float(oy * h), float(oz * h)};
-    const int Q = mat->Q;
-    const float c12f = float(mat->c12), c44f = float(mat->c44), cdf = float(mat->cd);
-    bool first_chunk = true;
-    // adaptive tree: two different split leaves interact through their adjacent children
-    // only (the others through the M2L one level down): the targets go child by child and
-    // each target child meets the children of B adjacent to it
-    int rA = -1, rB = -1;
-    if (ref_start && !self) {
-        if (ref_start[Aleaf + 1] > ref_start[Aleaf]) rA = ref_start[Aleaf];
-        if (ref_start[Bleaf + 1] > ref_start[Bleaf]) rB = ref_start[Bleaf];
+// a sum in the kernel's precision: two-float or FP64
+template <typename R>
+struct Acc;
+template <>
+struct Acc<float> {
+    float hi, lo;
+    __device__ __forceinline__ void zero() { hi = lo = 0.f; }
+    __device__ __forceinline__ void add(float v) { tsum(hi, lo, v); }
+    __device__ __forceinline__ void add(const Acc &o) { tsum2(hi, lo, o.hi, o.lo); }
+    __device__ __forceinline__ Acc shfl_xor(int o) const {
+        return Acc{__shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o)};
     }
-    const bool fine = rA >= 0 && rB >= 0;
-    if (fine) {
-        // B's reverse slots then collect several target children: they start from zero
-        for (int k = lane; k < (sB1 - sB0) * 6; k += 32)
-            part[(int64_t(slot_r) * N + sB0 + k / 6) * 6 + k % 6] = 0.0;
-        __syncwarp();
+    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+};
+template <>
+struct Acc<double> {
+    double v;
+    __device__ __forceinline__ void zero() { v = 0.0; }
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add(const Acc &o) { v += o.v; }
+    __device__ __forceinline__ Acc shfl_xor(int o) const { return Acc{__shfl_xor_sync(0xffffffffu, v, o)}; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+// a point in registers
+template <typename R>
+struct Pt;
+template <>
+struct Pt<float> {
+    float hi[3], lo[3], b[3], S[3], len2;
+    int seg;
+};
+template <>
+struct Pt<double> {
+    double hi[3], b[3], S[3], len2;
+    long long seg;
+};
+
+// rows of staged points in shared memory
+template <typename R, int N>
+struct Stage;
+template <int N>
+struct Stage<float, N> {
+    float4 r[4][N];
+    __device__ __forceinline__ void load_target(const void *rec, int64_t n, int64_t i, int k, bool full) {
+        const float4 *g = static_cast<const float4 *>(rec);
+        r[0][k] = __ldg(g + i);
+        r[1][k] = __ldg(g + n + i);
+        if (full) {
+            r[2][k] = __ldg(g + 2 * n + i);
+            r[3][k] = __ldg(g + 3 * n + i);
+        }
     }
-    for (int ts = 0; ts < (fine ? 8 : 1); ++ts) {
-    const int tA0 = fine ? child_start[9 * rA + ts] : sA0, tA1 = fine ? child_start[9 * rA + ts + 1] : sA1;
-    for (int r0 = tA0, nrem = 0; r0 < tA1; r0 += nrem) {
-        // nrem targets in this chunk on tg lanes (a power of two), 32 / tg lanes per
-        // target splitting the sources.  A chunk costs max(1, tg / 4) warp steps per
-        // 8 sources, so the targets left are cut into power-of-two chunks where that
-        // is cheaper than rounding them up (20 targets: 16 + 4, five steps instead
-        // of eight; 30 targets: one chunk of 32)
-        const int left = tA1 - r0;
-        const int tg = left >= 29 ? 32 : left >= 13 ? 16 : left >= 5 ? 8 : left >= 3 ? 4 : left;
-        nrem = min(tg, left);
-        const int ls = 32 / tg, ti = lane % tg, tj = lane / tg;
-        const int i = r0 + ti;
-        const bool vi = i < tA1;
-        // stage the lanes' own source tensors, one 432-byte row per target: the
-        // 16-byte reads of 8 consecutive rows fall in 8 different bank quads
-        __syncwarp();
-        {
-            const float4 *src = reinterpret_cast<const float4 *>(c32 + int64_t(108) * r0);
-            float4 *dst = reinterpret_cast<float4 *>(wPA);
-            for (int k = lane; k < nrem * 27; k += 32) dst[k] = __ldg(src + k);
-        }
-        __syncwarp();
-        float4 yi = make_float4(0.f, 0.f, 0.f, 0.f);
-        double xi[3] = {0.0, 0.0, 0.0};
-        int segi = -2;
-        if (vi) {
-            yi = yrel[i];
-            xi[0] = ys[3 * int64_t(i)], xi[1] = ys[3 * int64_t(i) + 1], xi[2] = ys[3 * int64_t(i) + 2];
-            segi = int(ssid[i]);
-        }
-        float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float accC[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, accCl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // close pairs
-        const float4 *Pi4 = reinterpret_cast<const float4 *>(wPA + 108 * ti);
-        for (int ss = 0; ss < (fine ? 8 : 1); ++ss) {
-        int jb0 = self ? r0 : sB0, jb1 = sB1;  // own leaf: pairs j > i only
-        if (fine) {
-            // B's child ss against A's child ts: adjacent at the children's level?
-            const int dx = 2 * ox + (ss & 1) - (ts & 1), dy = 2 * oy + ((ss >> 1) & 1) - ((ts >> 1) & 1),
-                      dz = 2 * oz + (ss >> 2) - (ts >> 2);
-            if (abs(dx) > 1 || abs(dy) > 1 || abs(dz) > 1) continue;
-            jb0 = child_start[9 * rB + ss];
-            jb1 = child_start[9 * rB + ss + 1];
-        }
-        for (int j0 = jb0; j0 < jb1; j0 += SYM_SCH) {
-            const int nj = min(SYM_SCH, jb1 - j0);
-            __syncwarp();
-            if (lane < nj) {
-                syB[warp][lane] = yrel[j0 + lane];
-                sdB[warp][lane] = int(ssid[j0 + lane]);
-            }
-            for (int k = lane; k < nj * 3; k += 32) (&sxB[warp][0][0])[k] = ys[3 * int64_t(j0) + k];
-            for (int k = lane; k < SYM_SCH * 6; k += 32) {
-                (&saccB[warp][0][0])[k] = 0.f;
-                (&saccCB[warp][0][0])[k] = make_float2(0.f, 0.f);
-            }
-            {
-                const float4 *src = reinterpret_cast<const float4 *>(c32 + int64_t(108) * j0);
-                float4 *dst = reinterpret_cast<float4 *>(wPB);
-                for (int k = lane; k < nj * 27; k += 32) dst[k] = __ldg(src + k);
-            }
-            __syncwarp();
-            for (int jj = 0; jj < nj; jj += ls) {
-                const int jl = jj + tj;  // this lane's source within the chunk
-                const int j = j0 + jl;
-                bool on = vi && jl < nj && (!self || j > i);
-                float4 yj = make_float4(0.f, 0.f, 0.f, 1.f);
-                if (on) {
-                    yj = syB[warp][jl];
-                    on = sdB[warp][jl] != segi;
-                }
-                float d3[3] = {yi.x - (yj.x + bsh[0]), yi.y - (yj.y + bsh[1]), yi.z - (yj.z + bsh[2])};
-                const float r2 = d3[0] * d3[0] + d3[1] * d3[1] + d3[2] * d3[2];
-                const float lmax = fmaxf(yi.w, yj.w);
-                const bool close = on && r2 < near2 * lmax * lmax;
-                float ir = 1.f;
-                if (close) {
-                    // the separation from the FP64 positions (no cancellation in the
-                    // leaf-relative FP32 coordinates); its length in FP32
-                    d3[0] = float(xi[0] - sxB[warp][jl][0]);
-                    d3[1] = float(xi[1] - sxB[warp][jl][1]);
-                    d3[2] = float(xi[2] - sxB[warp][jl][2]);
-                    const float rr = d3[0] * d3[0] + d3[1] * d3[1] + d3[2] * d3[2];
-                    if (rr == 0.f) on = false;
-                    ir = rr > 0.f ? rsqrtf(rr) : 1.f;
-                } else if (on) {
-                    ir = rsqrtf(r2);
-                }
-                float fw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, rv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                if (on) {
-                    float T[3] = {d3[0] * ir, d3[1] * ir, d3[2] * ir};
-                    float hs[18];
-                    if (HM == HM_CUBIC) {
-                        if (packed)
-                            h_cubic_f32x2(c12f + c44f, c44f, cdf, Q, reinterpret_cast<const float4 *>(sTab), T, hs);
-                        else
-                            h_cubic_f32(c12f + c44f, c44f, cdf, Q, sTab, T, hs);
-                    } else {
-                        h_circle_sym<float, float>(sC, Q, T, hs);
-                    }
-                    const float ir2 = ir * ir;
-                    const float4 *Pj4 = reinterpret_cast<const float4 *>(wPB + 108 * jl);
-                    // both contractions over the 108 entries in 16-byte pieces (entry c = 18 ab + k)
-#pragma unroll
-                    for (int c4 = 0; c4 < 27; ++c4) {
-                        const float4 pj = Pj4[c4], pi = Pi4[c4];
-                        const float vj[4] = {pj.x, pj.y, pj.z, pj.w}, vi4[4] = {pi.x, pi.y, pi.z, pi.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int c = 4 * c4 + e;
-                            fw[c / 18] = fmaf(vj[e], hs[c % 18], fw[c / 18]);
-                            rv[c / 18] = fmaf(vi4[e], hs[c % 18], rv[c / 18]);
-                        }
-                    }
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) {
-                        fw[ab] *= ir2;
-                        rv[ab] *= -ir2;
-                    }
-                    if (close) {
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) tsum(accC[ab], accCl[ab], fw[ab]);
-                    } else {
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) acc[ab] += fw[ab];
-                    }
-                }
-                // reverse: sum over the tg lanes that share source jl (fixed order); close
-                // pairs go through two-float sums, only when the warp has one
-                if (__any_sync(0xffffffffu, close)) {
-                    float ch[6], cl[6];
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) {
-                        ch[ab] = close ? rv[ab] : 0.f;
-                        cl[ab] = 0.f;
-                        if (close) rv[ab] = 0.f;
-                    }
-                    for (int off = 1; off < tg; off <<= 1)
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) {
-                            const float oh = __shfl_xor_sync(0xffffffffu, ch[ab], off);
-                            const float ol = __shfl_xor_sync(0xffffffffu, cl[ab], off);
-                            tsum2(ch[ab], cl[ab], oh, ol);
-                        }
-                    if (ti == 0 && jl < nj)
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) {
-                            float2 &a = saccCB[warp][jl][ab];
-                            tsum2(a.x, a.y, ch[ab], cl[ab]);
-                        }
-                }
-                for (int off = 1; off < tg; off <<= 1)
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) rv[ab] += __shfl_xor_sync(0xffffffffu, rv[ab], off);
-                if (ti == 0 && jl < nj) {
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) saccB[warp][jl][ab] += rv[ab];
-                }
-            }
-            __syncwarp();
-            // reverse partials of this chunk's sources: this warp is their only writer; the
-            // first target chunk stores, later ones add (in the own leaf the first chunk
-            // visits every source, later chunks only j >= r0)
-            for (int k = lane; k < nj * 6; k += 32) {
-                const int jl = k / 6, ab = k % 6;
-                double *dst = part + (int64_t(slot_r) * N + (j0 + jl)) * 6 + ab;
-                const float2 cc = saccCB[warp][jl][ab];
-                const double v = double(saccB[warp][jl][ab]) + (double(cc.x) + double(cc.y));
-                *dst = (first_chunk && !fine) ? v : *dst + v;
-            }
-        }
-        }
-        first_chunk = false;
-        // forward: sum over the lanes that share target i (fixed order)
-        for (int off = tg; off < 32; off <<= 1)
-#pragma unroll
-            for (int ab = 0; ab < 6; ++ab) {
-                acc[ab] += __shfl_xor_sync(0xffffffffu, acc[ab], off);
-                const float oh = __shfl_xor_sync(0xffffffffu, accC[ab], off);
-                const float ol = __shfl_xor_sync(0xffffffffu, accCl[ab], off);
-                tsum2(accC[ab], accCl[ab], oh, ol);
-            }
-        if (vi && tj == 0)
-#pragma unroll
-            for (int ab = 0; ab < 6; ++ab)
-                part[(int64_t(slot_f) * N + i) * 6 + ab] = double(acc[ab]) + (double(accC[ab]) + double(accCl[ab]));
+    // position moved by o leaf edges (eh + el, two floats) to the target leaf's centre
+    __device__ __forceinline__ void load_source(const void *rec, int64_t n, int64_t i, int k, int ox, int oy, int oz,
+                                                float eh, float el) {
+        const float4 *g = static_cast<const float4 *>(rec);
+        float4 a = __ldg(g + i), c = __ldg(g + n + i);
+        tsum2(a.x, c.x, float(ox) * eh, float(ox) * el);
+        tsum2(a.y, c.y, float(oy) * eh, float(oy) * el);
+        tsum2(a.z, c.z, float(oz) * eh, float(oz) * el);
+        r[0][k] = a;
+        r[1][k] = c;
+        r[2][k] = __ldg(g + 2 * n + i);
+        r[3][k] = __ldg(g + 3 * n + i);
     }
+    __device__ __forceinline__ Pt<float> get(int k, bool full) const {
+        Pt<float> p;
+        const float4 a = r[0][k], c = r[1][k];
+        p.hi[0] = a.x, p.hi[1] = a.y, p.hi[2] = a.z, p.len2 = a.w;
+        p.lo[0] = c.x, p.lo[1] = c.y, p.lo[2] = c.z, p.seg = __float_as_int(c.w);
+        if (full) {
+            const float4 b = r[2][k], s = r[3][k];
+            p.b[0] = b.x, p.b[1] = b.y, p.b[2] = b.z;
+            p.S[0] = s.x, p.S[1] = s.y, p.S[2] = s.z;
+        }
+        return p;
     }
+};
+template <int N>
+struct Stage<double, N> {
+    double2 r[5][N];
+    __device__ __forceinline__ void load_target(const void *rec, int64_t n, int64_t i, int k, bool full) {
+        const double2 *g = static_cast<const double2 *>(rec);
+        for (int q = 0; q < (full ? 5 : 2); ++q) r[q][k] = __ldg(g + q * n + i);
+    }
+    __device__ __forceinline__ void load_source(const void *rec, int64_t n, int64_t i, int k, int, int, int, float,
+                                                float) {
+        load_target(rec, n, i, k, true);
+    }
+    __device__ __forceinline__ Pt<double> get(int k, bool full) const {
+        Pt<double> p;
+        p.hi[0] = r[0][k].x, p.hi[1] = r[0][k].y, p.hi[2] = r[1][k].x;
+        p.seg = __double_as_longlong(r[1][k].y);
+        if (full) {
+            p.b[0] = r[2][k].x, p.b[1] = r[2][k].y, p.b[2] = r[3][k].x;
+            p.S[0] = r[3][k].y, p.S[1] = r[4][k].x, p.S[2] = r[4][k].y;
+        }
+        return p;
+    }
+};
+
+// separation x_i - y_j
+__device__ __forceinline__ void separation(const Pt<float> &p, const Pt<float> &s, float d[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d[k] = (p.hi[k] - s.hi[k]) + (p.lo[k] - s.lo[k]);
+}
+__device__ __forceinline__ void separation(const Pt<double> &p, const Pt<double> &s, double d[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d[k] = p.hi[k] - s.hi[k];
 }
 
-// FP64 form of the symmetric near field for the FP64 pass: the same leaf-pair
-// work items, target chunks and partial slots as k_near_sym, with FP64
-// positions, source tensors (P of k_precontract<double>), h and sums.  The
-// cubic rule takes its circle points from a shared table; the general
-// medium uses h_circle_sym.  FP64 arithmetic is the bound, so two warps per
-// block and the full 108-entry tensors staged as doubles suffice.
-constexpr int S64_WARPS = 2, S64_SCH = 8;
+constexpr int kTargets = 64;  // targets of an item staged at a time
+constexpr int kRanges = 112;  // list ranges of one target leaf: 14 leaves x 8 children
 
-template <int HM>
-__global__ void __launch_bounds__(S64_WARPS * 32) k_near_sym64(
-    int L, const TreeBox *__restrict__ box, const DevMaterial *__restrict__ mat, const int *__restrict__ sstart,
-    const double *__restrict__ ys, const double *__restrict__ P64, const int64_t *__restrict__ ssid,
-    double *__restrict__ part, int64_t N, const int2 *__restrict__ items, const int *__restrict__ n_items) {
-    extern __shared__ __align__(16) double sm_s64[];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    double *wPA = sm_s64 + warp * (32 * 108 + S64_SCH * 108);  // [32][108]: the chunk's target tensors
-    double *wPB = wPA + 32 * 108;                               // [SCH][108]: staged sources
-    __shared__ double sxB[S64_WARPS][S64_SCH][3];
-    __shared__ int64_t sdB[S64_WARPS][S64_SCH];
-    __shared__ double saccB[S64_WARPS][S64_SCH][6];
-    __shared__ double sC[81];
-    __shared__ double sTc[256], sTs[256];
-    if (HM == HM_GENERIC)
-        for (int i = threadIdx.x; i < 81; i += blockDim.x) sC[i] = mat->C[i];
-    if (HM == HM_CUBIC)
-        for (int i = threadIdx.x; i < mat->Q && i < 256; i += blockDim.x) sincospi(double(i) / double(mat->Q), &sTs[i], &sTc[i]);
-    __syncthreads();
-    const int64_t item = blockIdx.x * int64_t(S64_WARPS) + warp;
-    if (item >= *n_items) return;
-    const int2 wi = items[item];
-    const int64_t Aleaf = wi.x;
-    const int d = wi.y;
-    const int nlv = 1 << (L - 1);
-    int ax, ay, az;
-    cell_xyz3(Aleaf, nlv, ax, ay, az);
-    const int nb = 13 + d;
-    const int ox = nb % 3 - 1, oy = (nb / 3) % 3 - 1, oz = nb / 9 - 1;
-    const int64_t Bleaf = (int64_t(az + oz) * nlv + (ay + oy)) * nlv + (ax + ox);
-    const bool self = d == 0;
-    const int sA0 = sstart[Aleaf], sA1 = sstart[Aleaf + 1];
-    const int sB0 = sstart[Bleaf], sB1 = sstart[Bleaf + 1];
-    const int slot_f = nb, slot_r = self ? 27 : 26 - nb;
-    const int Q = mat->Q;
-    const double cp = mat->c12 + mat->c44, c44 = mat->c44, cd = mat->cd;
-    bool first_chunk = true;
-    for (int r0 = sA0, nrem = 0; r0 < sA1; r0 += nrem) {
-        const int left = sA1 - r0;
-        const int tg = left >= 29 ? 32 : left >= 13 ? 16 : left >= 5 ? 8 : left >= 3 ? 4 : left;
-        nrem = min(tg, left);
-        const int ls = 32 / tg, ti = lane % tg, tj = lane / tg;
-        const int i = r0 + ti;
-        const bool vi = i < sA1;
-        __syncwarp();
-        {
-            const double2 *src = reinterpret_cast<const double2 *>(P64 + int64_t(108) * r0);
-            double2 *dst = reinterpret_cast<double2 *>(wPA);
-            for (int k = lane; k < nrem * 54; k += 32) dst[k] = __ldg(src + k);
-        }
-        __syncwarp();
-        double xi[3] = {0.0, 0.0, 0.0};
-        int64_t segi = -2;
-        if (vi) {
-            xi[0] = ys[3 * int64_t(i)], xi[1] = ys[3 * int64_t(i) + 1], xi[2] = ys[3 * int64_t(i) + 2];
-            segi = ssid[i];
-        }
-        double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        const double *Pi = wPA + 108 * ti;
-        const int jb0 = self ? r0 : sB0;
-        for (int j0 = jb0; j0 < sB1; j0 += S64_SCH) {
-            const int nj = min(S64_SCH, sB1 - j0);
-            __syncwarp();
-            if (lane < nj) sdB[warp][lane] = ssid[j0 + lane];
-            for (int k = lane; k < nj * 3; k += 32) (&sxB[warp][0][0])[k] = ys[3 * int64_t(j0) + k];
-            for (int k = lane; k < S64_SCH * 6; k += 32) (&saccB[warp][0][0])[k] = 0.0;
-            {
-                const double2 *src = reinterpret_cast<const double2 *>(P64 + int64_t(108) * j0);
-                double2 *dst = reinterpret_cast<double2 *>(wPB);
-                for (int k = lane; k < nj * 54; k += 32) dst[k] = __ldg(src + k);
-            }
-            __syncwarp();
-            for (int jj = 0; jj < nj; jj += ls) {
-                const int jl = jj + tj;
-                const int j = j0 + jl;
-                const bool on = vi && jl < nj && (!self || j > i) && sdB[warp][jl] != segi;
-                double fw[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, rv[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-                if (on) {
-                    const double d3[3] = {xi[0] - sxB[warp][jl][0], xi[1] - sxB[warp][jl][1], xi[2] - sxB[warp][jl][2]};
-                    const double r2 = d3[0] * d3[0] + d3[1] * d3[1] + d3[2] * d3[2];
-                    if (r2 > 0.0) {
-                        const double ir = rsqrt(r2);
-                        const double T[3] = {d3[0] * ir, d3[1] * ir, d3[2] * ir};
-                        double hs[18];
-                        if (HM == HM_CUBIC)
-                            h_cubic_tab<double>(cp, c44, cd, Q, sTc, sTs, T, hs);
-                        else
-                            h_circle_sym<double, double>(sC, Q, T, hs);
-                        const double *Pj = wPB + 108 * jl;
-#pragma unroll
-                        for (int c = 0; c < 108; ++c) {
-                            fw[c / 18] = fma(Pj[c], hs[c % 18], fw[c / 18]);
-                            rv[c / 18] = fma(Pi[c], hs[c % 18], rv[c / 18]);
-                        }
-                        const double ir2 = ir * ir;
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) {
-                            acc[ab] += fw[ab] * ir2;
-                            rv[ab] *= -ir2;
-                        }
-                    }
-                }
-                for (int off = 1; off < tg; off <<= 1)
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) rv[ab] += __shfl_xor_sync(0xffffffffu, rv[ab], off);
-                if (ti == 0 && jl < nj)
-#pragma unroll
-                    for (int ab = 0; ab < 6; ++ab) saccB[warp][jl][ab] += rv[ab];
-            }
-            __syncwarp();
-            for (int k = lane; k < nj * 6; k += 32) {
-                const int jl = k / 6, ab = k % 6;
-                double *dst = part + (int64_t(slot_r) * N + (j0 + jl)) * 6 + ab;
-                const double v = saccB[warp][jl][ab];
-                *dst = first_chunk ? v : *dst + v;
-            }
-        }
-        first_chunk = false;
-        for (int off = tg; off < 32; off <<= 1)
-#pragma unroll
-            for (int ab = 0; ab < 6; ++ab) acc[ab] += __shfl_xor_sync(0xffffffffu, acc[ab], off);
-        if (vi && tj == 0)
-#pragma unroll
-            for (int ab = 0; ab < 6; ++ab) part[(int64_t(slot_f) * N + i) * 6 + ab] = acc[ab];
-    }
+template <typename R, bool SYM, bool LEARN>
+struct WarpShared {
+    static constexpr int kEntries = LEARN ? 64 : 32;  // list entries staged at a time
+    Stage<R, kTargets> tg;
+    Stage<R, kEntries> sr;
+    Acc<R> fwd[6][kTargets];
+    Acc<R> rev[SYM ? 6 : 1][SYM ? kEntries : 1];
+    int src[kEntries], pos[kEntries];  // sorted index and list position of the staged entries
+    int rstart[kRanges], rpos[kRanges], rpre[kRanges + 1];
+    unsigned char rdir[kRanges];
+    unsigned short queue[LEARN ? 2 : 1][LEARN ? 64 : 2];  // queued pairs: the plain rule's, the network's
+};
+
+// learned h: accepted bins, their polynomials, and the smallest distance squared over |S|^2
+struct NearLearned {
+    const uint32_t *binmask;  // bit set: the bin takes the plain rule
+    const float4 *poly;       // [bin][27]: 18 components x 6 coefficients (mlp.cu)
+    float rmin2, m2;
+};
+
+struct NearTree {
+    int L;
+    int64_t N;            // source points
+    int64_t n_t;          // target points
+    const TreeBox *box;
+    const int *tstart, *sstart;
+    const int *ref_start, *child_start;  // adaptive tree (else null)
+    const void *trec, *srec;
+    const NearPlan *plan;
+    const int *lp;
+    const NearItem *items;
+    unsigned long long *cnt;
+    double *rows;
+};
+
+template <typename R>
+constexpr int near_warps() { return sizeof(R) == 4 ? 4 : 2; }
+template <typename R>
+constexpr int near_blocks() { return sizeof(R) == 4 ? 3 : 4; }
+
+// h of one pair by the plain rule
+template <typename R, int HM>
+__device__ __forceinline__ void h_plain(const NearMedium<R> &md, const R *tab, const R T[3], R hs[18]) {
+    if constexpr (HM == HM_ISO)
+        h_iso_sym<R>(R(1), md.ha, T, hs);
+    else if constexpr (HM == HM_CUBIC)
+        h_cubic_moments<R>(md, tab, T, hs);
+    else if constexpr (HM == HM_POINTS)
+        h_general_points(md, tab, T, hs);
+    else
+        h_general_moments<R>(md, tab, T, hs);
 }
 
-// far field (L2P) plus the partial slots, in a fixed order
-__global__ void k_near_combine(int p, int nodes, int L, int64_t N, const TreeBox *__restrict__ box,
-                               const int *__restrict__ sstart, const int *__restrict__ pleaf,
-                               const double *__restrict__ xt, const float *__restrict__ S,
-                               const double *__restrict__ S64, const double *__restrict__ part,
-                               double *__restrict__ sig, const int *__restrict__ pfine,
-                               const float *__restrict__ S7) {
-    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (t >= N) return;
-    const int nlv = 1 << (L - 1);
-    const int64_t leaf = pleaf[t];
-    int cx, cy, cz;
-    cell_xyz3(leaf, nlv, cx, cy, cz);
-    double out[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (L >= 3 && S64) {
-        // FP64 local values (GBFMM_MIXED_F64T): interpolate in FP64
-        const int P3 = p * p * p;
-        const double h = box->H / nlv, ih = double(nlv) / box->H;
-        double bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP];
-        lagrange_1d<double>(p, (xt[3 * t] - (box->origin[0] + cx * h)) * ih, bx, nodes);
-        lagrange_1d<double>(p, (xt[3 * t + 1] - (box->origin[1] + cy * h)) * ih, by, nodes);
-        lagrange_1d<double>(p, (xt[3 * t + 2] - (box->origin[2] + cz * h)) * ih, bz, nodes);
-        const double *Sl = S64 + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 6;
-        for (int lz = 0; lz < p; ++lz)
-            for (int ly = 0; ly < p; ++ly) {
-                const double wyz = by[ly] * bz[lz];
-                for (int lx = 0; lx < p; ++lx) {
-                    const double w = bx[lx] * wyz;
-                    const double *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
-                    for (int ab = 0; ab < 6; ++ab) out[ab] += w * s6[ab];
-                }
-            }
-    } else if (L >= 3) {
-        const int P3 = p * p * p;
-        double h = box->H / nlv, ih = double(nlv) / box->H;
-        double c0[3] = {box->origin[0] + cx * h, box->origin[1] + cy * h, box->origin[2] + cz * h};
-        const float *Sl = S + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 6;
-        const int f = pfine ? pfine[t] : -1;
-        if (f >= 0) {
-            // a point of a split leaf: its child's local values and cell (adaptive tree)
-            h *= 0.5;
-            ih *= 2.0;
-            c0[0] += (f & 1) * h;
-            c0[1] += ((f >> 1) & 1) * h;
-            c0[2] += ((f >> 2) & 1) * h;
-            Sl = S7 + int64_t(f) * P3 * 6;
-        }
-        float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        float bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP];
-        lagrange_1d<float>(p, float((xt[3 * t] - c0[0]) * ih), bx, nodes);
-        lagrange_1d<float>(p, float((xt[3 * t + 1] - c0[1]) * ih), by, nodes);
-        lagrange_1d<float>(p, float((xt[3 * t + 2] - c0[2]) * ih), bz, nodes);
-        for (int lz = 0; lz < p; ++lz)
-            for (int ly = 0; ly < p; ++ly) {
-                const float wyz = by[ly] * bz[lz];
-                for (int lx = 0; lx < p; ++lx) {
-                    const float w = bx[lx] * wyz;
-                    const float *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
-                    for (int ab = 0; ab < 6; ++ab) acc[ab] += w * __ldg(s6 + ab);
-                }
-            }
-        for (int ab = 0; ab < 6; ++ab) out[ab] = double(acc[ab]);
-    }
-    for (int s = 0; s < kSlots; ++s) {
-        const int nb = s == 27 ? 13 : s;
-        const int bx = cx + nb % 3 - 1, by = cy + (nb / 3) % 3 - 1, bz = cz + nb / 9 - 1;
-        if (bx < 0 || by < 0 || bz < 0 || bx >= nlv || by >= nlv || bz >= nlv) continue;
-        const int64_t B = (int64_t(bz) * nlv + by) * nlv + bx;
-        if (sstart[B + 1] == sstart[B]) continue;
-        const double *ps = part + (int64_t(s) * N + t) * 6;
-        for (int ab = 0; ab < 6; ++ab) out[ab] += ps[ab];
-    }
-    for (int ab = 0; ab < 6; ++ab) sig[6 * t + ab] = out[ab];
-}
-
-// leaf-pair work items (A, d), heaviest first (log2 of |A| |B| buckets)
-__global__ void k_pairs_count(int64_t nl, int L, const int *__restrict__ sstart, int *__restrict__ cnt) {
-    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (l >= nl) return;
-    const int nA = sstart[l + 1] - sstart[l];
-    int c = 0;
-    if (nA > 0) {
-        const int nlv = 1 << (L - 1);
-        int x, y, z;
-        cell_xyz3(l, nlv, x, y, z);
-        for (int d = 0; d < 14; ++d) {
-            const int nb = 13 + d;
-            const int bx = x + nb % 3 - 1, by = y + (nb / 3) % 3 - 1, bz = z + nb / 9 - 1;
-            if (bx < 0 || by < 0 || bz < 0 || bx >= nlv || by >= nlv || bz >= nlv) continue;
-            const int64_t B = (int64_t(bz) * nlv + by) * nlv + bx;
-            if (sstart[B + 1] > sstart[B]) ++c;
-        }
-    }
-    cnt[l] = c;
-}
-
-__global__ void k_pairs_fill(int64_t nl, int L, const int *__restrict__ sstart, const int *__restrict__ off,
-                             int2 *__restrict__ items, int *__restrict__ keys, int *__restrict__ hist) {
-    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (l >= nl) return;
-    const int nA = sstart[l + 1] - sstart[l];
-    if (nA == 0) return;
-    const int nlv = 1 << (L - 1);
-    int x, y, z;
-    cell_xyz3(l, nlv, x, y, z);
-    int o = off[l];
-    for (int d = 0; d < 14; ++d) {
-        const int nb = 13 + d;
-        const int bx = x + nb % 3 - 1, by = y + (nb / 3) % 3 - 1, bz = z + nb / 9 - 1;
-        if (bx < 0 || by < 0 || bz < 0 || bx >= nlv || by >= nlv || bz >= nlv) continue;
-        const int64_t B = (int64_t(bz) * nlv + by) * nlv + bx;
-        const int nB = sstart[B + 1] - sstart[B];
-        if (nB == 0) continue;
-        const int64_t cost = d == 0 ? int64_t(nA) * nA / 2 + 1 : int64_t(nA) * nB;
-        const int key = 63 - (63 - __clzll(cost));
-        items[o] = make_int2(int(l), d);
-        keys[o] = key;
-        atomicAdd(&hist[key], 1);
-        ++o;
-    }
-}
-
-// ---------------------------------------------------------------- near field with the learned h
-// Angular bin of a folded direction (upper half-space): dominant axis face
-// (+z, +x, -x, +y, -y) and a 16 x 16 grid of the two other components.
-__device__ __forceinline__ int dir_bin(float x, float y, float z) {
+// Angular bin of a direction folded into the upper half-space (h is odd): dominant axis face
+// (+z, +x, -x, +y, -y) and a 16 x 16 grid of the two other components; (u, v): the place in the
+// bin, -1 .. 1; the sign of the fold is returned.  Any length.
+__device__ __forceinline__ float dir_bin(const float d[3], int &bin, float &u, float &v) {
+    const float sg = (d[2] > 0.f || (d[2] == 0.f && (d[1] > 0.f || (d[1] == 0.f && d[0] >= 0.f)))) ? 1.f : -1.f;
+    const float x = sg * d[0], y = sg * d[1], z = sg * d[2];
     const float ax = fabsf(x), ay = fabsf(y), az = fabsf(z);
     int f;
-    float u, v, m;
+    float p, q, m;
     if (az >= ax && az >= ay) {
-        f = 0, u = x, v = y, m = az;
+        f = 0, p = x, q = y, m = az;
     } else if (ax >= ay) {
-        f = x > 0.f ? 1 : 2, u = y, v = z, m = ax;
+        f = x > 0.f ? 1 : 2, p = y, q = z, m = ax;
     } else {
-        f = y > 0.f ? 3 : 4, u = x, v = z, m = ay;
+        f = y > 0.f ? 3 : 4, p = x, q = z, m = ay;
     }
-    const int bu = min(15, max(0, int((u / m + 1.f) * 8.f)));
-    const int bv = min(15, max(0, int((v / m + 1.f) * 8.f)));
-    return f * 256 + bu * 16 + bv;
+    const float im = recip(m), tp = (p * im + 1.f) * 8.f, tq = (q * im + 1.f) * 8.f;
+    const int bu = min(15, max(0, int(tp))), bv = min(15, max(0, int(tq)));
+    bin = f * 256 + bu * 16 + bv;
+    u = 2.f * (tp - float(bu)) - 1.f;
+    v = 2.f * (tq - float(bv)) - 1.f;
+    return sg;
 }
 
-constexpr int MSCH = 16;  // sources staged per warp chunk in the network kernel
-
-// Pairs at distance >= rmin x (source segment length) whose direction lies in
-// an angular bin the plain evaluator accepted use the network; the rest take
-// the plain path of k_near_mixed (FP32 cubic or generic rule, FP64
-// separation for close pairs).  Network pairs are queued per warp and
-// evaluated sixteen at a time by warp MMAs; every queued contribution is
-// added by the lane that queued it, in queue order (deterministic).
-template <bool CUBIC>
-__global__ void __launch_bounds__(WARPS * 32) k_near_mlp(
-    int p, int nodes, int L, int64_t nl, float near2, float rmin2, const TreeBox *__restrict__ box,
-    const DevMaterial *__restrict__ mat, const int *__restrict__ tstart, const double *__restrict__ xt,
-    const int64_t *__restrict__ tsid, const int *__restrict__ sstart, const float4 *__restrict__ yrel,
-    const double *__restrict__ ys, const float *__restrict__ c32, const int64_t *__restrict__ ssid,
-    const float *__restrict__ S, double *__restrict__ sig, const __nv_bfloat16 *__restrict__ th,
-    const float *__restrict__ th32, const float *__restrict__ hscale, const uint32_t *__restrict__ binmask,
-    const int2 *__restrict__ items, const int *__restrict__ n_items) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    mlpw::Weights &Wt = *reinterpret_cast<mlpw::Weights *>(dsm);
-    __shared__ __align__(16) float sP[WARPS][MSCH * 108];
-    __shared__ float4 sy[WARPS][MSCH];
-    __shared__ int ssd[WARPS][MSCH];
-    __shared__ float4 qd[WARPS][48];
-    __shared__ int qj[WARPS][48], ql[WARPS][48];
-    __shared__ float qc[WARPS][16][6];
-    __shared__ float sC[81];
-    __shared__ float2 sTab[128];
-    __shared__ uint32_t sBin[48];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int g = lane >> 2, tq = lane & 3;
-    mlpw::load(Wt, th, th32, hscale);
-    for (int i = threadIdx.x; i < 81; i += blockDim.x) sC[i] = float(mat->C[i]);
-    for (int i = threadIdx.x; i < mat->Q && i < 128; i += blockDim.x) {
-        float sn, cs;
-        sincospif(float(i) / float(mat->Q), &sn, &cs);
-        sTab[i] = make_float2(cs, sn);
+// h of one pair by the network's polynomial in its bin
+__device__ __forceinline__ void h_learned(const NearLearned &ln, const float d[3], float hs[18]) {
+    int bin;
+    float u, v;
+    const float sg = dir_bin(d, bin, u, v);
+    const float b1 = u, b2 = v, b3 = u * u - ln.m2, b4 = u * v, b5 = v * v - ln.m2;
+    const float4 *q = ln.poly + 27 * bin;
+#pragma unroll
+    for (int k = 0; k < 18; k += 2) {
+        const float4 a = __ldg(q + 3 * (k / 2)), b = __ldg(q + 3 * (k / 2) + 1), c = __ldg(q + 3 * (k / 2) + 2);
+        hs[k] = sg * (a.x + a.y * b1 + a.z * b2 + a.w * b3 + b.x * b4 + b.y * b5);
+        hs[k + 1] = sg * (b.z + b.w * b1 + c.x * b2 + c.y * b3 + c.z * b4 + c.w * b5);
     }
-    for (int i = threadIdx.x; i < 48; i += blockDim.x) sBin[i] = binmask[i];
-    __syncthreads();
-    // one work item per warp: up to 32 targets of one leaf, heaviest first
-    const int64_t item = blockIdx.x * int64_t(WARPS) + warp;
-    if (item >= *n_items) return;
-    const int2 wi = items[item];
-    const int64_t leaf = wi.x;
-    const int t0 = wi.y, t1 = min(wi.y + 32, tstart[leaf + 1]);
-    const int P3 = p * p * p;
-    const int nlv = 1 << (L - 1);
-    int cx, cy, cz;
-    cell_xyz3(leaf, nlv, cx, cy, cz);
-    const bool far = L >= 3;
-    const double h = box->H / nlv, ih = double(nlv) / box->H;
-    const double c0[3] = {box->origin[0] + cx * h, box->origin[1] + cy * h, box->origin[2] + cz * h};
-    const int Q = mat->Q;
-    const float c12f = float(mat->c12), c44f = float(mat->c44), cdf = float(mat->cd);
-    const float *Sl = S + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 6;
-    float *wP = sP[warp];
-    float4 *wy = sy[warp];
-    int *wsd = ssd[warp];
-    float4 *wq = qd[warp];
-    int *wj = qj[warp], *wl = ql[warp];
-    float(*wc)[6] = qc[warp];
-    for (int r0 = t0; r0 < t1; r0 += 32) {
-        const int nrem = min(32, t1 - r0);
-        int tg = 1;
-        while (tg < nrem) tg <<= 1;
-        const int ls = 32 / tg, tl = lane % tg, ph = lane / tg;
-        const int t = r0 + tl;
-        const bool valid = tl < nrem;
-        double x[3] = {0, 0, 0};
-        float xr[3] = {0.f, 0.f, 0.f};
-        float acc[6] = {0, 0, 0, 0, 0, 0};
-        double acc64[6] = {0, 0, 0, 0, 0, 0};
-        int myseg = -1;
-        if (valid) {
-            for (int d = 0; d < 3; ++d) {
-                x[d] = xt[3 * int64_t(t) + d];
-                xr[d] = float(x[d] - (c0[d] + 0.5 * h));
+}
+
+// A block of nt targets (from point tb) against the ns staged entries with the learned h.  The
+// pairs are visited along the diagonals of an M x M square (M = 32, or 64 where either side is
+// longer), classified, and queued by kind; 32 queued pairs make a step.  Pairs fewer than M - 1
+// places apart on that path share neither target nor entry, so a step whose pairs are adds to
+// the sums directly (the plain queue nearly always); otherwise lanes that share one add in the
+// order of their numbers.  Sorting costs ~90 instructions a visited pair and saves the ~1,900 of
+// the general rule for each learned one (100,000 segments in a turned crystal, Q = 32, a fifth
+// of the pairs learned; with the network's layers evaluated per pair, one-sided: 2,236 ms).
+template <int HM, bool SYM, typename Shared>
+__device__ __forceinline__ void learned_block(Shared &ws, const NearMedium<float> &md, const NearLearned &ln,
+                                              const float *tab, const uint32_t *mask, int tb, int nt, int ns, int lane) {
+    const int sh = nt > 32 || ns > 32 ? 6 : 5, M = 1 << sh;
+    const unsigned below = (1u << lane) - 1u;
+    int n0 = 0, n1 = 0;  // queued: plain, learned
+    for (int q0 = 0; q0 < M * M; q0 += 32) {
+        const int ti = (q0 + lane) & (M - 1), jl = (ti + (q0 >> sh)) & (M - 1);
+        if ((q0 & (M - 1)) < nt) {
+            bool on = ti < nt && jl < ns, net = false;
+            if (SYM) on = on && ws.src[jl] > tb + ti;
+            if (on) {
+                const Pt<float> pi = ws.tg.get(ti, false), pj = ws.sr.get(jl, false);
+                float d[3], u, v;
+                separation(pi, pj, d);
+                const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                on = pj.seg != pi.seg && r2 > 0.f;
+                int bin;
+                dir_bin(d, bin, u, v);
+                net = r2 >= ln.rmin2 * fmaxf(pi.len2, pj.len2) && !((mask[bin >> 5] >> (bin & 31)) & 1u);
             }
-            myseg = tsid ? int(tsid[t]) : -1;
+            const unsigned m0 = __ballot_sync(0xffffffffu, on && !net), m1 = __ballot_sync(0xffffffffu, on && net);
+            if (on) ws.queue[net][net ? n1 + __popc(m1 & below) : n0 + __popc(m0 & below)] = (unsigned short)(q0 + lane);
+            n0 += __popc(m0);
+            n1 += __popc(m1);
         }
-        if (far && ph == 0) {
-            float bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP];
-            lagrange_1d<float>(p, float((x[0] - c0[0]) * ih), bx, nodes);
-            lagrange_1d<float>(p, float((x[1] - c0[1]) * ih), by, nodes);
-            lagrange_1d<float>(p, float((x[2] - c0[2]) * ih), bz, nodes);
-            for (int lz = 0; lz < p; ++lz)
-                for (int ly = 0; ly < p; ++ly) {
-                    const float wyz = by[ly] * bz[lz];
-                    for (int lx = 0; lx < p; ++lx) {
-                        const float w = bx[lx] * wyz;
-                        const float *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
-                        for (int ab = 0; ab < 6; ++ab) acc[ab] += w * __ldg(s6 + ab);
+        const bool last = q0 + 32 >= M * M;
+#pragma unroll 1
+        for (int w = 0; w < 2; ++w) {
+            int n = w ? n1 : n0;
+            while (n >= 32 || (last && n > 0)) {
+                __syncwarp();
+                const int cnt = min(n, 32);
+                const bool on = lane < cnt;
+                const int place = on ? ws.queue[w][lane] : 0;
+                const int span = ws.queue[w][cnt - 1] - ws.queue[w][0];
+                const int it = place & (M - 1), je = (it + (place >> sh)) & (M - 1);
+                float ef[6], er[6];
+                if (on) {
+                    const Pt<float> pi = ws.tg.get(it, SYM), pj = ws.sr.get(je, true);
+                    float d[3];
+                    separation(pi, pj, d);
+                    const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                    const float ir = rsqrt_refined(r2), ir2 = ir * ir;
+                    float hs[18], Y[3][6];
+                    if (w == 0) {
+                        const float T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+                        h_plain<float, HM>(md, tab, T, hs);
+                    } else {
+                        h_learned(ln, d, hs);
                     }
+                    stress_rows<float, HM >= HM_POINTS>(md, hs, Y);
+                    strain_of<float>(Y, pj.b[0], pj.b[1], pj.b[2], ir2 * pj.S[0], ir2 * pj.S[1], ir2 * pj.S[2], ef);
+                    if (SYM)
+                        strain_of<float>(Y, pi.b[0], pi.b[1], pi.b[2], -ir2 * pi.S[0], -ir2 * pi.S[1], -ir2 * pi.S[2],
+                                         er);
                 }
-        }
-        int qn = 0;  // queued network pairs (warp-uniform)
-        for (int nb = 0; nb < 27; ++nb) {
-            const int dxn = nb % 3 - 1, dyn = (nb / 3) % 3 - 1, dzn = nb / 9 - 1;
-            const int ax = cx + dxn, ay = cy + dyn, az = cz + dzn;
-            if (ax < 0 || ay < 0 || az < 0 || ax >= nlv || ay >= nlv || az >= nlv) continue;
-            const int64_t A = (int64_t(az) * nlv + ay) * nlv + ax;
-            const int s0 = sstart[A], s1 = sstart[A + 1];
-            const float xs[3] = {xr[0] - float(dxn * h), xr[1] - float(dyn * h), xr[2] - float(dzn * h)};
-            for (int j0 = s0; j0 < s1; j0 += MSCH) {
-                const int nj = min(MSCH, s1 - j0);
-                __syncwarp();
-                if (lane < nj) {
-                    wy[lane] = yrel[j0 + lane];
-                    wsd[lane] = int(ssid[j0 + lane]);
+                int ri = on ? 0 : -1, rj = ri, rounds = 0;  // this lane's turn at its target and its entry
+                if (span >= M - 1) {
+                    ri = __popc(__match_any_sync(0xffffffffu, on ? it : 64 + lane) & below);
+                    rj = __popc(__match_any_sync(0xffffffffu, on ? je : 64 + lane) & below);
+                    if (!on) ri = rj = -1;
+                    rounds = __reduce_max_sync(0xffffffffu, max(ri, rj));
                 }
-                {
-                    const float4 *src = reinterpret_cast<const float4 *>(c32 + int64_t(108) * j0);
-                    float4 *dst = reinterpret_cast<float4 *>(wP);
-                    for (int i = lane; i < nj * 27; i += 32) dst[i] = __ldg(src + i);
-                }
-                __syncwarp();
-                const int nit = (nj + ls - 1) / ls;
-                for (int it = 0; it < nit; ++it) {
-                    const int j = ph + it * ls;
-                    bool eligible = false;
-                    float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (valid && j < nj && wsd[j] != myseg) {
-                        const float4 yj = wy[j];
-                        float d[3] = {xs[0] - yj.x, xs[1] - yj.y, xs[2] - yj.z};
-                        const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                        const bool close = r2 < near2 * yj.w * yj.w;
-                        bool ok = true;
-                        float ir;
-                        if (close) {
-                            const int64_t jj = j0 + j;
-                            const double dd0 = x[0] - ys[3 * jj], dd1 = x[1] - ys[3 * jj + 1], dd2 = x[2] - ys[3 * jj + 2];
-                            const double rr = dd0 * dd0 + dd1 * dd1 + dd2 * dd2;
-                            ok = rr != 0.0;
-                            d[0] = float(dd0);
-                            d[1] = float(dd1);
-                            d[2] = float(dd2);
-                            ir = ok ? float(rsqrt(rr)) : 0.f;
-                        } else {
-                            ir = rsqrtf(r2);
+#pragma unroll 1
+                for (int r = 0; r <= rounds; ++r) {
+                    // learned values carry the network's error: FP32 additions
+                    if (ri == r)
+#pragma unroll
+                        for (int e = 0; e < 6; ++e) {
+                            Acc<float> &a = ws.fwd[e][it];
+                            if (w) a.hi += ef[e];
+                            else a.add(ef[e]);
                         }
-                        if (ok) {
-                            const float T0 = d[0] * ir, T1 = d[1] * ir, T2 = d[2] * ir;
-                            const float sg = mlpw::fold_sign(T0, T1, T2);
-                            const int bin = dir_bin(sg * T0, sg * T1, sg * T2);
-                            const bool net = !close && r2 >= rmin2 * yj.w * yj.w && !((sBin[bin >> 5] >> (bin & 31)) & 1u);
-                            if (net) {
-                                eligible = true;
-                                qv = make_float4(T0, T1, T2, ir * ir);
-                            } else {
-                                float part[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                                if (CUBIC)
-                                    pair_generic<HM_CUBIC, float, float>(d, ir, wP + 108 * j, sC, Q, c12f, c44f, cdf,
-                                                                         part, sTab);
-                                else
-                                    pair_generic<HM_GENERIC, float, float>(d, ir, wP + 108 * j, sC, Q, c12f, c44f,
-                                                                           cdf, part, sTab);
-                                if (close) {
-                                    for (int ab = 0; ab < 6; ++ab) acc64[ab] += double(part[ab]);
-                                } else {
-                                    for (int ab = 0; ab < 6; ++ab) acc[ab] += part[ab];
+                    if (SYM && rj == r)
+#pragma unroll
+                        for (int e = 0; e < 6; ++e) {
+                            Acc<float> &a = ws.rev[e][je];
+                            if (w) a.hi += er[e];
+                            else a.add(er[e]);
+                        }
+                    __syncwarp();
+                }
+                // the rest of the queue moves up
+                n -= cnt;
+                const unsigned short rest = lane < n ? ws.queue[w][32 + lane] : (unsigned short)0;
+                __syncwarp();
+                if (lane < n) ws.queue[w][lane] = rest;
+            }
+            if (w) n1 = n;
+            else n0 = n;
+        }
+    }
+    __syncwarp();
+}
+
+template <typename R, int HM, bool SYM, bool LEARN>
+__global__ void __launch_bounds__(near_warps<R>() * 32, near_blocks<R>())
+    k_near_pairs(const __grid_constant__ NearTree tr, const __grid_constant__ NearMedium<R> md,
+                 const __grid_constant__ NearLearned ln) {
+    constexpr int NW = near_warps<R>(), D0 = SYM ? 13 : 0, ND = 27 - D0;
+    extern __shared__ __align__(16) unsigned char sm_near[];
+    typedef WarpShared<R, SYM, LEARN> Shared;
+    Shared &ws = reinterpret_cast<Shared *>(sm_near)[threadIdx.x / 32];
+    R *tab = reinterpret_cast<R *>(sm_near + NW * sizeof(Shared));
+    const int lane = threadIdx.x % 32;
+    __shared__ uint32_t s_mask[LEARN ? 48 : 1];
+    if constexpr (HM == HM_POINTS)
+        point_table(md.Q, tab);
+    else if (HM != HM_ISO)
+        moment_table<R>(md.Q, md.np, tab);
+    if (LEARN)
+        for (int i = threadIdx.x; i < 40; i += blockDim.x) s_mask[i] = ln.binmask[i];
+    __syncthreads();
+    const int nlv = 1 << (tr.L - 1);
+    const double edge = tr.box->H / nlv;
+    const float eh = float(edge), el = float(edge - double(eh));
+    const long long n_items = (long long)tr.cnt[kCntItems];
+    while (true) {
+        long long it = 0;
+        if (lane == 0) it = (long long)atomicAdd(&tr.cnt[kCntNext], 1ull);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= n_items) return;
+        const NearItem item = tr.items[it];
+        const int64_t A = item.leaf;
+        const NearPlan pl = tr.plan[A];
+        const int tA0 = tr.tstart[A], tA1 = tr.tstart[A + 1], nt = tA1 - tA0;
+        int ax, ay, az;
+        cell_xyz3(A, nlv, ax, ay, az);
+        const int s0 = item.b * pl.sb, s1 = min(pl.ns, s0 + pl.sb);
+        const long long fbase = pl.base + (long long)item.b * nt;
+        const long long rbase = pl.base + (long long)pl.cb * nt + (long long)item.a * pl.ns;
+        const int rA = SYM && tr.ref_start && tr.ref_start[A + 1] > tr.ref_start[A] ? tr.ref_start[A] : -1;
+        bool add = false;  // reverse rows: store, or add to what an earlier target block stored
+        if (SYM && rA >= 0) {
+            // a split leaf's children meet different parts of the list: the rows start from zero
+            for (int k = s0 + lane; k < s1; k += 32)
+                for (int e = 0; e < 6; ++e) tr.rows[(rbase + k) * 6 + e] = 0.0;
+            add = true;
+            __syncwarp();
+        }
+        const int g0 = rA >= 0 ? item.a * pl.ta : 0, g1 = rA >= 0 ? g0 + pl.ta : 1;  // children of the tile
+        for (int ch = g0; ch < g1; ++ch) {
+            const int b0 = rA >= 0 ? tr.child_start[9 * rA + ch] : tA0 + item.a * pl.ta;
+            const int b1 = rA >= 0 ? tr.child_start[9 * rA + ch + 1] : min(tA1, tA0 + (item.a + 1) * pl.ta);
+            for (int tb = b0; tb < b1; tb += kTargets) {
+                const int nb_t = min(kTargets, b1 - tb);
+                __syncwarp();
+                // the block's part of the list: whole leaves, or (two split leaves) the children
+                // adjacent to this one; in the own leaf only entries from the block's start on
+                int nr = 0, total = 0;
+                const int ne = rA >= 0 ? ND * 8 : ND;
+                for (int e0 = 0; e0 < ne; e0 += 32) {
+                    const int e = e0 + lane;
+                    int len = 0, start = 0, lpos = 0, dir = 0;
+                    if (e < ne) {
+                        dir = rA >= 0 ? e / 8 : e;
+                        const int ss = rA >= 0 ? e % 8 : 0, nb = D0 + dir;
+                        const int64_t B = neighbour(ax, ay, az, nb, nlv);
+                        if (B >= 0) {
+                            const int sB0 = tr.sstart[B], sB1 = tr.sstart[B + 1];
+                            lpos = tr.lp[ND * A + dir];
+                            const int rB = rA >= 0 && dir > 0 && tr.ref_start[B + 1] > tr.ref_start[B] ? tr.ref_start[B] : -1;
+                            if (rB >= 0) {
+                                const int ox = nb % 3 - 1, oy = (nb / 3) % 3 - 1, oz = nb / 9 - 1;
+                                const int dx = 2 * ox + (ss & 1) - (ch & 1),
+                                          dy = 2 * oy + ((ss >> 1) & 1) - ((ch >> 1) & 1),
+                                          dz = 2 * oz + (ss >> 2) - (ch >> 2);
+                                if (abs(dx) <= 1 && abs(dy) <= 1 && abs(dz) <= 1) {
+                                    start = tr.child_start[9 * rB + ss];
+                                    len = tr.child_start[9 * rB + ss + 1] - start;
+                                    lpos += start - sB0;
+                                }
+                            } else if (ss == 0) {
+                                start = sB0, len = sB1 - sB0;
+                            }
+                            int skip = max(0, s0 - lpos);
+                            if (SYM && dir == 0) skip = max(skip, tb - tA0);
+                            len = max(0, min(len, s1 - lpos) - skip);
+                            start += skip, lpos += skip;
+                        }
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, len > 0);
+                    int pre = len;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+                        if (lane >= o) pre += v;
+                    }
+                    if (len > 0) {
+                        const int k = nr + __popc(m & ((1u << lane) - 1u));
+                        ws.rstart[k] = start, ws.rpos[k] = lpos, ws.rpre[k] = total + pre - len;
+                        ws.rdir[k] = (unsigned char)(D0 + dir);
+                    }
+                    nr += __popc(m);
+                    total += __shfl_sync(0xffffffffu, pre, 31);
+                }
+                for (int k = lane; k < nb_t; k += 32) {
+                    ws.tg.load_target(tr.trec, tr.n_t, tb + k, k, SYM);
+                    for (int e = 0; e < 6; ++e) ws.fwd[e][k].zero();
+                }
+                for (int m0 = 0; m0 < total; m0 += Shared::kEntries) {
+                    const int ns = min(Shared::kEntries, total - m0);
+                    __syncwarp();
+                    for (int k = lane; k < ns; k += 32) {
+                        int lo = 0, hi = nr;  // last range that starts at or before this entry
+                        while (hi - lo > 1) {
+                            const int mid = (lo + hi) >> 1;
+                            if (ws.rpre[mid] <= m0 + k) lo = mid;
+                            else hi = mid;
+                        }
+                        const int off = m0 + k - ws.rpre[lo], j = ws.rstart[lo] + off, nb = ws.rdir[lo];
+                        ws.src[k] = j;
+                        ws.pos[k] = ws.rpos[lo] + off;
+                        ws.sr.load_source(tr.srec, tr.N, j, k, nb % 3 - 1, (nb / 3) % 3 - 1, nb / 9 - 1, eh, el);
+                    }
+                    if (SYM)
+                        for (int k = lane; k < Shared::kEntries; k += 32)
+                            for (int e = 0; e < 6; ++e) ws.rev[e][k].zero();
+                    __syncwarp();
+                    if constexpr (LEARN) learned_block<HM, SYM>(ws, md, ln, tab, s_mask, tb, nb_t, ns, lane);
+                    for (int c0 = LEARN ? nb_t : 0; c0 < nb_t;) {
+                        // tg steps cover tg targets: the next power of two where that wastes at most
+                        // two steps, else the largest that fits
+                        const int left = nb_t - c0;
+                        const int tg = left >= 30 ? 32 : left >= 15 ? 16 : left >= 7 ? 8 : left >= 3 ? 4 : left;
+                        const int ti = lane & (tg - 1), tj = lane / tg;
+                        const int i = tb + c0 + ti;
+                        const bool vi = ti < left;
+                        const Pt<R> pi = ws.tg.get(vi ? c0 + ti : 0, SYM);
+                        Acc<R> f[6];
+#pragma unroll
+                        for (int e = 0; e < 6; ++e) f[e].zero();
+                        for (int s = 0; s < tg; ++s) {
+                            const int jl = tj * tg + ((ti + s) & (tg - 1));
+                            bool on = vi && jl < ns;
+                            if (SYM) on = on && ws.src[jl] > i;
+                            if (on) {
+                                const Pt<R> pj = ws.sr.get(jl, true);
+                                R d[3];
+                                separation(pi, pj, d);
+                                const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                                if (pj.seg != pi.seg && r2 > R(0)) {
+                                    const R ir = rsqrt_refined(r2), ir2 = ir * ir;
+                                    const R T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+                                    R hs[18];
+                                    h_plain<R, HM>(md, tab, T, hs);
+                                    R Y[3][6], e6[6];
+                                    stress_rows<R, HM >= HM_POINTS>(md, hs, Y);
+                                    strain_of<R>(Y, pj.b[0], pj.b[1], pj.b[2], ir2 * pj.S[0], ir2 * pj.S[1],
+                                                 ir2 * pj.S[2], e6);
+#pragma unroll
+                                    for (int e = 0; e < 6; ++e) f[e].add(e6[e]);
+                                    if (SYM) {
+                                        strain_of<R>(Y, pi.b[0], pi.b[1], pi.b[2], -ir2 * pi.S[0], -ir2 * pi.S[1],
+                                                     -ir2 * pi.S[2], e6);
+#pragma unroll
+                                        for (int e = 0; e < 6; ++e) {
+                                            Acc<R> a = ws.rev[e][jl];
+                                            a.add(e6[e]);
+                                            ws.rev[e][jl] = a;
+                                        }
+                                    }
                                 }
                             }
+                            if (SYM) __syncwarp();
                         }
-                    }
-                    // enqueue this iteration's network pairs in lane order
-                    const unsigned m = __ballot_sync(0xffffffffu, eligible);
-                    if (eligible) {
-                        const int pos = qn + __popc(m & ((1u << lane) - 1u));
-                        wq[pos] = qv;
-                        wj[pos] = j;
-                        wl[pos] = lane;
-                    }
-                    qn += __popc(m);
-                    __syncwarp();
-                    // evaluate full tiles of 16 (and the remainder at the chunk's end)
-                    while (qn >= 16 || (qn > 0 && it == nit - 1)) {
-                        const int nrow = min(16, qn);
-                        const bool vlo = g < nrow, vhi = g + 8 < nrow;
-                        const float4 ql4 = vlo ? wq[g] : make_float4(0.f, 0.f, 1.f, 0.f);
-                        const float4 qh4 = vhi ? wq[g + 8] : make_float4(0.f, 0.f, 1.f, 0.f);
-                        const float slo = mlpw::fold_sign(ql4.x, ql4.y, ql4.z);
-                        const float shi = mlpw::fold_sign(qh4.x, qh4.y, qh4.z);
-                        const float dlo[3] = {slo * ql4.x, slo * ql4.y, slo * ql4.z};
-                        const float dhi[3] = {shi * qh4.x, shi * qh4.y, shi * qh4.z};
-                        float olo[8], ohi[8];
-                        mlpw::eval16(Wt, dlo, dhi, g, tq, olo, ohi);
-                        float plo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, phi[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                        const float *Plo = wP + 108 * (vlo ? wj[g] : 0), *Phi = wP + 108 * (vhi ? wj[g + 8] : 0);
+                        // the lanes that share a target (fixed order), then the block's sums
+                        for (int o = tg; o < 32; o <<= 1)
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const int col = 8 * (e >> 1) + 2 * tq + (e & 1);
-                            if (col >= 27) continue;
-                            const int v = col / 9, pp = (col / 3) % 3, q = col % 3;
-                            constexpr int PIX[9] = {0, 5, 4, 5, 1, 3, 4, 3, 2};
-                            const int k = 3 * PIX[v * 3 + pp] + q;
-                            const float wgt = (v == pp ? 1.f : 0.5f) * Wt.scale[col];
-                            const float hl = olo[e] * wgt * slo, hh = ohi[e] * wgt * shi;
+                            for (int e = 0; e < 6; ++e) f[e].add(f[e].shfl_xor(o));
+                        if (vi && tj == 0)
 #pragma unroll
-                            for (int ab = 0; ab < 6; ++ab) {
-                                plo[ab] += Plo[ab * 18 + k] * hl;
-                                phi[ab] += Phi[ab * 18 + k] * hh;
+                            for (int e = 0; e < 6; ++e) {
+                                Acc<R> a = ws.fwd[e][c0 + ti];
+                                a.add(f[e]);
+                                ws.fwd[e][c0 + ti] = a;
+                            }
+                        c0 += tg;
+                    }
+                    if (SYM) {
+                        __syncwarp();
+                        for (int k = lane; k < ns; k += 32) {
+                            double *row = tr.rows + (rbase + ws.pos[k]) * 6;
+                            for (int e = 0; e < 6; ++e) {
+                                const double v = ws.rev[e][k].value();
+                                row[e] = add ? row[e] + v : v;
                             }
                         }
-#pragma unroll
-                        for (int ab = 0; ab < 6; ++ab) {
-                            plo[ab] += __shfl_xor_sync(0xffffffffu, plo[ab], 1);
-                            plo[ab] += __shfl_xor_sync(0xffffffffu, plo[ab], 2);
-                            phi[ab] += __shfl_xor_sync(0xffffffffu, phi[ab], 1);
-                            phi[ab] += __shfl_xor_sync(0xffffffffu, phi[ab], 2);
-                        }
-                        if (tq == 0 && vlo)
-                            for (int ab = 0; ab < 6; ++ab) wc[g][ab] = plo[ab] * ql4.w;
-                        if (tq == 1 && vhi)
-                            for (int ab = 0; ab < 6; ++ab) wc[g + 8][ab] = phi[ab] * qh4.w;
-                        __syncwarp();
-                        for (int r = 0; r < nrow; ++r)
-                            if (wl[r] == lane)
-                                for (int ab = 0; ab < 6; ++ab) acc[ab] += wc[r][ab];
-                        __syncwarp();
-                        // drop the evaluated rows
-                        const int rest = qn - nrow;
-                        float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
-                        int mj = 0, ml = 0;
-                        if (lane < rest) {
-                            mv = wq[nrow + lane];
-                            mj = wj[nrow + lane];
-                            ml = wl[nrow + lane];
-                        }
-                        __syncwarp();
-                        if (lane < rest) {
-                            wq[lane] = mv;
-                            wj[lane] = mj;
-                            wl[lane] = ml;
-                        }
-                        qn = rest;
-                        __syncwarp();
                     }
                 }
+                __syncwarp();
+                for (int k = lane; k < nb_t; k += 32) {
+                    double *row = tr.rows + (fbase + (tb - tA0) + k) * 6;
+                    for (int e = 0; e < 6; ++e) row[e] = ws.fwd[e][k].value();
+                }
+                add = true;
             }
         }
-        for (int off = tg; off < 32; off <<= 1)
-            for (int ab = 0; ab < 6; ++ab) {
-                acc[ab] += __shfl_xor_sync(0xffffffffu, acc[ab], off);
-                acc64[ab] += __shfl_xor_sync(0xffffffffu, acc64[ab], off);
-            }
-        if (valid && ph == 0)
-            for (int ab = 0; ab < 6; ++ab) sig[6 * int64_t(t) + ab] = double(acc[ab]) + acc64[ab];
     }
 }
 
-// ---------------------------------------------------------------- work list
-// Items are (leaf, first target) for every 32 targets of a leaf; the cost of
-// an item is ~ (its targets) x (sources in the 27 neighbour leaves).  Items
-// are ordered by decreasing cost class (floor log2) so that the heaviest
-// start first and the uneven leaf populations of clustered networks do not
-// leave a long tail.
-__global__ void k_items_count(int64_t nl, int L, const int *__restrict__ tstart, const int *__restrict__ sstart,
-                              int *__restrict__ cnt, int *__restrict__ key_cnt) {
-    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (l >= nl) return;
-    const int nt = tstart[l + 1] - tstart[l];
-    cnt[l] = (nt + 31) / 32;
-    if (nt == 0) return;
-    const int nlv = 1 << (L - 1);
+// ---------------------------------------------------------------- combine
+// far field (L2P) plus the stress of the summed strain rows, in a fixed order
+template <typename SR>
+__device__ __forceinline__ void l2p(int p, int nodes, const double c0[3], double ih, const double *x,
+                                    const SR *__restrict__ Sl, double out[6]) {
+    SR bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP], acc[6];
+    for (int e = 0; e < 6; ++e) acc[e] = SR(0);
+    lagrange_1d<SR>(p, SR((x[0] - c0[0]) * ih), bx, nodes);
+    lagrange_1d<SR>(p, SR((x[1] - c0[1]) * ih), by, nodes);
+    lagrange_1d<SR>(p, SR((x[2] - c0[2]) * ih), bz, nodes);
+    for (int lz = 0; lz < p; ++lz)
+        for (int ly = 0; ly < p; ++ly) {
+            const SR wyz = by[ly] * bz[lz];
+            for (int lx = 0; lx < p; ++lx) {
+                const SR w = bx[lx] * wyz;
+                const SR *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
+                for (int e = 0; e < 6; ++e) acc[e] += w * __ldg(s6 + e);
+            }
+        }
+    for (int e = 0; e < 6; ++e) out[e] = double(acc[e]);
+}
+
+template <bool SYM>
+__global__ void k_near_combine(int p, int nodes, const __grid_constant__ NearTree tr, const double *__restrict__ C,
+                               const int *__restrict__ tleaf, const double *__restrict__ xt,
+                               const float *__restrict__ S, const double *__restrict__ S64, double *__restrict__ sig,
+                               const int *__restrict__ pfine, const float *__restrict__ S7) {
+    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (t >= tr.n_t) return;
+    const int nlv = 1 << (tr.L - 1);
+    const int64_t leaf = tleaf[t];
     int cx, cy, cz;
-    cell_xyz3(l, nlv, cx, cy, cz);
-    int64_t ns = 0;
-    for (int nb = 0; nb < 27; ++nb) {
-        const int ax = cx + nb % 3 - 1, ay = cy + (nb / 3) % 3 - 1, az = cz + nb / 9 - 1;
-        if (ax < 0 || ay < 0 || az < 0 || ax >= nlv || ay >= nlv || az >= nlv) continue;
-        const int64_t A = (int64_t(az) * nlv + ay) * nlv + ax;
-        ns += sstart[A + 1] - sstart[A];
-    }
-    const int64_t cost = int64_t(min(nt, 32)) * ns;
-    const int key = cost > 0 ? 63 - __clzll(cost) : 0;  // floor log2
-    key_cnt[l] = key;
-}
-
-__global__ void k_items_fill(int64_t nl, const int *__restrict__ tstart, const int *__restrict__ off,
-                             const int *__restrict__ key_of, int2 *__restrict__ items, int *__restrict__ keys,
-                             int *__restrict__ hist) {
-    const int64_t l = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (l >= nl) return;
-    const int t0 = tstart[l], t1 = tstart[l + 1];
-    const int key = 63 - key_of[l];
-    int o = off[l];
-    for (int r0 = t0; r0 < t1; r0 += 32, ++o) {
-        items[o] = make_int2(int(l), r0);
-        keys[o] = key;
-        atomicAdd(&hist[key], 1);
-    }
-}
-
-__global__ void k_items_order(int n_total_cap, const int *__restrict__ total, const int2 *__restrict__ items,
-                              const int *__restrict__ keys, const int *__restrict__ hist, int *__restrict__ cursor,
-                              int2 *__restrict__ sorted, int *__restrict__ n_items) {
-    __shared__ int base[64];
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int k = 0; k < 64; ++k) {
-            base[k] = run;
-            run += hist[k];
+    cell_xyz3(leaf, nlv, cx, cy, cz);
+    double far[6];
+    const int f = pfine ? pfine[t] : -1;
+    {
+        const int P3 = p * p * p;
+        double h = tr.box->H / nlv, ih = double(nlv) / tr.box->H;
+        double c0[3] = {tr.box->origin[0] + cx * h, tr.box->origin[1] + cy * h, tr.box->origin[2] + cz * h};
+        const int64_t cell = (cell_base_d(tr.L - 1) + leaf) * int64_t(P3) * 6;
+        if (S64) {
+            l2p<double>(p, nodes, c0, ih, xt + 3 * t, S64 + cell, far);
+        } else {
+            const float *Sl = S + cell;
+            if (f >= 0) {
+                // a point of a split leaf: its child's local values and cell (adaptive tree)
+                h *= 0.5;
+                ih *= 2.0;
+                c0[0] += (f & 1) * h;
+                c0[1] += ((f >> 1) & 1) * h;
+                c0[2] += ((f >> 2) & 1) * h;
+                Sl = S7 + int64_t(f) * P3 * 6;
+            }
+            l2p<float>(p, nodes, c0, ih, xt + 3 * t, Sl, far);
         }
     }
-    __syncthreads();
-    const int n = *total;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_items = n;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n && i < n_total_cap; i += gridDim.x * blockDim.x) {
-        const int k = keys[i];
-        sorted[base[k] + atomicAdd(&cursor[k], 1)] = items[i];
+    double e6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    auto add_row = [&](long long r) {
+        const double2 *q = reinterpret_cast<const double2 *>(tr.rows + r * 6);
+        const double2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+        e6[0] += a.x, e6[1] += a.y, e6[2] += b.x, e6[3] += b.y, e6[4] += c.x, e6[5] += c.y;
+    };
+    {
+        const NearPlan pl = tr.plan[leaf];
+        const int nt = tr.tstart[leaf + 1] - tr.tstart[leaf], k = int(t - tr.tstart[leaf]);
+        for (int b = 0; b < pl.cb; ++b) add_row(pl.base + (long long)b * nt + k);
     }
-}
-
-__global__ void k_scan_small(int64_t n, const int *__restrict__ cnt, int *__restrict__ start) {
-    // exclusive scan, one block of 1024 threads (cnt -> start[0..n])
-    __shared__ int part[1024];
-    const int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    const int64_t b = threadIdx.x * per, e = min(n, b + per);
-    int s = 0;
-    for (int64_t i = b; i < e; ++i) s += cnt[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int t = 0; t < int(blockDim.x); ++t) {
-            const int v = part[t];
-            part[t] = run;
-            run += v;
+    if (SYM) {
+        const int rank = int(t - tr.sstart[leaf]);
+        for (int d = 0; d < 14; ++d) {
+            // the leaf that holds this one in direction d of its list
+            const int64_t A = neighbour(cx, cy, cz, 13 - d, nlv);
+            if (A < 0) continue;
+            const int nt = tr.tstart[A + 1] - tr.tstart[A];
+            if (nt == 0) continue;
+            const NearPlan pl = tr.plan[A];
+            const long long r = pl.base + (long long)pl.cb * nt + tr.lp[14 * A + d] + rank;
+            const bool splitA = tr.ref_start && tr.ref_start[A + 1] > tr.ref_start[A];
+            // a plain leaf's tile meets its own leaf from the tile's first target on; a split
+            // leaf's rows were zeroed first
+            const int ca = splitA || d > 0 ? pl.ca : min(pl.ca, rank / pl.ta + 1);
+            const int nb = 13 + d, ox = nb % 3 - 1, oy = (nb / 3) % 3 - 1, oz = nb / 9 - 1;
+            const bool skip = splitA && pl.ca == 8 && f >= 0 && d > 0;  // one child per tile: adjacent ones only
+            for (int a = 0; a < ca; ++a) {
+                if (skip && (abs(2 * ox + (f & 1) - (a & 1)) > 1 || abs(2 * oy + ((f >> 1) & 1) - ((a >> 1) & 1)) > 1 ||
+                             abs(2 * oz + ((f >> 2) & 1) - (a >> 2)) > 1))
+                    continue;
+                add_row(r + (long long)a * pl.ns);
+            }
         }
-        start[n] = run;
     }
-    __syncthreads();
-    int run = part[threadIdx.x];
-    for (int64_t i = b; i < e; ++i) {
-        start[i] = run;
-        run += cnt[i];
+    for (int m = 0; m < 6; ++m) {
+        double s = far[m];
+        for (int e = 0; e < 6; ++e) s += C[6 * m + e] * e6[e];
+        sig[6 * t + m] = s;
     }
 }
 
 }  // namespace
 
-int near_coef_count(const gbfmm_ctx *ctx) { return ctx->mat.mode == GBFMM_H_ISO ? 80 : 108; }
+// ---------------------------------------------------------------- host side
+int mlp_tabulate(gbfmm_ctx *ctx);  // mlp.cu: the network's polynomials, when they are out of date
+float mlp_poly_m2();
 
+static bool near_learned(const gbfmm_ctx *ctx) {
+    return ctx->mat.mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64;
+}
+
+template <typename R>
+static NearMedium<R> near_medium(const DevMaterial &m) {
+    NearMedium<R> n{};
+    n.Q = m.Q;
+    n.np = (m.Q - 1) / 2;
+    n.ha = R(m.ha);
+    const double cp = m.c12 + m.c44, D = m.cd, c44 = m.c44;
+    const double d0 = c44 * c44 * (c44 + D + cp), d1 = c44 * D * (D + 2.0 * cp);
+    n.al = R(c44 * (c44 + D + cp));
+    n.be = R(c44 * (D + cp));
+    n.ga = R(D * (D + 2.0 * cp));
+    n.d1 = R(d1);
+    n.d2 = R(D * D * (D + 3.0 * cp));
+    n.e0 = R(d0 + 0.5 * d1);
+    n.c44 = R(c44);
+    n.cd = R(D);
+    n.mcp = R(-cp);
+    n.y12 = R(m.c12);
+    n.ydiag = R(D + 2.0 * c44);
+    n.y44 = R(c44);
+    static const int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
+    auto C = [&m](int i, int j, int k, int l) { return m.C[((i * 3 + j) * 3 + k) * 3 + l]; };
+    for (int a = 0; a < 6; ++a)
+        for (int x = 0; x < 6; ++x) {
+            n.C[6 * a + x] = R(m.V[6 * a + x]);
+            // (zz)_jk = z_i C_ijkl z_l
+            const int j = PV[a], k = PP[a], i = PV[x], l = PP[x];
+            n.Z[6 * a + x] = R(C(i, j, k, l) + (i != l ? C(l, j, k, i) : 0.0));
+        }
+    return n;
+}
+
+// rows and items that a pass may use: functions of the network's size alone (near_plan).  An
+// undivided plan needs 15 rows a point (forward one, 14 leaves hold it in their lists) and one
+// item per occupied leaf; the rest is room to divide the work.
+static int64_t rows_sym(int64_t N) { return 32 * N + std::min<int64_t>(int64_t(1) << 20, N * N / 8 + 64); }
+static int64_t rows_free(int64_t n) { return 4 * n + (int64_t(1) << 18); }
+static int64_t items_cap(int64_t n, int64_t nl) { return n / 2 + std::min(n, nl) + 65536; }
+
+// buffers of the pair kernel for n targets (records of the targets only when they are free)
+static int pairs_alloc(gbfmm_ctx *ctx, int64_t n, bool free_targets) {
+    NearWork &W = ctx->nw;
+    const bool f32 = ctx->opt.precision != GBFMM_FP64;
+    const int64_t nl = ctx->n_leaves, rows = free_targets ? rows_free(n) : rows_sym(n), it = items_cap(n, nl);
+    const size_t point = f32 ? 4 * sizeof(float4) : 5 * sizeof(double2), target = 2 * sizeof(float4);
+    if (int rc = grow_dev(ctx, W.rec_cap, ctx->N, {{&W.rec, size_t(ctx->N) * point}}, "near-field points")) return rc;
+    if (free_targets)
+        if (int rc = grow_dev(ctx, W.trec_cap, n, {{&W.trec, size_t(n) * target}}, "near-field targets")) return rc;
+    if (int rc = grow_dev(ctx, W.plan_cap, nl,
+                          {{(void **)&W.plan, size_t(nl) * sizeof(NearPlan)}, {(void **)&W.lp, size_t(nl) * 27 * sizeof(int)}},
+                          "near-field plan"))
+        return rc;
+    if (int rc = grow_dev(ctx, W.item_cap, it, {{(void **)&W.pitems, size_t(it) * sizeof(NearItem)}}, "near-field items"))
+        return rc;
+    if (int rc = grow_dev(ctx, W.row_cap, rows, {{(void **)&W.rows, size_t(rows) * 6 * sizeof(double)}}, "near-field sums"))
+        return rc;
+    if (!W.pcnt) CK(cudaMalloc(&W.pcnt, kCnt * sizeof(unsigned long long)));
+    return GBFMM_OK;
+}
+
+int near_alloc(gbfmm_ctx *ctx) { return pairs_alloc(ctx, ctx->N, false); }
+
+// the records of the source points
 int near_prepare(gbfmm_ctx *ctx) {
     const int64_t N = ctx->N;
     ++ctx->launches;
-    if (near_coef_count(ctx) == 80)
-        k_src_coef80<<<nblk(N, 128), 128, 0, ctx->stream>>>(N, ctx->d_q, ctx->d_Asym, float(ctx->mat.hc),
-                                                              float(ctx->mat.ha), ctx->d_Pf);
+    GaussWeights gw{};
+    gw.n = ctx->opt.n_gauss;
+    for (int i = 0; i < gw.n; ++i) gw.w[i] = ctx->gauss_w[i];
+    // h of the unit-circle rule is summed without its factor 1 / (4 pi Q), the isotropic one without hc
+    const double fac = ctx->mat.mode == GBFMM_H_ISO ? ctx->mat.hc : 1.0 / (4.0 * M_PI * ctx->mat.Q);
+    if (ctx->opt.precision == GBFMM_FP64)
+        k_near_records<double><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
+                                                                       ctx->d_pleaf, ctx->node_xyz, ctx->seg_nodes,
+                                                                       ctx->burgers, gw, fac, ctx->nw.rec);
     else
-        k_src_coef108<<<nblk(N, kCoefPts), 256, 0, ctx->stream>>>(N, ctx->d_q, ctx->d_Asym, ctx->d_Pf);
+        k_near_records<float><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
+                                                                      ctx->d_pleaf, ctx->node_xyz, ctx->seg_nodes,
+                                                                      ctx->burgers, gw, fac, ctx->nw.rec);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }
 
-// capacity of the near-field work list for n_targets targets: called when
-// the tree is built, so that an evaluation recorded into a CUDA graph
-// allocates nothing
-int near_alloc(gbfmm_ctx *ctx, int64_t n_targets) {
-    const int64_t nl = ctx->n_leaves;
-    const int64_t cap = nl + n_targets / 32 + 1;
-    NearWork &W = ctx->nw;
-    if (nl > W.cap_leaves) W.cap = 0;  // the per-leaf arrays grow with the item arrays
-    const int64_t cap0 = W.cap;
-    if (int rc = grow_dev(ctx, W.cap, cap,
-                          {{(void **)&W.items, cap * sizeof(int2)}, {(void **)&W.sorted, cap * sizeof(int2)},
-                           {(void **)&W.keys, cap * sizeof(int)}, {(void **)&W.cnt, nl * sizeof(int)},
-                           {(void **)&W.key_of, nl * sizeof(int)}, {(void **)&W.off, (nl + 1) * sizeof(int)},
-                           {(void **)&W.misc, 192 * sizeof(int)}},  // hist[64], cursor[64], n_items, total
-                          "near-field work list")) {
-        W.cap_leaves = 0;
-        return rc;
-    }
-    if (W.cap != cap0) W.cap_leaves = nl;
-    return GBFMM_OK;
-}
-
-// work list for the near kernels (no host synchronisation: the item count
-// stays on the device and surplus warps return)
-static int build_items(gbfmm_ctx *ctx, const int *tstart, int64_t n_targets, int *&n_items, int2 *&items,
-                       int64_t &cap) {
-    const int64_t nl = ctx->n_leaves;
-    cap = nl + n_targets / 32 + 1;
-    if (int rc = near_alloc(ctx, n_targets)) return rc;
-    NearWork &W = ctx->nw;
-    cudaStream_t st = ctx->stream;
-    CK(cudaMemsetAsync(W.misc, 0, 192 * sizeof(int), st));
-    CK(cudaMemsetAsync(W.key_of, 0, nl * sizeof(int), st));
-    ctx->launches += 4;
-    k_items_count<<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->L, tstart, ctx->d_leaf_start, W.cnt, W.key_of);
-    k_scan_small<<<1, 1024, 0, st>>>(nl, W.cnt, W.off);
-    k_items_fill<<<nblk(nl, 256), 256, 0, st>>>(nl, tstart, W.off, W.key_of, W.items, W.keys, W.misc);
-    k_items_order<<<nblk(cap, 256) < 1024 ? nblk(cap, 256) : 1024, 256, 0, st>>>(
-        int(cap), W.off + nl, W.items, W.keys, W.misc, W.misc + 64, W.sorted, W.misc + 128);
-    CK(cudaGetLastError());
-    n_items = W.misc + 128;
-    items = W.sorted;
-    return GBFMM_OK;
-}
-
-// the symmetric kernel applies to nodal forces with the unit-circle h
-static bool near_symmetric(const gbfmm_ctx *ctx) { return ctx->mat.mode == GBFMM_H_CIRCLE; }
-
-int near_sym_alloc(gbfmm_ctx *ctx) {
-    if (!near_symmetric(ctx)) return GBFMM_OK;
-    NearWork &W = ctx->nw;
-    const int64_t pcap = 14 * ctx->n_leaves;
-    if (int rc = grow_dev(ctx, W.pcap, pcap,
-                          {{(void **)&W.pitems, pcap * sizeof(int2)}, {(void **)&W.psorted, pcap * sizeof(int2)},
-                           {(void **)&W.pkeys, pcap * sizeof(int)}, {(void **)&W.pmisc, 192 * sizeof(int)}},
-                          "near-field leaf pairs"))
-        return rc;
-    if (int rc = grow_dev(ctx, W.part_cap, ctx->N,
-                          {{(void **)&W.part, size_t(kSlots) * ctx->N * 6 * sizeof(double)}}, "near-field partial sums"))
-        return rc;
-    return GBFMM_OK;
-}
-
-// leaf-pair work items of the symmetric near fields, heaviest first (count, scan, fill, order)
-static int build_pair_items(gbfmm_ctx *ctx) {
-    const int64_t nl = ctx->n_leaves, N = ctx->N;
-    if (int rc = near_alloc(ctx, N)) return rc;
-    if (int rc = near_sym_alloc(ctx)) return rc;
-    NearWork &W = ctx->nw;
-    cudaStream_t st = ctx->stream;
-    CK(cudaMemsetAsync(W.pmisc, 0, 192 * sizeof(int), st));
-    ctx->launches += 4;
-    k_pairs_count<<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->L, ctx->d_leaf_start, W.cnt);
-    k_scan_small<<<1, 1024, 0, st>>>(nl, W.cnt, W.off);
-    k_pairs_fill<<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->L, ctx->d_leaf_start, W.off, W.pitems, W.pkeys, W.pmisc);
-    k_items_order<<<nblk(W.pcap, 256) < 1024 ? nblk(W.pcap, 256) : 1024, 256, 0, st>>>(
-        int(W.pcap), W.off + nl, W.pitems, W.pkeys, W.pmisc, W.pmisc + 64, W.psorted, W.pmisc + 128);
-    CK(cudaGetLastError());
-    return GBFMM_OK;
-}
-
-// FP64 pass, nodal forces with the unit-circle h: symmetric near field in FP64, then
-// L2P from the FP64 local values and the partial slots (k_near_combine)
-int near_run_sym64(gbfmm_ctx *ctx, double *sig) {
-    if (int rc = build_pair_items(ctx)) return rc;
-    const int64_t N = ctx->N;
-    NearWork &W = ctx->nw;
-    cudaStream_t st = ctx->stream;
-    const size_t smem = size_t(S64_WARPS) * (32 + S64_SCH) * 108 * sizeof(double);
-    const unsigned grid = nblk(W.pcap, S64_WARPS);
-    ctx->launches += 2;
-    if (ctx->mat.cubic) {
-        CK(cudaFuncSetAttribute(k_near_sym64<HM_CUBIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        k_near_sym64<HM_CUBIC><<<grid, S64_WARPS * 32, smem, st>>>(ctx->L, ctx->d_box, ctx->d_mat, ctx->d_leaf_start,
-                                                                   ctx->d_y, ctx->d_P, ctx->d_sid, W.part, N,
-                                                                   W.psorted, W.pmisc + 128);
-    } else {
-        CK(cudaFuncSetAttribute(k_near_sym64<HM_GENERIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        k_near_sym64<HM_GENERIC><<<grid, S64_WARPS * 32, smem, st>>>(ctx->L, ctx->d_box, ctx->d_mat,
-                                                                     ctx->d_leaf_start, ctx->d_y, ctx->d_P, ctx->d_sid,
-                                                                     W.part, N, W.psorted, W.pmisc + 128);
-    }
-    k_near_combine<<<nblk(N, 256), 256, 0, st>>>(ctx->opt.p, ctx->opt.nodes, ctx->L, N, ctx->d_box, ctx->d_leaf_start, ctx->d_pleaf,
-                                                 ctx->d_y, nullptr, ctx->d_S, W.part, sig, nullptr, nullptr);
-    CK(cudaGetLastError());
-    return GBFMM_OK;
-}
-
-static int near_run_sym(gbfmm_ctx *ctx, double *sig) {
-    if (int rc = build_pair_items(ctx)) return rc;
-    // adaptive tree (nodal forces): split leaves, their children's ranges and local values
-    const int *ref_start = ctx->rf.on && ctx->L >= 3 ? ctx->rf.ref_start : nullptr;
-    const int64_t N = ctx->N;
-    NearWork &W = ctx->nw;
-    cudaStream_t st = ctx->stream;
-    ctx->launches += 2;
-    const float near2 = float(ctx->opt.near_fp64 * ctx->opt.near_fp64);
-    const size_t smem = size_t(SYM_WARPS) * (32 + SYM_SCH) * 108 * sizeof(float);
-    const unsigned grid = nblk(W.pcap, SYM_WARPS);
-    if (ctx->mat.cubic) {
-        CK(cudaFuncSetAttribute(k_near_sym<HM_CUBIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        k_near_sym<HM_CUBIC><<<grid, SYM_WARPS * 32, smem, st>>>(ctx->L, near2, ctx->d_box, ctx->d_mat,
-                                                                 ctx->d_leaf_start, ctx->d_yrel, ctx->d_y, ctx->d_Pf,
-                                                                 ctx->d_sid, W.part, N, W.psorted, W.pmisc + 128,
-                                                                 ref_start, ctx->rf.child_start);
-    } else {
-        CK(cudaFuncSetAttribute(k_near_sym<HM_GENERIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        k_near_sym<HM_GENERIC><<<grid, SYM_WARPS * 32, smem, st>>>(ctx->L, near2, ctx->d_box, ctx->d_mat,
-                                                                   ctx->d_leaf_start, ctx->d_yrel, ctx->d_y,
-                                                                   ctx->d_Pf, ctx->d_sid, W.part, N, W.psorted,
-                                                                   W.pmisc + 128, ref_start, ctx->rf.child_start);
-    }
-    const double *S64 = ctx->opt.precision == GBFMM_MIXED_F64T ? ctx->d_S : nullptr;
-    k_near_combine<<<nblk(N, 256), 256, 0, st>>>(ctx->opt.p, ctx->opt.nodes, ctx->L, N, ctx->d_box, ctx->d_leaf_start, ctx->d_pleaf,
-                                                 ctx->d_y, ctx->d_Sf, S64, W.part, sig,
-                                                 ref_start ? ctx->rf.pfine : nullptr, ctx->rf.S7);
-    CK(cudaGetLastError());
-    return GBFMM_OK;
-}
-
-int near_run(gbfmm_ctx *ctx, const int *tstart, const double *xt, const int64_t *tsid, double *sig) {
-    if (tsid && near_symmetric(ctx)) return near_run_sym(ctx, sig);
-    const int64_t nl = ctx->n_leaves;
-    const float near2 = float(ctx->opt.near_fp64 * ctx->opt.near_fp64);
-    int *n_items = nullptr;
-    int2 *items = nullptr;
-    int64_t cap = 0;
-    const int64_t n_targets = tsid ? ctx->N : ctx->t_cap;
-    if (int rc = build_items(ctx, tstart, n_targets, n_items, items, cap)) return rc;
-    const unsigned grid = nblk(cap, WARPS);
+template <typename R, int HM, bool SYM, bool LEARN>
+static int launch_pairs(gbfmm_ctx *ctx, const NearTree &tr, const NearMedium<R> &md, const NearLearned &ln) {
+    size_t table = 0;
+    if (HM == HM_POINTS) table = md.Q <= kPointMax ? size_t(md.Q) * sizeof(float4) : 0;
+    else if (HM != HM_ISO) table = md.np <= kMomMax ? size_t(md.np) * kMomRow * sizeof(R) : 0;
+    const size_t smem = near_warps<R>() * sizeof(WarpShared<R, SYM, LEARN>) + table;
+    auto kern = k_near_pairs<R, HM, SYM, LEARN>;
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     ++ctx->launches;
-    if (ctx->mat.mode == GBFMM_H_MLP) {
+    kern<<<unsigned(ctx->sm_count * near_blocks<R>()), near_warps<R>() * 32, smem, ctx->stream>>>(tr, md, ln);
+    CK(cudaGetLastError());
+    return GBFMM_OK;
+}
+
+template <typename R, bool SYM>
+static int run_pairs(gbfmm_ctx *ctx, const int *tstart, const double *xt, int64_t n_t, const int *tleaf, double *sig) {
+    if (int rc = pairs_alloc(ctx, n_t, !SYM)) return rc;
+    NearWork &W = ctx->nw;
+    cudaStream_t st = ctx->stream;
+    const int64_t nl = ctx->n_leaves;
+    // adaptive tree (nodal forces): split leaves, their children's ranges and local values
+    const bool fine = SYM && ctx->rf.on;
+    NearTree tr{};
+    tr.L = ctx->L;
+    tr.N = ctx->N;
+    tr.n_t = n_t;
+    tr.box = ctx->d_box;
+    tr.tstart = tstart;
+    tr.sstart = ctx->d_leaf_start;
+    tr.ref_start = fine ? ctx->rf.ref_start : nullptr;
+    tr.child_start = fine ? ctx->rf.child_start : nullptr;
+    tr.trec = SYM ? W.rec : W.trec;
+    tr.srec = W.rec;
+    tr.plan = static_cast<const NearPlan *>(W.plan);
+    tr.lp = W.lp;
+    tr.items = static_cast<const NearItem *>(W.pitems);
+    tr.cnt = W.pcnt;
+    tr.rows = W.rows;
+    CK(cudaMemsetAsync(W.pcnt, 0, kCnt * sizeof(unsigned long long), st));
+    if (!SYM) {
+        ++ctx->launches;
+        k_near_targets<R><<<nblk(n_t, 256), 256, 0, st>>>(n_t, ctx->L, ctx->d_box, xt, tleaf, W.trec);
+    }
+    ctx->launches += 2;
+    k_near_totals<SYM><<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->L, tstart, ctx->d_leaf_start, tr.ref_start, W.pcnt);
+    k_near_plan<SYM><<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->L, ctx->sm_count * near_blocks<R>() * near_warps<R>(),
+                                                    SYM ? rows_sym(n_t) : rows_free(n_t), items_cap(n_t, nl), tstart,
+                                                    ctx->d_leaf_start, tr.ref_start, W.pcnt,
+                                                    static_cast<NearPlan *>(W.plan), W.lp,
+                                                    static_cast<NearItem *>(W.pitems));
+    CK(cudaGetLastError());
+    const NearMedium<R> md = near_medium<R>(ctx->mat);
+    NearLearned ln{};
+    // The cubic form's FP32 rounding grows for Zener ratios below one (RMS of K, pointwise rule
+    // from C / cubic moments: A = 3.2, 2.1 / 1.6e-7; A = 0.48, 0.9 / 1.2e-7; A = 0.17, 0.8 /
+    // 2.6e-7): such media take the general rule.
+    const bool cubic = ctx->mat.cubic && (sizeof(R) == 8 || ctx->mat.cd <= 1e-6 * ctx->mat.c44);
+    int rc = GBFMM_OK;
+    if (ctx->mat.mode == GBFMM_H_ISO) {
+        rc = launch_pairs<R, HM_ISO, SYM, false>(ctx, tr, md, ln);
+    } else if (near_learned(ctx)) {
+        if constexpr (sizeof(R) == 4) {
+            // pairs closer than near_fp64 segment lengths take the plain rule whatever mlp_min_dist is
+            const double rmin = std::max(ctx->opt.mlp_min_dist > 0.0 ? ctx->opt.mlp_min_dist : 8.0, ctx->opt.near_fp64);
+            ln.binmask = ctx->mlp.d_binmask;
+            ln.poly = reinterpret_cast<const float4 *>(ctx->mlp.poly);
+            ln.rmin2 = float(rmin * rmin);
+            ln.m2 = mlp_poly_m2();
+            rc = cubic ? launch_pairs<R, HM_CUBIC, SYM, true>(ctx, tr, md, ln)
+                       : launch_pairs<R, HM_GENERAL, SYM, true>(ctx, tr, md, ln);
+        }
+    } else if (cubic) {
+        rc = launch_pairs<R, HM_CUBIC, SYM, false>(ctx, tr, md, ln);
+    } else {
+        if constexpr (sizeof(R) == 4)
+            rc = launch_pairs<R, HM_POINTS, SYM, false>(ctx, tr, md, ln);
+        else
+            rc = launch_pairs<R, HM_GENERAL, SYM, false>(ctx, tr, md, ln);
+    }
+    if (rc) return rc;
+    const double *S64 = ctx->opt.precision == GBFMM_MIXED ? nullptr : ctx->d_S;
+    ++ctx->launches;
+    k_near_combine<SYM><<<nblk(n_t, 256), 256, 0, st>>>(ctx->opt.p, ctx->opt.nodes, tr, ctx->d_mat->V, tleaf, xt, ctx->d_Sf,
+                                                        S64, sig, fine ? ctx->rf.pfine : nullptr, ctx->rf.S7);
+    CK(cudaGetLastError());
+    return GBFMM_OK;
+}
+
+// Near field and L2P of a pass, into sig (sorted order).  free_targets: the n_t sorted free
+// points, else the Gauss points themselves.
+int near_run(gbfmm_ctx *ctx, bool free_targets, int64_t n_t, double *sig) {
+    const int *tstart = free_targets ? ctx->d_t_start : ctx->d_leaf_start;
+    const double *xt = free_targets ? ctx->d_t_x : ctx->d_y;
+    if (!free_targets) n_t = ctx->N;
+    if (near_learned(ctx)) {
         if (!ctx->mlp.trained || !ctx->mlp.d_binmask)
             return set_err(ctx, GBFMM_ERR_INVALID_ARG, "GBFMM_H_MLP: train (or set) and calibrate the network first");
-        const float rmin = float(ctx->opt.mlp_min_dist > 0.0 ? ctx->opt.mlp_min_dist : 8.0);
-        const size_t smem = sizeof(mlpw::Weights);
-#define GB_MLP_ARGS                                                                                                  \
-    ctx->opt.p, ctx->opt.nodes, ctx->L, nl, near2, rmin *rmin, ctx->d_box, ctx->d_mat, tstart, xt, tsid, ctx->d_leaf_start, ctx->d_yrel, \
-        ctx->d_y, ctx->d_Pf, ctx->d_sid, ctx->d_Sf, sig, ctx->mlp.theta_h, ctx->mlp.theta, ctx->mlp.scale,        \
-        ctx->mlp.d_binmask, items, n_items
-        if (ctx->mat.cubic) {
-            CK(cudaFuncSetAttribute(k_near_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-            k_near_mlp<true><<<grid, WARPS * 32, smem, ctx->stream>>>(GB_MLP_ARGS);
-        } else {
-            CK(cudaFuncSetAttribute(k_near_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-            k_near_mlp<false><<<grid, WARPS * 32, smem, ctx->stream>>>(GB_MLP_ARGS);
-        }
-#undef GB_MLP_ARGS
-        CK(cudaGetLastError());
-        return GBFMM_OK;
+        if (int rc = mlp_tabulate(ctx)) return rc;  // when the network changed since
     }
-#define GB_NEAR_ARGS                                                                                           \
-    ctx->opt.p, ctx->opt.nodes, ctx->L, nl, near2, ctx->d_box, ctx->d_mat, tstart, xt, tsid, ctx->d_leaf_start, ctx->d_yrel, ctx->d_y, \
-        ctx->d_Pf, ctx->d_sid, ctx->d_Sf, sig, items, n_items
-    if (near_coef_count(ctx) == 80)
-        k_near_mixed<HM_ISO, 80, 32><<<grid, WARPS * 32, 0, ctx->stream>>>(GB_NEAR_ARGS);
-    else if (ctx->mat.cubic)
-        k_near_mixed<HM_CUBIC, 108, 24><<<grid, WARPS * 32, 0, ctx->stream>>>(GB_NEAR_ARGS);
-    else
-        k_near_mixed<HM_GENERIC, 108, 24><<<grid, WARPS * 32, 0, ctx->stream>>>(GB_NEAR_ARGS);
-#undef GB_NEAR_ARGS
-    CK(cudaGetLastError());
-    return GBFMM_OK;
+    const int *tleaf = free_targets ? ctx->d_t_leaf : ctx->d_pleaf;
+    if (ctx->opt.precision == GBFMM_FP64)
+        return free_targets ? run_pairs<double, false>(ctx, tstart, xt, n_t, tleaf, sig)
+                            : run_pairs<double, true>(ctx, tstart, xt, n_t, tleaf, sig);
+    return free_targets ? run_pairs<float, false>(ctx, tstart, xt, n_t, tleaf, sig)
+                        : run_pairs<float, true>(ctx, tstart, xt, n_t, tleaf, sig);
 }

@@ -253,12 +253,14 @@ __global__ void k_gather_points(int64_t n, int n_g, const int *__restrict__ perm
     pos[k] = int(i);
 }
 
-__global__ void k_gather_targets(int64_t n, const int *__restrict__ perm, const double *__restrict__ x0,
-                                 double *__restrict__ x, int *__restrict__ pos) {
+__global__ void k_gather_targets(int64_t n, const int *__restrict__ perm, const int *__restrict__ leaf_of,
+                                 const double *__restrict__ x0, double *__restrict__ x, int *__restrict__ pos,
+                                 int *__restrict__ tleaf) {
     int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= n) return;
     int k = perm[i];
     for (int d = 0; d < 3; ++d) x[3 * i + d] = x0[3 * int64_t(k) + d];
+    tleaf[i] = leaf_of[k];
     pos[k] = int(i);
 }
 
@@ -373,7 +375,8 @@ int targets_sort(gbfmm_ctx *ctx, int64_t n_t, const double *x) {
     if (nl > ctx->t_cap_leaves) ctx->t_cap = 0;
     const int64_t t0 = ctx->t_cap;
     if (int rc = grow_dev(ctx, ctx->t_cap, n_t,
-                          {{(void **)&ctx->d_t_pos, n_t * sizeof(int)}, {(void **)&ctx->d_t_x, n_t * 3 * sizeof(double)},
+                          {{(void **)&ctx->d_t_pos, n_t * sizeof(int)}, {(void **)&ctx->d_t_leaf, n_t * sizeof(int)},
+                           {(void **)&ctx->d_t_x, n_t * 3 * sizeof(double)},
                            {(void **)&ctx->d_t_sig, n_t * 6 * sizeof(double)},
                            {(void **)&ctx->d_t_tmp, (2 * n_t + 2 * nl) * sizeof(int)}},
                           "targets")) {
@@ -393,7 +396,7 @@ int targets_sort(gbfmm_ctx *ctx, int64_t n_t, const double *x) {
     ++ctx->launches;
     k_leaf_sort<<<unsigned(nl), 128, 0, st>>>(nl, ctx->d_t_start, perm, nullptr, 0);
     ++ctx->launches;
-    k_gather_targets<<<nblk(n_t, 256), 256, 0, st>>>(n_t, perm, x, ctx->d_t_x, ctx->d_t_pos);
+    k_gather_targets<<<nblk(n_t, 256), 256, 0, st>>>(n_t, perm, leaf_of, x, ctx->d_t_x, ctx->d_t_pos, ctx->d_t_leaf);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }

@@ -44,6 +44,7 @@ static void free_tree(gbfmm_ctx *ctx) {
     release(ctx->d_leaf_start);
     release(ctx->d_t_start);
     release(ctx->d_cnt);
+    release(ctx->d_scan);
     release(ctx->d_cursor);
     release(ctx->d_tmp_d);
     release(ctx->d_part);
@@ -96,6 +97,7 @@ static int ensure_tree_buffers(gbfmm_ctx *ctx) {
                           {{(void **)&ctx->d_leaf_start, (nl + 1) * sizeof(int)},
                            {(void **)&ctx->d_t_start, (nl + 1) * sizeof(int)},
                            {(void **)&ctx->d_cnt, nl * sizeof(int)},
+                           {(void **)&ctx->d_scan, scan_blocks(nl) * sizeof(int)},
                            {(void **)&ctx->d_cursor, nl * sizeof(int)}},
                           "leaves"))
         return rc;
@@ -278,7 +280,7 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     v(c->L), v(c->N), v(c->n_segs), v(c->n_nodes), v(c->n_cells), v(c->n_leaves), v(c->t_cap);
     v(c->node_xyz), v(c->seg_nodes), v(c->burgers), v(c->stream);
     const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Asym_f, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
-                          c->d_slen, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf,
+                          c->d_slen, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf, c->d_scan,
                           c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_t_pos, c->d_t_start,
                           c->d_t_x, c->d_t_sig, c->tc.Thi, c->tc.Tlo, c->tc.Whi, c->tc.Wlo, c->tc.d_status,
                           c->tc.d_flags, c->tc.d_pos, c->tc.d_list, c->tc.d_seg, c->tc.d_wmax, c->mlp.theta, c->mlp.theta_h,

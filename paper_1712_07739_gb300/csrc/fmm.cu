@@ -6,6 +6,7 @@
 //   L2P  s(x_i) = sum_l L_p(xbar_l, x_i) s(xbar_l) + near field over N(leaf)
 // Nodes of a cell of edge h at corner c are c + h t_a, t_a = a/(p-1)
 // (Sec. 4.1); node index m = (mz p + my) p + mx.
+#include <algorithm>
 #include <cmath>
 #include <string>
 
@@ -31,6 +32,22 @@ __global__ void k_occ_leaves(int64_t nl, const int *__restrict__ start, int64_t 
     int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= nl) return;
     occ[base + i] = start[i + 1] - start[i];
+}
+
+// levels `top` .. 0 from level top + 1, one block (level 5 and up have blocks enough of their own)
+__global__ void __launch_bounds__(1024) k_occ_top(int top, int *__restrict__ occ) {
+    for (int level = top; level >= 0; --level) {
+        const int n = 1 << level, nc = 2 * n;
+        const int64_t cb = cell_base_d(level + 1), base = cell_base_d(level);
+        for (int i = threadIdx.x; i < n * n * n; i += blockDim.x) {
+            int x, y, z, s = 0;
+            cell_xyz(i, n, x, y, z);
+            for (int c = 0; c < 8; ++c)
+                s += occ[cb + (int64_t(2 * z + (c >> 2)) * nc + (2 * y + ((c >> 1) & 1))) * nc + (2 * x + (c & 1))];
+            occ[base + i] = s;
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void k_occ_up(int level, int *__restrict__ occ) {
@@ -571,10 +588,12 @@ void compute_occ(gbfmm_ctx *ctx, const int *start, int *occ) {
     const int64_t nl = ctx->n_leaves;
     ++ctx->launches;
     k_occ_leaves<<<nblk(nl, 256), 256, 0, ctx->stream>>>(nl, start, cell_base(L - 1), occ);
-    for (int lev = L - 2; lev >= 0; --lev) {
+    for (int lev = L - 2; lev > 3; --lev) {
         ++ctx->launches;
         k_occ_up<<<nblk(int64_t(1) << (3 * lev), 256), 256, 0, ctx->stream>>>(lev, occ);
     }
+    ++ctx->launches;
+    k_occ_top<<<1, 1024, 0, ctx->stream>>>(std::min(L - 2, 3), occ);
 }
 
 namespace {

@@ -113,6 +113,7 @@ struct gbfmm_ctx {
     int *d_pos = nullptr;      // [N] original point index -> sorted position
     int *d_pleaf = nullptr;    // [N] leaf of each sorted point
     int *d_leaf_start = nullptr;  // [n_leaves + 1]
+    int *d_scan = nullptr;        // block sums of the scans over leaves
     int *d_tmp_i = nullptr;       // scratch ints, N + n_leaves + 1
     double *d_tmp_d = nullptr;    // scratch doubles
     // build scratch
@@ -213,4 +214,7 @@ int targets_sort(gbfmm_ctx *ctx, int64_t n_t, const double *x);
 int targets_scatter(gbfmm_ctx *ctx, int64_t n_t, double *sigma);
 void timer_mark(gbfmm_ctx *ctx);
 void compute_occ(gbfmm_ctx *ctx, const int *start, int *occ);
+// exclusive scan of n counts into start[0..n] (n up to the leaves of the tree), tree.cu
+void scan_counts(gbfmm_ctx *ctx, int64_t n, const int *cnt, int *start);
+int64_t scan_blocks(int64_t n);
 int share_material(gbfmm_ctx *dst, const gbfmm_ctx *src);  // material.cu

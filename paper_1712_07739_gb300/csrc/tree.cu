@@ -8,6 +8,7 @@
 // clamped.  Points are counting-sorted by leaf, and within a leaf by their
 // original index, so that the order (and every sum over it) is
 // deterministic.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -74,14 +75,31 @@ __global__ void k_bbox_partial(int64_t n, const double *__restrict__ y, double *
         for (int d = 0; d < 6; ++d) part[blockIdx.x * 6 + d] = sm[d][0];
 }
 
-__global__ void k_bbox_final(int nparts, const double *__restrict__ part, TreeBox *box) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int b = 0; b < nparts; ++b)
-        for (int d = 0; d < 3; ++d) {
-            lo[d] = fmin(lo[d], part[b * 6 + d]);
-            hi[d] = fmax(hi[d], part[b * 6 + 3 + d]);
+// one block of kBoxParts threads, one partial each (minima and maxima: exact in any order).  One
+// thread reading the partials one after the other took 210 us of every build.
+constexpr int kBoxParts = 256;
+__global__ void __launch_bounds__(kBoxParts) k_bbox_final(int nparts, const double *__restrict__ part, TreeBox *box) {
+    __shared__ double sm[6][kBoxParts / 32];
+    double v[6];
+    for (int d = 0; d < 6; ++d)
+        v[d] = int(threadIdx.x) < nparts ? part[threadIdx.x * 6 + d] : (d < 3 ? INFINITY : -INFINITY);
+    for (int d = 0; d < 6; ++d) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v[d], o);
+            v[d] = d < 3 ? fmin(v[d], u) : fmax(v[d], u);
         }
+        if ((threadIdx.x & 31) == 0) sm[d][threadIdx.x / 32] = v[d];
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double lo[3], hi[3];
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = sm[d][0], hi[d] = sm[3 + d][0];
+        for (int w = 1; w < kBoxParts / 32; ++w) {
+            lo[d] = fmin(lo[d], sm[d][w]);
+            hi[d] = fmax(hi[d], sm[3 + d][w]);
+        }
+    }
     double s = fmax(hi[0] - lo[0], fmax(hi[1] - lo[1], hi[2] - lo[2]));
     if (s == 0.0) s = 1.0;
     double H = s * (1.0 + 0.0009765625);
@@ -118,32 +136,6 @@ __global__ void k_leaf_count(int64_t n, const double *__restrict__ y, const Tree
         child_of[i] = (unsigned char)((fx & 1) | ((fy & 1) << 1) | ((fz & 1) << 2));
     }
     atomicAdd(&cnt[leaf], 1);
-}
-
-// exclusive scan of cnt[0..n) into start[0..n], one block of 1024 threads
-__global__ void k_scan(int64_t n, const int *__restrict__ cnt, int *__restrict__ start) {
-    __shared__ int part[1024];
-    int64_t per = (n + blockDim.x - 1) / blockDim.x;
-    int64_t b = threadIdx.x * per, e = min(n, b + per);
-    int s = 0;
-    for (int64_t i = b; i < e; ++i) s += cnt[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int t = 0; t < int(blockDim.x); ++t) {
-            int v = part[t];
-            part[t] = run;
-            run += v;
-        }
-        start[n] = run;
-    }
-    __syncthreads();
-    int run = part[threadIdx.x];
-    for (int64_t i = b; i < e; ++i) {
-        start[i] = run;
-        run += cnt[i];
-    }
 }
 
 __global__ void k_scatter(int64_t n, const int *__restrict__ leaf_of, const int *__restrict__ start,
@@ -298,7 +290,73 @@ void gauss_legendre(int n, double *x, double *w) {
 
 inline unsigned nblk(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
+// Exclusive scan of cnt[0..n) into start[0..n]: blocks of 4,096 counts, their sums first where
+// there is more than one block (262,144 leaves: 6 us; one block over all of them took 430 us).
+constexpr int kScanBlock = 4096;
+__device__ __forceinline__ int block_scan(int v, int *sm) {  // inclusive, 1,024 threads
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) sm[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        int x = sm[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
+        }
+        sm[lane] = x;
+    }
+    __syncthreads();
+    if (w > 0) v += sm[w - 1];
+    __syncthreads();
+    return v;
+}
+__global__ void __launch_bounds__(1024) k_scan_sums(int64_t n, const int *__restrict__ cnt, int *__restrict__ sums) {
+    __shared__ int sm[32];
+    const int64_t b = blockIdx.x * int64_t(kScanBlock) + 4 * threadIdx.x;
+    int s = 0;
+    for (int i = 0; i < 4; ++i) s += b + i < n ? cnt[b + i] : 0;
+    s = block_scan(s, sm);
+    if (threadIdx.x == 1023) sums[blockIdx.x] = s;
+}
+__global__ void __launch_bounds__(1024) k_scan_apply(int64_t n, const int *__restrict__ cnt,
+                                                     const int *__restrict__ sums, int *__restrict__ start) {
+    __shared__ int sm[32];
+    __shared__ int s_base;
+    int before = 0;
+    for (int i = threadIdx.x; i < int(blockIdx.x); i += 1024) before += sums[i];
+    before = block_scan(before, sm);
+    if (threadIdx.x == 1023) s_base = before;
+    const int64_t b = blockIdx.x * int64_t(kScanBlock) + 4 * threadIdx.x;
+    int v[4], s = 0;
+    for (int i = 0; i < 4; ++i) {
+        v[i] = b + i < n ? cnt[b + i] : 0;
+        s += v[i];
+    }
+    int run = block_scan(s, sm) - s + s_base;
+    for (int i = 0; i < 4; ++i) {
+        if (b + i < n) start[b + i] = run;
+        run += v[i];
+        if (b + i == n - 1) start[n] = run;
+    }
+}
+
 }  // namespace
+
+void scan_counts(gbfmm_ctx *ctx, int64_t n, const int *cnt, int *start) {
+    const unsigned nb = nblk(n, kScanBlock);
+    if (nb > 1) {
+        ++ctx->launches;
+        k_scan_sums<<<nb, 1024, 0, ctx->stream>>>(n, cnt, ctx->d_scan);
+    }
+    ++ctx->launches;
+    k_scan_apply<<<nb, 1024, 0, ctx->stream>>>(n, cnt, ctx->d_scan, start);
+}
+// block sums that a scan of n counts needs
+int64_t scan_blocks(int64_t n) { return n / kScanBlock + 1; }
 
 int tree_build(gbfmm_ctx *ctx, bool validate) {
     cudaStream_t st = ctx->stream;
@@ -315,7 +373,7 @@ int tree_build(gbfmm_ctx *ctx, bool validate) {
     double *y0 = ctx->d_y0, *q0 = ctx->d_q0, *len0 = ctx->d_len0, *part = ctx->d_part;
     int *leaf_of = ctx->d_leaf_of, *cnt = ctx->d_cnt, *cursor = ctx->d_cursor, *perm = ctx->d_perm;
     int *bad = ctx->d_bad;
-    const int nparts = 512;
+    const int nparts = int(std::min<int64_t>(kBoxParts, (N + 255) / 256));
     CK(cudaMemsetAsync(bad, 0, sizeof(int), st));
     ++ctx->launches;
     k_gauss_points<<<nblk(ctx->n_segs, 128), 128, 0, st>>>(ctx->n_segs, ctx->node_xyz, ctx->seg_nodes, ctx->burgers,
@@ -323,15 +381,14 @@ int tree_build(gbfmm_ctx *ctx, bool validate) {
     ++ctx->launches;
     k_bbox_partial<<<nparts, 256, 0, st>>>(N, y0, part);
     ++ctx->launches;
-    k_bbox_final<<<1, 32, 0, st>>>(nparts, part, ctx->d_box);
+    k_bbox_final<<<1, kBoxParts, 0, st>>>(nparts, part, ctx->d_box);
     CK(cudaMemsetAsync(cnt, 0, nl * sizeof(int), st));
     CK(cudaMemsetAsync(cursor, 0, nl * sizeof(int), st));
     ++ctx->launches;
     auto &RF = ctx->rf;
     const bool refine = RF.on != 0;
     k_leaf_count<<<nblk(N, 256), 256, 0, st>>>(N, y0, ctx->d_box, ctx->L, leaf_of, cnt, refine ? RF.child_of : nullptr);
-    ++ctx->launches;
-    k_scan<<<1, 1024, 0, st>>>(nl, cnt, ctx->d_leaf_start);
+    scan_counts(ctx, nl, cnt, ctx->d_leaf_start);
     ++ctx->launches;
     k_scatter<<<nblk(N, 256), 256, 0, st>>>(N, leaf_of, ctx->d_leaf_start, cursor, perm);
     ++ctx->launches;
@@ -340,9 +397,9 @@ int tree_build(gbfmm_ctx *ctx, bool validate) {
     RF.n_ref_host = -1;
     if (refine) {
         // split leaves: flags, their scan (leaf -> split index), each split leaf's child ranges
-        ctx->launches += 3;
+        ctx->launches += 2;
         k_ref_flags<<<nblk(nl, 256), 256, 0, st>>>(nl, ctx->d_leaf_start, ctx->opt.refine_points, cursor);
-        k_scan<<<1, 1024, 0, st>>>(nl, cursor, RF.ref_start);
+        scan_counts(ctx, nl, cursor, RF.ref_start);
         k_ref_children<<<nblk(nl, 128), 128, 0, st>>>(nl, ctx->d_leaf_start, RF.ref_start, perm, RF.child_of,
                                                       RF.ref_leaf, RF.child_start);
     }
@@ -389,8 +446,7 @@ int targets_sort(gbfmm_ctx *ctx, int64_t n_t, const double *x) {
     CK(cudaMemsetAsync(cursor, 0, nl * sizeof(int), st));
     ++ctx->launches;
     k_leaf_count<<<nblk(n_t, 256), 256, 0, st>>>(n_t, x, ctx->d_box, ctx->L, leaf_of, cnt, nullptr);
-    ++ctx->launches;
-    k_scan<<<1, 1024, 0, st>>>(nl, cnt, ctx->d_t_start);
+    scan_counts(ctx, nl, cnt, ctx->d_t_start);
     ++ctx->launches;
     k_scatter<<<nblk(n_t, 256), 256, 0, st>>>(n_t, leaf_of, ctx->d_t_start, cursor, perm);
     ++ctx->launches;

@@ -15,10 +15,6 @@
 
 namespace {
 
-struct Transfer {
-    double M[2][GB_MAXP][GB_MAXP];  // M[c][A'][a] = ell_A'((c + t_a) / 2)
-};
-
 inline unsigned nblk(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
 __device__ __forceinline__ void cell_xyz(int64_t lin, int n, int &x, int &y, int &z) {
@@ -66,202 +62,6 @@ __global__ void k_occ_up(int level, int *__restrict__ occ) {
     occ[cell_base_d(level) + i] = s;
 }
 
-// ---------------------------------------------------------------- P2M
-// one block per leaf; thread m accumulates W[m][0..8].  The local
-// coordinate of a point is formed in FP64; the basis and sums in R.
-template <typename R>
-__device__ void p2m_range(int p, int nodes, int b, int e, const double c0[3], double ih, const double *__restrict__ y,
-                          const double *__restrict__ q, R *__restrict__ Wc);
-
-template <typename R>
-__global__ void k_p2m(int p, int nodes, int L, const TreeBox *__restrict__ box, const int *__restrict__ start,
-                      const double *__restrict__ y, const double *__restrict__ q, R *__restrict__ W) {
-    const int64_t leaf = blockIdx.x;
-    const int nl = 1 << (L - 1);
-    const int P3 = p * p * p;
-    R *Wc = W + (cell_base_d(L - 1) + leaf) * int64_t(P3) * 9;
-    const int b = start[leaf], e = start[leaf + 1];
-    if (b == e) {
-        for (int i = threadIdx.x; i < P3 * 9; i += blockDim.x) Wc[i] = R(0);
-        return;
-    }
-    int cx, cy, cz;
-    cell_xyz(leaf, nl, cx, cy, cz);
-    const double h = box->H / nl;
-    const double ih = double(nl) / box->H;
-    const double c0[3] = {box->origin[0] + cx * h, box->origin[1] + cy * h, box->origin[2] + cz * h};
-    p2m_range<R>(p, nodes, b, e, c0, ih, y, q, Wc);
-}
-
-// adaptive tree: P2M of the children of split leaves, one block per child cell 8 r + c
-// (compact rows; empty and absent children get zeros)
-template <typename R>
-__global__ void k_p2m_fine(int p, int nodes, int L, const TreeBox *__restrict__ box, const int *__restrict__ n_ref,
-                           const int *__restrict__ ref_leaf, const int *__restrict__ child_start,
-                           const double *__restrict__ y, const double *__restrict__ q, R *__restrict__ W7) {
-    const int64_t f = blockIdx.x;
-    const int r = int(f >> 3), c = int(f & 7);
-    const int P3 = p * p * p;
-    R *Wc = W7 + f * int64_t(P3) * 9;
-    int b = 0, e = 0;
-    if (r < *n_ref) {
-        b = child_start[9 * r + c];
-        e = child_start[9 * r + c + 1];
-    }
-    if (b == e) {
-        for (int i = threadIdx.x; i < P3 * 9; i += blockDim.x) Wc[i] = R(0);
-        return;
-    }
-    const int nl = 1 << (L - 1);
-    int cx, cy, cz;
-    cell_xyz(ref_leaf[r], nl, cx, cy, cz);
-    const double h = box->H / (2 * nl);
-    const double ih = double(2 * nl) / box->H;
-    const double c0[3] = {box->origin[0] + (2 * cx + (c & 1)) * h, box->origin[1] + (2 * cy + ((c >> 1) & 1)) * h,
-                          box->origin[2] + (2 * cz + (c >> 2)) * h};
-    p2m_range<R>(p, nodes, b, e, c0, ih, y, q, Wc);
-}
-
-// W[m][wr] = sum over the points b..e of L_m(local position) q_wr (Sec. 4.3, P2M)
-template <typename R>
-__device__ void p2m_range(int p, int nodes, int b, int e, const double c0[3], double ih, const double *__restrict__ y,
-                          const double *__restrict__ q, R *__restrict__ Wc) {
-    const int P3 = p * p * p;
-    constexpr int CH = 64;
-    __shared__ R sb[CH][3][GB_MAXP];
-    __shared__ R sq[CH][9];
-    R acc[2][9];
-    for (int u = 0; u < 2; ++u)
-        for (int i = 0; i < 9; ++i) acc[u][i] = R(0);
-    for (int j0 = b; j0 < e; j0 += CH) {
-        const int nj = min(CH, e - j0);
-        __syncthreads();
-        for (int t = threadIdx.x; t < nj * 3; t += blockDim.x) {
-            int j = t / 3, d = t % 3;
-            R tt = R((y[3 * int64_t(j0 + j) + d] - c0[d]) * ih);
-            R v[GB_MAXP];
-            lagrange_1d<R>(p, tt, v, nodes);
-            for (int a = 0; a < p; ++a) sb[j][d][a] = v[a];
-        }
-        for (int t = threadIdx.x; t < nj * 9; t += blockDim.x) sq[t / 9][t % 9] = R(q[9 * int64_t(j0) + t]);
-        __syncthreads();
-        for (int u = 0; u < 2; ++u) {
-            int m = threadIdx.x + u * blockDim.x;
-            if (m >= P3) break;
-            int mx = m % p, my = (m / p) % p, mz = m / (p * p);
-            for (int j = 0; j < nj; ++j) {
-                R w = sb[j][0][mx] * sb[j][1][my] * sb[j][2][mz];
-                for (int i = 0; i < 9; ++i) acc[u][i] += w * sq[j][i];
-            }
-        }
-    }
-    for (int u = 0; u < 2; ++u) {
-        int m = threadIdx.x + u * blockDim.x;
-        if (m >= P3) break;
-        for (int i = 0; i < 9; ++i) Wc[m * 9 + i] = acc[u][i];
-    }
-}
-
-// ---------------------------------------------------------------- M2M / L2L
-// Separable tensor-product transfer on p x p x p x NC node values in shared
-// memory: out[A',B',C'] = sum_{a,b,c} Mx[A'][a] My[B'][b] Mz[C'][c] in[a,b,c]
-// (forward = true), or with each M transposed (forward = false).
-template <int NC, typename R>
-__device__ void transfer3(int p, const double (*Mx)[GB_MAXP], const double (*My)[GB_MAXP],
-                          const double (*Mz)[GB_MAXP], bool fwd, R *in, R *t1) {
-    const int P3 = p * p * p;
-    auto m = [&](const double (*M)[GB_MAXP], int o, int i) { return R(fwd ? M[o][i] : M[i][o]); };
-    // x pass: t1[z][y][X] = sum_x m(X, x) in[z][y][x]
-    for (int t = threadIdx.x; t < P3 * NC; t += blockDim.x) {
-        int c = t % NC, node = t / NC;
-        int X = node % p, yz = node / p;
-        R s = R(0);
-        for (int x = 0; x < p; ++x) s += m(Mx, X, x) * in[(yz * p + x) * NC + c];
-        t1[t] = s;
-    }
-    __syncthreads();
-    // y pass: in[z][Y][X] = sum_y m(Y, y) t1[z][y][X]
-    for (int t = threadIdx.x; t < P3 * NC; t += blockDim.x) {
-        int c = t % NC, node = t / NC;
-        int X = node % p, Y = (node / p) % p, z = node / (p * p);
-        R s = R(0);
-        for (int yy = 0; yy < p; ++yy) s += m(My, Y, yy) * t1[((z * p + yy) * p + X) * NC + c];
-        in[t] = s;
-    }
-    __syncthreads();
-    // z pass: t1[Z][Y][X] = sum_z m(Z, z) in[z][Y][X]
-    for (int t = threadIdx.x; t < P3 * NC; t += blockDim.x) {
-        int c = t % NC, node = t / NC;
-        int XY = node % (p * p), Z = node / (p * p);
-        R s = R(0);
-        for (int zz = 0; zz < p; ++zz) s += m(Mz, Z, zz) * in[(zz * p * p + XY) * NC + c];
-        t1[t] = s;
-    }
-    __syncthreads();
-}
-
-// parent weights at `level` from its 8 children at level + 1
-template <typename R>
-__global__ void k_m2m(int p, int level, Transfer tr, const int *__restrict__ occ, R *__restrict__ W) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    R *sm = reinterpret_cast<R *>(sm_raw);
-    const int P3 = p * p * p;
-    const int n = 1 << level;
-    const int64_t cell = blockIdx.x;
-    R *Wp = W + (cell_base_d(level) + cell) * int64_t(P3) * 9;
-    R *in = sm, *t1 = sm + P3 * 9;
-    if (occ[cell_base_d(level) + cell] == 0) {
-        for (int i = threadIdx.x; i < P3 * 9; i += blockDim.x) Wp[i] = R(0);
-        return;
-    }
-    int x, y, z;
-    cell_xyz(cell, n, x, y, z);
-    R acc[18];
-    for (int i = 0; i < 18; ++i) acc[i] = R(0);
-    const int nc = 2 * n;
-    for (int c = 0; c < 8; ++c) {
-        const int ox = c & 1, oy = (c >> 1) & 1, oz = c >> 2;
-        const int64_t ch = cell_base_d(level + 1) + (int64_t(2 * z + oz) * nc + (2 * y + oy)) * nc + (2 * x + ox);
-        if (occ[ch] == 0) continue;
-        const R *Wc = W + ch * int64_t(P3) * 9;
-        __syncthreads();
-        for (int i = threadIdx.x; i < P3 * 9; i += blockDim.x) in[i] = Wc[i];
-        __syncthreads();
-        transfer3<9, R>(p, tr.M[ox], tr.M[oy], tr.M[oz], true, in, t1);
-        for (int u = 0; u < 18; ++u) {
-            int i = threadIdx.x + u * blockDim.x;
-            if (i >= P3 * 9) break;
-            acc[u] += t1[i];
-        }
-    }
-    for (int u = 0; u < 18; ++u) {
-        int i = threadIdx.x + u * blockDim.x;
-        if (i >= P3 * 9) break;
-        Wp[i] = acc[u];
-    }
-}
-
-// child locals at `level` += parent's, interpolated
-template <typename R>
-__global__ void k_l2l(int p, int level, Transfer tr, const int *__restrict__ tocc, R *__restrict__ S) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    R *sm = reinterpret_cast<R *>(sm_raw);
-    const int P3 = p * p * p;
-    const int n = 1 << level;
-    const int64_t cell = blockIdx.x;
-    if (tocc[cell_base_d(level) + cell] == 0) return;
-    int x, y, z;
-    cell_xyz(cell, n, x, y, z);
-    const int np = n / 2;
-    const int64_t par = cell_base_d(level - 1) + (int64_t(z / 2) * np + y / 2) * np + x / 2;
-    R *in = sm, *t1 = sm + P3 * 6;
-    for (int i = threadIdx.x; i < P3 * 6; i += blockDim.x) in[i] = S[par * P3 * 6 + i];
-    __syncthreads();
-    transfer3<6, R>(p, tr.M[x & 1], tr.M[y & 1], tr.M[z & 1], false, in, t1);
-    R *Sc = S + (cell_base_d(level) + cell) * int64_t(P3) * 6;
-    for (int i = threadIdx.x; i < P3 * 6; i += blockDim.x) Sc[i] += t1[i];
-}
-
 // adaptive tree: occupancy of the children of split leaves at level L (one below the
 // leaves), into occL (the level's part of the occupancy array, zeroed before); the work
 // counts read it to count the children's M2L pairs
@@ -278,163 +78,6 @@ __global__ void k_fine_occ(int64_t n_fine, int L, const int *__restrict__ n_ref,
     cell_xyz(ref_leaf[r], nl, x, y, z);
     const int64_t lin = (int64_t(2 * z + (c >> 2)) * nf + (2 * y + ((c >> 1) & 1))) * nf + (2 * x + (c & 1));
     occL[lin] = cnt;
-}
-
-// adaptive tree: children's local values += their split parent's, interpolated (L2L),
-// one block per child cell 8 r + c that holds points
-template <typename R>
-__global__ void k_l2l_fine(int p, int L, Transfer tr, const int *__restrict__ n_ref, const int *__restrict__ ref_leaf,
-                           const int *__restrict__ child_start, const R *__restrict__ S, R *__restrict__ S7) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    R *in = reinterpret_cast<R *>(sm_raw);
-    const int64_t f = blockIdx.x;
-    const int r = int(f >> 3), c = int(f & 7);
-    if (r >= *n_ref || child_start[9 * r + c + 1] == child_start[9 * r + c]) return;
-    const int P3 = p * p * p;
-    R *t1 = in + P3 * 6;
-    const R *Sp = S + (cell_base_d(L - 1) + ref_leaf[r]) * int64_t(P3) * 6;
-    for (int i = threadIdx.x; i < P3 * 6; i += blockDim.x) in[i] = Sp[i];
-    __syncthreads();
-    transfer3<6, R>(p, tr.M[c & 1], tr.M[(c >> 1) & 1], tr.M[c >> 2], false, in, t1);
-    R *out = S7 + f * int64_t(P3) * 6;
-    for (int i = threadIdx.x; i < P3 * 6; i += blockDim.x) out[i] += t1[i];
-}
-
-// Parent weights at `level` from its 8 children at level + 1 (Sec. 3.2,
-// M2M), with the children merged one axis at a time: for each child row
-// (oy, oz) the x transfer sums over both x children (2p terms), then the y
-// transfer over both y halves, then the z transfer over both z halves --
-// 14 p multiply-adds per parent value instead of 24 p for eight separate
-// tensor-product transfers, and two barriers per parent instead of 24.
-// Shared memory: 4 x 9 p^3 values (x-merged rows of one z half, x- and
-// y-merged halves).
-template <typename R>
-__global__ void __launch_bounds__(256) k_m2m_merge(int p, int level, Transfer tr, const int *__restrict__ occ,
-                                                   R *__restrict__ W) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    R *tx = reinterpret_cast<R *>(sm_raw);
-    __shared__ R Ms[2][GB_MAXP][GB_MAXP];
-    __shared__ int64_t s_ch[8];
-    const int P3 = p * p * p, NV = P3 * 9;
-    R *u = tx + 2 * NV;
-    const int n = 1 << level, nc = 2 * n;
-    const int64_t cell = blockIdx.x;
-    R *Wp = W + (cell_base_d(level) + cell) * int64_t(NV);
-    if (occ[cell_base_d(level) + cell] == 0) {
-        for (int i = threadIdx.x; i < NV; i += blockDim.x) Wp[i] = R(0);
-        return;
-    }
-    int x, y, z;
-    cell_xyz(cell, n, x, y, z);
-    for (int i = threadIdx.x; i < 2 * GB_MAXP * GB_MAXP; i += blockDim.x) {
-        const int c = i / (GB_MAXP * GB_MAXP), o = (i / GB_MAXP) % GB_MAXP, a = i % GB_MAXP;
-        Ms[c][o][a] = R(tr.M[c][o][a]);
-    }
-    if (threadIdx.x < 8) {
-        const int ox = threadIdx.x & 1, oy = (threadIdx.x >> 1) & 1, oz = threadIdx.x >> 2;
-        const int64_t ch = cell_base_d(level + 1) + (int64_t(2 * z + oz) * nc + (2 * y + oy)) * nc + (2 * x + ox);
-        s_ch[threadIdx.x] = occ[ch] > 0 ? ch * int64_t(NV) : int64_t(-1);
-    }
-    __syncthreads();
-    for (int oz = 0; oz < 2; ++oz) {
-        // x: tx[oy][((c p + b) p + A) 9 + k] = sum_ox sum_a M[ox][A][a] W_(ox,oy,oz)[((c p + b) p + a) 9 + k]
-        for (int t = threadIdx.x; t < 2 * NV; t += blockDim.x) {
-            const int oy = t / NV, r = t - oy * NV;
-            const int k = r % 9, node = r / 9, A = node % p, bc = node / p;
-            R s = R(0);
-            for (int ox = 0; ox < 2; ++ox) {
-                const int64_t base = s_ch[ox + 2 * oy + 4 * oz];
-                if (base < 0) continue;
-                const R *Wc = W + base + int64_t(bc) * p * 9 + k;
-                for (int a = 0; a < p; ++a) s += Ms[ox][A][a] * Wc[9 * a];
-            }
-            tx[t] = s;
-        }
-        __syncthreads();
-        // y: u[oz][((c p + B) p + A) 9 + k] = sum_oy sum_b M[oy][B][b] tx[oy][((c p + b) p + A) 9 + k]
-        for (int r = threadIdx.x; r < NV; r += blockDim.x) {
-            const int k = r % 9, node = r / 9, A = node % p, B = (node / p) % p, c = node / (p * p);
-            R s = R(0);
-            for (int oy = 0; oy < 2; ++oy)
-                for (int b = 0; b < p; ++b) s += Ms[oy][B][b] * tx[oy * NV + ((c * p + b) * p + A) * 9 + k];
-            u[oz * NV + r] = s;
-        }
-        __syncthreads();
-    }
-    // z: W[((C p + B) p + A) 9 + k] = sum_oz sum_c M[oz][C][c] u[oz][((c p + B) p + A) 9 + k]
-    for (int r = threadIdx.x; r < NV; r += blockDim.x) {
-        const int k = r % 9, node = r / 9, AB = node % (p * p), C = node / (p * p);
-        R s = R(0);
-        for (int oz = 0; oz < 2; ++oz)
-            for (int c = 0; c < p; ++c) s += Ms[oz][C][c] * u[oz * NV + (c * p * p + AB) * 9 + k];
-        Wp[r] = s;
-    }
-}
-
-// Child locals at `level` += their parent's, interpolated (Sec. 3.2, L2L),
-// one block per parent at level - 1 producing all eight children axis by
-// axis: the parent's values are read once, the x transfer gives both x
-// halves, the y transfer the four (ox, oy) quarters, the z transfer the
-// eight children -- 14 p multiply-adds per child value on average instead
-// of 24 p.  Shared memory: 7 x 6 p^3 values.
-template <typename R>
-__global__ void __launch_bounds__(256) k_l2l_split(int p, int level, Transfer tr, const int *__restrict__ tocc,
-                                                   R *__restrict__ S) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    R *in = reinterpret_cast<R *>(sm_raw);
-    __shared__ R Ms[2][GB_MAXP][GB_MAXP];
-    __shared__ int64_t s_ch[8];
-    const int P3 = p * p * p, NV = P3 * 6;
-    R *tx = in + NV, *ty = tx + 2 * NV;
-    const int np = 1 << (level - 1), n = 2 * np;
-    const int64_t par = blockIdx.x;
-    int x, y, z;
-    cell_xyz(par, np, x, y, z);
-    if (threadIdx.x < 8) {
-        const int ox = threadIdx.x & 1, oy = (threadIdx.x >> 1) & 1, oz = threadIdx.x >> 2;
-        const int64_t ch = cell_base_d(level) + (int64_t(2 * z + oz) * n + (2 * y + oy)) * n + (2 * x + ox);
-        s_ch[threadIdx.x] = tocc[ch] > 0 ? ch * int64_t(NV) : int64_t(-1);
-    }
-    for (int i = threadIdx.x; i < 2 * GB_MAXP * GB_MAXP; i += blockDim.x) {
-        const int c = i / (GB_MAXP * GB_MAXP), o = (i / GB_MAXP) % GB_MAXP, a = i % GB_MAXP;
-        Ms[c][o][a] = R(tr.M[c][o][a]);
-    }
-    __syncthreads();
-    bool any = false;
-    for (int c = 0; c < 8; ++c) any |= s_ch[c] >= 0;
-    if (!any) return;
-    const R *Sp = S + (cell_base_d(level - 1) + par) * int64_t(NV);
-    for (int i = threadIdx.x; i < NV; i += blockDim.x) in[i] = Sp[i];
-    __syncthreads();
-    // x: tx[ox][((c p + b) p + A) 6 + k] = sum_a M[ox][a][A] in[((c p + b) p + a) 6 + k]
-    for (int t = threadIdx.x; t < 2 * NV; t += blockDim.x) {
-        const int ox = t / NV, r = t - ox * NV;
-        const int k = r % 6, node = r / 6, A = node % p, bc = node / p;
-        R s = R(0);
-        for (int a = 0; a < p; ++a) s += Ms[ox][a][A] * in[(bc * p + a) * 6 + k];
-        tx[t] = s;
-    }
-    __syncthreads();
-    // y: ty[ox + 2 oy][((c p + B) p + A) 6 + k] = sum_b M[oy][b][B] tx[ox][((c p + b) p + A) 6 + k]
-    for (int t = threadIdx.x; t < 4 * NV; t += blockDim.x) {
-        const int q = t / NV, r = t - q * NV, ox = q & 1, oy = q >> 1;
-        const int k = r % 6, node = r / 6, A = node % p, B = (node / p) % p, c = node / (p * p);
-        R s = R(0);
-        for (int b = 0; b < p; ++b) s += Ms[oy][b][B] * tx[ox * NV + ((c * p + b) * p + A) * 6 + k];
-        ty[t] = s;
-    }
-    __syncthreads();
-    // z: child (ox, oy, oz) += sum_c M[oz][c][C] ty[ox + 2 oy][((c p + B) p + A) 6 + k]
-    for (int t = threadIdx.x; t < 8 * NV; t += blockDim.x) {
-        const int ci = t / NV, r = t - ci * NV, oz = ci >> 2;
-        const int64_t base = s_ch[ci];
-        if (base < 0) continue;
-        const int k = r % 6, node = r / 6, AB = node % (p * p), C = node / (p * p);
-        const R *tq = ty + (ci & 3) * NV;
-        R s = R(0);
-        for (int c = 0; c < p; ++c) s += Ms[oz][c][C] * tq[(c * p * p + AB) * 6 + k];
-        S[base + r] += s;
-    }
 }
 
 // ---------------------------------------------------------------- M2L (FP64)
@@ -548,36 +191,6 @@ __global__ void k_scatter_targets(int64_t n, const int *__restrict__ pos, const 
     if (k >= n) return;
     const double *s = src + 6 * int64_t(pos[k]);
     for (int a = 0; a < 6; ++a) dst[6 * k + a] = s[a];
-}
-
-// M[c][A][a] = ell_A((c + t_a) / 2): the parent's basis function A at node a of child c
-// (equispaced nodes as before; Chebyshev nodes, the zeros of T_p on [0, 1])
-Transfer make_transfer(int p, int nodes) {
-    Transfer t{};
-    if (nodes == GBFMM_NODES_CHEBYSHEV) {
-        double tn[GB_MAXP];
-        for (int b = 0; b < p; ++b) tn[b] = 0.5 * (1.0 - std::cos(M_PI * double(2 * b + 1) / double(2 * p)));
-        for (int c = 0; c < 2; ++c)
-            for (int A = 0; A < p; ++A)
-                for (int a = 0; a < p; ++a) {
-                    const double x = (c + tn[a]) / 2.0;
-                    double v = 1.0;
-                    for (int b = 0; b < p; ++b)
-                        if (b != A) v *= (x - tn[b]) / (tn[A] - tn[b]);
-                    t.M[c][A][a] = v;
-                }
-        return t;
-    }
-    for (int c = 0; c < 2; ++c)
-        for (int A = 0; A < p; ++A)
-            for (int a = 0; a < p; ++a) {
-                double x = (c + double(a) / (p - 1)) / 2.0;
-                double v = 1.0;
-                for (int b = 0; b < p; ++b)
-                    if (b != A) v *= (x - double(b) / (p - 1)) / (double(A - b) / (p - 1));
-                t.M[c][A][a] = v;
-            }
-    return t;
 }
 
 }  // namespace
@@ -715,6 +328,11 @@ int work_counts(gbfmm_ctx *ctx, int64_t *res) {
     return GBFMM_OK;
 }
 
+template <typename R>
+int upward(gbfmm_ctx *ctx, const int *occ, R *W, int64_t n_fine);  // transfer.cu
+template <typename R>
+int downward(gbfmm_ctx *ctx, const int *tocc, R *S, int64_t n_fine);
+
 void timer_mark(gbfmm_ctx *ctx) {
     if (!ctx->timer.on || ctx->timer.n >= 16) return;
     cudaEventRecord(ctx->timer.ev[ctx->timer.n++], ctx->stream);
@@ -729,10 +347,8 @@ int near_run(gbfmm_ctx *ctx, bool free_targets, int64_t n_t, double *sig);   // 
 int fmm_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     cudaStream_t st = ctx->stream;
     const int p = ctx->opt.p, L = ctx->L, P3 = p * p * p;
-    const int64_t nl = ctx->n_leaves;
     int *occ = ctx->d_tmp_i;                 // [n_cells] sources per cell
     int *tocc = free_targets ? occ + ctx->n_cells : occ;
-    Transfer tr = make_transfer(p, ctx->opt.nodes);
 
     timer_mark(ctx);
     if (int rc = near_prepare(ctx)) return rc;
@@ -740,14 +356,7 @@ int fmm_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     if (free_targets) compute_occ(ctx, ctx->d_t_start, tocc);
     CK(cudaGetLastError());
     timer_mark(ctx);
-    if (L >= 3) {
-        ++ctx->launches;
-        k_p2m<double><<<unsigned(nl), 256, 0, st>>>(p, ctx->opt.nodes, L, ctx->d_box, ctx->d_leaf_start, ctx->d_y, ctx->d_q, ctx->d_W);
-        const size_t sm9 = size_t(2) * P3 * 9 * sizeof(double);
-        for (int lev = L - 2; lev >= 2; --lev)
-            { ++ctx->launches; k_m2m<double><<<unsigned(int64_t(1) << (3 * lev)), 256, sm9, st>>>(p, lev, tr, occ, ctx->d_W); }
-        CK(cudaGetLastError());
-    }
+    if (int rc = upward<double>(ctx, occ, ctx->d_W, 0)) return rc;
     timer_mark(ctx);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(st, &cap));
@@ -762,12 +371,7 @@ int fmm_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
         CK(cudaGetLastError());
     }
     timer_mark(ctx);
-    if (L >= 4) {
-        const size_t sm6 = size_t(2) * P3 * 6 * sizeof(double);
-        for (int lev = 3; lev <= L - 1; ++lev)
-            { ++ctx->launches; k_l2l<double><<<unsigned(int64_t(1) << (3 * lev)), 256, sm6, st>>>(p, lev, tr, tocc, ctx->d_S); }
-        CK(cudaGetLastError());
-    }
+    if (int rc = downward<double>(ctx, tocc, ctx->d_S, 0)) return rc;
     timer_mark(ctx);
     if (int rc = near_run(ctx, free_targets, n_t, free_targets ? ctx->d_t_sig : ctx->d_sig)) return rc;
     timer_mark(ctx);
@@ -798,13 +402,8 @@ int targets_scatter(gbfmm_ctx *ctx, int64_t n_t, double *sigma) {
     return GBFMM_OK;
 }
 
-int mixed_kernel_attrs(gbfmm_ctx *ctx);
-
 int fmm_kernel_attrs(gbfmm_ctx *ctx) {
-    if (int rc = mixed_kernel_attrs(ctx)) return rc;
     const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
-    CK(cudaFuncSetAttribute(k_m2m<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(2 * P3 * 9 * sizeof(double))));
-    CK(cudaFuncSetAttribute(k_l2l<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(2 * P3 * 6 * sizeof(double))));
     CK(cudaFuncSetAttribute(k_m2l_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, int(P3 * 9 * sizeof(double))));
     return GBFMM_OK;
 }
@@ -830,49 +429,23 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
         if (int rc = m2l_tc_setup(ctx)) return rc;
         if (int rc = m2l_tc_prepare(ctx)) return rc;
     }
-    cudaStream_t st = ctx->stream;
     const bool t64 = ctx->opt.precision == GBFMM_MIXED_F64T;  // FP64 P2M, M2M, L2L, L2P
-    const int p = ctx->opt.p, L = ctx->L, P3 = p * p * p;
-    const int64_t nl = ctx->n_leaves;
+    const int L = ctx->L;
     int *occ = ctx->d_tmp_i;
     int *tocc = free_targets ? occ + ctx->n_cells : occ;
-    Transfer tr = make_transfer(p, ctx->opt.nodes);
     // adaptive tree: the children of split leaves take part in nodal-force passes (free
     // targets keep the uniform tree, whose near field covers whole leaves)
     auto &RF = ctx->rf;
     const int64_t n_fine = RF.fine_rows();
     const bool fine = RF.on && !free_targets && L >= 3 && n_fine > 0;
-    const int *n_ref = RF.ref_start ? RF.ref_start + nl : nullptr;
     timer_mark(ctx);
     if (int rc = near_prepare(ctx)) return rc;
     compute_occ(ctx, ctx->d_leaf_start, occ);
     if (free_targets) compute_occ(ctx, ctx->d_t_start, tocc);
     CK(cudaGetLastError());
     timer_mark(ctx);
-    if (L >= 3) {
-        ++ctx->launches;
-        if (t64)
-            k_p2m<double><<<unsigned(nl), 256, 0, st>>>(p, ctx->opt.nodes, L, ctx->d_box, ctx->d_leaf_start, ctx->d_y, ctx->d_q,
-                                                        ctx->d_W);
-        else
-            k_p2m<float><<<unsigned(nl), 256, 0, st>>>(p, ctx->opt.nodes, L, ctx->d_box, ctx->d_leaf_start, ctx->d_y, ctx->d_q,
-                                                       ctx->d_Wf);
-        for (int lev = L - 2; lev >= 2; --lev) {
-            ++ctx->launches;
-            const unsigned g = unsigned(int64_t(1) << (3 * lev));
-            if (t64)
-                k_m2m<double><<<g, 256, size_t(2) * P3 * 9 * sizeof(double), st>>>(p, lev, tr, occ, ctx->d_W);
-            else
-                k_m2m_merge<float><<<g, 256, size_t(4) * P3 * 9 * sizeof(float), st>>>(p, lev, tr, occ, ctx->d_Wf);
-        }
-        if (fine) {
-            // the children of split leaves: their multipole values
-            ++ctx->launches;
-            k_p2m_fine<float><<<unsigned(n_fine), 256, 0, st>>>(p, ctx->opt.nodes, L, ctx->d_box, n_ref, RF.ref_leaf,
-                                                                RF.child_start, ctx->d_y, ctx->d_q, RF.W7);
-        }
-        CK(cudaGetLastError());
-    }
+    if (int rc = t64 ? upward<double>(ctx, occ, ctx->d_W, 0) : upward<float>(ctx, occ, ctx->d_Wf, fine ? n_fine : 0))
+        return rc;
     timer_mark(ctx);
     if (L >= 3) {
         int rc = m2l_tc_run(ctx, ctx->d_Wf, t64 ? ctx->d_W : nullptr, occ, tocc, ctx->d_Sf, t64 ? ctx->d_S : nullptr,
@@ -880,38 +453,11 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
         if (rc) return rc;
     }
     timer_mark(ctx);
-    if (L >= 4) {
-        for (int lev = 3; lev <= L - 1; ++lev) {
-            ++ctx->launches;
-            const unsigned g = unsigned(int64_t(1) << (3 * lev));
-            if (t64)
-                k_l2l<double><<<g, 256, size_t(2) * P3 * 6 * sizeof(double), st>>>(p, lev, tr, tocc, ctx->d_S);
-            else  // one block per parent
-                k_l2l_split<float><<<g / 8, 256, size_t(7) * P3 * 6 * sizeof(float), st>>>(p, lev, tr, tocc,
-                                                                                          ctx->d_Sf);
-        }
-        CK(cudaGetLastError());
-    }
-    if (fine) {
-        // the children's local values (the level-L M2L, written by m2l_tc_run) += the parent's
-        ++ctx->launches;
-        k_l2l_fine<float><<<unsigned(n_fine), 256, size_t(2) * P3 * 6 * sizeof(float), st>>>(
-            p, L, tr, n_ref, RF.ref_leaf, RF.child_start, ctx->d_Sf, RF.S7);
-        CK(cudaGetLastError());
-    }
+    // (the children's local values, the level-L M2L, were written by m2l_tc_run)
+    if (int rc = t64 ? downward<double>(ctx, tocc, ctx->d_S, 0) : downward<float>(ctx, tocc, ctx->d_Sf, fine ? n_fine : 0))
+        return rc;
     timer_mark(ctx);
     if (int rc = near_run(ctx, free_targets, n_t, free_targets ? ctx->d_t_sig : ctx->d_sig)) return rc;
     timer_mark(ctx);
-    return GBFMM_OK;
-}
-
-int mixed_kernel_attrs(gbfmm_ctx *ctx) {
-    const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
-    CK(cudaFuncSetAttribute(k_m2m_merge<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            int(4 * P3 * 9 * sizeof(float))));
-    CK(cudaFuncSetAttribute(k_l2l_split<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            int(7 * P3 * 6 * sizeof(float))));
-    CK(cudaFuncSetAttribute(k_l2l_fine<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            int(2 * P3 * 6 * sizeof(float))));
     return GBFMM_OK;
 }

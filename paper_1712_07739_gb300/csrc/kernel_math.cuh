@@ -6,6 +6,8 @@
 // components are kept, in the order k = 3 * pair + q with pairs
 // (0,0) (1,1) (2,2) (1,2) (0,2) (0,1).
 #pragma once
+#include <cmath>
+
 #include "internal.cuh"
 
 // Isotropic medium: derivative of the Kelvin Green's function
@@ -196,39 +198,38 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 // footnote); nodes = GBFMM_NODES_CHEBYSHEV, the zeros of the Chebyshev
 // polynomial T_p mapped to [0, 1], t_a = (1 - cos((2a + 1) pi / (2p))) / 2
 // (the nodes of the Chebyshev FMM, Sec. 3).
-template <typename R>
-__device__ __forceinline__ R cheb_node(int a, int p) {
-    if constexpr (sizeof(R) == 8)
-        return 0.5 * (1.0 - cospi(double(2 * a + 1) / double(2 * p)));
-    else
-        return 0.5f * (1.0f - cospif(float(2 * a + 1) / float(2 * p)));
+__device__ __forceinline__ double cheb_node(int a, int p) {
+    return 0.5 * (1.0 - cospi(double(2 * a + 1) / double(2 * p)));
 }
 
+// The nodes and the inverse denominators of the basis, made on the host in FP64 and passed by
+// value (kernel parameters): one product of p factors per value.
 template <typename R>
-__device__ __forceinline__ void lagrange_1d(int p, R t, R *out, int nodes) {
-    if (nodes == GBFMM_NODES_CHEBYSHEV) {
-        // node positions recomputed in the loops: a local table of them, inlined into
-        // the near-field kernels next to the three output arrays, gave wrong basis values
-        // there (measured: the y-axis values equalled the z-axis ones)
-        for (int a = 0; a < p; ++a) {
-            const R ta = cheb_node<R>(a, p);
-            R v = R(1);
-            for (int b = 0; b < p; ++b)
-                if (b != a) {
-                    const R tb = cheb_node<R>(b, p);
-                    v *= (t - tb) / (ta - tb);
-                }
-            out[a] = v;
-        }
-        return;
-    }
-    const R inv = R(1) / R(p - 1);
+struct NodeTab {
+    R t[GB_MAXP], w[GB_MAXP];
+};
+template <typename R>
+inline NodeTab<R> make_nodes(int p, int nodes) {
+    NodeTab<R> n{};
+    double t[GB_MAXP];
+    for (int a = 0; a < p; ++a)
+        t[a] = nodes == GBFMM_NODES_CHEBYSHEV ? 0.5 * (1.0 - std::cos(M_PI * double(2 * a + 1) / double(2 * p)))
+                                              : double(a) / double(p - 1);
     for (int a = 0; a < p; ++a) {
-        R v = R(1);
+        double d = 1.0;
         for (int b = 0; b < p; ++b)
-            if (b != a) v *= (t - R(b) * inv) / (R(a - b) * inv);
-        out[a] = v;
+            if (b != a) d *= t[a] - t[b];
+        n.t[a] = R(t[a]);
+        n.w[a] = R(1.0 / d);
     }
+    return n;
+}
+template <typename R>
+__device__ __forceinline__ R lagrange_at(const NodeTab<R> &n, int p, int a, R t) {
+    R v = n.w[a];
+    for (int b = 0; b < p; ++b)
+        if (b != a) v *= t - n.t[b];
+    return v;
 }
 
 // The kernel of Sec. 2, Eq. "kernel" at separation d (FP64, 54 values

@@ -74,9 +74,9 @@ __global__ void k_node_ops(int p, int nodes, int o0, int nc, const int *__restri
         const int mx = mm % p, my = (mm / p) % p, mz = mm / (p * p);
         double K[54];
         if (nodes == GBFMM_NODES_CHEBYSHEV) {
-            const double d[3] = {ox + cheb_node<double>(lx, p) - cheb_node<double>(mx, p),
-                                 oy + cheb_node<double>(ly, p) - cheb_node<double>(my, p),
-                                 oz + cheb_node<double>(lz, p) - cheb_node<double>(mz, p)};
+            const double d[3] = {ox + cheb_node(lx, p) - cheb_node(mx, p),
+                                 oy + cheb_node(ly, p) - cheb_node(my, p),
+                                 oz + cheb_node(lz, p) - cheb_node(mz, p)};
             kernel_at(mat, Asym, d, K);
         } else {
             const int R0 = (lat_n - 1) / 2;

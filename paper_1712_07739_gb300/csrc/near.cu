@@ -830,34 +830,59 @@ __global__ void __launch_bounds__(near_warps<R>() * 32, near_blocks<R>())
 }
 
 // ---------------------------------------------------------------- combine
-// far field (L2P) plus the stress of the summed strain rows, in a fixed order
-template <typename SR>
-__device__ __forceinline__ void l2p(int p, int nodes, const double c0[3], double ih, const double *x,
-                                    const SR *__restrict__ Sl, double out[6]) {
-    SR bx[GB_MAXP], by[GB_MAXP], bz[GB_MAXP], acc[6];
-    for (int e = 0; e < 6; ++e) acc[e] = SR(0);
-    lagrange_1d<SR>(p, SR((x[0] - c0[0]) * ih), bx, nodes);
-    lagrange_1d<SR>(p, SR((x[1] - c0[1]) * ih), by, nodes);
-    lagrange_1d<SR>(p, SR((x[2] - c0[2]) * ih), bz, nodes);
-    for (int lz = 0; lz < p; ++lz)
-        for (int ly = 0; ly < p; ++ly) {
-            const SR wyz = by[ly] * bz[lz];
-            for (int lx = 0; lx < p; ++lx) {
-                const SR w = bx[lx] * wyz;
-                const SR *s6 = Sl + ((lz * p + ly) * p + lx) * 6;
-                for (int e = 0; e < 6; ++e) acc[e] += w * __ldg(s6 + e);
+// Far field (L2P) plus the stress of the summed strain rows, LANES threads per point.  Eight lanes
+// share a point's 3 p basis values, take every eighth (y, z) row of the p^3 local values and every
+// eighth of its rows, and are added by a fixed tree: in the smallest calls one thread's chain is
+// the time (157 segments 64 -> 27 us, FP64 167 us).  One thread per point where there are enough
+// points to fill the GPU: the 32 points of a warp then mostly read the same local values (4M
+// points: 7.3 ms with eight lanes).
+constexpr int64_t kCombinePoints = 65536;  // up to this many points: eight lanes
+
+template <int LANES, typename SR>
+__device__ __forceinline__ void l2p(int p, const NodeTab<SR> &nt, SR *basis, int g, const double c0[3], double ih,
+                                    const double *x, const SR *__restrict__ Sl, double out[6]) {
+    for (int i = g; i < 3 * p; i += LANES) {
+        const int d = i / p;
+        basis[i] = lagrange_at<SR>(nt, p, i - d * p, SR((x[d] - (d == 0 ? c0[0] : d == 1 ? c0[1] : c0[2])) * ih));
+    }
+    __syncwarp();
+    SR acc[6] = {SR(0), SR(0), SR(0), SR(0), SR(0), SR(0)};
+    for (int r = g; r < p * p; r += LANES) {
+        const SR wyz = basis[p + r % p] * basis[2 * p + r / p];
+        SR v[6] = {SR(0), SR(0), SR(0), SR(0), SR(0), SR(0)};
+        for (int lx = 0; lx < p; ++lx) {
+            const SR w = basis[lx];
+            const SR *s6 = Sl + (r * p + lx) * 6;  // 24 or 48 bytes, read in pairs
+            if constexpr (sizeof(SR) == 4) {
+                const float2 *q = reinterpret_cast<const float2 *>(s6);
+                const float2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+                v[0] += w * a.x, v[1] += w * a.y, v[2] += w * b.x, v[3] += w * b.y, v[4] += w * c.x, v[5] += w * c.y;
+            } else {
+                const double2 *q = reinterpret_cast<const double2 *>(s6);
+                const double2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+                v[0] += w * a.x, v[1] += w * a.y, v[2] += w * b.x, v[3] += w * b.y, v[4] += w * c.x, v[5] += w * c.y;
             }
         }
-    for (int e = 0; e < 6; ++e) out[e] = double(acc[e]);
+        for (int e = 0; e < 6; ++e) acc[e] += wyz * v[e];
+    }
+    for (int e = 0; e < 6; ++e) {
+        for (int o = LANES / 2; o > 0; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+        out[e] = double(acc[e]);
+    }
 }
 
-template <bool SYM>
-__global__ void k_near_combine(int p, int nodes, const __grid_constant__ NearTree tr, const double *__restrict__ C,
-                               const int *__restrict__ tleaf, const double *__restrict__ xt,
-                               const float *__restrict__ S, const double *__restrict__ S64, double *__restrict__ sig,
-                               const int *__restrict__ pfine, const float *__restrict__ S7) {
-    const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (t >= tr.n_t) return;
+template <bool SYM, int LANES, typename SR>
+__global__ void __launch_bounds__(256) k_near_combine(int p, const __grid_constant__ NodeTab<SR> nt,
+                                                      const __grid_constant__ NearTree tr,
+                                                      const double *__restrict__ C, const int *__restrict__ tleaf,
+                                                      const double *__restrict__ xt, const SR *__restrict__ S,
+                                                      double *__restrict__ sig, const int *__restrict__ pfine,
+                                                      const SR *__restrict__ S7) {
+    __shared__ SR s_basis[256 / LANES][3 * GB_MAXP + 1];  // (+ 1: one thread per point would meet one bank)
+    const int64_t t0 = (blockIdx.x * int64_t(256) + threadIdx.x) / LANES;
+    const int g = threadIdx.x % LANES;
+    const bool valid = t0 < tr.n_t;
+    const int64_t t = valid ? t0 : tr.n_t - 1;  // surplus lanes repeat the last point
     const int nlv = 1 << (tr.L - 1);
     const int64_t leaf = tleaf[t];
     int cx, cy, cz;
@@ -868,22 +893,17 @@ __global__ void k_near_combine(int p, int nodes, const __grid_constant__ NearTre
         const int P3 = p * p * p;
         double h = tr.box->H / nlv, ih = double(nlv) / tr.box->H;
         double c0[3] = {tr.box->origin[0] + cx * h, tr.box->origin[1] + cy * h, tr.box->origin[2] + cz * h};
-        const int64_t cell = (cell_base_d(tr.L - 1) + leaf) * int64_t(P3) * 6;
-        if (S64) {
-            l2p<double>(p, nodes, c0, ih, xt + 3 * t, S64 + cell, far);
-        } else {
-            const float *Sl = S + cell;
-            if (f >= 0) {
-                // a point of a split leaf: its child's local values and cell (adaptive tree)
-                h *= 0.5;
-                ih *= 2.0;
-                c0[0] += (f & 1) * h;
-                c0[1] += ((f >> 1) & 1) * h;
-                c0[2] += ((f >> 2) & 1) * h;
-                Sl = S7 + int64_t(f) * P3 * 6;
-            }
-            l2p<float>(p, nodes, c0, ih, xt + 3 * t, Sl, far);
+        const SR *Sl = S + (cell_base_d(tr.L - 1) + leaf) * int64_t(P3) * 6;
+        if (f >= 0) {
+            // a point of a split leaf: its child's local values and cell (adaptive tree)
+            h *= 0.5;
+            ih *= 2.0;
+            c0[0] += (f & 1) * h;
+            c0[1] += ((f >> 1) & 1) * h;
+            c0[2] += ((f >> 2) & 1) * h;
+            Sl = S7 + int64_t(f) * P3 * 6;
         }
+        l2p<LANES, SR>(p, nt, s_basis[threadIdx.x / LANES], g, c0, ih, xt + 3 * t, Sl, far);
     }
     double e6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     auto add_row = [&](long long r) {
@@ -893,19 +913,19 @@ __global__ void k_near_combine(int p, int nodes, const __grid_constant__ NearTre
     };
     {
         const NearPlan pl = tr.plan[leaf];
-        const int nt = tr.tstart[leaf + 1] - tr.tstart[leaf], k = int(t - tr.tstart[leaf]);
-        for (int b = 0; b < pl.cb; ++b) add_row(pl.base + (long long)b * nt + k);
+        const int nt_l = tr.tstart[leaf + 1] - tr.tstart[leaf], k = int(t - tr.tstart[leaf]);
+        for (int b = g; b < pl.cb; b += LANES) add_row(pl.base + (long long)b * nt_l + k);
     }
     if (SYM) {
         const int rank = int(t - tr.sstart[leaf]);
-        for (int d = 0; d < 14; ++d) {
+        for (int d = g; d < 14; d += LANES) {
             // the leaf that holds this one in direction d of its list
             const int64_t A = neighbour(cx, cy, cz, 13 - d, nlv);
             if (A < 0) continue;
-            const int nt = tr.tstart[A + 1] - tr.tstart[A];
-            if (nt == 0) continue;
+            const int nt_a = tr.tstart[A + 1] - tr.tstart[A];
+            if (nt_a == 0) continue;
             const NearPlan pl = tr.plan[A];
-            const long long r = pl.base + (long long)pl.cb * nt + tr.lp[14 * A + d] + rank;
+            const long long r = pl.base + (long long)pl.cb * nt_a + tr.lp[14 * A + d] + rank;
             const bool splitA = tr.ref_start && tr.ref_start[A + 1] > tr.ref_start[A];
             // a plain leaf's tile meets its own leaf from the tile's first target on; a split
             // leaf's rows were zeroed first
@@ -920,10 +940,16 @@ __global__ void k_near_combine(int p, int nodes, const __grid_constant__ NearTre
             }
         }
     }
+    __syncwarp();
+    for (int e = 0; e < 6; ++e)
+        for (int o = LANES / 2; o > 0; o >>= 1) e6[e] += __shfl_xor_sync(0xffffffffu, e6[e], o);
+    if (!valid) return;
+#pragma unroll
     for (int m = 0; m < 6; ++m) {
-        double s = far[m];
+        if (LANES > 1 && g != m) continue;
+        double s = 0.0;
         for (int e = 0; e < 6; ++e) s += C[6 * m + e] * e6[e];
-        sig[6 * t + m] = s;
+        sig[6 * t + m] = s + far[m];
     }
 }
 
@@ -1034,6 +1060,21 @@ static int launch_pairs(gbfmm_ctx *ctx, const NearTree &tr, const NearMedium<R> 
     return GBFMM_OK;
 }
 
+template <bool SYM, typename SR>
+static int launch_combine(gbfmm_ctx *ctx, const NearTree &tr, const int *tleaf, const double *xt, const SR *S, double *sig,
+                          const int *pfine, const SR *S7) {
+    const NodeTab<SR> nt = make_nodes<SR>(ctx->opt.p, ctx->opt.nodes);
+    ++ctx->launches;
+    if (tr.n_t <= kCombinePoints)
+        k_near_combine<SYM, 8, SR><<<nblk(tr.n_t * 8, 256), 256, 0, ctx->stream>>>(ctx->opt.p, nt, tr, ctx->d_mat->V, tleaf,
+                                                                                    xt, S, sig, pfine, S7);
+    else
+        k_near_combine<SYM, 1, SR><<<nblk(tr.n_t, 256), 256, 0, ctx->stream>>>(ctx->opt.p, nt, tr, ctx->d_mat->V, tleaf, xt,
+                                                                               S, sig, pfine, S7);
+    CK(cudaGetLastError());
+    return GBFMM_OK;
+}
+
 template <typename R, bool SYM>
 static int run_pairs(gbfmm_ctx *ctx, const int *tstart, const double *xt, int64_t n_t, const int *tleaf, double *sig) {
     if (int rc = pairs_alloc(ctx, n_t, !SYM)) return rc;
@@ -1100,12 +1141,9 @@ static int run_pairs(gbfmm_ctx *ctx, const int *tstart, const double *xt, int64_
             rc = launch_pairs<R, HM_GENERAL, SYM, false>(ctx, tr, md, ln);
     }
     if (rc) return rc;
-    const double *S64 = ctx->opt.precision == GBFMM_MIXED ? nullptr : ctx->d_S;
-    ++ctx->launches;
-    k_near_combine<SYM><<<nblk(n_t, 256), 256, 0, st>>>(ctx->opt.p, ctx->opt.nodes, tr, ctx->d_mat->V, tleaf, xt, ctx->d_Sf,
-                                                        S64, sig, fine ? ctx->rf.pfine : nullptr, ctx->rf.S7);
-    CK(cudaGetLastError());
-    return GBFMM_OK;
+    const int *pfine = fine ? ctx->rf.pfine : nullptr;
+    if (ctx->opt.precision == GBFMM_MIXED) return launch_combine<SYM, float>(ctx, tr, tleaf, xt, ctx->d_Sf, sig, pfine, ctx->rf.S7);
+    return launch_combine<SYM, double>(ctx, tr, tleaf, xt, ctx->d_S, sig, nullptr, nullptr);  // FP64 local values
 }
 
 // Near field and L2P of a pass, into sig (sorted order).  free_targets: the n_t sorted free

@@ -106,7 +106,8 @@ typedef struct {
                               many consecutive runs, each accumulated in tensor memory from
                               zero and added to the local values in FP32 (FP64 with
                               GBFMM_MIXED_F64T); shorter accumulation chains, one launch per
-                              run.  0 = 1; fmm_default_options: 7. */
+                              run.  0 = 1; fmm_default_options: 7.  Levels 2 .. 4 are summed
+                              together over the 316 offsets, in at least this many runs. */
     int m2l_basis;         /* MIXED: operands of the tensor-core M2L.  0 = the node values of
                               Eq. "m2l" (multipole values at the source cell's nodes); 1 = the
                               Legendre moments of each source cell, sum_j P_k(y_j) q_j with

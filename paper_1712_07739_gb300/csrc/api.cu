@@ -97,7 +97,7 @@ static int ensure_tree_buffers(gbfmm_ctx *ctx) {
                           {{(void **)&ctx->d_leaf_start, (nl + 1) * sizeof(int)},
                            {(void **)&ctx->d_t_start, (nl + 1) * sizeof(int)},
                            {(void **)&ctx->d_cnt, nl * sizeof(int)},
-                           {(void **)&ctx->d_scan, scan_blocks(nl) * sizeof(int)},
+                           {(void **)&ctx->d_scan, scan_blocks(2 * nl) * sizeof(int)},
                            {(void **)&ctx->d_cursor, nl * sizeof(int)}},
                           "leaves"))
         return rc;
@@ -290,11 +290,11 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
                           c->tc.Xh, c->tc.Xl, c->tc.d_scal, c->tc.d_bits, c->tc.Wc, c->tc.Sc, c->tc.blas_ws,
                           c->rf.child_of, c->rf.ref_start, c->rf.ref_leaf, c->rf.child_start, c->rf.pfine,
                           c->rf.W7, c->rf.S7, c->rf.Wc7, c->rf.Sc7, c->tc.d_pcnt, c->tc.d_pairs, c->tc.Gh,
-                          c->tc.Gl, c->tc.Yf};
+                          c->tc.Gl, c->tc.Yf, c->tc.few_list, c->tc.few_part};
     mix(ptrs, sizeof(ptrs));
     v(c->mat.mode), v(c->mat.Q), v(c->mat.cubic), v(c->tc.n_work), v(c->tc.split), v(c->tc.tf32);
     mix(c->tc.wofs, sizeof(c->tc.wofs));
-    v(c->tc.n_slots), v(c->tc.n_seg), v(c->mlp.trained);
+    v(c->tc.n_slots), v(c->tc.n_seg), v(c->tc.few_top), v(c->tc.few_work), v(c->mlp.trained);
     v(c->tc.r1), v(c->tc.r2), v(c->rf.cap_ref), v(c->rf.n_ref_host), v(c->tc.blas);
     return h;
 }

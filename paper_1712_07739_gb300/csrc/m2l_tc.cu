@@ -31,6 +31,14 @@
 // modes: TF32 operands; FP16 operands with a power-of-two scale per level for
 // W and one for the operators (FP16 carries 3 more mantissa bits than BF16).
 //
+// Few cells.  Levels 2 .. 4 hold 8 classes of at most 8, 64 and 512 cells, so their tiles above are
+// mostly padding and every CTA streams its operator rows of 189 offsets for a handful of cells
+// (6,011 segments, p = 6: 23 GB of operators for 68 GFLOP of products, 8.7 of 9.5 ms).  k_m2l_few
+// takes the cells of these levels together, 384 to a CTA whatever their level and class, all 316
+// offsets, and spreads the offsets over CTAs (sections of the offset list) so that one set of
+// cells occupies the GPU; each operator byte is then read once per set.  The sections' sums go to
+// scratch and are added in their order (k_few_sum).
+//
 // Warp roles (192 threads): warp 0 loads the operator rows by TMA, warp 1
 // owns TMEM and issues the MMAs, warps 2-5 gather the multipole rows (each
 // thread waits for its copies, fences them to the async proxy and arrives on
@@ -591,6 +599,317 @@ __global__ void __launch_bounds__(192, 1)
     }
 }
 
+// ---------------------------------------------------------------- few cells
+constexpr int kFewTop = 4;     // deepest level taken together: 64 + 512 + 4,096 cells at most
+constexpr int kFewRows = 384;  // cells per CTA (three tiles of 128)
+constexpr int kFewSections = 64;
+struct FewCount {
+    int cells, sets, sections;
+};
+struct FewParams {
+    M2LParams P;
+    short lo[316];  // residual operator of an offset, -1 without
+    int groups;
+};
+__constant__ signed char c_o316[316][3];
+
+// sections of the offset list for a number of cell sets: about four CTAs per SM, no fewer than
+// m2l_chunks (each section is one accumulation in tensor memory)
+__host__ __device__ inline int few_sections(int sets, int groups, int chunks, int sms) {
+    const int want = (4 * sms + sets * groups - 1) / (sets * groups);
+    const int top = chunks > kFewSections ? chunks : kFewSections;
+    return want < chunks ? chunks : (want > top ? top : want);
+}
+
+// cells of levels 2 .. top that hold targets, in level and linear order: x | y << 5 | z << 10 | level << 15
+__global__ void __launch_bounds__(1024) k_few_list(int top, int groups, int chunks, int sms, const int *__restrict__ tocc,
+                                                   int *__restrict__ list, FewCount *__restrict__ cnt) {
+    __shared__ int s_warp[32], s_base;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_base = 0;
+    __syncthreads();
+    const int n_all = int(cell_base_d(top + 1) - cell_base_d(2));
+    for (int i0 = 0; i0 < n_all; i0 += 1024) {
+        const int i = i0 + threadIdx.x;
+        int code = 0;
+        bool on = false;
+        if (i < n_all) {
+            const int64_t g = cell_base_d(2) + i;
+            int l = 2;
+            while (l < top && g >= cell_base_d(l + 1)) ++l;
+            const int c = int(g - cell_base_d(l)), n = 1 << l;
+            on = tocc[g] > 0;
+            code = (c & (n - 1)) | (((c >> l) & (n - 1)) << 5) | ((c >> (2 * l)) << 10) | (l << 15);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) s_warp[w] = __popc(m);
+        __syncthreads();
+        int before = s_base;
+        for (int k = 0; k < w; ++k) before += s_warp[k];
+        if (on) list[before + __popc(m & ((1u << lane) - 1u))] = code;
+        __syncthreads();
+        if (threadIdx.x == 1023) s_base = before + s_warp[31];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const int n = s_base, sets = (n + kFewRows - 1) / kFewRows;
+        *cnt = FewCount{n, sets, sets ? few_sections(sets, groups, chunks, sms) : 0};
+    }
+}
+
+// byte offset of the packed multipole row of cell (x, y, z) of a level
+__device__ __forceinline__ int64_t packed_row(const M2LParams &P, int level, int x, int y, int z) {
+    const int m = 1 << (level - 1), cls = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
+    return P.wofs[level] + (((int64_t(cls) * m + z / 2) * m + y / 2) * m + x / 2) * P.row_bytes;
+}
+
+// the source at cell - o when it lies in the cell's interaction list and holds segments
+__device__ __forceinline__ bool few_source(int code, int ox, int oy, int oz, const int *__restrict__ occ, int &level,
+                                           int &x, int &y, int &z) {
+    const int tx = code & 31, ty = (code >> 5) & 31, tz = (code >> 10) & 31;
+    level = code >> 15;
+    const int n = 1 << level;
+    x = tx - ox, y = ty - oy, z = tz - oz;
+    if (x < 0 || y < 0 || z < 0 || x >= n || y >= n || z >= n) return false;
+    if (abs((tx >> 1) - (x >> 1)) > 1 || abs((ty >> 1) - (y >> 1)) > 1 || abs((tz >> 1) - (z >> 1)) > 1) return false;
+    return occ[cell_base_d(level) + (int64_t(z) * n + y) * n + x] > 0;
+}
+
+// Item (section, operator group, cell set), the sets fastest: CTAs that run together read the same
+// operator rows.  Levels up to 4 go here whatever their cells: with few of them the operators' bytes
+// bound the time (6,011 segments, p = 6: 8.6 -> 1.2 ms; 157 segments, p = 4: 390 -> 60 us; 50,000
+// segments, L = 5, p = 5, free targets: 6.2 -> 2.8 ms), and a level 4 full of cells is 13 sets of 316
+// offsets against 16 tiles of 189, better spread (a million segments: whole pass 166.1 -> 163.6 ms).
+// Level 5 would be 86 sets against 96 tiles that already fill the GPU.  Roles, stages and barriers as in k_m2l_tc with the cells as A.
+template <bool TF32>
+__global__ void __launch_bounds__(192, 1)
+    k_m2l_few(const __grid_constant__ FewParams F, const FewCount *__restrict__ cnt, const int *__restrict__ list,
+              const int *__restrict__ occ, float *__restrict__ part, int Np, int *__restrict__ status, int stages) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const M2LParams &P = F.P;
+    constexpr int TPC = 3, kStageA = TPC * kTileA;
+    const int stageB = P.ncta * 128, stage_bytes = kStageA + stageB;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * stages + 1);
+    __shared__ int s_code[kFewRows];
+    __shared__ uint32_t s_active[10];
+    __shared__ int s_stop;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int sets = cnt->sets, sections = cnt->sections, cells = cnt->cells;
+    if (threadIdx.x == 0) s_stop = *reinterpret_cast<volatile int *>(status) != 0;
+    if (threadIdx.x < 10) s_active[threadIdx.x] = 0u;
+    __syncthreads();
+    if (int(blockIdx.x) >= sets * F.groups * sections || s_stop) return;  // surplus block, or an earlier time-out
+    const int set = blockIdx.x % sets, group = (blockIdx.x / sets) % F.groups, sec = blockIdx.x / (sets * F.groups);
+    const int nrow = min(kFewRows, cells - set * kFewRows), tiles = (nrow + 127) / 128;
+    const int o_lo = 316 * sec / sections, o_hi = 316 * (sec + 1) / sections;
+    for (int r = threadIdx.x; r < kFewRows; r += 192) s_code[r] = r < nrow ? list[set * kFewRows + r] : -1;
+    __syncthreads();
+    for (int o = o_lo + warp; o < o_hi; o += 6) {
+        const int ox = c_o316[o][0], oy = c_o316[o][1], oz = c_o316[o][2];
+        bool hit = false;
+        for (int r = lane; r < nrow && !hit; r += 32) {
+            int l, x, y, z;
+            hit = few_source(s_code[r], ox, oy, oz, occ, l, x, y, z);
+        }
+        if (__any_sync(0xffffffffu, hit) && lane == 0) atomicOr(&s_active[o / 32], 1u << (o % 32));
+    }
+    if (threadIdx.x == 0) {
+        // full: the operator-load thread (expect_tx) + 128 gathering threads; empty: the MMA commit
+        for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&bars[s]), 129);
+        for (int s = stages; s < 2 * stages + 1; ++s) mbar_init(smem_u32(&bars[s]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(P.tmem_cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[stages]), accb = smem_u32(&bars[2 * stages]);
+    const uint32_t smem0 = smem_u32(smem);
+    auto active = [&](int o) { return (s_active[o / 32] >> (o % 32)) & 1u; };
+    uint32_t o_act = 0u;  // offsets of this section with a source
+    for (int i = 0; i < 10; ++i) o_act |= s_active[i];
+
+    if (warp == 0 && lane == 0) {
+        // ---------------- operator rows (B) by TMA
+        int it = 0;
+        bool ok = true;
+        for (int o = o_lo; o < o_hi && ok; ++o) {
+            if (!active(o)) continue;
+            const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+            for (int pass = 0; pass < np && ok; ++pass) {
+                const CUtensorMap *tb = pass == 2 ? &P.tmTlo : &P.tmT;
+                const int tidx = pass == 2 ? F.lo[o] : o;
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
+                    const int s = it % stages;
+                    if (!mbar_wait(empty0 + 8 * s, ((it / stages) & 1) ^ 1, status)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_expect_tx(full0 + 8 * s, uint32_t(stageB));
+                    if (P.drop_first && it == 0) continue;  // the MMA warp's wait on this stage runs out
+                    tma_load_3d(smem0 + s * stage_bytes + kStageA, tb, kb * P.kstep, group * P.ncta, tidx, full0 + 8 * s);
+                }
+            }
+        }
+    } else if (warp == 1 && lane == 0) {
+        // ---------------- MMA issuer
+        int it = 0;
+        bool ok = true;
+        for (int o = o_lo; o < o_hi && ok; ++o) {
+            if (!active(o)) continue;
+            const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+            for (int pass = 0; pass < np && ok; ++pass)
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
+                    const int s = it % stages;
+                    if (!mbar_wait(full0 + 8 * s, (it / stages) & 1, status)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t a = smem0 + s * stage_bytes;
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const uint64_t bd = sw128_desc(a + kStageA + kk * 32);
+                        for (int t = 0; t < tiles; ++t)
+                            mma_issue<TF32>(tmem + t * P.nsub, sw128_desc(a + t * kTileA + kk * 32), bd, P.idesc,
+                                            (it > 0 || kk > 0) ? 1u : 0u);
+                    }
+                    mma_commit(empty0 + 8 * s);
+                }
+        }
+        // fires when every MMA issued above has completed
+        if (o_act) mma_commit(accb);
+    } else if (warp >= 2) {
+        const int row = threadIdx.x - 64;
+        const bool any = o_act != 0u;
+        {
+            // ---------------- multipole rows (A), as in k_m2l_tc: each thread finds the source of its
+            // own rows, the copies go by 8 lanes per 128-byte row piece
+            const int lag = 1;
+            int it = 0, done = 0;
+            bool ok = true;
+            const int c = lane & 7, wrow0 = row - lane;
+            for (int o = o_lo; o < o_hi && ok; ++o) {
+                if (!active(o)) continue;
+                const int ox = c_o316[o][0], oy = c_o316[o][1], oz = c_o316[o][2];
+                int64_t own[TPC];
+                uint32_t own_nb = 0;  // bits t: a source; 4 + t: one whose level has the residual passes
+#pragma unroll
+                for (int t = 0; t < TPC; ++t) {
+                    own[t] = 0;
+                    const int code = s_code[t * 128 + row];
+                    int l, x, y, z;
+                    if (code >= 0 && few_source(code, ox, oy, oz, occ, l, x, y, z)) {
+                        own[t] = packed_row(P, l, x, y, z);
+                        own_nb |= (1u << t) | (((P.split_levels >> l) & 1) ? 16u << t : 0u);
+                    }
+                }
+                int64_t srcoff[8][TPC];
+                uint32_t nbm = 0, nbr = 0;  // bit 8 t + i: row 4 i + lane / 8 of tile t has a source
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int from = 4 * i + (lane >> 3);
+                    const uint32_t f = __shfl_sync(0xffffffffu, own_nb, from);
+#pragma unroll
+                    for (int t = 0; t < TPC; ++t) {
+                        srcoff[i][t] = __shfl_sync(0xffffffffu, own[t], from);
+                        nbm |= ((f >> t) & 1u) << (8 * t + i);
+                        nbr |= ((f >> (4 + t)) & 1u) << (8 * t + i);
+                    }
+                }
+                const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+                for (int pass = 0; pass < np && ok; ++pass) {
+                    const uint8_t *wb = pass == 1 ? P.Wlo : P.Whi;
+                    const uint32_t have = pass == 0 ? nbm : nbr;
+                    for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
+                        const int s = it % stages;
+                        if (!mbar_wait(empty0 + 8 * s, ((it / stages) & 1) ^ 1, status)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t sbase = smem0 + s * stage_bytes;
+                        const uint8_t *wk = wb + kb * 128 + 16 * c;
+#pragma unroll
+                        for (int t = 0; t < TPC; ++t)
+                            if (t < tiles)
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    const int r = wrow0 + 4 * i + (lane >> 3);
+                                    const bool on = (have >> (8 * t + i)) & 1u;
+                                    cp_async16(sbase + t * kTileA + r * 128 + ((c ^ (r & 7)) << 4),
+                                               on ? wk + srcoff[i][t] : wk, on ? 16u : 0u);
+                                }
+                        cp_async_commit();
+                        if (it - done >= lag) {
+                            cp_async_wait(lag);
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            mbar_arrive(full0 + 8 * (done % stages));
+                            ++done;
+                        }
+                    }
+                }
+            }
+            cp_async_wait(0);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            for (; done < it; ++done) mbar_arrive(full0 + 8 * (done % stages));
+        }
+        // ---------------- epilogue: TMEM -> this section's sums
+        const bool ok = any ? mbar_wait(accb, 0, status) : true;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const int q = warp % 4, trow = q * 32 + lane;
+        for (int t = 0; t < tiles; ++t) {
+            const int r = t * 128 + trow;
+            float *dst = part + ((int64_t(sec) * sets + set) * kFewRows + r) * Np + group * P.ncta;
+            for (int c0 = 0; c0 < P.nsub; c0 += 16) {
+                float v[16];
+                for (int i = 0; i < 16; ++i) v[i] = 0.f;
+                if (ok && any) tmem_ld16(tmem + (uint32_t(q * 32) << 16) + uint32_t(t * P.nsub + c0), v);
+                if (ok && r < nrow)
+                    for (int i = 0; i < 4; ++i)
+                        reinterpret_cast<float4 *>(dst + c0)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2],
+                                                                              v[4 * i + 3]);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(P.tmem_cols));
+    }
+}
+
+// local values of the listed cells: the sections' sums in their order (two-float), scaled
+__global__ void k_few_sum(const FewCount *__restrict__ cnt, const int *__restrict__ list, const float *__restrict__ part,
+                          int Np, int nvalid, const unsigned *__restrict__ wmax, float inv_op_scale,
+                          const TreeBox *__restrict__ box, float *__restrict__ S, double *__restrict__ S64) {
+    const int cell = blockIdx.x;
+    if (cell >= cnt->cells) return;
+    const int code = list[cell], level = code >> 15, n = 1 << level;
+    const int64_t g = cell_base_d(level) + (int64_t((code >> 10) & 31) * n + ((code >> 5) & 31)) * n + (code & 31);
+    float sc = float(double(n) / box->H) * float(double(n) / box->H);
+    if (wmax) sc *= inv_op_scale / wscale_of(wmax[level]);
+    const int64_t step = int64_t(cnt->sets) * kFewRows * Np;
+    for (int k = threadIdx.x; k < nvalid; k += blockDim.x) {
+        const float *p = part + int64_t(cell) * Np + k;
+        float hi = 0.f, lo = 0.f;
+        for (int s = 0; s < cnt->sections; ++s) {
+            const float b = __ldg(p + s * step), t = hi + b, bb = t - hi;
+            lo += (hi - (t - bb)) + (b - bb);
+            hi = t;
+        }
+        if (S64) S64[g * nvalid + k] = (double(hi) + double(lo)) * double(sc);
+        else S[g * nvalid + k] = (hi + lo) * sc;
+    }
+}
+
 // ---------------------------------------------------------------- operators
 // T_o[n = l*6 + ab][k = m*9 + wr] = Klat[o (p-1) + l - m][ab][wr] (unit cell);
 // hi = bf16(T), lo = bf16(T - hi) (residual table only for split offsets).
@@ -729,12 +1048,11 @@ __global__ void k_build_ops_modal(int p, int lat_n, int Np, int Kp, int Kp_lo, c
     }
 }
 
-// Node values -> Legendre moments, in place, for the occupied cells of one level
+// Node values -> Legendre moments, in place, for the occupied cells of levels 2 + blockIdx.y
 template <typename TW>
-__global__ void k_w_modal(int level, int p, const __grid_constant__ BasisMats B, TW *__restrict__ W,
-                          const int *__restrict__ occ) {
+__global__ void k_w_modal(int p, const __grid_constant__ BasisMats B, TW *__restrict__ W, const int *__restrict__ occ) {
     extern __shared__ __align__(16) unsigned char sm_wm[];
-    const int P3 = p * p * p;
+    const int P3 = p * p * p, level = 2 + blockIdx.y;
     TW *a = reinterpret_cast<TW *>(sm_wm), *b = a + 9 * P3;
     const int64_t cells = int64_t(1) << (3 * level), base = cell_base_d(level);
     for (int64_t lin = blockIdx.x; lin < cells; lin += gridDim.x) {
@@ -762,14 +1080,20 @@ __global__ void k_w_modal(int level, int p, const __grid_constant__ BasisMats B,
 }
 
 // W (FP32, [cell][kv]: kv = 9 p^3 node values or moments, or r2 compressed values) ->
-// parity-split hi / lo, [class][mz][my][mx][Kp] per level, one block per cell at a time.
-// Rows of cells without segments are not written: the gather never reads them (their
-// copies are zero fills).
+// parity-split hi / lo, [class][mz][my][mx][Kp] per level, one block per cell at a time, levels
+// 2 + blockIdx.y.  Rows of cells without segments are not written: the gather never reads them
+// (their copies are zero fills).
+struct PackArgs {
+    int64_t ofs[GB_TC_MAXLEV];  // elements
+    int split_levels;           // levels with residuals
+};
 template <typename E, typename TW>
-__global__ void k_pack_w(int level, int kv, int Kp, const TW *__restrict__ W, const int *__restrict__ occ,
-                         const unsigned *__restrict__ wmax, E *__restrict__ hi, E *__restrict__ lo) {
-    const int n = 1 << level, m = n / 2;
+__global__ void k_pack_w(const __grid_constant__ PackArgs A, int kv, int Kp, const TW *__restrict__ W,
+                         const int *__restrict__ occ, const unsigned *__restrict__ wmax, E *__restrict__ Whi,
+                         E *__restrict__ Wlo) {
+    const int level = 2 + blockIdx.y, n = 1 << level, m = n / 2;
     const double s = wmax ? double(wscale_of(wmax[level])) : 1.0;
+    E *hi = Whi + A.ofs[level], *lo = (A.split_levels >> level) & 1 ? Wlo + A.ofs[level] : nullptr;
     const int64_t cells = int64_t(n) * n * n;
     for (int64_t lin = blockIdx.x; lin < cells; lin += gridDim.x) {
         const int64_t g = cell_base_d(level) + lin;
@@ -787,11 +1111,11 @@ __global__ void k_pack_w(int level, int kv, int Kp, const TW *__restrict__ W, co
     }
 }
 
-// largest |W| over the occupied cells of one level (non-negative floats order
-// like their bit patterns), one block per cell at a time
+// largest |W| over the occupied cells of every level (non-negative floats order like their bit
+// patterns), one block per cell at a time, levels 2 + blockIdx.y
 template <typename TW>
-__global__ void k_wmax(int level, int kv, const TW *__restrict__ W, const int *__restrict__ occ,
-                       unsigned *__restrict__ wmax) {
+__global__ void k_wmax(int kv, const TW *__restrict__ W, const int *__restrict__ occ, unsigned *__restrict__ wmax) {
+    const int level = 2 + blockIdx.y;
     const int64_t cells = int64_t(1) << (3 * level), base = cell_base_d(level);
     float mx = 0.f;
     for (int64_t lin = blockIdx.x; lin < cells; lin += gridDim.x) {
@@ -826,40 +1150,6 @@ __global__ void k_mb_flags(int level, const int *__restrict__ tocc, int *__restr
                               (morton_part(uint32_t(z >> 1)) << 2);
         flags[slot_base(level) + cls * m3 + code] = tocc[cell_base_d(level) + lin] > 0 ? 1 : 0;
     }
-}
-
-// exclusive scan of n flags into pos[0..n] (one block)
-__global__ void k_scan_flags(int n, const int *__restrict__ flags, int *__restrict__ pos) {
-    __shared__ int part[1024];
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < n; base += 1024 * 8) {
-        int v[8], sum = 0;
-        for (int i = 0; i < 8; ++i) {
-            const int k = base + threadIdx.x * 8 + i;
-            v[i] = k < n ? flags[k] : 0;
-            sum += v[i];
-        }
-        part[threadIdx.x] = sum;
-        __syncthreads();
-        for (int off = 1; off < 1024; off <<= 1) {
-            const int t = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-            __syncthreads();
-            part[threadIdx.x] += t;
-            __syncthreads();
-        }
-        int run = carry + part[threadIdx.x] - sum;
-        for (int i = 0; i < 8; ++i) {
-            const int k = base + threadIdx.x * 8 + i;
-            if (k < n) pos[k] = run;
-            run += v[i];
-        }
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += part[1023];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) pos[n] = carry;
 }
 
 // compact list of the flagged slots (Morton code of the cell within its class)
@@ -1059,6 +1349,10 @@ int m2l_tc_setup(gbfmm_ctx *ctx) {
         if (cnt != 189) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "m2l setup: class offset count != 189");
     }
     CK(cudaMemcpyToSymbol(c_offs, ent, sizeof(ent)));
+    signed char o316[316][3];
+    for (int i = 0; i < 316; ++i)
+        for (int d = 0; d < 3; ++d) o316[i][d] = (signed char)off[3 * i + d];
+    CK(cudaMemcpyToSymbol(c_o316, o316, sizeof(o316)));
     int *d_off = nullptr, *d_lo = nullptr;
     CK(cudaMalloc(&d_off, off.size() * sizeof(int)));
     CK(cudaMalloc(&d_lo, lo_of.size() * sizeof(int)));
@@ -1192,6 +1486,13 @@ static int encode(gbfmm_ctx *ctx, CUtensorMap *tm, void *base, int rank, const c
     return GBFMM_OK;
 }
 
+// deepest level whose cells k_m2l_few takes (1: none): with the cells as A, and runs of offsets
+// that its scratch is sized for
+static int few_top_of(const gbfmm_ctx *ctx) {
+    if (ctx->tc.swap || ctx->opt.m2l_chunks > kFewSections) return 1;
+    return std::min(ctx->L - 1, kFewTop);
+}
+
 // Per-tree buffers: packed W (hi / lo), tensor maps, work list.
 int m2l_tc_prepare(gbfmm_ctx *ctx) {
     TcPlan &T = ctx->tc;
@@ -1205,10 +1506,29 @@ int m2l_tc_prepare(gbfmm_ctx *ctx) {
     if (int rc = grow_dev(ctx, T.w_cap, tot, {{&T.Whi, size_t(tot) * T.esz}, {&T.Wlo, size_t(tot) * T.esz}},
                           "packed multipole values"))
         return rc;
+    // levels 2 .. few_top go through k_m2l_few: its cell list, counts and the sections' sums, for
+    // every number of cell sets up to the levels' cells
+    T.few_top = few_top_of(ctx);
+    if (T.few_top >= 2) {
+        const int chunks = std::max(1, ctx->opt.m2l_chunks);
+        const int64_t cells = cell_base(T.few_top + 1) - cell_base(2), sets_max = (cells + kFewRows - 1) / kFewRows;
+        int64_t rows = 0;
+        T.few_work = 0;
+        for (int64_t k = 1; k <= sets_max; ++k) {
+            const int64_t sec = few_sections(int(k), T.groups, chunks, ctx->sm_count);
+            rows = std::max(rows, k * sec * kFewRows);
+            T.few_work = std::max<int>(T.few_work, int(k * sec * T.groups));
+        }
+        if (int rc = grow_dev(ctx, T.few_cap, rows * T.Np,
+                              {{(void **)&T.few_part, size_t(rows) * T.Np * sizeof(float)}}, "M2L sections"))
+            return rc;
+        if (!T.few_list)
+            CK(cudaMalloc(&T.few_list, (cell_base(kFewTop + 1) - cell_base(2)) * sizeof(int) + sizeof(FewCount) + 16));
+    }
     // cell slots, target list and segment table (filled on the device per pass)
     const int64_t slots = slot_base(L);
     int64_t tiles = 0;  // CTAs per operator group, upper bound: every cell holds targets
-    for (int l = 2; l < L; ++l) tiles += 8 * ((((int64_t(1) << (3 * (l - 1))) + 127) / 128 + T.tpc - 1) / T.tpc);
+    for (int l = std::max(2, T.few_top + 1); l < L; ++l) tiles += 8 * ((((int64_t(1) << (3 * (l - 1))) + 127) / 128 + T.tpc - 1) / T.tpc);
     if (int rc = grow_dev(ctx, T.slot_cap, slots,
                           {{(void **)&T.d_flags, slots * sizeof(int)}, {(void **)&T.d_pos, (slots + 1) * sizeof(int)},
                            {(void **)&T.d_list, slots * sizeof(int)}},
@@ -1238,61 +1558,51 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
         if (int rc = svd_transform_w(ctx, Wf, fine)) return rc;
     const float *Wsrc = T.svd ? T.Wc : Wf;
     const int kv = T.svd ? T.r2 : 9 * P3;  // valid values per cell row
+    PackArgs pk{};
+    pk.split_levels = T.split ? split_levels : 0;
     for (int l = 2; l < L; ++l) {
-        const bool split_l = T.split && ((split_levels >> l) & 1);  // residual W only where it is read
-        const int64_t cells_l = int64_t(1) << (3 * l);
-        void *whi = (char *)T.Whi + T.wofs[l] * T.esz, *wlo = (char *)T.Wlo + T.wofs[l] * T.esz;
-        const unsigned gb = unsigned(std::min<int64_t>(cells_l, 8 * 152));  // blocks stride over the cells
-        if (T.modal && !T.svd) {
-            // node values -> Legendre moments (in place: nothing reads these W after the M2L)
-            ++ctx->launches;
-            if (W64)
-                k_w_modal<double><<<gb, 256, size_t(2) * 9 * P3 * sizeof(double), ctx->stream>>>(
-                    l, p, B, const_cast<double *>(W64), occ);
-            else
-                k_w_modal<float><<<gb, 256, size_t(2) * 9 * P3 * sizeof(float), ctx->stream>>>(
-                    l, p, B, const_cast<float *>(Wf), occ);
-        }
-        if (T.tf32) {
-            ++ctx->launches;
-            if (W64)
-                k_pack_w<float><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, W64, occ, nullptr, (float *)whi, (float *)nullptr);
-            else
-                k_pack_w<float><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, Wsrc, occ, nullptr, (float *)whi, (float *)nullptr);
-        } else if (T.fp16) {
-            const unsigned gm = gb;
-            __half *lo = split_l ? (__half *)wlo : nullptr;
-            ctx->launches += 2;
-            if (W64) {
-                k_wmax<<<gm, 256, 0, ctx->stream>>>(l, kv, W64, occ, T.d_wmax);
-                k_pack_w<__half><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, W64, occ, T.d_wmax, (__half *)whi, lo);
-            } else {
-                k_wmax<<<gm, 256, 0, ctx->stream>>>(l, kv, Wsrc, occ, T.d_wmax);
-                k_pack_w<__half><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, Wsrc, occ, T.d_wmax, (__half *)whi, lo);
-            }
-        } else {
-            __nv_bfloat16 *lo = split_l ? (__nv_bfloat16 *)wlo : nullptr;
-            ++ctx->launches;
-            if (W64)
-                k_pack_w<__nv_bfloat16><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, W64, occ, nullptr,
-                                                                     (__nv_bfloat16 *)whi, lo);
-            else
-                k_pack_w<__nv_bfloat16><<<gb, 256, 0, ctx->stream>>>(l, kv, T.Kp, Wsrc, occ, nullptr,
-                                                                     (__nv_bfloat16 *)whi, lo);
-        }
+        pk.ofs[l] = T.wofs[l];
         prm.wofs[l] = T.wofs[l] * T.esz;
     }
+    // blocks stride over the cells of a level, one row of blocks per level
+    const dim3 gw(unsigned(std::min<int64_t>(int64_t(1) << (3 * (L - 1)), 8 * 152)), unsigned(L - 2));
+    cudaStream_t st = ctx->stream;
+    if (T.modal && !T.svd) {
+        // node values -> Legendre moments (in place: nothing reads these W after the M2L)
+        ++ctx->launches;
+        if (W64)
+            k_w_modal<double><<<gw, 256, size_t(2) * 9 * P3 * sizeof(double), st>>>(p, B, const_cast<double *>(W64), occ);
+        else
+            k_w_modal<float><<<gw, 256, size_t(2) * 9 * P3 * sizeof(float), st>>>(p, B, const_cast<float *>(Wf), occ);
+    }
+    if (T.tf32) {
+        ++ctx->launches;
+        if (W64)
+            k_pack_w<float><<<gw, 256, 0, st>>>(pk, kv, T.Kp, W64, occ, nullptr, (float *)T.Whi, (float *)nullptr);
+        else
+            k_pack_w<float><<<gw, 256, 0, st>>>(pk, kv, T.Kp, Wsrc, occ, nullptr, (float *)T.Whi, (float *)nullptr);
+    } else if (T.fp16) {
+        ctx->launches += 2;
+        if (W64) {
+            k_wmax<<<gw, 256, 0, st>>>(kv, W64, occ, T.d_wmax);
+            k_pack_w<__half><<<gw, 256, 0, st>>>(pk, kv, T.Kp, W64, occ, T.d_wmax, (__half *)T.Whi, (__half *)T.Wlo);
+        } else {
+            k_wmax<<<gw, 256, 0, st>>>(kv, Wsrc, occ, T.d_wmax);
+            k_pack_w<__half><<<gw, 256, 0, st>>>(pk, kv, T.Kp, Wsrc, occ, T.d_wmax, (__half *)T.Whi, (__half *)T.Wlo);
+        }
+    } else {
+        ++ctx->launches;
+        if (W64)
+            k_pack_w<__nv_bfloat16><<<gw, 256, 0, st>>>(pk, kv, T.Kp, W64, occ, nullptr, (__nv_bfloat16 *)T.Whi,
+                                                        (__nv_bfloat16 *)T.Wlo);
+        else
+            k_pack_w<__nv_bfloat16><<<gw, 256, 0, st>>>(pk, kv, T.Kp, Wsrc, occ, nullptr, (__nv_bfloat16 *)T.Whi,
+                                                        (__nv_bfloat16 *)T.Wlo);
+    }
+    CK(cudaGetLastError());
     prm.Whi = static_cast<const uint8_t *>(T.Whi);
     prm.Wlo = static_cast<const uint8_t *>(T.Wlo);
     prm.row_bytes = T.Kp * T.esz;
-    for (int l = 2; l < L; ++l) {
-        ++ctx->launches;
-        k_mb_flags<<<nblk(int64_t(1) << (3 * l), 256), 256, 0, ctx->stream>>>(l, tocc, T.d_flags);
-    }
-    ctx->launches += 3;
-    k_scan_flags<<<1, 1024, 0, ctx->stream>>>(int(T.n_slots), T.d_flags, T.d_pos);
-    k_mb_list<<<nblk(T.n_slots, 256), 256, 0, ctx->stream>>>(int(T.n_slots), L, T.d_flags, T.d_pos, T.d_list);
-    k_seg_table<<<1, 32, 0, ctx->stream>>>(L, T.tpc, T.d_pos, T.d_seg);
     {
         const cuuint64_t dims[3] = {cuuint64_t(T.Kp), cuuint64_t(T.Np), cuuint64_t(T.n_off)};
         const cuuint64_t strides[2] = {cuuint64_t(T.Kp) * T.esz, cuuint64_t(T.Kp) * T.esz * T.Np};
@@ -1323,32 +1633,68 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
     const int stage_bytes = T.tpc * kTileA + (T.swap ? 2 * kTileA : T.ncta * 128);
     // as many stages as fit in the shared memory a block may opt into, next to the
     // kernel's static arrays, the 1 KB alignment pad and the barriers
-    int dev = 0, optin = 0;
+    int dev = 0, optin = 0, stages = 0;
+    size_t smem = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    auto kern = T.tf32 ? (T.swap ? k_m2l_tc<true, true> : k_m2l_tc<true, false>)
-                       : (T.swap ? k_m2l_tc<false, true> : k_m2l_tc<false, false>);
-    cudaFuncAttributes fa;
-    CK(cudaFuncGetAttributes(&fa, kern));
-    const int64_t room = int64_t(optin) - int64_t(fa.sharedSizeBytes) - 1024 - (2 * 6 + 2) * 8 - 64;
-    const int stages = int(std::min<int64_t>(6, room / stage_bytes));
-    if (stages < 2) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "tensor-core M2L: operator block too large");
-    const size_t smem = size_t(stages) * stage_bytes + 1024 + (2 * stages + 2) * 8 + 64;
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    // offset chunks: each launch accumulates a run of consecutive offsets of every class's list
-    // in tensor memory; the chunks' sums are added outside the tensor cores, in the local values
-    const int chunks = std::max(1, std::min(189, ctx->opt.m2l_chunks));
+    auto fit = [&](const void *kern) -> int {
+        cudaFuncAttributes fa;
+        CK(cudaFuncGetAttributes(&fa, kern));
+        const int64_t room = int64_t(optin) - int64_t(fa.sharedSizeBytes) - 1024 - (2 * 6 + 2) * 8 - 64;
+        stages = int(std::min<int64_t>(6, room / stage_bytes));
+        if (stages < 2) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "tensor-core M2L: operator block too large");
+        smem = size_t(stages) * stage_bytes + 1024 + (2 * stages + 2) * 8 + 64;
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+        return GBFMM_OK;
+    };
     float *Sout = T.svd ? T.Sc : Sf;  // compressed: the r1 coefficients of every target cell
-    if (T.svd) CK(cudaMemsetAsync(T.Sc, 0, size_t(ctx->n_cells) * T.r1 * sizeof(float), ctx->stream));
-    for (int c = 0; c < chunks; ++c) {
-        prm.o_lo = (189 * c) / chunks;
-        prm.o_hi = (189 * (c + 1)) / chunks;
-        prm.accumulate = c > 0 ? 1 : 0;
-        if (c > 0) prm.drop_first = 0;
-        ++ctx->launches;
-        kern<<<T.n_work, 192, smem, ctx->stream>>>(prm, T.d_seg, 8 * (L - 2), T.d_list, occ, tocc, ctx->d_box, Sout,
-                                                   S64, T.d_status, stages, T.groups);
+    if (T.svd) CK(cudaMemsetAsync(T.Sc, 0, size_t(ctx->n_cells) * T.r1 * sizeof(float), st));
+    const int few = T.few_top;
+    if (few >= 2) {
+        FewParams fp;
+        fp.P = prm;
+        fp.P.split = T.split && (split_levels & ((2 << few) - 4));
+        fp.groups = T.groups;
+        for (int i = 0; i < 316; ++i) fp.lo[i] = T.lo_host[i];
+        auto kern = T.tf32 ? k_m2l_few<true> : k_m2l_few<false>;
+        if (int rc = fit((const void *)kern)) return rc;
+        FewCount *cnt = reinterpret_cast<FewCount *>(T.few_list);
+        int *list = reinterpret_cast<int *>(T.few_list) + 4;
+        ctx->launches += 3;
+        k_few_list<<<1, 1024, 0, st>>>(few, T.groups, std::max(1, ctx->opt.m2l_chunks), ctx->sm_count, tocc, list, cnt);
+        kern<<<T.few_work, 192, smem, st>>>(fp, cnt, list, occ, T.few_part, T.Np, T.d_status, stages);
+        k_few_sum<<<unsigned(cell_base(few + 1) - cell_base(2)), 256, 0, st>>>(
+            cnt, list, T.few_part, T.Np, prm.nvalid, prm.wmax, prm.inv_op_scale, ctx->d_box, Sout, S64);
         CK(cudaGetLastError());
+        prm.drop_first = 0;
+    }
+    if (L - 1 > few) {
+        // target cells of the deeper levels: flags by slot, their scan, the list and the segments
+        if (few >= 2) CK(cudaMemsetAsync(T.d_flags, 0, slot_base(few + 1) * sizeof(int), st));
+        for (int l = std::max(2, few + 1); l < L; ++l) {
+            ++ctx->launches;
+            k_mb_flags<<<nblk(int64_t(1) << (3 * l), 256), 256, 0, st>>>(l, tocc, T.d_flags);
+        }
+        scan_counts(ctx, T.n_slots, T.d_flags, T.d_pos);
+        ctx->launches += 2;
+        k_mb_list<<<nblk(T.n_slots, 256), 256, 0, st>>>(int(T.n_slots), L, T.d_flags, T.d_pos, T.d_list);
+        k_seg_table<<<1, 32, 0, st>>>(L, T.tpc, T.d_pos, T.d_seg);
+        auto kern = T.tf32 ? (T.swap ? k_m2l_tc<true, true> : k_m2l_tc<true, false>)
+                           : (T.swap ? k_m2l_tc<false, true> : k_m2l_tc<false, false>);
+        if (int rc = fit((const void *)kern)) return rc;
+        // offset chunks: each launch accumulates a run of consecutive offsets of every class's list
+        // in tensor memory; the chunks' sums are added outside the tensor cores, in the local values
+        const int chunks = std::max(1, std::min(189, ctx->opt.m2l_chunks));
+        for (int c = 0; c < chunks; ++c) {
+            prm.o_lo = (189 * c) / chunks;
+            prm.o_hi = (189 * (c + 1)) / chunks;
+            prm.accumulate = c > 0 ? 1 : 0;
+            if (c > 0) prm.drop_first = 0;
+            ++ctx->launches;
+            kern<<<T.n_work, 192, smem, st>>>(prm, T.d_seg, 8 * (L - 2), T.d_list, occ, tocc, ctx->d_box, Sout, S64,
+                                              T.d_status, stages, T.groups);
+            CK(cudaGetLastError());
+        }
     }
     if (T.svd) {
         if (fine)
@@ -1371,7 +1717,8 @@ int m2l_tc_status(gbfmm_ctx *ctx, int *out) {
 void m2l_tc_free(gbfmm_ctx *ctx) {
     TcPlan &T = ctx->tc;
     svd_free(ctx, ctx->borrowed_material);
-    void *ps[] = {T.Thi, T.Tlo, T.Whi, T.Wlo, T.d_status, T.d_flags, T.d_pos, T.d_list, T.d_seg, T.d_wmax};
+    void *ps[] = {T.Thi, T.Tlo, T.Whi, T.Wlo, T.d_status, T.d_flags, T.d_pos, T.d_list, T.d_seg, T.d_wmax,
+                  T.few_list, T.few_part};
     for (void *q : ps)
         if (q) cudaFree(q);
     T = TcPlan{};

@@ -36,6 +36,12 @@ struct TcPlan {
     int4 *d_seg = nullptr;     // per (level, class): first list entry, count, first tile
     int64_t slot_cap = 0, n_slots = 0;
     int n_seg = 0;
+    // few cells (k_m2l_few): deepest level taken, CTAs of the largest launch, counts and cell list,
+    // the sections' sums
+    int few_top = 1, few_work = 0;
+    void *few_list = nullptr;
+    float *few_part = nullptr;
+    int64_t few_cap = 0;
     // SVD-compressed M2L (gbfmm_options.m2l_svd_tol > 0, m2l_svd.cu): the GEMM runs on
     // r2 source and r1 target coefficients per cell
     int svd = 0;

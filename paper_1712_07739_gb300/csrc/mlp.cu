@@ -9,10 +9,11 @@
 // flat FP32 master vector (W1 [128x3], b1, W2 [128x128], b2, W3, b3,
 // W4 [32x128] (rows 27..31 stay zero), b4 [32]) with a BF16 copy for compute.
 //
-// Training: Adam on the mean-squared error in scaled units.  Every matrix
-// product of the forward and backward passes runs in k_gemm_bf16 (warp
-// mma.m16n8k16, BF16 in, FP32 accumulate); the first layer (3 inputs) and
-// the element-wise steps are plain kernels.
+// Evaluation is one kernel: a warp takes 16 directions through all four layers in registers, the
+// weights in shared memory (mlp_warp.cuh), so a direction moves 12 bytes in and 108 out instead of
+// its 384 activations.  Training: Adam on the mean-squared error in scaled units; a step's forward
+// and backward chain is the same kernel form, the weight gradients (sums over the batch) one split
+// product and one ordered sum.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -24,181 +25,299 @@
 
 #include "internal.cuh"
 #include "kernel_math.cuh"
+#include "mlp_warp.cuh"
 
 namespace {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int OFF_W1 = 0, OFF_B1 = 384, OFF_W2 = 512, OFF_B2 = 16896, OFF_W3 = 17024, OFF_B3 = 33408,
-              OFF_W4 = 33536, OFF_B4 = 37632, NPAR = 37664;
+using mlpw::NPAR;
+using mlpw::OFF_B1;
+using mlpw::OFF_B2;
+using mlpw::OFF_B3;
+using mlpw::OFF_B4;
+using mlpw::OFF_W1;
+using mlpw::OFF_W2;
+using mlpw::OFF_W3;
+using mlpw::OFF_W4;
 
 inline unsigned nblk(int64_t n, int b) { return unsigned(std::min<int64_t>((n + b - 1) / b, 1 << 22)); }
 
-// SiLU through the hardware tanh (the same form the near-field kernel uses):
-// sigmoid(z) = (1 + tanh(z/2)) / 2, silu = z sigmoid(z), silu' = s (1 + z (1 - s))
-__device__ __forceinline__ float tanh_hw(float x) {
-    float y;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float silu(float z) { return 0.5f * z * (1.f + tanh_hw(0.5f * z)); }
-__device__ __forceinline__ float dsilu(float z) {
-    const float s = 0.5f * (1.f + tanh_hw(0.5f * z));
-    return s * (1.f + z * (1.f - s));
+// Bound by the weight fragments' way out of shared memory (its pipe 83 % busy, the tensor pipe 37 %):
+// sixteen directions per warp at 128 registers, two blocks of eight warps per SM.  32 directions per
+// warp would halve the fragment loads but leave 8 to 12 warps an SM, too few to cover the chain
+// (254 us).  1,000,003 directions: 224 us, 2,561 us as seven kernels per 262,144 directions with the
+// activations in memory.  Blocks stride over the tiles: the weights load once per block.
+constexpr int kEvalWarps = 8;
+struct EvalSmem {
+    mlpw::Weights w;
+    float out[kEvalWarps][16 * 27];
+};
+__global__ void __launch_bounds__(32 * kEvalWarps, 2)
+    k_mlp_eval(int64_t n, const float *__restrict__ dirs, const bf16 *__restrict__ th, const float *__restrict__ th32,
+               const float *__restrict__ scale, float *__restrict__ h) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    EvalSmem &sm = *reinterpret_cast<EvalSmem *>(sm_raw);
+    mlpw::load(sm.w, th, th32, scale);
+    __syncthreads();
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
+    const int64_t tiles = (n + 15) / 16;
+    // neighbouring tiles to different blocks: a small call spreads over the SMs
+    for (int64_t tile = int64_t(warp) * gridDim.x + blockIdx.x; tile < tiles; tile += int64_t(gridDim.x) * kEvalWarps) {
+        float d[2][3], s[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int64_t b = min(tile * 16 + g + 8 * r, n - 1);  // rows past the end repeat the last
+            const float x = __ldg(dirs + 3 * b), y = __ldg(dirs + 3 * b + 1), z = __ldg(dirs + 3 * b + 2);
+            s[r] = mlpw::half_space_sign(x, y, z);
+            d[r][0] = s[r] * x, d[r][1] = s[r] * y, d[r][2] = s[r] * z;
+        }
+        uint32_t a[8][4];
+        float z[16][4];
+        mlpw::first(sm.w, d[0], d[1], z, t);
+        mlpw::silu_all(z);
+        mlpw::pack_a<8>(a, z);
+        mlpw::layer<16, 8, false>(sm.w.W2, a, z, lane);
+        mlpw::add_bias<16>(sm.w.b2, z, t);
+        mlpw::silu_all(z);
+        mlpw::pack_a<8>(a, z);
+        mlpw::layer<16, 8, false>(sm.w.W3, a, z, lane);
+        mlpw::add_bias<16>(sm.w.b3, z, t);
+        mlpw::silu_all(z);
+        mlpw::pack_a<8>(a, z);
+        mlpw::layer<4, 8, false>(sm.w.W4, a, z, lane);
+        mlpw::add_bias<4>(sm.w.b4, z, t);
+        // scaled output -> h (sign of the half-space restored), rows put together in shared memory
+        float *out = sm.out[warp];
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 8 * nt + 2 * t + (j & 1);
+                if (c < 27) out[(g + 8 * (j >> 1)) * 27 + c] = s[j >> 1] * sm.w.scale[c] * z[nt][j];
+            }
+        __syncwarp();
+        const int rows = int(min(int64_t(16), n - tile * 16));
+        for (int i = lane; i < rows * 27; i += 32) h[tile * 16 * 27 + i] = out[i];
+        __syncwarp();
+    }
 }
 
-__device__ __forceinline__ float half_space_sign(float x, float y, float z) {
-    return (z > 0.f || (z == 0.f && (y > 0.f || (y == 0.f && x >= 0.f)))) ? 1.f : -1.f;
+// Forward and backward chain of one batch.  A warp takes 16 samples through the network and back
+// in registers (the transposed products read the same weights by transposing loads) and leaves
+// what the weight gradients read: inputs x, activations a1 .. a3 and the gradients of the
+// pre-activations g1 .. g3, go, in BF16 rows, g1 also in FP32.  The pre-activations go through
+// memory in the lane's own order.  loss = mean_{b,c} (o - s y / scale)^2, one partial per tile.
+// Two warps a block: a batch of 8,192 is 512 tiles, about three warps for every SM, whose serial
+// chain is the time.  The whole gradient of 8,192 samples: 78 us, 1,926 us as 22 kernels with the
+// activations in memory (this one 32 us, k_mlp_wgrad 15, k_grad_sum 8).
+constexpr int kTrainWarps = 2;
+struct TrainArgs {
+    float *x, *z, *g32, *lossp;  // [n][3], [tile][3][16][32][4], [n][128], [tiles]
+    bf16 *a[3], *g[3], *go;      // [n][128] each (g[0] = g1), [n][32]
+};
+__device__ __forceinline__ void store_rows(bf16 *__restrict__ dst, int ld, const uint32_t (*a)[4], int KT, int64_t r0,
+                                           int64_t n, int g, int t) {
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk)
+        if (kk < KT)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t r = r0 + g + 8 * (j & 1);
+                if (r < n) *reinterpret_cast<uint32_t *>(dst + r * ld + kk * 16 + 2 * t + 8 * (j >> 1)) = a[kk][j];
+            }
+}
+__global__ void __launch_bounds__(32 * kTrainWarps)
+    k_mlp_train(int n, const float *__restrict__ dirs, const float *__restrict__ y, const bf16 *__restrict__ th,
+                const float *__restrict__ th32, const float *__restrict__ scale, const __grid_constant__ TrainArgs T) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    mlpw::Weights &w = *reinterpret_cast<mlpw::Weights *>(sm_raw);
+    mlpw::load(w, th, th32, scale);
+    __syncthreads();
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
+    const int64_t tiles = (int64_t(n) + 15) / 16;
+    for (int64_t tile = int64_t(blockIdx.x) * kTrainWarps + warp; tile < tiles; tile += int64_t(gridDim.x) * kTrainWarps) {
+        const int64_t r0 = tile * 16;
+        float d[2][3], s[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int64_t b = r0 + g + 8 * r, bb = min(b, int64_t(n) - 1);
+            const float x = __ldg(dirs + 3 * bb), yy = __ldg(dirs + 3 * bb + 1), z = __ldg(dirs + 3 * bb + 2);
+            s[r] = mlpw::half_space_sign(x, yy, z);
+            d[r][0] = s[r] * x, d[r][1] = s[r] * yy, d[r][2] = s[r] * z;
+            if (t < 3 && b < n) T.x[3 * b + t] = t == 0 ? d[r][0] : t == 1 ? d[r][1] : d[r][2];
+        }
+        float4 *zs = reinterpret_cast<float4 *>(T.z) + tile * (3 * 16 * 32) + lane;
+        uint32_t a[8][4];
+        float z[16][4];
+        auto keep = [&](int l) {  // pre-activations to memory, activations to rows and to A fragments
+#pragma unroll
+            for (int nt = 0; nt < 16; ++nt) zs[(l * 16 + nt) * 32] = make_float4(z[nt][0], z[nt][1], z[nt][2], z[nt][3]);
+            mlpw::silu_all(z);
+            mlpw::pack_a<8>(a, z);
+            store_rows(T.a[l], 128, a, 8, r0, n, g, t);
+        };
+        mlpw::first(w, d[0], d[1], z, t);
+        keep(0);
+        mlpw::layer<16, 8, false>(w.W2, a, z, lane);
+        mlpw::add_bias<16>(w.b2, z, t);
+        keep(1);
+        mlpw::layer<16, 8, false>(w.W3, a, z, lane);
+        mlpw::add_bias<16>(w.b3, z, t);
+        keep(2);
+        float o[4][4];
+        mlpw::layer<4, 8, false>(w.W4, a, o, lane);
+        mlpw::add_bias<4>(w.b4, o, t);
+        float loss = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 8 * nt + 2 * t + (j & 1);
+                const int64_t b = r0 + g + 8 * (j >> 1);
+                float gv = 0.f;
+                if (c < 27 && b < n) {
+                    const float r = o[nt][j] - s[j >> 1] * y[b * 27 + c] / w.scale[c];
+                    gv = 2.f * r / (float(n) * 27.f);
+                    loss += r * r / (float(n) * 27.f);
+                }
+                o[nt][j] = gv;
+            }
+        for (int k = 16; k > 0; k >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, k);
+        if (lane == 0) T.lossp[tile] = loss;
+        mlpw::pack_a<2>(a, o);
+        store_rows(T.go, 32, a, 2, r0, n, g, t);
+        auto back = [&](int l) {  // z holds dL/da of layer l + 1: times silu' of its pre-activations
+#pragma unroll
+            for (int nt = 0; nt < 16; ++nt) {
+                const float4 v = zs[(l * 16 + nt) * 32];
+                z[nt][0] *= mlpw::dsilu(v.x), z[nt][1] *= mlpw::dsilu(v.y);
+                z[nt][2] *= mlpw::dsilu(v.z), z[nt][3] *= mlpw::dsilu(v.w);
+            }
+            mlpw::pack_a<8>(a, z);
+            store_rows(T.g[l], 128, a, 8, r0, n, g, t);
+        };
+        mlpw::layer<16, 2, true>(w.W4, a, z, lane);
+        back(2);
+        mlpw::layer<16, 8, true>(w.W3, a, z, lane);
+        back(1);
+        mlpw::layer<16, 8, true>(w.W2, a, z, lane);
+        back(0);
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (r0 + g + 8 * r < n)
+                    *reinterpret_cast<float2 *>(T.g32 + (r0 + g + 8 * r) * 128 + 8 * nt + 2 * t) =
+                        make_float2(z[nt][2 * r], z[nt][2 * r + 1]);
+    }
 }
 
-// C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n]); A(m,k) = A[m sam + k sak],
-// B(k,n) = B[k sbk + n sbn], BF16 in, FP32 out.  64 x 64 block tile, 4 warps,
-// each warp 16 rows x 64 columns as 8 mma.m16n8k16 per 16-wide K step.
-__global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const bf16 *__restrict__ A, int64_t sam,
-                                                   int64_t sak, const bf16 *__restrict__ B, int64_t sbk, int64_t sbn,
-                                                   const float *__restrict__ bias, float *__restrict__ C, int64_t ldc) {
-    __shared__ __align__(16) bf16 As[64][24];
-    __shared__ __align__(16) bf16 Bs[64][24];
+// Weight gradients of one run of samples (blockIdx.y), blockIdx.x: 0 .. 3 the halves (output rows
+// 0..63, 64..127) of dW3 and dW2, 4 dW4, 5 the first layer.  dW[o][i] = sum_b g[b][o] a[b][i] with
+// both operands read from sample rows by transposing ldmatrix; the bias gradients are column sums.
+// The runs' sums (at most kGradRuns of the whole parameter vector) are added in their order by
+// k_grad_sum: one block per output tile summing all 8,192 samples took 2.2 ms.
+constexpr int kGradRuns = 64, kGradRows = 64;  // runs at most; samples in shared memory at a time
+__global__ void __launch_bounds__(256)
+    k_mlp_wgrad(int n, int run, const __grid_constant__ TrainArgs T, float *__restrict__ part) {
+    __shared__ __align__(16) bf16 Gs[kGradRows][72];         // 64 output columns of g
+    __shared__ __align__(16) bf16 As[kGradRows][mlpw::LD];   // the layer's inputs
+    const int64_t b0 = int64_t(blockIdx.y) * run, b1 = min(int64_t(n), b0 + run);
+    float *out = part + int64_t(blockIdx.y) * NPAR;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+    const int job = blockIdx.x;
+    if (job == 5) {
+        // dW1[o][i] = sum_b g1[b][o] x[b][i] (FP32), db1 from the BF16 g1: a thread per output and half run
+        __shared__ float red[128][4];
+        const int o = tid & 127, half = tid >> 7;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+        for (int64_t b = b0 + half; b < b1; b += 2) {
+            const float gv = T.g32[b * 128 + o];
+            v[0] += gv * T.x[3 * b], v[1] += gv * T.x[3 * b + 1], v[2] += gv * T.x[3 * b + 2];
+            v[3] += __bfloat162float(T.g[0][b * 128 + o]);
+        }
+        if (half)
+            for (int j = 0; j < 4; ++j) red[o][j] = v[j];
+        __syncthreads();
+        if (!half) {
+            for (int j = 0; j < 3; ++j) out[OFF_W1 + 3 * o + j] = v[j] + red[o][j];
+            out[OFF_B1 + o] = v[3] + red[o][3];
+        }
+        return;
+    }
+    const bf16 *G = job == 4 ? T.go : T.g[job < 2 ? 2 : 1], *A = T.a[job == 4 ? 2 : job < 2 ? 1 : 0];
+    const int cols = job == 4 ? 32 : 64, ldg = job == 4 ? 32 : 128, c0 = job == 4 ? 0 : 64 * (job & 1);
+    const int w0 = job == 4 ? OFF_W4 : job < 2 ? OFF_W3 : OFF_W2, bias0 = job == 4 ? OFF_B4 : job < 2 ? OFF_B3 : OFF_B2;
+    // warp: 16 output rows x 64 inputs
+    const int m0 = 16 * (warp & 3), i0 = 64 * (warp >> 2), mat = lane >> 3, r = lane & 7;
+    const bool busy = m0 < cols;
     float acc[8][4];
-    for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    const bf16 zero = __float2bfloat16(0.f);
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int i = tid; i < 64 * 16; i += 128) {
-            const int r = i / 16, c = i % 16, m = m0 + r, k = k0 + c;
-            As[r][c] = (m < M && k < K) ? A[m * sam + k * sak] : zero;
-            const int n = n0 + r;
-            Bs[r][c] = (n < N && k < K) ? B[k * sbk + n * sbn] : zero;
-        }
-        __syncthreads();
-        const int r0 = warp * 16;
-        uint32_t a[4];
-        a[0] = *reinterpret_cast<const uint32_t *>(&As[r0 + g][2 * t]);
-        a[1] = *reinterpret_cast<const uint32_t *>(&As[r0 + g + 8][2 * t]);
-        a[2] = *reinterpret_cast<const uint32_t *>(&As[r0 + g][2 * t + 8]);
-        a[3] = *reinterpret_cast<const uint32_t *>(&As[r0 + g + 8][2 * t + 8]);
-        for (int nt = 0; nt < 8; ++nt) {
-            uint32_t b0 = *reinterpret_cast<const uint32_t *>(&Bs[nt * 8 + g][2 * t]);
-            uint32_t b1 = *reinterpret_cast<const uint32_t *>(&Bs[nt * 8 + g][2 * t + 8]);
-            asm volatile(
-                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-                "{%0, %1, %2, %3};"
-                : "+f"(acc[nt][0]), "+f"(acc[nt][1]), "+f"(acc[nt][2]), "+f"(acc[nt][3])
-                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-        }
-        __syncthreads();
-    }
-    const int r0 = m0 + warp * 16;
     for (int nt = 0; nt < 8; ++nt)
-        for (int j = 0; j < 4; ++j) {
-            const int m = r0 + g + (j >= 2 ? 8 : 0), n = n0 + nt * 8 + 2 * t + (j & 1);
-            if (m < M && n < N) C[m * ldc + n] = acc[nt][j] + (bias ? bias[n] : 0.f);
+        for (int j = 0; j < 4; ++j) acc[nt][j] = 0.f;
+    float db = 0.f;
+    for (int64_t s0 = b0; s0 < b1; s0 += kGradRows) {
+        const int rows = int(min(int64_t(kGradRows), b1 - s0));
+        const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < kGradRows * 16; i += 256) {
+            const int b = i / 16, c = 8 * (i % 16);
+            *reinterpret_cast<uint4 *>(&As[b][c]) =
+                b < rows ? *reinterpret_cast<const uint4 *>(A + (s0 + b) * 128 + c) : none;
         }
-}
-
-void gemm(cudaStream_t st, int M, int N, int K, const bf16 *A, int64_t sam, int64_t sak, const bf16 *B, int64_t sbk,
-          int64_t sbn, const float *bias, float *C, int64_t ldc) {
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    k_gemm_bf16<<<grid, 128, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, bias, C, ldc);
-}
-
-// first layer on canonical inputs: z1 = W1 x + b1, a1 = silu(z1)
-__global__ void k_layer1(int n, const float *__restrict__ dirs, const bf16 *__restrict__ th,
-                         const float *__restrict__ th32, float *__restrict__ x, float *__restrict__ z1,
-                         bf16 *__restrict__ a1) {
-    const int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (idx >= int64_t(n) * 128) return;
-    const int b = int(idx / 128), o = int(idx % 128);
-    const float tx = dirs[3 * b], ty = dirs[3 * b + 1], tz = dirs[3 * b + 2];
-    const float s = half_space_sign(tx, ty, tz);
-    const float xx = s * tx, xy = s * ty, xz = s * tz;
-    if (o == 0 && x) {
-        x[3 * b] = xx;
-        x[3 * b + 1] = xy;
-        x[3 * b + 2] = xz;
-    }
-    const float z = __bfloat162float(th[OFF_W1 + 3 * o]) * xx + __bfloat162float(th[OFF_W1 + 3 * o + 1]) * xy +
-                    __bfloat162float(th[OFF_W1 + 3 * o + 2]) * xz + th32[OFF_B1 + o];
-    if (z1) z1[idx] = z;
-    a1[idx] = __float2bfloat16(silu(z));
-}
-
-__global__ void k_silu(int64_t n, const float *__restrict__ z, bf16 *__restrict__ a) {
-    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i < n) a[i] = __float2bfloat16(silu(z[i]));
-}
-
-// scaled output -> h (sign of the half-space restored)
-__global__ void k_output(int n, const float *__restrict__ dirs, const float *__restrict__ o32,
-                         const float *__restrict__ scale, float *__restrict__ h) {
-    const int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (idx >= int64_t(n) * 27) return;
-    const int b = int(idx / 27), c = int(idx % 27);
-    const float s = half_space_sign(dirs[3 * b], dirs[3 * b + 1], dirs[3 * b + 2]);
-    h[idx] = s * scale[c] * o32[int64_t(b) * 32 + c];
-}
-
-// d loss / d o for loss = mean_{b,c} (o - s y / scale)^2
-__global__ void k_loss_grad(int n, const float *__restrict__ dirs, const float *__restrict__ o32,
-                            const float *__restrict__ y, const float *__restrict__ scale, bf16 *__restrict__ go,
-                            float *__restrict__ loss) {
-    const int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    float l = 0.f;
-    if (idx < int64_t(n) * 32) {
-        const int b = int(idx / 32), c = int(idx % 32);
-        float gval = 0.f;
-        if (c < 27) {
-            const float s = half_space_sign(dirs[3 * b], dirs[3 * b + 1], dirs[3 * b + 2]);
-            const float r = o32[idx] - s * y[int64_t(b) * 27 + c] / scale[c];
-            gval = 2.f * r / (float(n) * 27.f);
-            l = r * r / (float(n) * 27.f);
+        for (int i = tid; i < kGradRows * cols / 8; i += 256) {
+            const int b = i / (cols / 8), c = 8 * (i % (cols / 8));
+            *reinterpret_cast<uint4 *>(&Gs[b][c]) =
+                b < rows ? *reinterpret_cast<const uint4 *>(G + (s0 + b) * ldg + c0 + c) : none;
         }
-        go[idx] = __float2bfloat16(gval);
-    }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.f) atomicAdd(loss, l);
-}
-
-__global__ void k_dsilu_mul(int64_t n, const float *__restrict__ da, const float *__restrict__ z,
-                            bf16 *__restrict__ g, float *__restrict__ g32) {
-    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i >= n) return;
-    const float v = da[i] * dsilu(z[i]);
-    g[i] = __float2bfloat16(v);
-    if (g32) g32[i] = v;
-}
-
-// db[c] = sum_b g[b][c]  (g given as BF16 rows of width ld)
-__global__ void k_colsum(int n, int cols, int ld, const bf16 *__restrict__ g, float *__restrict__ db) {
-    const int c = blockIdx.x;
-    float s = 0.f;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) s += __bfloat162float(g[int64_t(b) * ld + c]);
-    __shared__ float sm[256];
-    sm[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
+        __syncthreads();
+        if (busy)
+#pragma unroll
+            for (int kk = 0; kk < kGradRows / 16; ++kk) {
+                uint32_t a[4], b[4];
+                // A[o][b] from rows of samples: pieces (o low, b low), (o high, b low), (o low, b high), ..
+                mlpw::ldsm4<true>(a, &Gs[kk * 16 + (mat >> 1) * 8 + r][m0 + (mat & 1) * 8]);
+#pragma unroll
+                for (int nt = 0; nt < 8; nt += 2) {
+                    mlpw::ldsm4<true>(b, &As[kk * 16 + (mat & 1) * 8 + r][i0 + (nt + (mat >> 1)) * 8]);
+                    mlpw::mma16816(acc[nt], a, b[0], b[1]);
+                    mlpw::mma16816(acc[nt + 1], a, b[2], b[3]);
+                }
+            }
+        if (tid < cols)
+            for (int b = 0; b < rows; ++b) db += __bfloat162float(Gs[b][tid]);
         __syncthreads();
     }
-    if (threadIdx.x == 0 && c < cols) db[c] = sm[0];
+    if (tid < cols) out[bias0 + c0 + tid] = db;
+    if (busy)
+        for (int nt = 0; nt < 8; ++nt)
+            for (int j = 0; j < 4; ++j)
+                out[w0 + (c0 + m0 + (lane >> 2) + 8 * (j >> 1)) * 128 + i0 + 8 * nt + 2 * (lane & 3) + (j & 1)] = acc[nt][j];
 }
 
-// dW1[o][i] = sum_b g1[b][o] x[b][i]
-__global__ void k_dw1(int n, const float *__restrict__ g1, const float *__restrict__ x, float *__restrict__ dW1) {
-    const int o = blockIdx.x / 3, i = blockIdx.x % 3;
-    float s = 0.f;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) s += g1[int64_t(b) * 128 + o] * x[3 * b + i];
-    __shared__ float sm[256];
-    sm[threadIdx.x] = s;
-    __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if (threadIdx.x < k) sm[threadIdx.x] += sm[threadIdx.x + k];
+// gradient = the runs' sums in order; the last block adds the tiles' losses
+__global__ void __launch_bounds__(256) k_grad_sum(int runs, const float *__restrict__ part, float *__restrict__ grad,
+                                                  int64_t tiles, const float *__restrict__ lossp,
+                                                  float *__restrict__ loss) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float sm[256];
+        float s = 0.f;
+        for (int64_t i = threadIdx.x; i < tiles; i += 256) s += lossp[i];
+        sm[threadIdx.x] = s;
         __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *loss = sm[0];
+        return;
     }
-    if (threadIdx.x == 0) dW1[3 * o + i] = sm[0];
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= NPAR) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < runs; ++r) s += part[int64_t(r) * NPAR + i];
+    grad[i] = s;
 }
 
 __global__ void k_adam(int n, float *__restrict__ th, const float *__restrict__ g, float *__restrict__ m,
@@ -285,9 +404,9 @@ __global__ void k_bin_poly(const float *__restrict__ h, float m2, float fac, flo
 
 // ---------------------------------------------------------------- host side
 struct MlpBuffers {
-    int cap = 0;
-    float *x = nullptr, *z1 = nullptr, *z2 = nullptr, *z3 = nullptr, *o = nullptr, *da = nullptr, *g32 = nullptr;
-    bf16 *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *go = nullptr, *g = nullptr;
+    int64_t cap = 0;  // samples, a multiple of 16
+    TrainArgs t{};
+    float *part = nullptr;  // [kGradRuns][NPAR]
 };
 
 static MlpBuffers &bufs(gbfmm_ctx *ctx) { return *reinterpret_cast<MlpBuffers *>(ctx->mlp.bufs); }
@@ -306,76 +425,47 @@ static int mlp_alloc_state(gbfmm_ctx *ctx) {
     return GBFMM_OK;
 }
 
+// buffers of a training batch of n samples
 static int mlp_alloc_batch(gbfmm_ctx *ctx, int n) {
     MlpBuffers &B = bufs(ctx);
-    if (n <= B.cap) return GBFMM_OK;
-    void *ps[] = {B.x, B.z1, B.z2, B.z3, B.o, B.da, B.g32, B.a1, B.a2, B.a3, B.go, B.g};
-    for (void *p : ps)
-        if (p) cudaFree(p);
-    const int64_t n128 = int64_t(n) * 128;
-    CK(cudaMalloc(&B.x, int64_t(n) * 3 * sizeof(float)));
-    CK(cudaMalloc(&B.z1, n128 * sizeof(float)));
-    CK(cudaMalloc(&B.z2, n128 * sizeof(float)));
-    CK(cudaMalloc(&B.z3, n128 * sizeof(float)));
-    CK(cudaMalloc(&B.o, int64_t(n) * 32 * sizeof(float)));
-    CK(cudaMalloc(&B.da, n128 * sizeof(float)));
-    CK(cudaMalloc(&B.g32, n128 * sizeof(float)));
-    CK(cudaMalloc(&B.a1, n128 * sizeof(bf16)));
-    CK(cudaMalloc(&B.a2, n128 * sizeof(bf16)));
-    CK(cudaMalloc(&B.a3, n128 * sizeof(bf16)));
-    CK(cudaMalloc(&B.go, int64_t(n) * 32 * sizeof(bf16)));
-    CK(cudaMalloc(&B.g, n128 * sizeof(bf16)));
-    B.cap = n;
-    return GBFMM_OK;
+    TrainArgs &T = B.t;
+    if (!B.part) CK(cudaMalloc(&B.part, size_t(kGradRuns) * NPAR * sizeof(float)));
+    const size_t m = (size_t(n) + 15) / 16 * 16;
+    return grow_dev(ctx, B.cap, int64_t(m),
+                    {{(void **)&T.x, m * 3 * sizeof(float)}, {(void **)&T.z, m * 384 * sizeof(float)},
+                     {(void **)&T.g32, m * 128 * sizeof(float)}, {(void **)&T.lossp, m / 16 * sizeof(float)},
+                     {(void **)&T.a[0], m * 128 * sizeof(bf16)}, {(void **)&T.a[1], m * 128 * sizeof(bf16)},
+                     {(void **)&T.a[2], m * 128 * sizeof(bf16)}, {(void **)&T.g[0], m * 128 * sizeof(bf16)},
+                     {(void **)&T.g[1], m * 128 * sizeof(bf16)}, {(void **)&T.g[2], m * 128 * sizeof(bf16)},
+                     {(void **)&T.go, m * 32 * sizeof(bf16)}},
+                    "network batch");
 }
 
-// forward of n directions (batch buffers hold the activations): BF16
-// weight matrices, FP32 biases, FP32 accumulation
-static int mlp_forward(gbfmm_ctx *ctx, int n, const float *dirs) {
-    MlpState &M = ctx->mlp;
-    MlpBuffers &B = bufs(ctx);
-    cudaStream_t st = ctx->stream;
-    const bf16 *th = M.theta_h;
-    const float *b = M.theta;
-    ctx->launches += 6;
-    k_layer1<<<nblk(int64_t(n) * 128, 256), 256, 0, st>>>(n, dirs, th, b, B.x, B.z1, B.a1);
-    gemm(st, n, 128, 128, B.a1, 128, 1, th + OFF_W2, 1, 128, b + OFF_B2, B.z2, 128);
-    k_silu<<<nblk(int64_t(n) * 128, 256), 256, 0, st>>>(int64_t(n) * 128, B.z2, B.a2);
-    gemm(st, n, 128, 128, B.a2, 128, 1, th + OFF_W3, 1, 128, b + OFF_B3, B.z3, 128);
-    k_silu<<<nblk(int64_t(n) * 128, 256), 256, 0, st>>>(int64_t(n) * 128, B.z3, B.a3);
-    gemm(st, n, 32, 128, B.a3, 128, 1, th + OFF_W4, 1, 128, b + OFF_B4, B.o, 32);
+// network outputs of n directions (BF16 weight matrices, FP32 biases, FP32 accumulation)
+static int mlp_forward(gbfmm_ctx *ctx, int64_t n, const float *dirs, float *h) {
+    const MlpState &M = ctx->mlp;
+    CK(cudaFuncSetAttribute(k_mlp_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(EvalSmem))));
+    ++ctx->launches;
+    k_mlp_eval<<<unsigned(std::min<int64_t>((n + 15) / 16, 2 * ctx->sm_count)), 32 * kEvalWarps, sizeof(EvalSmem), ctx->stream>>>(
+        n, dirs, M.theta_h, M.theta, M.scale, h);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }
 
 // gradient of the loss on one batch into M.grad; loss (scaled units) into M.loss
-static int mlp_backward(gbfmm_ctx *ctx, int n, const float *dirs, const float *y) {
+static int mlp_gradient(gbfmm_ctx *ctx, int n, const float *dirs, const float *y) {
     MlpState &M = ctx->mlp;
     MlpBuffers &B = bufs(ctx);
-    cudaStream_t st = ctx->stream;
-    const bf16 *th = M.theta_h;
-    const int64_t n128 = int64_t(n) * 128;
-    CK(cudaMemsetAsync(M.loss, 0, sizeof(float), st));
-    ctx->launches += 16;
-    k_loss_grad<<<nblk(int64_t(n) * 32, 256), 256, 0, st>>>(n, dirs, B.o, y, M.scale, B.go, M.loss);
-    // layer 4
-    gemm(st, 32, 128, n, B.go, 1, 32, B.a3, 128, 1, nullptr, M.grad + OFF_W4, 128);
-    k_colsum<<<32, 256, 0, st>>>(n, 32, 32, B.go, M.grad + OFF_B4);
-    gemm(st, n, 128, 32, B.go, 32, 1, th + OFF_W4, 128, 1, nullptr, B.da, 128);
-    k_dsilu_mul<<<nblk(n128, 256), 256, 0, st>>>(n128, B.da, B.z3, B.g, nullptr);
-    // layer 3
-    gemm(st, 128, 128, n, B.g, 1, 128, B.a2, 128, 1, nullptr, M.grad + OFF_W3, 128);
-    k_colsum<<<128, 256, 0, st>>>(n, 128, 128, B.g, M.grad + OFF_B3);
-    gemm(st, n, 128, 128, B.g, 128, 1, th + OFF_W3, 128, 1, nullptr, B.da, 128);
-    k_dsilu_mul<<<nblk(n128, 256), 256, 0, st>>>(n128, B.da, B.z2, B.g, nullptr);
-    // layer 2
-    gemm(st, 128, 128, n, B.g, 1, 128, B.a1, 128, 1, nullptr, M.grad + OFF_W2, 128);
-    k_colsum<<<128, 256, 0, st>>>(n, 128, 128, B.g, M.grad + OFF_B2);
-    gemm(st, n, 128, 128, B.g, 128, 1, th + OFF_W2, 128, 1, nullptr, B.da, 128);
-    k_dsilu_mul<<<nblk(n128, 256), 256, 0, st>>>(n128, B.da, B.z1, B.g, B.g32);
-    // layer 1 (3 inputs)
-    k_dw1<<<384, 256, 0, st>>>(n, B.g32, B.x, M.grad + OFF_W1);
-    k_colsum<<<128, 256, 0, st>>>(n, 128, 128, B.g, M.grad + OFF_B1);
+    const int64_t tiles = (int64_t(n) + 15) / 16, blocks = (tiles + kTrainWarps - 1) / kTrainWarps;
+    const size_t smem = sizeof(mlpw::Weights);
+    CK(cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const int64_t run = std::max<int64_t>(128, ((int64_t(n) + kGradRuns - 1) / kGradRuns + 15) / 16 * 16);
+    const int runs = int((n + run - 1) / run);
+    ctx->launches += 3;
+    k_mlp_train<<<unsigned(std::min<int64_t>(blocks, 2 * ctx->sm_count)), 32 * kTrainWarps, smem, ctx->stream>>>(
+        n, dirs, y, M.theta_h, M.theta, M.scale, B.t);
+    k_mlp_wgrad<<<dim3(6, unsigned(runs)), 256, 0, ctx->stream>>>(n, int(run), B.t, B.part);
+    k_grad_sum<<<nblk(NPAR, 256) + 1, 256, 0, ctx->stream>>>(runs, B.part, M.grad, tiles, B.t.lossp, M.loss);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }
@@ -389,19 +479,7 @@ static void sync_params(gbfmm_ctx *ctx) {
 int mlp_eval_device(gbfmm_ctx *ctx, int64_t n, const float *dirs, float *h) {
     MlpState &M = ctx->mlp;
     if (!M.trained) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "fmm_mlp_eval: network not trained or set");
-    const int chunk = 1 << 18;
-    int rc = mlp_alloc_batch(ctx, int(std::min<int64_t>(n, chunk)));
-    if (rc) return rc;
-    for (int64_t b0 = 0; b0 < n; b0 += chunk) {
-        const int nb = int(std::min<int64_t>(chunk, n - b0));
-        rc = mlp_forward(ctx, nb, dirs + 3 * b0);
-        if (rc) return rc;
-        ++ctx->launches;
-        k_output<<<nblk(int64_t(nb) * 27, 256), 256, 0, ctx->stream>>>(nb, dirs + 3 * b0, bufs(ctx).o, M.scale,
-                                                                         h + 27 * b0);
-    }
-    CK(cudaGetLastError());
-    return GBFMM_OK;
+    return mlp_forward(ctx, n, dirs, h);
 }
 
 extern "C" int fmm_mlp_set(gbfmm_ctx *ctx, const float *theta, const float *scale) {
@@ -449,9 +527,7 @@ extern "C" int fmm_mlp_grad(gbfmm_ctx *ctx, int n, const float *dirs, const floa
     if (!ctx->mlp.trained) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "fmm_mlp_grad: set parameters first");
     int rc = mlp_alloc_batch(ctx, n);
     if (rc) return rc;
-    rc = mlp_forward(ctx, n, dirs);
-    if (rc) return rc;
-    rc = mlp_backward(ctx, n, dirs, y);
+    rc = mlp_gradient(ctx, n, dirs, y);
     if (rc) return rc;
     CK(cudaMemcpyAsync(grad, ctx->mlp.grad, NPAR * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
     if (loss) {
@@ -532,9 +608,7 @@ extern "C" int fmm_mlp_train(gbfmm_ctx *ctx, int64_t n, const float *dirs, int e
             ctx->launches += 2;
             k_gather_rows<<<nblk(int64_t(batch) * 3, 256), 256, 0, st>>>(batch, 3, perm + int64_t(s) * batch, dirs, bd);
             k_gather_rows<<<nblk(int64_t(batch) * 27, 256), 256, 0, st>>>(batch, 27, perm + int64_t(s) * batch, y, by);
-            rc = mlp_forward(ctx, batch, bd);
-            if (rc) return rc;
-            rc = mlp_backward(ctx, batch, bd, by);
+            rc = mlp_gradient(ctx, batch, bd, by);
             if (rc) return rc;
             ++M.step;
             const double frac = double(M.step) / double(total);
@@ -675,7 +749,8 @@ void mlp_free(gbfmm_ctx *ctx) {
         if (p) cudaFree(p);
     if (M.bufs) {
         MlpBuffers &B = bufs(ctx);
-        void *qs[] = {B.x, B.z1, B.z2, B.z3, B.o, B.da, B.g32, B.a1, B.a2, B.a3, B.go, B.g};
+        const TrainArgs &T = B.t;
+        void *qs[] = {T.x, T.z, T.g32, T.lossp, T.a[0], T.a[1], T.a[2], T.g[0], T.g[1], T.g[2], T.go, B.part};
         for (void *p : qs)
             if (p) cudaFree(p);
         delete &B;
@@ -685,31 +760,9 @@ void mlp_free(gbfmm_ctx *ctx) {
 
 // ---------------------------------------------------------------- no-allocation evaluation
 // fmm_mlp_eval_noalloc: the network evaluation of fmm_mlp_eval for callers
-// that must not allocate device memory during the call (see gbfmm.h).  The
-// activations live in one file-scope device array; its device address is
-// looked up once per device.
-#define GB_NOALLOC_CHUNK 4096                      // directions per pass over the scratch
+// that must not allocate device memory during the call (see gbfmm.h): the
+// evaluation keeps no activations in memory.
 #define GB_NOALLOC_MAX (int64_t(1) << 24)          // largest n accepted per call
-static constexpr size_t kNoallocZ = size_t(GB_NOALLOC_CHUNK) * 128 * sizeof(float);   // pre-activations
-static constexpr size_t kNoallocA = size_t(GB_NOALLOC_CHUNK) * 128 * sizeof(bf16);    // one activation buffer
-static constexpr size_t kNoallocO = size_t(GB_NOALLOC_CHUNK) * 32 * sizeof(float);    // outputs
-static constexpr size_t kNoallocBytes = kNoallocZ + 2 * kNoallocA + kNoallocO;         // 4.5 MiB
-
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
-
-static unsigned char *noalloc_base(gbfmm_ctx *ctx) {
-    // one lookup per device, made with that device current (the context's)
-    static unsigned char *base[64] = {nullptr};
-    const int dev = ctx->device;
-    int cur = -1;
-    if (cudaGetDevice(&cur) != cudaSuccess || cur != dev || dev < 0 || dev >= 64) return nullptr;
-    if (!base[dev]) {
-        void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess) return nullptr;
-        base[dev] = static_cast<unsigned char *>(p);
-    }
-    return base[dev];
-}
 
 extern "C" int fmm_mlp_eval_noalloc(gbfmm_ctx *ctx, int64_t n, const float *dirs, float *h) {
     if (!ctx) return GBFMM_ERR_INVALID_ARG;
@@ -721,31 +774,8 @@ extern "C" int fmm_mlp_eval_noalloc(gbfmm_ctx *ctx, int64_t n, const float *dirs
                            std::to_string(GB_NOALLOC_MAX) + " directions per call");
     if (!ctx->mlp.trained) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "fmm_mlp_eval_noalloc: network not set");
     if (n == 0) return GBFMM_OK;
-    unsigned char *base = noalloc_base(ctx);
-    if (!base)
-        return set_err(ctx, GBFMM_ERR_CUDA,
-                       "fmm_mlp_eval_noalloc: scratch address lookup failed (is the context's device current?)");
-    float *z = reinterpret_cast<float *>(base);
-    bf16 *a = reinterpret_cast<bf16 *>(base + kNoallocZ);
-    bf16 *b = reinterpret_cast<bf16 *>(base + kNoallocZ + kNoallocA);
-    float *o = reinterpret_cast<float *>(base + kNoallocZ + 2 * kNoallocA);
-    cudaStream_t st = ctx->stream;
-    const MlpState &M = ctx->mlp;
-    const bf16 *th = M.theta_h;
-    const float *bias = M.theta;
-    for (int64_t b0 = 0; b0 < n; b0 += GB_NOALLOC_CHUNK) {
-        const int nb = int(std::min<int64_t>(GB_NOALLOC_CHUNK, n - b0));
-        const int64_t e = int64_t(nb) * 128;
-        const float *d = dirs + 3 * b0;
-        ctx->launches += 7;
-        k_layer1<<<nblk(e, 256), 256, 0, st>>>(nb, d, th, bias, nullptr, nullptr, a);
-        gemm(st, nb, 128, 128, a, 128, 1, th + OFF_W2, 1, 128, bias + OFF_B2, z, 128);
-        k_silu<<<nblk(e, 256), 256, 0, st>>>(e, z, b);
-        gemm(st, nb, 128, 128, b, 128, 1, th + OFF_W3, 1, 128, bias + OFF_B3, z, 128);
-        k_silu<<<nblk(e, 256), 256, 0, st>>>(e, z, a);
-        gemm(st, nb, 32, 128, a, 128, 1, th + OFF_W4, 1, 128, bias + OFF_B4, o, 32);
-        k_output<<<nblk(int64_t(nb) * 27, 256), 256, 0, st>>>(nb, d, o, M.scale, h + 27 * b0);
-    }
-    CK(cudaGetLastError());
-    return GBFMM_OK;
+    int cur = -1;
+    if (cudaGetDevice(&cur) != cudaSuccess || cur != ctx->device)
+        return set_err(ctx, GBFMM_ERR_CUDA, "fmm_mlp_eval_noalloc: is the context's device current?");
+    return mlp_forward(ctx, n, dirs, h);
 }

@@ -1,11 +1,13 @@
-// Warp-level evaluation of the angular network inside the near-field loop.
+// Warp-level layers of the angular network.
 //
-// Sixteen queued pair directions form the rows of one m16n8k16 tile; the
-// layers run as warp MMAs (BF16 in, FP32 accumulate) with weights in shared
-// memory and activations kept in registers: the FP32 accumulator fragment of
-// one layer, passed through SiLU and packed to BF16 pairs, is exactly the A
-// fragment of the next layer for the same lane.  Layout of the parameter
-// vector as in mlp.cu (W1 [128x3], b1, W2 [128x128], b2, W3, b3, W4 [32x128], b4).
+// Sixteen directions form the rows of one m16n8k16 tile; the layers run as warp MMAs (BF16 in,
+// FP32 accumulate) with the weights in shared memory and the activations in registers: the FP32
+// accumulator fragment of one layer, passed through SiLU and packed to BF16 pairs, is exactly the
+// A fragment of the next layer for the same lane (row g = lane / 4 and g + 8, columns
+// 8 nt + 2 t, + 1 with t = lane % 4).  B fragments come by ldmatrix, four 8 x 8 pieces (two
+// column tiles) an instruction, transposed for the products with the weights' transpose; rows of
+// 136 elements keep them free of bank conflicts.  Layout of the parameter vector: W1 [128x3], b1,
+// W2 [128x128], b2, W3, b3, W4 [32x128] (rows 27..31 zero), b4 [32].
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -13,45 +15,57 @@
 namespace mlpw {
 
 constexpr int OFF_W1 = 0, OFF_B1 = 384, OFF_W2 = 512, OFF_B2 = 16896, OFF_W3 = 17024, OFF_B3 = 33408,
-              OFF_W4 = 33536, OFF_B4 = 37632;
-constexpr int LD = 136;  // padded row (bf16) of the weight matrices: conflict-free fragment loads
+              OFF_W4 = 33536, OFF_B4 = 37632, NPAR = 37664;
+constexpr int LD = 136;  // padded row (bf16) of the weight matrices
 
 struct Weights {
     __nv_bfloat16 W2[128 * LD];
     __nv_bfloat16 W3[128 * LD];
     __nv_bfloat16 W4[32 * LD];
-    float W1[128 * 3];
-    float b1[128], b2[128], b3[128], b4[32], scale[32];
+    float4 W1[128];  // row and bias
+    float b2[128], b3[128], b4[32], scale[32];
 };
 
-// cooperative copy of the parameters into shared memory (whole block)
+// cooperative copy of the parameters into shared memory (whole block); the parameter vector's
+// matrices start on 16-byte boundaries
 __device__ inline void load(Weights &w, const __nv_bfloat16 *__restrict__ th, const float *__restrict__ th32,
                             const float *__restrict__ scale) {
-    for (int i = threadIdx.x; i < 128 * 128; i += blockDim.x) {
-        const int r = i / 128, c = i % 128;
-        w.W2[r * LD + c] = th[OFF_W2 + i];
-        w.W3[r * LD + c] = th[OFF_W3 + i];
+    for (int i = threadIdx.x; i < 128 * 16; i += blockDim.x) {
+        const int r = i / 16, c = 8 * (i % 16);
+        *reinterpret_cast<uint4 *>(&w.W2[r * LD + c]) = *reinterpret_cast<const uint4 *>(th + OFF_W2 + 8 * i);
+        *reinterpret_cast<uint4 *>(&w.W3[r * LD + c]) = *reinterpret_cast<const uint4 *>(th + OFF_W3 + 8 * i);
+        if (i < 32 * 16)
+            *reinterpret_cast<uint4 *>(&w.W4[r * LD + c]) = *reinterpret_cast<const uint4 *>(th + OFF_W4 + 8 * i);
     }
-    for (int i = threadIdx.x; i < 32 * 128; i += blockDim.x) w.W4[(i / 128) * LD + (i % 128)] = th[OFF_W4 + i];
-    for (int i = threadIdx.x; i < 384; i += blockDim.x) w.W1[i] = __bfloat162float(th[OFF_W1 + i]);
     for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-        w.b1[i] = th32[OFF_B1 + i];
+        w.W1[i] = make_float4(__bfloat162float(th[OFF_W1 + 3 * i]), __bfloat162float(th[OFF_W1 + 3 * i + 1]),
+                              __bfloat162float(th[OFF_W1 + 3 * i + 2]), th32[OFF_B1 + i]);
         w.b2[i] = th32[OFF_B2 + i];
         w.b3[i] = th32[OFF_B3 + i];
     }
     for (int i = threadIdx.x; i < 32; i += blockDim.x) {
         w.b4[i] = th32[OFF_B4 + i];
-        w.scale[i] = i < 27 ? scale[i] : 0.f;
+        w.scale[i] = scale[i];
     }
 }
 
-// SiLU through the hardware tanh: silu(z) = z sigmoid(z) = z (1 + tanh(z/2)) / 2
-__device__ __forceinline__ float tanh_approx(float x) {
+// SiLU through the hardware tanh: sigmoid(z) = (1 + tanh(z/2)) / 2, silu = z sigmoid(z),
+// silu' = s (1 + z (1 - s))
+__device__ __forceinline__ float tanh_hw(float x) {
     float y;
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float silu_t(float z) { return 0.5f * z * (1.f + tanh_approx(0.5f * z)); }
+__device__ __forceinline__ float silu(float z) { return 0.5f * z * (1.f + tanh_hw(0.5f * z)); }
+__device__ __forceinline__ float dsilu(float z) {
+    const float s = 0.5f * (1.f + tanh_hw(0.5f * z));
+    return s * (1.f + z * (1.f - s));
+}
+
+// sign of the half-space fold (h is odd)
+__device__ __forceinline__ float half_space_sign(float x, float y, float z) {
+    return (z > 0.f || (z == 0.f && (y > 0.f || (y == 0.f && x >= 0.f)))) ? 1.f : -1.f;
+}
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -66,88 +80,81 @@ __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], uint32
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// one hidden 128 -> 128 layer: a (A fragments, 8 k-steps) -> next A fragments
-__device__ __forceinline__ void hidden(const __nv_bfloat16 *__restrict__ W, const float *__restrict__ b,
-                                       uint32_t a[8][4], int g, int t) {
-    float acc[16][4];
+template <bool T>
+__device__ __forceinline__ void ldsm4(uint32_t r[4], const __nv_bfloat16 *p) {
+    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    if (T)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// acc[nt] = a (KT steps of 16) times the transpose of W (rows = outputs), or W itself (TR: rows =
+// inputs), NT column tiles of 8; sums in ascending k from zero
+template <int NT, int KT, bool TR>
+__device__ __forceinline__ void layer(const __nv_bfloat16 *__restrict__ W, const uint32_t (*a)[4], float (*acc)[4],
+                                      int lane) {
+    const int mat = lane >> 3, r = lane & 7;
 #pragma unroll
-    for (int nt = 0; nt < 16; ++nt) {
-        const float b0 = b[nt * 8 + 2 * t], b1 = b[nt * 8 + 2 * t + 1];
-        acc[nt][0] = b0;
-        acc[nt][1] = b1;
-        acc[nt][2] = b0;
-        acc[nt][3] = b1;
-    }
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk)
+        for (int j = 0; j < 4; ++j) acc[nt][j] = 0.f;
 #pragma unroll
-        for (int nt = 0; nt < 16; ++nt) {
-            const __nv_bfloat16 *row = W + (nt * 8 + g) * LD + kk * 16 + 2 * t;
-            mma16816(acc[nt], a[kk], *reinterpret_cast<const uint32_t *>(row),
-                     *reinterpret_cast<const uint32_t *>(row + 8));
+    for (int kk = 0; kk < KT; ++kk)
+#pragma unroll
+        for (int nt = 0; nt < NT; nt += 2) {
+            uint32_t b[4];
+            // pieces in order: (nt, k low half), (nt, k high half), (nt + 1, low), (nt + 1, high)
+            ldsm4<TR>(b, TR ? W + (kk * 16 + (mat & 1) * 8 + r) * LD + (nt + (mat >> 1)) * 8
+                            : W + ((nt + (mat >> 1)) * 8 + r) * LD + kk * 16 + (mat & 1) * 8);
+            mma16816(acc[nt], a[kk], b[0], b[1]);
+            mma16816(acc[nt + 1], a[kk], b[2], b[3]);
         }
+}
+
+// accumulator fragments -> A fragments of the next product
+template <int KT>
+__device__ __forceinline__ void pack_a(uint32_t (*a)[4], const float (*v)[4]) {
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-        a[kk][0] = pack2(silu_t(acc[2 * kk][0]), silu_t(acc[2 * kk][1]));
-        a[kk][1] = pack2(silu_t(acc[2 * kk][2]), silu_t(acc[2 * kk][3]));
-        a[kk][2] = pack2(silu_t(acc[2 * kk + 1][0]), silu_t(acc[2 * kk + 1][1]));
-        a[kk][3] = pack2(silu_t(acc[2 * kk + 1][2]), silu_t(acc[2 * kk + 1][3]));
+    for (int kk = 0; kk < KT; ++kk) {
+        a[kk][0] = pack2(v[2 * kk][0], v[2 * kk][1]);
+        a[kk][1] = pack2(v[2 * kk][2], v[2 * kk][3]);
+        a[kk][2] = pack2(v[2 * kk + 1][0], v[2 * kk + 1][1]);
+        a[kk][3] = pack2(v[2 * kk + 1][2], v[2 * kk + 1][3]);
     }
 }
 
-// sign of the half-space fold (h is odd)
-__device__ __forceinline__ float fold_sign(float x, float y, float z) {
-    return (z > 0.f || (z == 0.f && (y > 0.f || (y == 0.f && x >= 0.f)))) ? 1.f : -1.f;
+// pre-activations of the first layer (3 inputs) for the folded directions dlo (row g), dhi (row g + 8)
+__device__ __forceinline__ void first(const Weights &w, const float dlo[3], const float dhi[3], float (*z)[4], int t) {
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float4 v = w.W1[8 * nt + 2 * t + e];
+            z[nt][e] = v.x * dlo[0] + v.y * dlo[1] + v.z * dlo[2] + v.w;
+            z[nt][2 + e] = v.x * dhi[0] + v.y * dhi[1] + v.z * dhi[2] + v.w;
+        }
 }
 
-// Network outputs for rows g and g + 8 of a 16-direction tile.  dlo, dhi:
-// the two directions this lane's rows hold (already folded, |T| = 1).
-// out[e]: for e = 0..7, column 8 (e / 2) + 2 t + (e & 1), row g (lo) / g + 8 (hi).
-__device__ __forceinline__ void eval16(const Weights &w, const float dlo[3], const float dhi[3], int g, int t,
-                                       float olo[8], float ohi[8]) {
-    uint32_t a[8][4];
+template <int NT>
+__device__ __forceinline__ void add_bias(const float *__restrict__ b, float (*z)[4], int t) {
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-        float z[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int c = kk * 16 + 2 * t + (e & 1) + (e >> 1) * 8;
-            const float w0 = w.W1[3 * c], w1 = w.W1[3 * c + 1], w2 = w.W1[3 * c + 2], bb = w.b1[c];
-            z[2 * e] = silu_t(fmaf(w0, dlo[0], fmaf(w1, dlo[1], fmaf(w2, dlo[2], bb))));
-            z[2 * e + 1] = silu_t(fmaf(w0, dhi[0], fmaf(w1, dhi[1], fmaf(w2, dhi[2], bb))));
-        }
-        // e = 0: col 2t (lo, hi); e = 1: col 2t+1; e = 2: col 2t+8; e = 3: col 2t+9
-        a[kk][0] = pack2(z[0], z[2]);
-        a[kk][1] = pack2(z[1], z[3]);
-        a[kk][2] = pack2(z[4], z[6]);
-        a[kk][3] = pack2(z[5], z[7]);
+    for (int nt = 0; nt < NT; ++nt) {
+        const float2 v = *reinterpret_cast<const float2 *>(b + 8 * nt + 2 * t);
+        z[nt][0] += v.x;
+        z[nt][1] += v.y;
+        z[nt][2] += v.x;
+        z[nt][3] += v.y;
     }
-    hidden(w.W2, w.b2, a, g, t);
-    hidden(w.W3, w.b3, a, g, t);
-    float acc[4][4];
+}
+
+__device__ __forceinline__ void silu_all(float (*z)[4]) {
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float b0 = w.b4[nt * 8 + 2 * t], b1 = w.b4[nt * 8 + 2 * t + 1];
-        acc[nt][0] = b0;
-        acc[nt][1] = b1;
-        acc[nt][2] = b0;
-        acc[nt][3] = b1;
-    }
+    for (int nt = 0; nt < 16; ++nt)
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const __nv_bfloat16 *row = w.W4 + (nt * 8 + g) * LD + kk * 16 + 2 * t;
-            mma16816(acc[nt], a[kk], *reinterpret_cast<const uint32_t *>(row),
-                     *reinterpret_cast<const uint32_t *>(row + 8));
-        }
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        olo[2 * nt] = acc[nt][0];
-        olo[2 * nt + 1] = acc[nt][1];
-        ohi[2 * nt] = acc[nt][2];
-        ohi[2 * nt + 1] = acc[nt][3];
-    }
+        for (int j = 0; j < 4; ++j) z[nt][j] = silu(z[nt][j]);
 }
 
 }  // namespace mlpw

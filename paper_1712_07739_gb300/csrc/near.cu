@@ -300,12 +300,6 @@ __global__ void __launch_bounds__(256) k_near_plan(int64_t nl, int L, int warps,
 // Two-float sums: the value is hi + lo, and each addition keeps its exact rounding error
 // (Knuth's two-sum), so a sum of FP32 terms carries ~48 mantissa bits without FP64 arithmetic
 // (FP64 runs at a small fraction of the FP32 rate on this part).
-__device__ __forceinline__ void tsum(float &hi, float &lo, float b) {
-    const float s = hi + b;
-    const float bb = s - hi;
-    lo += (hi - (s - bb)) + (b - bb);
-    hi = s;
-}
 __device__ __forceinline__ void tsum2(float &hi, float &lo, float bhi, float blo) {
     const float s = hi + bhi;
     const float bb = s - hi;
@@ -320,7 +314,13 @@ template <>
 struct Acc<float> {
     float hi, lo;
     __device__ __forceinline__ void zero() { hi = lo = 0.f; }
-    __device__ __forceinline__ void add(float v) { tsum(hi, lo, v); }
+    // a pair's value: Kahan's form (four operations), whose error stays that of perturbing each term
+    // by its own rounding; a two-sum is kept where sums meet sums
+    __device__ __forceinline__ void add(float v) {
+        const float s = hi + v;
+        lo += v - (s - hi);
+        hi = s;
+    }
     __device__ __forceinline__ void add(const Acc &o) { tsum2(hi, lo, o.hi, o.lo); }
     __device__ __forceinline__ Acc shfl_xor(int o) const {
         return Acc{__shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o)};
@@ -468,17 +468,19 @@ constexpr int near_warps() { return sizeof(R) == 4 ? 4 : 2; }
 template <typename R>
 constexpr int near_blocks() { return sizeof(R) == 4 ? 3 : 4; }
 
-// h of one pair by the plain rule
+// stress rows of one pair by the plain rule
 template <typename R, int HM>
-__device__ __forceinline__ void h_plain(const NearMedium<R> &md, const R *tab, const R T[3], R hs[18]) {
-    if constexpr (HM == HM_ISO)
-        h_iso_sym<R>(R(1), md.ha, T, hs);
-    else if constexpr (HM == HM_CUBIC)
-        h_cubic_moments<R>(md, tab, T, hs);
-    else if constexpr (HM == HM_POINTS)
-        h_general_points(md, tab, T, hs);
-    else
-        h_general_moments<R>(md, tab, T, hs);
+__device__ __forceinline__ void rows_plain(const NearMedium<R> &md, const R *tab, const R T[3], R Y[3][6]) {
+    if constexpr (HM == HM_CUBIC) {
+        rows_cubic<R>(md, tab, T, Y);
+    } else {
+        R hs[18];
+        if constexpr (HM == HM_POINTS)
+            h_general_points(md, tab, T, hs);
+        else
+            h_general_moments<R>(md, tab, T, hs);
+        stress_rows<R, true>(md, hs, Y);
+    }
 }
 
 // Angular bin of a direction folded into the upper half-space (h is odd): dominant axis face
@@ -572,14 +574,15 @@ __device__ __forceinline__ void learned_block(Shared &ws, const NearMedium<float
                     separation(pi, pj, d);
                     const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
                     const float ir = rsqrt_refined(r2), ir2 = ir * ir;
-                    float hs[18], Y[3][6];
+                    float Y[3][6];
                     if (w == 0) {
                         const float T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
-                        h_plain<float, HM>(md, tab, T, hs);
+                        rows_plain<float, HM>(md, tab, T, Y);
                     } else {
+                        float hs[18];
                         h_learned(ln, d, hs);
+                        stress_rows<float, HM >= HM_POINTS>(md, hs, Y);
                     }
-                    stress_rows<float, HM >= HM_POINTS>(md, hs, Y);
                     strain_of<float>(Y, pj.b[0], pj.b[1], pj.b[2], ir2 * pj.S[0], ir2 * pj.S[1], ir2 * pj.S[2], ef);
                     if (SYM)
                         strain_of<float>(Y, pi.b[0], pi.b[1], pi.b[2], -ir2 * pi.S[0], -ir2 * pi.S[1], -ir2 * pi.S[2],
@@ -772,17 +775,21 @@ __global__ void __launch_bounds__(near_warps<R>() * 32, near_blocks<R>())
                                 if (pj.seg != pi.seg && r2 > R(0)) {
                                     const R ir = rsqrt_refined(r2), ir2 = ir * ir;
                                     const R T[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
-                                    R hs[18];
-                                    h_plain<R, HM>(md, tab, T, hs);
                                     R Y[3][6], e6[6];
-                                    stress_rows<R, HM >= HM_POINTS>(md, hs, Y);
-                                    strain_of<R>(Y, pj.b[0], pj.b[1], pj.b[2], ir2 * pj.S[0], ir2 * pj.S[1],
-                                                 ir2 * pj.S[2], e6);
+                                    if constexpr (HM != HM_ISO) rows_plain<R, HM>(md, tab, T, Y);
+                                    auto strain = [&](const Pt<R> &p, R f) {
+                                        if constexpr (HM == HM_ISO)
+                                            strain_iso<R>(md, T, p.b[0], p.b[1], p.b[2], f * p.S[0], f * p.S[1],
+                                                          f * p.S[2], e6);
+                                        else
+                                            strain_of<R>(Y, p.b[0], p.b[1], p.b[2], f * p.S[0], f * p.S[1], f * p.S[2],
+                                                         e6);
+                                    };
+                                    strain(pj, ir2);
 #pragma unroll
                                     for (int e = 0; e < 6; ++e) f[e].add(e6[e]);
                                     if (SYM) {
-                                        strain_of<R>(Y, pi.b[0], pi.b[1], pi.b[2], -ir2 * pi.S[0], -ir2 * pi.S[1],
-                                                     -ir2 * pi.S[2], e6);
+                                        strain(pi, -ir2);
 #pragma unroll
                                         for (int e = 0; e < 6; ++e) {
                                             Acc<R> a = ws.rev[e][jl];
@@ -968,20 +975,24 @@ static NearMedium<R> near_medium(const DevMaterial &m) {
     NearMedium<R> n{};
     n.Q = m.Q;
     n.np = (m.Q - 1) / 2;
-    n.ha = R(m.ha);
-    const double cp = m.c12 + m.c44, D = m.cd, c44 = m.c44;
+    const double cp = m.c12 + m.c44, D = m.cd, c44 = m.c44, ydiag = D + 2.0 * c44;
+    n.k1 = R(m.V[1] * (1.0 - m.ha) + 2.0 * m.V[21]);
+    n.k3 = R(m.V[21] * (1.0 - m.ha));
+    n.k6 = R(6.0 * m.V[21]);
+    // adj_ii = al - be z_i^2 + ga z_j^2 z_k^2, adj_ij = mcp z_i z_j (c44 + D z_k^2)
+    const double al = c44 * (c44 + D + cp), be = c44 * (D + cp), ga = D * (D + 2.0 * cp), mcp = -cp;
     const double d0 = c44 * c44 * (c44 + D + cp), d1 = c44 * D * (D + 2.0 * cp);
-    n.al = R(c44 * (c44 + D + cp));
-    n.be = R(c44 * (D + cp));
-    n.ga = R(D * (D + 2.0 * cp));
     n.d1 = R(d1);
     n.d2 = R(D * D * (D + 3.0 * cp));
     n.e0 = R(d0 + 0.5 * d1);
-    n.c44 = R(c44);
-    n.cd = R(D);
-    n.mcp = R(-cp);
+    // sum_p h_cpp = (al + mcp c44) lin_c - (be + mcp c44) c1_c + (ga + 2 mcp D) x2_c
+    const double t0 = m.c12 * (al + mcp * c44), t1 = -m.c12 * (be + mcp * c44), t2 = m.c12 * (ga + 2.0 * mcp * D);
+    n.rc[0] = R(t0 + ydiag * al), n.rc[1] = R(t1 - ydiag * be), n.rc[2] = R(t2 + ydiag * ga);
+    n.rn[0] = R(t0), n.rn[1] = R(t1), n.rn[2] = R(t2 + ydiag * mcp * D), n.rn[3] = R(ydiag * mcp * c44);
+    n.re[0] = R(c44 * mcp * (2.0 * c44 + D)), n.re[1] = R(-c44 * mcp * D);
+    n.rs[0] = R(c44 * al), n.rs[1] = R(c44 * mcp * D), n.rs[2] = R(c44 * (mcp * c44 - be)), n.rs[3] = R(c44 * ga);
     n.y12 = R(m.c12);
-    n.ydiag = R(D + 2.0 * c44);
+    n.ydiag = R(ydiag);
     n.y44 = R(c44);
     static const int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
     auto C = [&m](int i, int j, int k, int l) { return m.C[((i * 3 + j) * 3 + k) * 3 + l]; };

@@ -30,10 +30,9 @@
 template <typename R>
 struct NearMedium {
     int Q, np;                   // circle points; pairs (phi, -phi) with 0 < phi < pi / 2
-    R ha;                        // isotropic: 3 - 4 nu (the factor hc is folded into the Burgers vectors)
-    R al, be, ga;                // cubic: adj_ii = al - be z_i^2 + ga z_j^2 z_k^2 (|z| = 1)
+    R k1, k3, k6;                // isotropic: strain_iso's factors (1 / (16 pi mu (1 - nu)) is folded into the Burgers vectors)
     R d1, d2, e0;                // cubic: det = d0 + d1 s2 + d2 s3 with s2, s3 the symmetric functions of z_i^2; e0 = d0 + d1 / 2
-    R c44, cd, mcp;              // cubic: adj_ij = mcp z_i z_j (c44 + cd z_k^2), mcp = -(C12 + C44)
+    R rc[3], rn[4], re[2], rs[4];  // cubic: factors of rows_cubic
     R y12, ydiag, y44;           // cubic: C12, C11 - C12, C44 (contraction)
     R C[36];                     // Voigt stiffness
     R Z[36];                     // (zz)_m = sum_x Z[6 m + x] (z z)_x, pairs in the order of hs
@@ -62,7 +61,14 @@ __device__ __forceinline__ float recip(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// Newton's iteration from the hardware's approximation: two steps square its error of 2^-20 twice,
+// four multiply-adds where the correctly rounded quotient takes a longer chain with its range checks
+__device__ __forceinline__ double recip(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(fma(-x, y, 1.0), y, y);
+    return fma(fma(-x, y, 1.0), y, y);
+}
 
 // the rows 1 .. np of a block's table (nothing for a rule too large for it)
 template <typename R>
@@ -180,13 +186,23 @@ struct Cubic {
 // L on a cubic polynomial, given its moments F (of y) and G (of w)
 template <typename R>
 __device__ __forceinline__ R apply3(const R F[4], const R G[3], const Cubic<R> &p) {
-    const R u = F[0] * p.P[0] + F[1] * p.P[1] + F[2] * p.P[2] + F[3] * p.P[3];
-    return u - (G[0] * p.E[0] + G[1] * p.E[1] + G[2] * p.E[2]);
+    R u = F[0] * p.P[0] + F[1] * p.P[1] + F[2] * p.P[2] + F[3] * p.P[3];
+    u -= G[0] * p.E[0];
+    u -= G[1] * p.E[1];
+    u -= G[2] * p.E[2];
+    return u;
 }
 
-// h of a cubic medium with axes along x, y, z, times 4 pi Q
+// A cubic medium with axes along x, y, z: the stress rows Y (see stress_rows) of 4 pi Q h without
+// h itself.  With adj_ii = al - be z_i^2 + ga z_j^2 z_k^2 and adj_ij = mcp z_i z_j (c44 + cd z_k^2)
+// every row is a combination of L on monomials: lin_q = L[z_q], c1_q = L[z_q^3],
+// c2_qk = L[z_q z_k^2], c3 = L[z_0 z_1 z_2], x2_q = L[z_q z_j^2 z_k^2], x3_q = L[z_i z_j z_q^3] and
+// t_qk = L[z_q^3 z_k^2]; components of h that meet in a row share its terms, so the 18 rows cost 48
+// multiply-adds where h and its contraction cost 92 (with Kahan sums of the pairs, whole pass of 250,000
+// segments, Q = 16: 46.6 -> 44.6 ms; 3,000 segments in FP64, Q = 32: 17.7 -> 17.0 ms), and round less
+// (rows of random directions, FP32, C11 = 1.684, C12 = 1.214, C44 = 0.754: 3.0e-7 by way of h, 2.5e-7).
 template <typename R>
-__device__ __forceinline__ void h_cubic_moments(const NearMedium<R> &md, const R *tab, const R T[3], R hs[18]) {
+__device__ __forceinline__ void rows_cubic(const NearMedium<R> &md, const R *tab, const R T[3], R Y[3][6]) {
     R a[3], b[3];
     circle_axes<R>(T, a, b);
     R aa[3], ab[3], bb[3];  // z_i^2: aa c^2 + ab c s + bb s^2 (ab = 2 a b)
@@ -277,12 +293,14 @@ __device__ __forceinline__ void h_cubic_moments(const NearMedium<R> &md, const R
     R F2[3][4], G2[3][3];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const R t2 = R(2) * T[k];
-        R u[4];
+        const R t2 = R(2) * T[k], ta = t2 * a[k], tb = t2 * b[k];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) u[i] = a[k] * Th[i] + b[k] * Th[i + 1];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) F2[k][i] = aa[k] * Ps[i] + ab[k] * Ps[i + 1] + bb[k] * Ps[i + 2] - t2 * u[i];
+        for (int i = 0; i < 4; ++i) {
+            R u = aa[k] * Ps[i] + ab[k] * Ps[i + 1] + bb[k] * Ps[i + 2];
+            u -= ta * Th[i];
+            u -= tb * Th[i + 1];
+            F2[k][i] = u;
+        }
 #pragma unroll
         for (int i = 0; i < 3; ++i) G2[k][i] = aa[k] * Th[i] + ab[k] * Th[i + 1] + bb[k] * Th[i + 2];
     }
@@ -290,37 +308,48 @@ __device__ __forceinline__ void h_cubic_moments(const NearMedium<R> &md, const R
     for (int i = 0; i < 4; ++i) F2[2][i] = F[i] - F2[0][i] - F2[1][i];
 #pragma unroll
     for (int i = 0; i < 3; ++i) G2[2][i] = G[i] - G2[0][i] - G2[1][i];
-    R x2[3], x3[3];  // z_q z_j^2 z_k^2 and z_i z_j z_k^3
+    R x2[3], x3[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const int j = (q + 2) % 3;
         x2[q] = apply3<R>(F2[j], G2[j], zq[q]);
-        x3[q] = apply3<R>(F2[q], G2[q], p3);
+        x3[q] = q < 2 ? apply3<R>(F2[q], G2[q], p3) : c3 - x3[0] - x3[1];  // |z|^2 = 1
     }
-    constexpr int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
 #pragma unroll
-    for (int pr = 0; pr < 6; ++pr) {
-        const int v = PV[pr], p = PP[pr];
+    for (int c = 0; c < 3; ++c) {
+        const R v = md.rn[0] * lin[c] + md.rn[1] * c1[c] + md.rn[2] * x2[c];
+        Y[c][c] = md.rc[0] * lin[c] + md.rc[1] * c1[c] + md.rc[2] * x2[c];
+        Y[c][(c + 1) % 3] = v + md.rn[3] * c2[c][(c + 1) % 3];
+        Y[c][(c + 2) % 3] = v + md.rn[3] * c2[c][(c + 2) % 3];
+        Y[c][3 + c] = md.re[0] * c3 + md.re[1] * x3[c];
+        const R u = md.rs[0] * lin[c] + md.rs[1] * x2[c];  // shear rows with z_c as the odd factor
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (v == p) {
-                if (q == v) {
-                    hs[3 * pr + q] = md.al * lin[q] - md.be * c1[q] + md.ga * x2[q];
-                } else {
-                    const int k = 3 - v - q;
-                    hs[3 * pr + q] = md.al * lin[q] - md.be * c2[q][v] + md.ga * apply3<R>(F2[k], G2[k], z3[q]);
-                }
-            } else {
-                const int k = 3 - v - p;
-                if (q == k) {
-                    hs[3 * pr + q] = md.mcp * (md.c44 * c3 + md.cd * x3[k]);
-                } else {
-                    const int o = q == v ? p : v;
-                    hs[3 * pr + q] = md.mcp * (md.c44 * c2[o][q] + md.cd * x2[o]);
-                }
-            }
+        for (int n = 1; n < 3; ++n) {
+            const int r = (c + n) % 3, k = (c + 3 - n) % 3;
+            Y[r][3 + k] = u + md.rs[2] * c2[c][r] + md.rs[3] * apply3<R>(F2[k], G2[k], z3[c]);
         }
     }
+}
+
+// An isotropic medium: with h_cpq = -3 T_c T_p T_q - ha d_cp T_q + d_cq T_p + d_pq T_c (ha = 3 - 4 nu) the
+// contraction of strain_of leaves, up to an antisymmetric part that the strain does not see, the
+// symmetric part of T (x) S x (k1 b - k6 (T.b) T) + k3 b (x) (S x T): 43 multiply-adds a direction and
+// no rows (2,000 segments in FP64, whose near field is bound by its arithmetic: whole
+// pass 5.35 -> 3.89 ms; FP32 rounding 1.7e-7 by way of the rows, 0.9e-7).
+template <typename R>
+__device__ __forceinline__ void strain_iso(const NearMedium<R> &md, const R T[3], R b0, R b1, R b2, R S0, R S1, R S2,
+                                           R e[6]) {
+    const R x0 = S1 * T[2] - S2 * T[1], x1 = S2 * T[0] - S0 * T[2], x2 = S0 * T[1] - S1 * T[0];  // S x T
+    const R f = md.k6 * (T[0] * b0 + T[1] * b1 + T[2] * b2);
+    const R u0 = md.k1 * (S1 * b2 - S2 * b1) - f * x0, u1 = md.k1 * (S2 * b0 - S0 * b2) - f * x1,
+            u2 = md.k1 * (S0 * b1 - S1 * b0) - f * x2;
+    const R w0 = md.k3 * x0, w1 = md.k3 * x1, w2 = md.k3 * x2;
+    e[0] = T[0] * u0 + b0 * w0;
+    e[1] = T[1] * u1 + b1 * w1;
+    e[2] = T[2] * u2 + b2 * w2;
+    e[3] = (T[1] * u2 + b1 * w2) + (T[2] * u1 + b2 * w1);
+    e[4] = (T[0] * u2 + b0 * w2) + (T[2] * u0 + b2 * w0);
+    e[5] = (T[0] * u1 + b0 * w1) + (T[1] * u0 + b1 * w0);
 }
 
 // product of two quadratic forms, A and B: coefficients of c^2, c s, s^2, then of c eps, s eps;

@@ -244,9 +244,11 @@ __global__ void __launch_bounds__(256) k_near_totals(int64_t nl, int L, const in
 }
 
 // The size is the smallest candidate whose rows and items fit the buffers and that leaves a
-// resident warp about eight items (a warp's last item is then a small part of its time), but
-// not above 32,768 pairs where the buffers allow (about 1 ms of a warp): every quantity
-// depends on the network and the options alone, so results do not depend on a buffer's history.
+// resident warp at most sixteen items (four at least: a warp's last item is then a small part of its
+// time; 50,000 segments, near field: 9.3 ms with eight to two items, 8.5 with these, 8.6 with twice
+// as many), but not above 32,768 pairs where the buffers allow (about 1 ms of a warp): every
+// quantity depends on the network and the options alone, so results do not depend on a buffer's
+// history.
 template <bool SYM>
 __global__ void __launch_bounds__(256) k_near_plan(int64_t nl, int L, int warps, long long cap_rows, long long cap_items,
                                                    const int *__restrict__ tstart, const int *__restrict__ sstart,
@@ -267,7 +269,7 @@ __global__ void __launch_bounds__(256) k_near_plan(int64_t nl, int L, int warps,
             lp[ND * l + d] = ns;
             if (B >= 0) ns += sstart[B + 1] - sstart[B];
         }
-        int64_t want = int64_t(cnt[0] / (8ull * (unsigned long long)warps));
+        int64_t want = int64_t(cnt[0] / (16ull * (unsigned long long)warps));
         want = min(want, int64_t(32768));
         int k = 0;
         while (k < kPlanSizes - 1 && (plan_size(k) < want || (long long)cnt[1 + k] > cap_rows ||

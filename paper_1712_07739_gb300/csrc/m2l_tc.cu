@@ -39,13 +39,18 @@
 // cells occupies the GPU; each operator byte is then read once per set.  The sections' sums go to
 // scratch and are added in their order (k_few_sum).
 //
-// Warp roles (192 threads): warp 0 loads the operator rows by TMA, warp 1
-// owns TMEM and issues the MMAs, warps 2-5 gather the multipole rows (each
-// thread waits for its copies, fences them to the async proxy and arrives on
-// the stage's barrier) and then read the accumulator out (warp w reads TMEM
-// lanes 32 (w % 4) .. 32 (w % 4) + 31).  Every mbarrier wait is bounded; on
-// time-out a device status word gets GBFMM_ERR_TIMEOUT and the block winds
-// down, freeing its tensor memory.
+// Warp roles (320 threads): warp 0 loads the operator rows by TMA, warp 1
+// owns TMEM and issues the MMAs, warps 2-9 gather the multipole rows (the
+// copies count in the stage's barrier as they arrive) and then read the accumulator out (warp w reads TMEM
+// lanes 32 (w % 4) .. 32 (w % 4) + 31, every second 16 columns).  The
+// bookkeeping of single threads bounds a stage: with the ring's position by
+// division and descriptors formed for every MMA the tensor pipe was 44 % busy
+// (levels 2-4 of 50,000 segments, p = 5, free targets, 2.8 ms) whatever the
+// gathering did; counted rings and descriptors a constant apart make it 56 %
+// (1.7 ms).  Gathering by TMA (tile::gather4) instead is slower (6,011
+// segments, p = 6, whole pass 1.92 ms against 1.43).  Every mbarrier wait is
+// bounded; on time-out a device status word gets
+// GBFMM_ERR_TIMEOUT and the block winds down, freeing its tensor memory.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -72,8 +77,8 @@ struct OffsetEntry {
 __constant__ OffsetEntry c_offs[8][189];
 
 struct M2LParams {
-    const uint8_t *Whi, *Wlo;         // packed W (hi, residual), level l at byte wofs[l]
-    int64_t wofs[GB_TC_MAXLEV];
+    const uint8_t *Whi, *Wlo;         // packed W (hi, residual)
+    int wrow[GB_TC_MAXLEV];           // first row of a level
     int row_bytes;                    // K_pad x element size
     CUtensorMap tmT;                  // T hi: (Kp, Np, 316)
     CUtensorMap tmTlo;                // T residual: (Kp, Np, n_lo)
@@ -113,6 +118,7 @@ __device__ __forceinline__ float wscale_of(unsigned bits) {
 //    operands (TMA) of two MMAs that share the CTA's two tiles of target cells as one
 //    N = 256 operand, so a gathered row feeds 256 instead of nsub output columns and a
 //    stage gathers 32 instead of 48 KB for about the same tensor work.
+constexpr int kTcThreads = 320;  // warps: operators, MMA, eight for the multipole rows and the epilogue
 constexpr int kTileA = 128 * 128;  // one tile's multipole rows per stage: 16 KB
 template <bool SWAP> constexpr int tpc_of() { return SWAP ? 2 : 3; }  // tiles of 128 cells per CTA
 
@@ -161,21 +167,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *st
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// wait until at most n groups of this thread are pending (n is 0..5)
-__device__ __forceinline__ void cp_async_wait(int n) {
-    switch (n) {
-        case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-        case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-        case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-        case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-        case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-        default: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-    }
+// this thread's copies so far count once in the barrier when they have arrived
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, int c2,
                                             uint32_t bar) {
@@ -269,8 +265,70 @@ constexpr int kMaxSeg = 8 * GB_TC_MAXLEV;
 // split: the residual passes apply at this level
 __device__ __forceinline__ int passes_of(const OffsetEntry &e, int split) { return (split && e.lo >= 0) ? 3 : 1; }
 
+// the stage a role works on and its phase: counted, not divided (a division by the run-time number
+// of stages costs more than the rest of a stage's bookkeeping)
+struct Ring {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int stages) {
+        if (++s == stages) s = 0, ph ^= 1u;
+    }
+};
+
+// one stage's MMAs with the cells as A: the tiles in tm, four K steps each; begun: tiles whose
+// accumulator holds a sum.  Descriptors of a stage differ in the address field only.
+template <bool TF32, int TPC>
+__device__ __forceinline__ void mma_tiles(uint32_t tmem, int nsub, uint32_t rows, uint32_t ops, uint32_t idesc, uint32_t tm,
+                                          uint32_t begun) {
+    const uint64_t ad = sw128_desc(rows), bd = sw128_desc(ops);
+#pragma unroll
+    for (int t = 0; t < TPC; ++t)
+        if ((tm >> t) & 1u)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                mma_issue<TF32>(tmem + t * nsub, ad + uint32_t(t * (kTileA >> 4) + 2 * kk), bd + uint32_t(2 * kk), idesc,
+                                kk > 0 ? 1u : (begun >> t) & 1u);
+}
+
+// which of a CTA's tiles take part in an offset: those with a source (operators as A: all of them,
+// the tiles are one operand)
+template <bool SWAP, int TPC, int W>
+__device__ __forceinline__ uint32_t tiles_at(const uint32_t (&act)[TPC][W], int o) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int t = 0; t < TPC; ++t) m |= ((act[t][o / 32] >> (o % 32)) & 1u) << t;
+    return SWAP ? (1u << TPC) - 1u : m;
+}
+
+// A warp's share of a stage's multipole rows: rows 16 g .. 16 g + 15 of every tile, as copies of 8
+// lanes per 128-byte row piece (lane l moves piece l % 8 of rows 4 i + l / 8).  take_rows spreads the
+// table rows that the lanes found (lane l: for row l % 16 of tile l / 16, then of tile 2; -1 without) to the copying lanes: addresses and sizes (0 writes zeros).
+template <int TPC>
+__device__ __forceinline__ void take_rows(const int own[2], int lane, const uint8_t *table, int row_bytes,
+                                          const uint8_t *(&src)[TPC][4], uint32_t (&size)[TPC][4]) {
+#pragma unroll
+    for (int t = 0; t < TPC; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int v = __shfl_sync(0xffffffffu, own[t / 2], 16 * (t & 1) + 4 * i + (lane >> 3));
+            src[t][i] = table + 16 * (lane & 7) + int64_t(max(v, 0)) * row_bytes;
+            size[t][i] = v < 0 ? 0u : 16u;
+        }
+}
+// one stage's copies of the tiles in tm; dst: this lane's place in the stage's first tile for even and
+// odd i (16-byte piece c of row r lies at (c ^ (r & 7)) * 16)
+template <int TPC>
+__device__ __forceinline__ void copy_rows(uint32_t tm, const uint32_t dst[2], int64_t at, const uint8_t *const (&src)[TPC][4],
+                                          const uint32_t (&size)[TPC][4]) {
+#pragma unroll
+    for (int t = 0; t < TPC; ++t)
+        if ((tm >> t) & 1u)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async16(dst[i & 1] + t * kTileA + i * 512, src[t][i] + at, size[t][i]);
+}
+
 template <bool TF32, bool SWAP>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
     k_m2l_tc(const __grid_constant__ M2LParams P, const int4 *__restrict__ seg, int n_seg,
              const int *__restrict__ list, const int *__restrict__ occ, const int *__restrict__ tocc,
              const TreeBox *__restrict__ box, float *__restrict__ S, double *__restrict__ S64,
@@ -288,7 +346,8 @@ __global__ void __launch_bounds__(192, 1)
 
     __shared__ int s_level, s_cls, s_rows, s_nrow, s_stop;  // s_rows, s_nrow: first list entry, cells of the CTA
     __shared__ short s_tgt[TPC][128][3];  // sub-grid positions of the tiles' target cells
-    __shared__ uint32_t s_active[6];   // offsets with at least one occupied source cell
+    __shared__ uint32_t s_active[6];      // offsets with at least one occupied source cell
+    __shared__ uint32_t s_tact[TPC][6];   // the same, of one tile
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int tile = blockIdx.x / groups, group = blockIdx.x % groups;
     if (threadIdx.x == 0) {
@@ -307,7 +366,10 @@ __global__ void __launch_bounds__(192, 1)
                 }
             }
     }
-    if (threadIdx.x < 6) s_active[threadIdx.x] = 0u;
+    if (threadIdx.x < 6) {
+        s_active[threadIdx.x] = 0u;
+        for (int t = 0; t < TPC; ++t) s_tact[t][threadIdx.x] = 0u;
+    }
     __syncthreads();
     if (s_level < 0 || s_stop) return;  // surplus block, or an earlier block timed out
     const int level = s_level, cls = s_cls, nrow = s_nrow;
@@ -327,24 +389,29 @@ __global__ void __launch_bounds__(192, 1)
     __syncthreads();
 
     // active offsets: lane r of warp w checks rows 4r .. 4r + 3 of every tile
-    for (int oi = P.o_lo + warp; oi < P.o_hi; oi += 6) {
+    for (int oi = P.o_lo + warp; oi < P.o_hi; oi += kTcThreads / 32) {
         const OffsetEntry e = c_offs[cls][oi];
         const int ccx = e.cls & 1, ccy = (e.cls >> 1) & 1, ccz = e.cls >> 2;
-        bool hit = false;
-        for (int q = 0; q < 4 * TPC; ++q) {
-            const int t = q / 4, row = 4 * lane + q % 4;
-            const int px = s_tgt[t][row][0] + e.sx, py = s_tgt[t][row][1] + e.sy, pz = s_tgt[t][row][2] + e.sz;
-            if (px >= 0 && py >= 0 && pz >= 0 && px < m && py < m && pz < m) {
-                const int64_t g = cbase + (int64_t(2 * pz + ccz) * n + (2 * py + ccy)) * n + (2 * px + ccx);
-                hit |= occ[g] > 0;
+        for (int t = 0; t < TPC; ++t) {
+            bool hit = false;
+            for (int q = 0; q < 4; ++q) {
+                const int row = 4 * lane + q;
+                const int px = s_tgt[t][row][0] + e.sx, py = s_tgt[t][row][1] + e.sy, pz = s_tgt[t][row][2] + e.sz;
+                if (px >= 0 && py >= 0 && pz >= 0 && px < m && py < m && pz < m) {
+                    const int64_t g = cbase + (int64_t(2 * pz + ccz) * n + (2 * py + ccy)) * n + (2 * px + ccx);
+                    hit |= occ[g] > 0;
+                }
+            }
+            if (__any_sync(0xffffffffu, hit) && lane == 0) {
+                atomicOr(&s_active[oi / 32], 1u << (oi % 32));
+                atomicOr(&s_tact[t][oi / 32], 1u << (oi % 32));
             }
         }
-        if (__any_sync(0xffffffffu, hit) && lane == 0) atomicOr(&s_active[oi / 32], 1u << (oi % 32));
     }
 
     if (threadIdx.x == 0) {
-        // full: the operator-load thread (expect_tx) + 128 gathering threads; empty: the MMA commit
-        for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&bars[s]), 129);
+        // full: the operator-load thread (expect_tx) + 256 gathering threads; empty: the MMA commit
+        for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&bars[s]), 257);
         for (int s = stages; s < 2 * stages + 1; ++s) mbar_init(smem_u32(&bars[s]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -363,25 +430,27 @@ __global__ void __launch_bounds__(192, 1)
 
     if (warp == 0 && lane == 0) {
         // ---------------- operator rows (B) by TMA
-        int it = 0;
-        bool ok = true;
-        for (int oi = 0; oi < 189 && ok; ++oi) {
+        Ring rg;
+        bool ok = true, drop = P.drop_first != 0;
+        for (int oi = P.o_lo; oi < P.o_hi && ok; ++oi) {
             if (!((s_active[oi / 32] >> (oi % 32)) & 1u)) continue;
             const OffsetEntry e = c_offs[cls][oi];
             const int np = passes_of(e, split);
             for (int pass = 0; pass < np && ok; ++pass) {
                 const CUtensorMap *tb = (pass == 2) ? &P.tmTlo : &P.tmT;
                 const int tidx = (pass == 2) ? e.lo : e.top;
-                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                    const int s = it % stages;
-                    const uint32_t ph = (it / stages) & 1;
-                    if (!mbar_wait(empty0 + 8 * s, ph ^ 1, status)) {
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                    const int s = rg.s;
+                    if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
                         ok = false;
                         break;
                     }
                     const uint32_t fb = full0 + 8 * s;
                     mbar_expect_tx(fb, uint32_t(SWAP ? mbc * kTileA : stageB));
-                    if (P.drop_first && it == 0) continue;  // the MMA warp's wait on this stage runs out
+                    if (drop) {  // the MMA warp's wait on this stage runs out
+                        drop = false;
+                        continue;
+                    }
                     if (SWAP)
                         for (int mb = 0; mb < mbc; ++mb)
                             tma_load_3d(smem0 + s * stage_bytes + kStageA + mb * kTileA, tb, kb * P.kstep,
@@ -394,38 +463,39 @@ __global__ void __launch_bounds__(192, 1)
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
         const uint32_t idesc = P.idesc;
-        int it = 0;
+        Ring rg;
+        uint32_t begun = 0u;  // tiles whose accumulator holds a sum
         bool ok = true;
-        for (int oi = 0; oi < 189 && ok; ++oi) {
+        for (int oi = P.o_lo; oi < P.o_hi && ok; ++oi) {
             if (!((s_active[oi / 32] >> (oi % 32)) & 1u)) continue;
+            const uint32_t tm = tiles_at<SWAP>(s_tact, oi);
             const OffsetEntry e = c_offs[cls][oi];
             const int np = passes_of(e, split);
             for (int pass = 0; pass < np && ok; ++pass) {
-                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                    const int s = it % stages;
-                    const uint32_t ph = (it / stages) & 1;
-                    if (!mbar_wait(full0 + 8 * s, ph, status)) {
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                    const int s = rg.s;
+                    if (!mbar_wait(full0 + 8 * s, rg.ph, status)) {
                         ok = false;
                         break;
                     }
+                    // the gathered rows were written through the generic proxy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     const uint32_t a = smem0 + s * stage_bytes;
-                    for (int kk = 0; kk < 4; ++kk) {
-                        if (SWAP) {
-                            // the two tiles' 256 rows (contiguous, 1024 B per 8 rows) are the N operand
-                            const uint64_t bd = sw128_desc(a + kk * 32);
-                            for (int mb = 0; mb < mbc; ++mb) {
-                                const uint64_t ad = sw128_desc(a + kStageA + mb * kTileA + kk * 32);
-                                mma_issue<TF32>(tmem + mb * 256, ad, bd, idesc, (it > 0 || kk > 0) ? 1u : 0u);
-                            }
-                        } else {
-                            const uint64_t bd = sw128_desc(a + kStageA + kk * 32);
-                            for (int t = 0; t < TPC; ++t) {
-                                const uint64_t ad = sw128_desc(a + t * kTileA + kk * 32);
-                                mma_issue<TF32>(tmem + t * P.nsub, ad, bd, idesc, (it > 0 || kk > 0) ? 1u : 0u);
-                            }
+                    if (SWAP) {
+                        // the two tiles' 256 rows (contiguous, 1024 B per 8 rows) are the N operand
+                        const uint64_t bd = sw128_desc(a);
+                        for (int mb = 0; mb < mbc; ++mb) {
+                            const uint64_t ad = sw128_desc(a + kStageA + mb * kTileA);
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                mma_issue<TF32>(tmem + mb * 256, ad + uint32_t(2 * kk), bd + uint32_t(2 * kk), idesc,
+                                                (begun || kk > 0) ? 1u : 0u);
                         }
+                    } else {
+                        mma_tiles<TF32, TPC>(tmem, P.nsub, a, a + kStageA, idesc, tm, begun);
                     }
+                    begun |= tm;
                     mma_commit(empty0 + 8 * s);
                 }
             }
@@ -433,93 +503,61 @@ __global__ void __launch_bounds__(192, 1)
         // fires when every MMA issued above has completed (no MMA, no wait: see the epilogue)
         if (s_active[0] | s_active[1] | s_active[2] | s_active[3] | s_active[4] | s_active[5]) mma_commit(accb);
     } else if (warp >= 2) {
-        const int row = threadIdx.x - 64;  // 0..127: this thread's tile row
+        const int wrow0 = 16 * (warp - 2);  // this warp's first row of every tile
+        const uint32_t place[2] = {uint32_t((wrow0 + (lane >> 3)) * 128 + (((lane & 7) ^ (lane >> 3)) << 4)),
+                                   uint32_t((wrow0 + (lane >> 3)) * 128 + (((lane & 7) ^ (4 + (lane >> 3))) << 4))};
         {
             // ---------------- multipole rows (A): gathered by cp.async into the 128-byte
-            // swizzled K-major layout (16-byte piece c of row r at (c ^ (r & 7)) * 16);
-            // sources outside the sub-grid, or empty, read as zeros.  Each thread finds
-            // the source of its own row; the copies go by 8 lanes per row (lane l moves
-            // piece l % 8 of rows 4 i + l / 8 of its warp's 32), so a warp instruction
-            // reads four whole 128-byte row pieces.  A thread signals stage j full once it
-            // has issued stage j + 1: issuing stage j + lag waits for the MMAs of stage
-            // j + lag - stages, so with lag = stages - 1 the MMAs of stage j could not be
-            // issued before those of stage j - 1 had finished; with lag = 1 they wait only
-            // for stage j - 2, and two stages of copies stay in flight.
-            const int lag = 1;
-            int it = 0, done = 0;
+            // swizzled K-major layout; sources outside the sub-grid, or empty, read as zeros.  Each
+            // warp finds the sources of its 16 rows of every tile once per offset.  A stage's copies
+            // count in its barrier when they arrive, so no thread waits for them and every stage
+            // stays in flight; the MMA thread orders them before the tensor core's reads.
+            Ring rg;
             bool ok = true;
-            const int c = lane & 7, wrow0 = row - lane;  // this warp's first tile row
-            for (int oi = 0; oi < 189 && ok; ++oi) {
+            for (int oi = P.o_lo; oi < P.o_hi && ok; ++oi) {
                 if (!((s_active[oi / 32] >> (oi % 32)) & 1u)) continue;
+                const uint32_t tm = tiles_at<SWAP>(s_tact, oi);
                 const OffsetEntry e = c_offs[cls][oi];
-                int64_t own[TPC];
-                uint32_t own_nb = 0;
+                int own[2] = {-1, -1};
 #pragma unroll
-                for (int t = 0; t < TPC; ++t) {
-                    const int px = s_tgt[t][row][0] + e.sx, py = s_tgt[t][row][1] + e.sy,
-                              pz = s_tgt[t][row][2] + e.sz;
-                    bool have = px >= 0 && py >= 0 && pz >= 0 && px < m && py < m && pz < m;
-                    own[t] = 0;
-                    if (have) {
+                for (int k = 0; k < (TPC + 1) / 2; ++k) {
+                    const int t = 2 * k + lane / 16, r = wrow0 + lane % 16;
+                    if (t >= TPC) continue;
+                    const int px = s_tgt[t][r][0] + e.sx, py = s_tgt[t][r][1] + e.sy, pz = s_tgt[t][r][2] + e.sz;
+                    if (px >= 0 && py >= 0 && pz >= 0 && px < m && py < m && pz < m) {
                         const int ccx = e.cls & 1, ccy = (e.cls >> 1) & 1, ccz = e.cls >> 2;
-                        have = occ[cbase + (int64_t(2 * pz + ccz) * n + (2 * py + ccy)) * n + (2 * px + ccx)] > 0;
-                        own[t] = (((int64_t(e.cls) * m + pz) * m + py) * m + px) * P.row_bytes;
-                    }
-                    own_nb |= have ? (1u << t) : 0u;
-                }
-                int64_t srcoff[8][TPC];
-                uint32_t nbm = 0;  // bit 8 t + i: row 4 i + lane / 8 of tile t has a source
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int from = 4 * i + (lane >> 3);
-                    const uint32_t f = __shfl_sync(0xffffffffu, own_nb, from);
-#pragma unroll
-                    for (int t = 0; t < TPC; ++t) {
-                        srcoff[i][t] = __shfl_sync(0xffffffffu, own[t], from);
-                        nbm |= ((f >> t) & 1u) << (8 * t + i);
+                        if (occ[cbase + (int64_t(2 * pz + ccz) * n + (2 * py + ccy)) * n + (2 * px + ccx)] > 0)
+                            own[k] = P.wrow[level] + ((e.cls * m + pz) * m + py) * m + px;
                     }
                 }
+                __syncwarp();
                 const int np = passes_of(e, split);
                 for (int pass = 0; pass < np && ok; ++pass) {
-                    const uint8_t *wb = ((pass == 1) ? P.Wlo : P.Whi) + P.wofs[level];
-                    for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                        const int s = it % stages;
-                        const uint32_t ph = (it / stages) & 1;
-                        if (!mbar_wait(empty0 + 8 * s, ph ^ 1, status)) {
+                    const uint8_t *src[TPC][4];
+                    uint32_t size[TPC][4];
+                    take_rows<TPC>(own, lane, pass == 1 ? P.Wlo : P.Whi, P.row_bytes, src, size);
+                    for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                        const int s = rg.s;
+                        if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
                             ok = false;
                             break;
                         }
-                        const uint32_t sbase = smem0 + s * stage_bytes;
-                        const uint8_t *wk = wb + kb * 128 + 16 * c;
-#pragma unroll
-                        for (int t = 0; t < TPC; ++t)
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const int r = wrow0 + 4 * i + (lane >> 3);
-                                cp_async16(sbase + t * kTileA + r * 128 + ((c ^ (r & 7)) << 4), wk + srcoff[i][t],
-                                           ((nbm >> (8 * t + i)) & 1u) ? 16u : 0u);
-                            }
-                        cp_async_commit();
-                        if (it - done >= lag) {
-                            // the copies of stage `done` are complete: make them visible to the
-                            // tensor cores, then count this thread in that stage's full barrier
-                            cp_async_wait(lag);
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            mbar_arrive(full0 + 8 * (done % stages));
-                            ++done;
-                        }
+                        const uint32_t dst[2] = {smem0 + s * stage_bytes + place[0], smem0 + s * stage_bytes + place[1]};
+                        copy_rows<TPC>(tm, dst, int64_t(kb) * 128, src, size);
+                        cp_async_arrive(full0 + 8 * s);
                     }
+                    ok = __all_sync(0xffffffffu, ok);
                 }
             }
-            cp_async_wait(0);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            for (; done < it; ++done) mbar_arrive(full0 + 8 * (done % stages));
+            cp_async_wait_all();
         }
+        __syncwarp();
         // ---------------- epilogue: TMEM -> scaled FP32 local values of the tile's target cells
         bool any_src = false;
         for (int i = 0; i < 6; ++i) any_src |= s_active[i] != 0u;
         const bool ok = any_src ? mbar_wait(accb, 0, status) : true;
         asm volatile("tcgen05.fence::after_thread_sync;");
+        const int half = (warp - 2) / 4;  // two warps share a quadrant's rows: every second 16 columns
         const int q = warp % 4;
         const int trow = q * 32 + lane;  // TMEM lane = tile row
         float sc = float(double(n) / box->H) * float(double(n) / box->H);
@@ -530,7 +568,7 @@ __global__ void __launch_bounds__(192, 1)
             for (int mb = 0; mb < mbc; ++mb) {
                 const int nr = group * 256 + mb * 128 + trow;  // this thread's operator row
                 const bool rv = nr < P.nvalid;
-                for (int c0 = 0; c0 < 256; c0 += 16) {
+                for (int c0 = 16 * half; c0 < 256; c0 += 32) {
                     float v[16];
                     if (ok && any_src) tmem_ld16(tmem + (uint32_t(q * 32) << 16) + uint32_t(mb * 256 + c0), v);
                     for (int i = 0; i < 16; ++i) {
@@ -564,15 +602,17 @@ __global__ void __launch_bounds__(192, 1)
                     (2 * s_tgt[t][trow][0] + cx);
             float *dst = S + g * int64_t(P.nvalid);
             double *dst64 = S64 ? S64 + g * int64_t(P.nvalid) : nullptr;  // FP64 local values, when kept
-            if (ok && !any_src) {
+            bool any_t = false;
+            for (int i = 0; i < 6; ++i) any_t |= s_tact[t][i] != 0u;
+            if (ok && !any_t) {
                 // no occupied source among this launch's offsets: zero local values (or nothing to add)
                 if (valid && !P.accumulate)
-                    for (int col = group * P.ncta; col < min(P.nvalid, (group + 1) * P.ncta); ++col) {
+                    for (int col = group * P.ncta + half; col < min(P.nvalid, (group + 1) * P.ncta); col += 2) {
                         if (dst64) dst64[col] = 0.0;
                         else dst[col] = 0.f;
                     }
             } else if (ok) {
-                for (int c0 = 0; c0 < P.nsub; c0 += 16) {
+                for (int c0 = 16 * half; c0 < P.nsub; c0 += 32) {
                     float v[16];
                     tmem_ld16(tmem + (uint32_t(q * 32) << 16) + uint32_t(t * P.nsub + c0), v);
                     const int col = group * P.ncta + c0;
@@ -603,6 +643,7 @@ __global__ void __launch_bounds__(192, 1)
 constexpr int kFewTop = 4;     // deepest level taken together: 64 + 512 + 4,096 cells at most
 constexpr int kFewRows = 384;  // cells per CTA (three tiles of 128)
 constexpr int kFewSections = 64;
+constexpr int kFewSetsMax = (64 + 512 + 4096 + kFewRows - 1) / kFewRows;
 struct FewCount {
     int cells, sets, sections;
 };
@@ -610,6 +651,7 @@ struct FewParams {
     M2LParams P;
     short lo[316];  // residual operator of an offset, -1 without
     int groups;
+    const uint32_t *masks;  // [tile][10]: offsets with a source, by k_few_mask
 };
 __constant__ signed char c_o316[316][3];
 
@@ -621,25 +663,29 @@ __host__ __device__ inline int few_sections(int sets, int groups, int chunks, in
     return want < chunks ? chunks : (want > top ? top : want);
 }
 
-// cells of levels 2 .. top that hold targets, in level and linear order: x | y << 5 | z << 10 | level << 15
+// cells of levels 2 .. top that hold targets, in slot order (level, class, Morton code), so that the
+// 128 cells of a tile mostly share a class, whose list has 189 of the 316 offsets:
+// x | y << 5 | z << 10 | level << 15
 __global__ void __launch_bounds__(1024) k_few_list(int top, int groups, int chunks, int sms, const int *__restrict__ tocc,
                                                    int *__restrict__ list, FewCount *__restrict__ cnt) {
     __shared__ int s_warp[32], s_base;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_base = 0;
     __syncthreads();
-    const int n_all = int(cell_base_d(top + 1) - cell_base_d(2));
+    const int n_all = int(slot_base(top + 1));
     for (int i0 = 0; i0 < n_all; i0 += 1024) {
         const int i = i0 + threadIdx.x;
         int code = 0;
         bool on = false;
         if (i < n_all) {
-            const int64_t g = cell_base_d(2) + i;
             int l = 2;
-            while (l < top && g >= cell_base_d(l + 1)) ++l;
-            const int c = int(g - cell_base_d(l)), n = 1 << l;
-            on = tocc[g] > 0;
-            code = (c & (n - 1)) | (((c >> l) & (n - 1)) << 5) | ((c >> (2 * l)) << 10) | (l << 15);
+            while (l < top && i >= int(slot_base(l + 1))) ++l;
+            const int m3 = 1 << (3 * (l - 1)), k = i - int(slot_base(l)), cls = k / m3, n = 1 << l;
+            const uint32_t mc = uint32_t(k % m3);
+            const int x = 2 * int(morton_compact(mc)) + (cls & 1), y = 2 * int(morton_compact(mc >> 1)) + ((cls >> 1) & 1),
+                      z = 2 * int(morton_compact(mc >> 2)) + (cls >> 2);
+            on = tocc[cell_base_d(l) + (int64_t(z) * n + y) * n + x] > 0;
+            code = x | (y << 5) | (z << 10) | (l << 15);
         }
         const unsigned m = __ballot_sync(0xffffffffu, on);
         if (lane == 0) s_warp[w] = __popc(m);
@@ -657,10 +703,10 @@ __global__ void __launch_bounds__(1024) k_few_list(int top, int groups, int chun
     }
 }
 
-// byte offset of the packed multipole row of cell (x, y, z) of a level
-__device__ __forceinline__ int64_t packed_row(const M2LParams &P, int level, int x, int y, int z) {
+// table row of cell (x, y, z) of a level
+__device__ __forceinline__ int packed_row(const M2LParams &P, int level, int x, int y, int z) {
     const int m = 1 << (level - 1), cls = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
-    return P.wofs[level] + (((int64_t(cls) * m + z / 2) * m + y / 2) * m + x / 2) * P.row_bytes;
+    return P.wrow[level] + ((cls * m + z / 2) * m + y / 2) * m + x / 2;
 }
 
 // the source at cell - o when it lies in the cell's interaction list and holds segments
@@ -675,14 +721,37 @@ __device__ __forceinline__ bool few_source(int code, int ox, int oy, int oz, con
     return occ[cell_base_d(level) + (int64_t(z) * n + y) * n + x] > 0;
 }
 
+// offsets at which a tile of 128 listed cells has a source; one block per tile and 32 offsets
+__global__ void __launch_bounds__(512) k_few_mask(const FewCount *__restrict__ cnt, const int *__restrict__ list,
+                                                  const int *__restrict__ occ, uint32_t *__restrict__ masks) {
+    const int cells = cnt->cells, r0 = blockIdx.x * 128, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (r0 >= cells) return;
+    __shared__ uint32_t s_m;
+    if (threadIdx.x == 0) s_m = 0u;
+    __syncthreads();
+    for (int b = w; b < 32; b += 16) {
+        const int o = 32 * blockIdx.y + b;
+        bool hit = false;
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + 32 * q + lane;
+            int l, x, y, z;
+            if (o < 316 && r < cells) hit |= few_source(list[r], c_o316[o][0], c_o316[o][1], c_o316[o][2], occ, l, x, y, z);
+        }
+        if (__any_sync(0xffffffffu, hit) && lane == 0) atomicOr(&s_m, 1u << b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) masks[10 * blockIdx.x + blockIdx.y] = s_m;
+}
+
 // Item (section, operator group, cell set), the sets fastest: CTAs that run together read the same
 // operator rows.  Levels up to 4 go here whatever their cells: with few of them the operators' bytes
-// bound the time (6,011 segments, p = 6: 8.6 -> 1.2 ms; 157 segments, p = 4: 390 -> 60 us; 50,000
-// segments, L = 5, p = 5, free targets: 6.2 -> 2.8 ms), and a level 4 full of cells is 13 sets of 316
-// offsets against 16 tiles of 189, better spread (a million segments: whole pass 166.1 -> 163.6 ms).
-// Level 5 would be 86 sets against 96 tiles that already fill the GPU.  Roles, stages and barriers as in k_m2l_tc with the cells as A.
+// bound the time (6,011 segments, p = 6: 8.6 ms per class, 0.8 here; 157 segments, p = 4: 390 and 16
+// us; 50,000 segments, L = 5, p = 5, free targets: 6.2 and 1.7 ms), and a level 4 full of cells is 13
+// sets, better spread than 16 tiles (a million segments: whole pass 166.1 and 163.6 ms).  Level 5
+// would be 86 sets against 96 tiles that already fill the GPU.  Tiles of one class skip the offsets
+// of the others' lists (27 % of the gathered rows had a source without that).
 template <bool TF32>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
     k_m2l_few(const __grid_constant__ FewParams F, const FewCount *__restrict__ cnt, const int *__restrict__ list,
               const int *__restrict__ occ, float *__restrict__ part, int Np, int *__restrict__ status, int stages) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -693,31 +762,45 @@ __global__ void __launch_bounds__(192, 1)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + stages * stage_bytes);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * stages + 1);
     __shared__ int s_code[kFewRows];
-    __shared__ uint32_t s_active[10];
+    __shared__ short s_off[316];  // the section's offsets in order, with the tiles that have a source: o | tiles << 9
+    __shared__ int s_noff;
     __shared__ int s_stop;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int sets = cnt->sets, sections = cnt->sections, cells = cnt->cells;
     if (threadIdx.x == 0) s_stop = *reinterpret_cast<volatile int *>(status) != 0;
-    if (threadIdx.x < 10) s_active[threadIdx.x] = 0u;
     __syncthreads();
     if (int(blockIdx.x) >= sets * F.groups * sections || s_stop) return;  // surplus block, or an earlier time-out
     const int set = blockIdx.x % sets, group = (blockIdx.x / sets) % F.groups, sec = blockIdx.x / (sets * F.groups);
     const int nrow = min(kFewRows, cells - set * kFewRows), tiles = (nrow + 127) / 128;
-    const int o_lo = 316 * sec / sections, o_hi = 316 * (sec + 1) / sections;
-    for (int r = threadIdx.x; r < kFewRows; r += 192) s_code[r] = r < nrow ? list[set * kFewRows + r] : -1;
+    for (int r = threadIdx.x; r < kFewRows; r += kTcThreads) s_code[r] = r < nrow ? list[set * kFewRows + r] : -1;
     __syncthreads();
-    for (int o = o_lo + warp; o < o_hi; o += 6) {
-        const int ox = c_o316[o][0], oy = c_o316[o][1], oz = c_o316[o][2];
-        bool hit = false;
-        for (int r = lane; r < nrow && !hit; r += 32) {
-            int l, x, y, z;
-            hit = few_source(s_code[r], ox, oy, oz, occ, l, x, y, z);
+    if (warp == 0) {
+        // the set's offsets (any tile's) are cut into sections of equal length; word w of lane w
+        uint32_t own[TPC] = {0u, 0u, 0u}, u = 0u;
+        if (lane < 10)
+            for (int t = 0; t < TPC; ++t) {
+                if (t < tiles) own[t] = F.masks[10 * (TPC * set + t) + lane];
+                u |= own[t];
+            }
+        int rank = __popc(u);
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, rank, d);
+            if (lane >= d) rank += v;
         }
-        if (__any_sync(0xffffffffu, hit) && lane == 0) atomicOr(&s_active[o / 32], 1u << (o % 32));
+        const int total = __shfl_sync(0xffffffffu, rank, 31), lo = total * sec / sections,
+                  hi = total * (sec + 1) / sections;
+        rank -= __popc(u) + lo;
+        for (uint32_t b = u; b; b &= b - 1, ++rank)
+            if (rank >= 0 && rank < hi - lo) {
+                const int k = __ffs(b) - 1;
+                s_off[rank] = short((32 * lane + k) | (((own[0] >> k) & 1u) << 9) | (((own[1] >> k) & 1u) << 10) |
+                                    (((own[2] >> k) & 1u) << 11));
+            }
+        if (lane == 0) s_noff = hi - lo;
     }
     if (threadIdx.x == 0) {
-        // full: the operator-load thread (expect_tx) + 128 gathering threads; empty: the MMA commit
-        for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&bars[s]), 129);
+        // full: the operator-load thread (expect_tx) + 256 gathering threads; empty: the MMA commit
+        for (int s = 0; s < stages; ++s) mbar_init(smem_u32(&bars[s]), 257);
         for (int s = stages; s < 2 * stages + 1; ++s) mbar_init(smem_u32(&bars[s]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -733,144 +816,120 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t tmem = *tmem_slot;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[stages]), accb = smem_u32(&bars[2 * stages]);
     const uint32_t smem0 = smem_u32(smem);
-    auto active = [&](int o) { return (s_active[o / 32] >> (o % 32)) & 1u; };
-    uint32_t o_act = 0u;  // offsets of this section with a source
-    for (int i = 0; i < 10; ++i) o_act |= s_active[i];
+    const int noff = s_noff;
 
     if (warp == 0 && lane == 0) {
         // ---------------- operator rows (B) by TMA
-        int it = 0;
-        bool ok = true;
-        for (int o = o_lo; o < o_hi && ok; ++o) {
-            if (!active(o)) continue;
+        Ring rg;
+        bool ok = true, drop = P.drop_first != 0;
+        for (int oi = 0; oi < noff && ok; ++oi) {
+            const int o = s_off[oi] & 511;
             const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
             for (int pass = 0; pass < np && ok; ++pass) {
                 const CUtensorMap *tb = pass == 2 ? &P.tmTlo : &P.tmT;
                 const int tidx = pass == 2 ? F.lo[o] : o;
-                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                    const int s = it % stages;
-                    if (!mbar_wait(empty0 + 8 * s, ((it / stages) & 1) ^ 1, status)) {
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                    const int s = rg.s;
+                    if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
                         ok = false;
                         break;
                     }
                     mbar_expect_tx(full0 + 8 * s, uint32_t(stageB));
-                    if (P.drop_first && it == 0) continue;  // the MMA warp's wait on this stage runs out
+                    if (drop) {  // the MMA warp's wait on this stage runs out
+                        drop = false;
+                        continue;
+                    }
                     tma_load_3d(smem0 + s * stage_bytes + kStageA, tb, kb * P.kstep, group * P.ncta, tidx, full0 + 8 * s);
                 }
             }
         }
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        int it = 0;
+        Ring rg;
+        uint32_t begun = 0u;
         bool ok = true;
-        for (int o = o_lo; o < o_hi && ok; ++o) {
-            if (!active(o)) continue;
+        for (int oi = 0; oi < noff && ok; ++oi) {
+            const int o = s_off[oi] & 511;
+            const uint32_t tm = uint32_t(s_off[oi]) >> 9;
             const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
             for (int pass = 0; pass < np && ok; ++pass)
-                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                    const int s = it % stages;
-                    if (!mbar_wait(full0 + 8 * s, (it / stages) & 1, status)) {
+                for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                    const int s = rg.s;
+                    if (!mbar_wait(full0 + 8 * s, rg.ph, status)) {
                         ok = false;
                         break;
                     }
+                    // the gathered rows were written through the generic proxy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     const uint32_t a = smem0 + s * stage_bytes;
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const uint64_t bd = sw128_desc(a + kStageA + kk * 32);
-                        for (int t = 0; t < tiles; ++t)
-                            mma_issue<TF32>(tmem + t * P.nsub, sw128_desc(a + t * kTileA + kk * 32), bd, P.idesc,
-                                            (it > 0 || kk > 0) ? 1u : 0u);
-                    }
+                    mma_tiles<TF32, TPC>(tmem, P.nsub, a, a + kStageA, P.idesc, tm, begun);
+                    begun |= tm;
                     mma_commit(empty0 + 8 * s);
                 }
         }
         // fires when every MMA issued above has completed
-        if (o_act) mma_commit(accb);
+        if (noff > 0) mma_commit(accb);
     } else if (warp >= 2) {
-        const int row = threadIdx.x - 64;
-        const bool any = o_act != 0u;
+        const bool any = noff > 0;
+        const int wrow0 = 16 * (warp - 2);
+        const uint32_t place[2] = {uint32_t((wrow0 + (lane >> 3)) * 128 + (((lane & 7) ^ (lane >> 3)) << 4)),
+                                   uint32_t((wrow0 + (lane >> 3)) * 128 + (((lane & 7) ^ (4 + (lane >> 3))) << 4))};
         {
-            // ---------------- multipole rows (A), as in k_m2l_tc: each thread finds the source of its
-            // own rows, the copies go by 8 lanes per 128-byte row piece
-            const int lag = 1;
-            int it = 0, done = 0;
+            // ---------------- multipole rows (A), as in k_m2l_tc
+            Ring rg;
             bool ok = true;
-            const int c = lane & 7, wrow0 = row - lane;
-            for (int o = o_lo; o < o_hi && ok; ++o) {
-                if (!active(o)) continue;
+            for (int oi = 0; oi < noff && ok; ++oi) {
+                const int o = s_off[oi] & 511;
+                const uint32_t tm = uint32_t(s_off[oi]) >> 9;
                 const int ox = c_o316[o][0], oy = c_o316[o][1], oz = c_o316[o][2];
-                int64_t own[TPC];
-                uint32_t own_nb = 0;  // bits t: a source; 4 + t: one whose level has the residual passes
+                int own[2] = {-1, -1}, res[2] = {-1, -1};  // res: in levels with residual passes
 #pragma unroll
-                for (int t = 0; t < TPC; ++t) {
-                    own[t] = 0;
-                    const int code = s_code[t * 128 + row];
+                for (int k = 0; k < 2; ++k) {
+                    const int t = 2 * k + lane / 16;
+                    const int code = t < TPC ? s_code[t * 128 + wrow0 + lane % 16] : -1;
                     int l, x, y, z;
                     if (code >= 0 && few_source(code, ox, oy, oz, occ, l, x, y, z)) {
-                        own[t] = packed_row(P, l, x, y, z);
-                        own_nb |= (1u << t) | (((P.split_levels >> l) & 1) ? 16u << t : 0u);
+                        own[k] = packed_row(P, l, x, y, z);
+                        if ((P.split_levels >> l) & 1) res[k] = own[k];
                     }
                 }
-                int64_t srcoff[8][TPC];
-                uint32_t nbm = 0, nbr = 0;  // bit 8 t + i: row 4 i + lane / 8 of tile t has a source
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int from = 4 * i + (lane >> 3);
-                    const uint32_t f = __shfl_sync(0xffffffffu, own_nb, from);
-#pragma unroll
-                    for (int t = 0; t < TPC; ++t) {
-                        srcoff[i][t] = __shfl_sync(0xffffffffu, own[t], from);
-                        nbm |= ((f >> t) & 1u) << (8 * t + i);
-                        nbr |= ((f >> (4 + t)) & 1u) << (8 * t + i);
-                    }
-                }
+                __syncwarp();
                 const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
                 for (int pass = 0; pass < np && ok; ++pass) {
-                    const uint8_t *wb = pass == 1 ? P.Wlo : P.Whi;
-                    const uint32_t have = pass == 0 ? nbm : nbr;
-                    for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, ++it) {
-                        const int s = it % stages;
-                        if (!mbar_wait(empty0 + 8 * s, ((it / stages) & 1) ^ 1, status)) {
+                    const uint8_t *src[TPC][4];
+                    uint32_t size[TPC][4];
+                    take_rows<TPC>(pass == 0 ? own : res, lane, pass == 1 ? P.Wlo : P.Whi, P.row_bytes, src, size);
+                    for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
+                        const int s = rg.s;
+                        if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
                             ok = false;
                             break;
                         }
-                        const uint32_t sbase = smem0 + s * stage_bytes;
-                        const uint8_t *wk = wb + kb * 128 + 16 * c;
-#pragma unroll
-                        for (int t = 0; t < TPC; ++t)
-                            if (t < tiles)
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const int r = wrow0 + 4 * i + (lane >> 3);
-                                    const bool on = (have >> (8 * t + i)) & 1u;
-                                    cp_async16(sbase + t * kTileA + r * 128 + ((c ^ (r & 7)) << 4),
-                                               on ? wk + srcoff[i][t] : wk, on ? 16u : 0u);
-                                }
-                        cp_async_commit();
-                        if (it - done >= lag) {
-                            cp_async_wait(lag);
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            mbar_arrive(full0 + 8 * (done % stages));
-                            ++done;
-                        }
+                        const uint32_t dst[2] = {smem0 + s * stage_bytes + place[0], smem0 + s * stage_bytes + place[1]};
+                        copy_rows<TPC>(tm, dst, int64_t(kb) * 128, src, size);
+                        cp_async_arrive(full0 + 8 * s);
                     }
+                    ok = __all_sync(0xffffffffu, ok);
                 }
             }
-            cp_async_wait(0);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            for (; done < it; ++done) mbar_arrive(full0 + 8 * (done % stages));
+            cp_async_wait_all();
         }
+        __syncwarp();
         // ---------------- epilogue: TMEM -> this section's sums
+        uint32_t t_act = 0u;  // tiles with a source in this section
+        for (int oi = 0; oi < noff; ++oi) t_act |= uint32_t(s_off[oi]) >> 9;
         const bool ok = any ? mbar_wait(accb, 0, status) : true;
         asm volatile("tcgen05.fence::after_thread_sync;");
+        const int half = (warp - 2) / 4;  // two warps share a quadrant's rows: every second 16 columns
         const int q = warp % 4, trow = q * 32 + lane;
         for (int t = 0; t < tiles; ++t) {
             const int r = t * 128 + trow;
             float *dst = part + ((int64_t(sec) * sets + set) * kFewRows + r) * Np + group * P.ncta;
-            for (int c0 = 0; c0 < P.nsub; c0 += 16) {
+            for (int c0 = 16 * half; c0 < P.nsub; c0 += 32) {
                 float v[16];
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
-                if (ok && any) tmem_ld16(tmem + (uint32_t(q * 32) << 16) + uint32_t(t * P.nsub + c0), v);
+                if (ok && ((t_act >> t) & 1u)) tmem_ld16(tmem + (uint32_t(q * 32) << 16) + uint32_t(t * P.nsub + c0), v);
                 if (ok && r < nrow)
                     for (int i = 0; i < 4; ++i)
                         reinterpret_cast<float4 *>(dst + c0)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2],
@@ -1523,7 +1582,8 @@ int m2l_tc_prepare(gbfmm_ctx *ctx) {
                               {{(void **)&T.few_part, size_t(rows) * T.Np * sizeof(float)}}, "M2L sections"))
             return rc;
         if (!T.few_list)
-            CK(cudaMalloc(&T.few_list, (cell_base(kFewTop + 1) - cell_base(2)) * sizeof(int) + sizeof(FewCount) + 16));
+            CK(cudaMalloc(&T.few_list, 16 + (cell_base(kFewTop + 1) - cell_base(2)) * sizeof(int) +
+                                           (kFewSetsMax * 3 * 10) * sizeof(uint32_t)));
     }
     // cell slots, target list and segment table (filled on the device per pass)
     const int64_t slots = slot_base(L);
@@ -1562,7 +1622,7 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
     pk.split_levels = T.split ? split_levels : 0;
     for (int l = 2; l < L; ++l) {
         pk.ofs[l] = T.wofs[l];
-        prm.wofs[l] = T.wofs[l] * T.esz;
+        prm.wrow[l] = int(T.wofs[l] / T.Kp);
     }
     // blocks stride over the cells of a level, one row of blocks per level
     const dim3 gw(unsigned(std::min<int64_t>(int64_t(1) << (3 * (L - 1)), 8 * 152)), unsigned(L - 2));
@@ -1660,9 +1720,12 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
         if (int rc = fit((const void *)kern)) return rc;
         FewCount *cnt = reinterpret_cast<FewCount *>(T.few_list);
         int *list = reinterpret_cast<int *>(T.few_list) + 4;
-        ctx->launches += 3;
+        fp.masks = reinterpret_cast<const uint32_t *>(list + (cell_base(kFewTop + 1) - cell_base(2)));
+        ctx->launches += 4;
         k_few_list<<<1, 1024, 0, st>>>(few, T.groups, std::max(1, ctx->opt.m2l_chunks), ctx->sm_count, tocc, list, cnt);
-        kern<<<T.few_work, 192, smem, st>>>(fp, cnt, list, occ, T.few_part, T.Np, T.d_status, stages);
+        k_few_mask<<<dim3(unsigned((cell_base(few + 1) - cell_base(2) + 127) / 128), 10), 512, 0, st>>>(
+            cnt, list, occ, const_cast<uint32_t *>(fp.masks));
+        kern<<<T.few_work, kTcThreads, smem, st>>>(fp, cnt, list, occ, T.few_part, T.Np, T.d_status, stages);
         k_few_sum<<<unsigned(cell_base(few + 1) - cell_base(2)), 256, 0, st>>>(
             cnt, list, T.few_part, T.Np, prm.nvalid, prm.wmax, prm.inv_op_scale, ctx->d_box, Sout, S64);
         CK(cudaGetLastError());
@@ -1691,7 +1754,7 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
             prm.accumulate = c > 0 ? 1 : 0;
             if (c > 0) prm.drop_first = 0;
             ++ctx->launches;
-            kern<<<T.n_work, 192, smem, st>>>(prm, T.d_seg, 8 * (L - 2), T.d_list, occ, tocc, ctx->d_box, Sout, S64,
+            kern<<<T.n_work, kTcThreads, smem, st>>>(prm, T.d_seg, 8 * (L - 2), T.d_list, occ, tocc, ctx->d_box, Sout, S64,
                                               T.d_status, stages, T.groups);
             CK(cudaGetLastError());
         }

@@ -91,14 +91,37 @@ def near_flops(wl, work):
     return work["near_pairs"] * near_pair_flops("mixed", wl["h_mode"], q, cubic) + l2p, name
 
 
-# DRAM bytes per target point of one k_near_sym launch (cubic rule, Q = 16), from
+def near_work(wl, work):
+    """FLOP that the pair kernel (k_near_pairs) executes for the near field (+ L2P)
+    of one pass, a multiply-add as two.  Nodal forces evaluate a pair once for
+    both directions.  Unit-circle rule: 37 multiply-adds and two reciprocals per
+    pair of circle points (phi, -phi) beside about 430 (cubic medium) or 850 (any
+    other in FP64) a pair, or 93 per circle point beside 300 (any other in FP32);
+    isotropic: 43 a direction beside 30; learned: 108 from the bin's polynomial
+    beside 220.  ``near_flops`` counts the same pairs by the pointwise rule."""
+    p, q, pairs = wl["p"], wl.get("circle_q", 64), work["near_pairs"] / 2.0
+    l2p = work["points"] * (12 * p ** 3 + 30 * p)
+    if wl["h_mode"] == "iso":
+        return pairs * 2 * (2 * 43 + 30) + l2p, "k_near_pairs"
+    if wl["h_mode"] == "mlp":
+        return pairs * 2 * (108 + 220) + l2p, "k_near_pairs"
+    if is_cubic_aligned(wl["C"]()):
+        per = 39 * ((q - 1) // 2) + 430
+    elif wl["precision"] == "fp64":
+        per = 39 * ((q - 1) // 2) + 850
+    else:
+        per = 93 * q + 300
+    return pairs * 2 * per + l2p, "k_near_pairs"
+
+
+# DRAM bytes per target point of one near-field launch (k_near_pairs, cubic rule, Q = 16), from
 # one ncu capture on the 250,000-segment slab network (dram__bytes_read.sum +
-# dram__bytes_write.sum = 6.494 + 1.347 GB for 1,000,000 points); valid for the
+# dram__bytes_write.sum = 0.161 + 0.760 GB for 1,000,000 points); valid for the
 # kernel version the capture was taken of
-NEAR_SYM_DRAM_BYTES_PER_POINT = (6.493849e9 + 1.346746e9) / 1.0e6
+NEAR_SYM_DRAM_BYTES_PER_POINT = (1.60587e8 + 7.60081e8) / 1.0e6
 # the same two counters for the headline's launch itself (1M segments, adaptive tree at
 # threshold 128; a one-pass capture of the full-size run)
-NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES = 21815144704 + 4425026816
+NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES = 1112050432 + 3203101952
 
 
 def measured_alu_peaks():
@@ -447,7 +470,7 @@ def run_batch(args, wl):
     work = f.work_counts()
     p = wl["p"]
     if st[4] >= st[2]:
-        flops, kname = near_flops(wl, work)
+        flops, kname = near_work(wl, work)
         pk = measured_alu_peaks()
         roof = {"bound": "alu", "kernel": kname + " (largest network alone)", "achieved": flops / (st[4] / 1e3) / 1e12,
                 "peak": pk["fp32_tflops"], "unit": "TFLOP/s", "peak_source": pk["source"]}
@@ -676,14 +699,15 @@ def roofline_of(wl, work, m2l_ms, leaf_ms, m2l_fft, peaks, ranks=None):
     alu_peak = peaks["fp64_tflops"] if fp64 else peaks["fp32_tflops"]
     traffic, traffic_src = None, None
     if leaf_ms >= m2l_ms:
-        flops, kname = near_flops(wl, work)
+        flops, kname = near_work(wl, work)
         achieved = flops / (leaf_ms / 1e3) / 1e12
+        nodal = near_flops(wl, work)[1] == "k_near_sym"  # the passes the captures below describe
         dom, bound, peak, src = kname + " (L2P + near-field P2P)", "alu", alu_peak, peaks["source"]
-        if kname == "k_near_sym" and wl.get("circle_q") == 16 and not wl.get("refine_points"):
+        if nodal and wl.get("circle_q") == 16 and not wl.get("refine_points"):
             traffic = NEAR_SYM_DRAM_BYTES_PER_POINT * work["points"]
-            traffic_src = ("dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of k_near_sym on the "
+            traffic_src = ("dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of k_near_pairs on the "
                            "250k-segment slab network, scaled by points")
-        elif (kname == "k_near_sym" and wl.get("refine_points") == 128 and work["points"] == 4_000_000
+        elif (nodal and wl.get("refine_points") == 128 and work["points"] == 4_000_000
               and NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES):
             traffic = NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES
             traffic_src = ("dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of this launch "
@@ -707,8 +731,8 @@ def roofline_of(wl, work, m2l_ms, leaf_ms, m2l_fft, peaks, ranks=None):
             peak, src = measured_bf16_peak()
     return {"bound": bound, "kernel": dom, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic, "traffic_source": traffic_src, "peak_source": src,
-            "work": "algorithmic: near pairs x FLOP/pair (h once per unordered pair when h is the unit-circle "
-                    "rule) + L2P, or M2L cell pairs x 2*54*p^6 (x 8*54*(2p)^2*(p+1) through transforms, "
+            "work": "near pairs x FLOP/pair as the pair kernel evaluates them (once per unordered pair, circle "
+                    "moments) + L2P, or M2L cell pairs x 2*54*p^6 (x 8*54*(2p)^2*(p+1) through transforms, "
                     "x 2*r1*r2 compressed)"}
 
 

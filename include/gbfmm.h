@@ -80,8 +80,9 @@ typedef struct {
     int h_mode;            /* GBFMM_H_ISO, GBFMM_H_CIRCLE or GBFMM_H_MLP */
     int circle_q;          /* trapezoid points on the half circle for GBFMM_H_CIRCLE; 0 = 64 */
     int leaf_segments;     /* with levels == 0: target mean segments per occupied leaf; 0 = 32 */
-    double near_fp64;      /* MIXED: near pairs closer than near_fp64 x (source segment length)
-                              are evaluated in FP64; 0 = 2.0 */
+    double near_fp64;      /* MIXED: with GBFMM_H_MLP, near pairs closer than near_fp64 x (the longer
+                              segment's length) take the plain rule whatever mlp_min_dist is;
+                              0 = 2.0.  Every near pair's separation and sums carry two floats. */
     int m2l_split;         /* MIXED: operand precision of the tensor-core M2L, GBFMM_M2L_*:
                               0 = BF16 with residual (split) passes on the offsets with
                               max |o_i| = 2, 1 = BF16 only, 2 = BF16 with residual passes on
@@ -91,8 +92,9 @@ typedef struct {
                               operators, 5 = as 4 plus residual passes
                               on the offsets with max |o_i| = 2, 6 = as 4 plus residual
                               passes on all 316 offsets (fmm_default_options) */
-    double mlp_min_dist;   /* GBFMM_H_MLP: near pairs closer than this many source segment
-                              lengths use the plain evaluator; 0 = 8 */
+    double mlp_min_dist;   /* GBFMM_H_MLP: near pairs closer than this many lengths of the longer
+                              segment use the plain evaluator; 0 = 8.  The others take the
+                              network's values as one quadratic per angular bin. */
     int m2l_fft;           /* FP64: 1 = M2L through the Toeplitz structure of the operators
                               (Sec. 4.1, Theorem 1): each offset's node-to-node map applied as
                               a convolution, by products of discrete Fourier transforms of size

@@ -17,9 +17,9 @@
 // matrix and forming F at every point; points phi and -phi share the even and odd
 // parts of every polynomial, so a pair of points costs 37 multiply-adds and two
 // reciprocals (the pointwise form: 114 and one reciprocal for each point).  The
-// coefficients before the loop and the 18 components after it cost about 500
-// multiply-adds in a cubic medium with axes along x, y, z and 850 in any other,
-// whatever Q is.  The sums run over the same points as the pointwise form, so the
+// coefficients before the loop and the rows of stress and two strains after it cost
+// about 430 multiply-adds in a cubic medium with axes along x, y, z and 850 in any
+// other, whatever Q is.  The sums run over the same points as the pointwise form, so the
 // two agree to rounding (FP64: 1e-15; FP32, chain from the separation to h / R^2
 // against FP64, C11 = 1.684, C12 = 1.214, C44 = 0.754: 1.6e-7 RMS here, 2.2e-7
 // pointwise with an unrefined reciprocal square root).

@@ -656,7 +656,8 @@ struct FewParams {
 __constant__ signed char c_o316[316][3];
 
 // sections of the offset list for a number of cell sets: about four CTAs per SM, no fewer than
-// m2l_chunks (each section is one accumulation in tensor memory)
+// m2l_chunks (each section is one accumulation in tensor memory).  M2L stage with two / three / four /
+// six per SM: 6,011 segments 0.95 / 0.93 / 0.96 / 0.99 ms, 50,000 segments 1.44 / 1.37 / 1.33 / 1.33
 __host__ __device__ inline int few_sections(int sets, int groups, int chunks, int sms) {
     const int want = (4 * sms + sets * groups - 1) / (sets * groups);
     const int top = chunks > kFewSections ? chunks : kFewSections;

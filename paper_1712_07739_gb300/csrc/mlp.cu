@@ -107,13 +107,16 @@ __global__ void __launch_bounds__(32 * kEvalWarps, 2)
 // in registers (the transposed products read the same weights by transposing loads) and leaves
 // what the weight gradients read: inputs x, activations a1 .. a3 and the gradients of the
 // pre-activations g1 .. g3, go, in BF16 rows, g1 also in FP32.  The pre-activations go through
-// memory in the lane's own order.  loss = mean_{b,c} (o - s y / scale)^2, one partial per tile.
+// memory in the lane's own order.  loss = mean_{b,c} (o - s y / scale)^2, one partial per tile: the
+// FP32 terms are summed in FP64 (13 additions a lane and tile), so the loss is theirs to its own
+// FP32 rounding in whatever order the tiles run (sums of 8,192 samples in FP32: up to 2e-6 off).
 // Two warps a block: a batch of 8,192 is 512 tiles, about three warps for every SM, whose serial
 // chain is the time.  The whole gradient of 8,192 samples: 78 us, 1,926 us as 22 kernels with the
 // activations in memory (this one 32 us, k_mlp_wgrad 15, k_grad_sum 8).
 constexpr int kTrainWarps = 2;
 struct TrainArgs {
-    float *x, *z, *g32, *lossp;  // [n][3], [tile][3][16][32][4], [n][128], [tiles]
+    float *x, *z, *g32;          // [n][3], [tile][3][16][32][4], [n][128]
+    double *lossp;               // [tiles]
     bf16 *a[3], *g[3], *go;      // [n][128] each (g[0] = g1), [n][32]
 };
 __device__ __forceinline__ void store_rows(bf16 *__restrict__ dst, int ld, const uint32_t (*a)[4], int KT, int64_t r0,
@@ -168,7 +171,7 @@ __global__ void __launch_bounds__(32 * kTrainWarps)
         float o[4][4];
         mlpw::layer<4, 8, false>(w.W4, a, o, lane);
         mlpw::add_bias<4>(w.b4, o, t);
-        float loss = 0.f;
+        double loss = 0.0;
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
@@ -179,7 +182,7 @@ __global__ void __launch_bounds__(32 * kTrainWarps)
                 if (c < 27 && b < n) {
                     const float r = o[nt][j] - s[j >> 1] * y[b * 27 + c] / w.scale[c];
                     gv = 2.f * r / (float(n) * 27.f);
-                    loss += r * r / (float(n) * 27.f);
+                    loss += double(r * r / (float(n) * 27.f));
                 }
                 o[nt][j] = gv;
             }
@@ -297,11 +300,11 @@ __global__ void __launch_bounds__(256)
 
 // gradient = the runs' sums in order; the last block adds the tiles' losses
 __global__ void __launch_bounds__(256) k_grad_sum(int runs, const float *__restrict__ part, float *__restrict__ grad,
-                                                  int64_t tiles, const float *__restrict__ lossp,
+                                                  int64_t tiles, const double *__restrict__ lossp,
                                                   float *__restrict__ loss) {
     if (blockIdx.x == gridDim.x - 1) {
-        __shared__ float sm[256];
-        float s = 0.f;
+        __shared__ double sm[256];
+        double s = 0.0;
         for (int64_t i = threadIdx.x; i < tiles; i += 256) s += lossp[i];
         sm[threadIdx.x] = s;
         __syncthreads();
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(256) k_grad_sum(int runs, const float *__restr
             if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
             __syncthreads();
         }
-        if (threadIdx.x == 0) *loss = sm[0];
+        if (threadIdx.x == 0) *loss = float(sm[0]);
         return;
     }
     const int i = blockIdx.x * 256 + threadIdx.x;
@@ -433,7 +436,7 @@ static int mlp_alloc_batch(gbfmm_ctx *ctx, int n) {
     const size_t m = (size_t(n) + 15) / 16 * 16;
     return grow_dev(ctx, B.cap, int64_t(m),
                     {{(void **)&T.x, m * 3 * sizeof(float)}, {(void **)&T.z, m * 384 * sizeof(float)},
-                     {(void **)&T.g32, m * 128 * sizeof(float)}, {(void **)&T.lossp, m / 16 * sizeof(float)},
+                     {(void **)&T.g32, m * 128 * sizeof(float)}, {(void **)&T.lossp, m / 16 * sizeof(double)},
                      {(void **)&T.a[0], m * 128 * sizeof(bf16)}, {(void **)&T.a[1], m * 128 * sizeof(bf16)},
                      {(void **)&T.a[2], m * 128 * sizeof(bf16)}, {(void **)&T.g[0], m * 128 * sizeof(bf16)},
                      {(void **)&T.g[1], m * 128 * sizeof(bf16)}, {(void **)&T.g[2], m * 128 * sizeof(bf16)},

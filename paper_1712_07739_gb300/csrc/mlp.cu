@@ -382,12 +382,12 @@ __global__ void k_gather_rows(int n, int w, const int *__restrict__ idx, const f
 // The network as polynomials for the near field: per angular bin the least-squares quadratic in
 // the bin's coordinates (u, v) through the network's values at 8 x 8 directions, on the basis
 // 1, u, v, u^2 - m2, uv, v^2 - m2, which is orthogonal on that grid (m2 = mean of u^2); the 18
-// components symmetric in (v, p), times fac.  One block per bin, a thread per coefficient.  A
+// components symmetric in (v, p).  One block per bin, a thread per coefficient.  A
 // pair of the near field then costs 108 multiply-adds instead of 37,000 (a bin is 1/16 of a face
 // wide: the quadratic follows the network's values within its own BF16 noise).
 constexpr int kBinGrid = 8;
 __host__ __device__ inline float grid_coord(int i) { return float(2 * i + 1 - kBinGrid) / float(kBinGrid); }
-__global__ void k_bin_poly(const float *__restrict__ h, float m2, float fac, float *__restrict__ poly) {
+__global__ void k_bin_poly(const float *__restrict__ h, float m2, float *__restrict__ poly) {
     constexpr int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
     const int t = threadIdx.x;
     if (t >= 108) return;
@@ -400,7 +400,7 @@ __global__ void k_bin_poly(const float *__restrict__ h, float m2, float fac, flo
         num += phi * 0.5f * (hb[27 * i + (v * 3 + p) * 3 + q] + hb[27 * i + (p * 3 + v) * 3 + q]);
         den += phi * phi;
     }
-    poly[108 * blockIdx.x + t] = fac * num / den;
+    poly[108 * blockIdx.x + t] = num / den;
 }
 
 }  // namespace
@@ -665,8 +665,8 @@ float mlp_poly_m2() {
     return s / float(kBinGrid);
 }
 
-// The near field's polynomials of the current network (h times 4 pi Q: the pair kernel's
-// Burgers vectors carry the inverse).  Rebuilt after the network changed; synchronises then.
+// The near field's polynomials of the current network.  Rebuilt after the network changed;
+// synchronises then.
 int mlp_tabulate(gbfmm_ctx *ctx) {
     MlpState &M = ctx->mlp;
     if (M.poly_ok && M.poly) return GBFMM_OK;
@@ -683,7 +683,7 @@ int mlp_tabulate(gbfmm_ctx *ctx) {
         CK(cudaMemcpyAsync(dd, dirs.data(), n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
         if (int r = mlp_eval_device(ctx, n, dd, h)) return r;
         ++ctx->launches;
-        k_bin_poly<<<kBins, 128, 0, ctx->stream>>>(h, mlp_poly_m2(), float(4.0 * M_PI * ctx->mat.Q), M.poly);
+        k_bin_poly<<<kBins, 128, 0, ctx->stream>>>(h, mlp_poly_m2(), M.poly);
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(ctx->stream));
         return GBFMM_OK;

@@ -448,6 +448,7 @@ struct NearLearned {
     const uint32_t *binmask;  // bit set: the bin takes the plain rule
     const float4 *poly;       // [bin][27]: 18 components x 6 coefficients (mlp.cu)
     float rmin2, m2;
+    float fac;                // 4 pi Q times the kernel's unit of the moduli: what the pairs' Burgers vectors leave out
 };
 
 struct NearTree {
@@ -509,11 +510,11 @@ __device__ __forceinline__ float dir_bin(const float d[3], int &bin, float &u, f
     return sg;
 }
 
-// h of one pair by the network's polynomial in its bin
+// h of one pair by the network's polynomial in its bin, in the pair kernel's unit
 __device__ __forceinline__ void h_learned(const NearLearned &ln, const float d[3], float hs[18]) {
     int bin;
     float u, v;
-    const float sg = dir_bin(d, bin, u, v);
+    const float sg = ln.fac * dir_bin(d, bin, u, v);
     const float b1 = u, b2 = v, b3 = u * u - ln.m2, b4 = u * v, b5 = v * v - ln.m2;
     const float4 *q = ln.poly + 27 * bin;
 #pragma unroll
@@ -972,15 +973,34 @@ static bool near_learned(const gbfmm_ctx *ctx) {
     return ctx->mat.mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64;
 }
 
+// The pair kernel's unit of the moduli: the power of two at their largest entry.  Its rules form
+// det(zz)^-2, the sixth power of a modulus, and FP32 holds that for moduli from 4e-7 to 2e6 only
+// (with moduli in Pa every term with it vanishes and h is finite and wrong); in this unit the moduli
+// are of order one whatever the caller's, and no rounding changes.
+static double near_unit(const DevMaterial &m) {
+    double v = 0.0;
+    for (int i = 0; i < 6; ++i) v = std::max(v, m.V[7 * i]);
+    return std::ldexp(1.0, std::ilogb(v));
+}
+
+// Burgers vectors carry the factor of h that its sums leave out: 1 / (4 pi Q) of the unit-circle
+// rule, the isotropic rule's factor (an inverse modulus, in the kernel's unit)
+static double near_factor(const DevMaterial &m) {
+    return m.mode == GBFMM_H_ISO ? m.hc * near_unit(m) : 1.0 / (4.0 * M_PI * m.Q);
+}
+
+// constants of a medium in the kernel's unit; the strain of a pair has none, so nothing is scaled
+// back but the network's h, whose unit is the caller's (NearLearned)
 template <typename R>
 static NearMedium<R> near_medium(const DevMaterial &m) {
     NearMedium<R> n{};
     n.Q = m.Q;
     n.np = (m.Q - 1) / 2;
-    const double cp = m.c12 + m.c44, D = m.cd, c44 = m.c44, ydiag = D + 2.0 * c44;
-    n.k1 = R(m.V[1] * (1.0 - m.ha) + 2.0 * m.V[21]);
-    n.k3 = R(m.V[21] * (1.0 - m.ha));
-    n.k6 = R(6.0 * m.V[21]);
+    const double iu = 1.0 / near_unit(m), c12 = iu * m.c12, c44 = iu * m.c44, D = iu * m.cd;
+    const double cp = c12 + c44, ydiag = D + 2.0 * c44;
+    n.k1 = R(iu * (m.V[1] * (1.0 - m.ha) + 2.0 * m.V[21]));
+    n.k3 = R(iu * m.V[21] * (1.0 - m.ha));
+    n.k6 = R(iu * 6.0 * m.V[21]);
     // adj_ii = al - be z_i^2 + ga z_j^2 z_k^2, adj_ij = mcp z_i z_j (c44 + D z_k^2)
     const double al = c44 * (c44 + D + cp), be = c44 * (D + cp), ga = D * (D + 2.0 * cp), mcp = -cp;
     const double d0 = c44 * c44 * (c44 + D + cp), d1 = c44 * D * (D + 2.0 * cp);
@@ -988,19 +1008,19 @@ static NearMedium<R> near_medium(const DevMaterial &m) {
     n.d2 = R(D * D * (D + 3.0 * cp));
     n.e0 = R(d0 + 0.5 * d1);
     // sum_p h_cpp = (al + mcp c44) lin_c - (be + mcp c44) c1_c + (ga + 2 mcp D) x2_c
-    const double t0 = m.c12 * (al + mcp * c44), t1 = -m.c12 * (be + mcp * c44), t2 = m.c12 * (ga + 2.0 * mcp * D);
+    const double t0 = c12 * (al + mcp * c44), t1 = -c12 * (be + mcp * c44), t2 = c12 * (ga + 2.0 * mcp * D);
     n.rc[0] = R(t0 + ydiag * al), n.rc[1] = R(t1 - ydiag * be), n.rc[2] = R(t2 + ydiag * ga);
     n.rn[0] = R(t0), n.rn[1] = R(t1), n.rn[2] = R(t2 + ydiag * mcp * D), n.rn[3] = R(ydiag * mcp * c44);
     n.re[0] = R(c44 * mcp * (2.0 * c44 + D)), n.re[1] = R(-c44 * mcp * D);
     n.rs[0] = R(c44 * al), n.rs[1] = R(c44 * mcp * D), n.rs[2] = R(c44 * (mcp * c44 - be)), n.rs[3] = R(c44 * ga);
-    n.y12 = R(m.c12);
+    n.y12 = R(c12);
     n.ydiag = R(ydiag);
     n.y44 = R(c44);
     static const int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
-    auto C = [&m](int i, int j, int k, int l) { return m.C[((i * 3 + j) * 3 + k) * 3 + l]; };
+    auto C = [&m, iu](int i, int j, int k, int l) { return iu * m.C[((i * 3 + j) * 3 + k) * 3 + l]; };
     for (int a = 0; a < 6; ++a)
         for (int x = 0; x < 6; ++x) {
-            n.C[6 * a + x] = R(m.V[6 * a + x]);
+            n.C[6 * a + x] = R(iu * m.V[6 * a + x]);
             // (zz)_jk = z_i C_ijkl z_l
             const int j = PV[a], k = PP[a], i = PV[x], l = PP[x];
             n.Z[6 * a + x] = R(C(i, j, k, l) + (i != l ? C(l, j, k, i) : 0.0));
@@ -1045,8 +1065,7 @@ int near_prepare(gbfmm_ctx *ctx) {
     GaussWeights gw{};
     gw.n = ctx->opt.n_gauss;
     for (int i = 0; i < gw.n; ++i) gw.w[i] = ctx->gauss_w[i];
-    // h of the unit-circle rule is summed without its factor 1 / (4 pi Q), the isotropic one without hc
-    const double fac = ctx->mat.mode == GBFMM_H_ISO ? ctx->mat.hc : 1.0 / (4.0 * M_PI * ctx->mat.Q);
+    const double fac = near_factor(ctx->mat);
     if (ctx->opt.precision == GBFMM_FP64)
         k_near_records<double><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
                                                                        ctx->d_pleaf, ctx->node_xyz, ctx->seg_nodes,
@@ -1142,6 +1161,7 @@ static int run_pairs(gbfmm_ctx *ctx, const int *tstart, const double *xt, int64_
             ln.poly = reinterpret_cast<const float4 *>(ctx->mlp.poly);
             ln.rmin2 = float(rmin * rmin);
             ln.m2 = mlp_poly_m2();
+            ln.fac = float(near_unit(ctx->mat) / near_factor(ctx->mat));
             rc = cubic ? launch_pairs<R, HM_CUBIC, SYM, true>(ctx, tr, md, ln)
                        : launch_pairs<R, HM_GENERAL, SYM, true>(ctx, tr, md, ln);
         }

@@ -26,11 +26,12 @@
 #pragma once
 #include "kernel_math.cuh"
 
-// Constants of a medium as the near-field kernels take them (by value, kernel parameters)
+// Constants of a medium as the near-field kernels take them (by value, kernel parameters), the moduli
+// divided by a power of two near the largest: the rules below form 1 / det^2, a sixth power
 template <typename R>
 struct NearMedium {
     int Q, np;                   // circle points; pairs (phi, -phi) with 0 < phi < pi / 2
-    R k1, k3, k6;                // isotropic: strain_iso's factors (1 / (16 pi mu (1 - nu)) is folded into the Burgers vectors)
+    R k1, k3, k6;                // isotropic: strain_iso's factors (1 / (16 pi mu (1 - nu)) in the same unit is folded into the Burgers vectors)
     R d1, d2, e0;                // cubic: det = d0 + d1 s2 + d2 s3 with s2, s3 the symmetric functions of z_i^2; e0 = d0 + d1 / 2
     R rc[3], rn[4], re[2], rs[4];  // cubic: factors of rows_cubic
     R y12, ydiag, y44;           // cubic: C12, C11 - C12, C44 (contraction)

@@ -49,7 +49,6 @@ struct MlpState {
     void *bufs = nullptr;              // batch activations
     uint32_t *d_binmask = nullptr;     // [48] angular bins where the plain evaluator is used
     float *poly = nullptr;             // [1280][108] the network as polynomials, one per angular bin (near field)
-    bool poly_ok = false;              // poly belongs to the current network
     double fallback_frac = 1.0;        // fraction of bins flagged by the last calibration
     bool trained = false;
     int64_t step = 0;

@@ -385,8 +385,20 @@ __global__ void k_gather_rows(int n, int w, const int *__restrict__ idx, const f
 // components symmetric in (v, p).  One block per bin, a thread per coefficient.  A
 // pair of the near field then costs 108 multiply-adds instead of 37,000 (a bin is 1/16 of a face
 // wide: the quadratic follows the network's values within its own BF16 noise).
-constexpr int kBinGrid = 8;
+constexpr int kBins = 5 * 256, kBinGrid = 8, kBinPer = kBinGrid * kBinGrid;
 __host__ __device__ inline float grid_coord(int i) { return float(2 * i + 1 - kBinGrid) / float(kBinGrid); }
+
+// the 8 x 8 directions of every angular bin (the near field's binning: dominant axis face +z, +x, -x,
+// +y, -y and a 16 x 16 grid of the other two components), [bin][64][3]
+__global__ void __launch_bounds__(kBinPer) k_bin_dirs(float *__restrict__ dirs) {
+    const int b = blockIdx.x, i = threadIdx.x, f = b / 256;
+    const float p = -1.f + (2.f * float((b / 16) % 16) + 1.f + grid_coord(i % kBinGrid)) / 16.f;
+    const float q = -1.f + (2.f * float(b % 16) + 1.f + grid_coord(i / kBinGrid)) / 16.f;
+    const float n = sqrtf(p * p + q * q + 1.f);
+    const float x = f == 0 || f >= 3 ? p : f == 1 ? 1.f : -1.f, y = f == 0 ? q : f <= 2 ? p : f == 3 ? 1.f : -1.f;
+    float *d = dirs + (int64_t(b) * kBinPer + i) * 3;
+    d[0] = x / n, d[1] = y / n, d[2] = (f == 0 ? 1.f : q) / n;
+}
 __global__ void k_bin_poly(const float *__restrict__ h, float m2, float *__restrict__ poly) {
     constexpr int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
     const int t = threadIdx.x;
@@ -485,8 +497,10 @@ int mlp_eval_device(gbfmm_ctx *ctx, int64_t n, const float *dirs, float *h) {
     return mlp_forward(ctx, n, dirs, h);
 }
 
-extern "C" int fmm_mlp_set(gbfmm_ctx *ctx, const float *theta, const float *scale) {
-    if (!ctx || !theta || !scale) return GBFMM_ERR_INVALID_ARG;
+static int mlp_changed(gbfmm_ctx *ctx);
+
+// parameters and scales (host) into the context
+static int mlp_load(gbfmm_ctx *ctx, const float *theta, const float *scale) {
     int rc = mlp_alloc_state(ctx);
     if (rc) return rc;
     std::vector<float> th(theta, theta + NPAR);
@@ -494,6 +508,7 @@ extern "C" int fmm_mlp_set(gbfmm_ctx *ctx, const float *theta, const float *scal
     for (int i = OFF_B4 + 27; i < NPAR; ++i) th[i] = 0.f;
     float sc[32] = {0};
     for (int i = 0; i < 27; ++i) sc[i] = scale[i];
+    ctx->mlp.trained = false;  // until mlp_changed
     CK(cudaMemcpy(ctx->mlp.theta, th.data(), NPAR * sizeof(float), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(ctx->mlp.scale, sc, sizeof(sc), cudaMemcpyHostToDevice));
     CK(cudaMemset(ctx->mlp.m, 0, NPAR * sizeof(float)));
@@ -502,10 +517,14 @@ extern "C" int fmm_mlp_set(gbfmm_ctx *ctx, const float *theta, const float *scal
     if (rc) return rc;
     sync_params(ctx);
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->mlp.trained = true;
-    ctx->mlp.poly_ok = false;
     ctx->mlp.step = 0;
     return GBFMM_OK;
+}
+
+extern "C" int fmm_mlp_set(gbfmm_ctx *ctx, const float *theta, const float *scale) {
+    if (!ctx || !theta || !scale) return GBFMM_ERR_INVALID_ARG;
+    if (int rc = mlp_load(ctx, theta, scale)) return rc;
+    return mlp_changed(ctx);
 }
 
 extern "C" int fmm_mlp_get(gbfmm_ctx *ctx, float *theta, float *scale) {
@@ -595,7 +614,7 @@ extern "C" int fmm_mlp_train(gbfmm_ctx *ctx, int64_t n, const float *dirs, int e
     fill(OFF_W2, 128, 128, 128);
     fill(OFF_W3, 128, 128, 128);
     fill(OFF_W4, 27, 128, 128);
-    rc = fmm_mlp_set(ctx, th.data(), sc);
+    rc = mlp_load(ctx, th.data(), sc);
     if (rc) return rc;
     // Adam with cosine decay of the learning rate
     const int steps_per_epoch = int(n / batch);
@@ -630,32 +649,8 @@ extern "C" int fmm_mlp_train(gbfmm_ctx *ctx, int64_t n, const float *dirs, int e
     cudaFree(by);
     cudaFree(perm);
     cudaFree(acc);
-    M.trained = true;
-    M.poly_ok = false;
     if (final_loss) *final_loss = last;
-    return GBFMM_OK;
-}
-
-constexpr int kBins = 5 * 256;
-
-// 8 x 8 directions of every angular bin (the near field's binning), [bin][64][3]
-static std::vector<float> bin_directions() {
-    const int per = kBinGrid * kBinGrid;
-    std::vector<float> dirs(size_t(kBins) * per * 3);
-    for (int b = 0; b < kBins; ++b) {
-        const int f = b / 256, bu = (b / 16) % 16, bv = b % 16;
-        for (int i = 0; i < per; ++i) {
-            const float u = -1.f + 2.f * (bu + (i % 8 + 0.5f) / 8.f) / 16.f;
-            const float v = -1.f + 2.f * (bv + (i / 8 + 0.5f) / 8.f) / 16.f;
-            float d[3];
-            if (f == 0) { d[0] = u; d[1] = v; d[2] = 1.f; }
-            else if (f <= 2) { d[0] = f == 1 ? 1.f : -1.f; d[1] = u; d[2] = v; }
-            else { d[0] = u; d[1] = f == 3 ? 1.f : -1.f; d[2] = v; }
-            const float n = std::sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-            for (int c = 0; c < 3; ++c) dirs[(size_t(b) * per + i) * 3 + c] = d[c] / n;
-        }
-    }
-    return dirs;
+    return mlp_changed(ctx);
 }
 
 // mean of grid_coord^2
@@ -665,76 +660,77 @@ float mlp_poly_m2() {
     return s / float(kBinGrid);
 }
 
-// The near field's polynomials of the current network.  Rebuilt after the network changed;
-// synchronises then.
-int mlp_tabulate(gbfmm_ctx *ctx) {
-    MlpState &M = ctx->mlp;
-    if (M.poly_ok && M.poly) return GBFMM_OK;
-    const std::vector<float> dirs = bin_directions();
-    const int64_t n = int64_t(dirs.size() / 3);
-    if (!M.poly) CK(cudaMalloc(&M.poly, size_t(kBins) * 108 * sizeof(float)));
-    float *dd = nullptr, *h = nullptr;
-    if (cudaMalloc(&dd, n * 3 * sizeof(float)) != cudaSuccess || cudaMalloc(&h, n * 27 * sizeof(float)) != cudaSuccess) {
-        cudaFree(dd);
-        return set_err(ctx, GBFMM_ERR_CUDA, "learned near field: out of device memory");
+// Scratch of a call that prepares or judges the near field's polynomials
+struct BinScratch {
+    float *dirs = nullptr, *h = nullptr, *y = nullptr;
+    ~BinScratch() {
+        for (float *p : {dirs, h, y})
+            if (p) cudaFree(p);
     }
-    int rc = GBFMM_OK;
-    auto run = [&]() -> int {
-        CK(cudaMemcpyAsync(dd, dirs.data(), n * 3 * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-        if (int r = mlp_eval_device(ctx, n, dd, h)) return r;
-        ++ctx->launches;
-        k_bin_poly<<<kBins, 128, 0, ctx->stream>>>(h, mlp_poly_m2(), M.poly);
-        CK(cudaGetLastError());
-        CK(cudaStreamSynchronize(ctx->stream));
-        return GBFMM_OK;
-    };
-    rc = run();
-    cudaFree(dd);
-    cudaFree(h);
-    if (!rc) M.poly_ok = true;
-    return rc;
+};
+
+// The near field's polynomials of the current network, built when it is set or trained: an
+// evaluation finds them ready.  Synchronises.
+static int mlp_tabulate(gbfmm_ctx *ctx) {
+    MlpState &M = ctx->mlp;
+    constexpr int64_t n = int64_t(kBins) * kBinPer;
+    BinScratch b;
+    if (!M.poly) CK(cudaMalloc(&M.poly, size_t(kBins) * 108 * sizeof(float)));
+    CK(cudaMalloc(&b.dirs, n * 3 * sizeof(float)));
+    CK(cudaMalloc(&b.h, n * 27 * sizeof(float)));
+    ctx->launches += 2;
+    k_bin_dirs<<<kBins, kBinPer, 0, ctx->stream>>>(b.dirs);
+    if (int rc = mlp_forward(ctx, n, b.dirs, b.h)) return rc;
+    k_bin_poly<<<kBins, 128, 0, ctx->stream>>>(b.h, mlp_poly_m2(), M.poly);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(ctx->stream));
+    return GBFMM_OK;
+}
+
+// after the parameters changed: the polynomials, where the near field reads them
+static int mlp_changed(gbfmm_ctx *ctx) {
+    if (ctx->opt.h_mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64)
+        if (int rc = mlp_tabulate(ctx)) return rc;
+    ctx->mlp.trained = true;
+    return GBFMM_OK;
 }
 
 // Assess the network per angular bin against the plain evaluator: 64 directions
-// per bin of the near-field kernel's binning (dominant axis face +z, +x, -x,
-// +y, -y and a 16 x 16 grid of the other two components); a bin whose largest
+// per bin of the near-field kernel's binning (k_bin_dirs); a bin whose largest
 // component error exceeds bin_tol x (RMS of h over all samples) is flagged
 // and its pairs take the plain evaluator.
 extern "C" int fmm_mlp_calibrate(gbfmm_ctx *ctx, double bin_tol, double *fallback_frac) {
     if (!ctx || !(bin_tol > 0.0)) return GBFMM_ERR_INVALID_ARG;
     if (!ctx->mlp.trained) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "fmm_mlp_calibrate: train or set the network first");
-    const int nb = kBins, per = kBinGrid * kBinGrid;
-    const std::vector<float> dirs = bin_directions();
-    const int64_t n = int64_t(nb) * per;
-    float *dd = nullptr, *y = nullptr, *hm = nullptr;
-    CK(cudaMalloc(&dd, n * 3 * sizeof(float)));
-    CK(cudaMalloc(&y, n * 27 * sizeof(float)));
-    CK(cudaMalloc(&hm, n * 27 * sizeof(float)));
-    CK(cudaMemcpy(dd, dirs.data(), n * 3 * sizeof(float), cudaMemcpyHostToDevice));
-    int rc = fmm_mlp_labels(ctx, n, dd, y);
+    const int nb = kBins, per = kBinPer;
+    constexpr int64_t n = int64_t(kBins) * kBinPer;
+    BinScratch b;
+    CK(cudaMalloc(&b.dirs, n * 3 * sizeof(float)));
+    CK(cudaMalloc(&b.y, n * 27 * sizeof(float)));
+    CK(cudaMalloc(&b.h, n * 27 * sizeof(float)));
+    ++ctx->launches;
+    k_bin_dirs<<<kBins, kBinPer, 0, ctx->stream>>>(b.dirs);
+    int rc = fmm_mlp_labels(ctx, n, b.dirs, b.y);
     if (rc) return rc;
-    rc = mlp_eval_device(ctx, n, dd, hm);
+    rc = mlp_eval_device(ctx, n, b.dirs, b.h);
     if (rc) return rc;
     std::vector<float> hy(n * 27), hh(n * 27);
-    CK(cudaMemcpyAsync(hy.data(), y, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(hh.data(), hm, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(hy.data(), b.y, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(hh.data(), b.h, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    cudaFree(dd);
-    cudaFree(y);
-    cudaFree(hm);
     double ss = 0.0;
     for (float v : hy) ss += double(v) * v;
     const double rms = std::sqrt(ss / double(hy.size()));
     uint32_t mask[48] = {0};
     int flagged = 0;
-    for (int b = 0; b < nb; ++b) {
+    for (int bin = 0; bin < nb; ++bin) {
         double e = 0.0;
         for (int i = 0; i < per * 27; ++i) {
-            const size_t k = size_t(b) * per * 27 + i;
+            const size_t k = size_t(bin) * per * 27 + i;
             e = std::max(e, std::fabs(double(hh[k]) - double(hy[k])));
         }
         if (e > bin_tol * rms) {
-            mask[b >> 5] |= 1u << (b & 31);
+            mask[bin >> 5] |= 1u << (bin & 31);
             ++flagged;
         }
     }
@@ -742,7 +738,7 @@ extern "C" int fmm_mlp_calibrate(gbfmm_ctx *ctx, double bin_tol, double *fallbac
     CK(cudaMemcpy(ctx->mlp.d_binmask, mask, sizeof(mask), cudaMemcpyHostToDevice));
     ctx->mlp.fallback_frac = double(flagged) / double(nb);
     if (fallback_frac) *fallback_frac = ctx->mlp.fallback_frac;
-    return mlp_tabulate(ctx);
+    return GBFMM_OK;
 }
 
 void mlp_free(gbfmm_ctx *ctx) {

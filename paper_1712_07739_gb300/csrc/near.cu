@@ -966,8 +966,7 @@ __global__ void __launch_bounds__(256) k_near_combine(int p, const __grid_consta
 }  // namespace
 
 // ---------------------------------------------------------------- host side
-int mlp_tabulate(gbfmm_ctx *ctx);  // mlp.cu: the network's polynomials, when they are out of date
-float mlp_poly_m2();
+float mlp_poly_m2();  // mlp.cu
 
 static bool near_learned(const gbfmm_ctx *ctx) {
     return ctx->mat.mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64;
@@ -1185,11 +1184,8 @@ int near_run(gbfmm_ctx *ctx, bool free_targets, int64_t n_t, double *sig) {
     const int *tstart = free_targets ? ctx->d_t_start : ctx->d_leaf_start;
     const double *xt = free_targets ? ctx->d_t_x : ctx->d_y;
     if (!free_targets) n_t = ctx->N;
-    if (near_learned(ctx)) {
-        if (!ctx->mlp.trained || !ctx->mlp.d_binmask)
-            return set_err(ctx, GBFMM_ERR_INVALID_ARG, "GBFMM_H_MLP: train (or set) and calibrate the network first");
-        if (int rc = mlp_tabulate(ctx)) return rc;  // when the network changed since
-    }
+    if (near_learned(ctx) && (!ctx->mlp.trained || !ctx->mlp.d_binmask))
+        return set_err(ctx, GBFMM_ERR_INVALID_ARG, "GBFMM_H_MLP: train (or set) and calibrate the network first");
     const int *tleaf = free_targets ? ctx->d_t_leaf : ctx->d_pleaf;
     if (ctx->opt.precision == GBFMM_FP64)
         return free_targets ? run_pairs<double, false>(ctx, tstart, xt, n_t, tleaf, sig)

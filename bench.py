@@ -96,7 +96,7 @@ def near_work(wl, work):
     of one pass, a multiply-add as two.  Nodal forces evaluate a pair once for
     both directions.  Unit-circle rule: 37 multiply-adds and two reciprocals per
     pair of circle points (phi, -phi) beside about 430 (cubic medium) or 850 (any
-    other in FP64) a pair, or 93 per circle point beside 300 (any other in FP32);
+    other in FP64) a pair, or 132 per circle point beside 190 (any other in FP32);
     isotropic: 43 a direction beside 30; learned: 108 from the bin's polynomial
     beside 220.  ``near_flops`` counts the same pairs by the pointwise rule."""
     p, q, pairs = wl["p"], wl.get("circle_q", 64), work["near_pairs"] / 2.0
@@ -110,7 +110,7 @@ def near_work(wl, work):
     elif wl["precision"] == "fp64":
         per = 39 * ((q - 1) // 2) + 850
     else:
-        per = 93 * q + 300
+        per = 132 * q + 190
     return pairs * 2 * per + l2p, "k_near_pairs"
 
 

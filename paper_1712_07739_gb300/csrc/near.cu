@@ -54,7 +54,7 @@ __device__ __forceinline__ void cell_xyz3(int64_t lin, int n, int &x, int &y, in
 }
 
 // h models of the near kernels: closed form; moment form of a cubic medium; any medium, point by
-// point (FP32) or in moment form (FP64, and FP32 beside the learned h, whose error covers its rounding)
+// point (FP32) or in moment form (FP64, and FP32 beside the learned h)
 constexpr int HM_ISO = 0, HM_CUBIC = 1, HM_POINTS = 2, HM_GENERAL = 3;
 
 // ---------------------------------------------------------------- point records
@@ -1016,6 +1016,7 @@ static NearMedium<R> near_medium(const DevMaterial &m) {
             // (zz)_jk = z_i C_ijkl z_l
             const int j = PV[a], k = PP[a], i = PV[x], l = PP[x];
             n.Z[6 * a + x] = R(C(i, j, k, l) + (i != l ? C(l, j, k, i) : 0.0));
+            n.Z2[6 * a + x] = make_float2(float(n.Z[6 * a + x]), float(n.Z[6 * a + x]));
         }
     return n;
 }
@@ -1073,7 +1074,7 @@ int near_prepare(gbfmm_ctx *ctx) {
 template <typename R, int HM, bool SYM, bool LEARN>
 static int launch_pairs(gbfmm_ctx *ctx, const NearTree &tr, const NearMedium<R> &md, const NearLearned &ln) {
     size_t table = 0;
-    if (HM == HM_POINTS) table = md.Q <= kPointMax ? size_t(md.Q) * sizeof(float4) : 0;
+    if (HM == HM_POINTS) table = md.Q <= kPointMax ? size_t((md.Q + 1) / 2) * sizeof(float4) : 0;
     else if (HM != HM_ISO) table = md.np <= kMomMax ? size_t(md.np) * kMomRow * sizeof(R) : 0;
     const size_t smem = near_warps<R>() * sizeof(WarpShared<R, SYM, LEARN>) + table;
     auto kern = k_near_pairs<R, HM, SYM, LEARN>;

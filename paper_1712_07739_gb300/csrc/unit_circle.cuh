@@ -37,6 +37,7 @@ struct NearMedium {
     R y12, ydiag, y44;           // cubic: C12, C11 - C12, C44 (contraction)
     R C[36];                     // Voigt stiffness
     R Z[36];                     // (zz)_m = sum_x Z[6 m + x] (z z)_x, pairs in the order of hs
+    float2 Z2[36];               // the same, twice, for packed arithmetic
 };
 
 // Rows of the moment table, one per pair (phi, -phi): ten pairs of values
@@ -451,84 +452,104 @@ __device__ __forceinline__ void h_general_moments(const NearMedium<R> &md, const
     }
 }
 
-// Points of the pointwise general rule: (cos 2phi, sin 2phi, cos phi, sin phi) of the Q points
-constexpr int kPointMax = 1024;  // kept in shared memory up to this many, else computed where used
-__device__ __noinline__ inline float4 circle_point4(int k, int Q) {
-    double s, c;
-    sincospi(double(k) / double(Q), &s, &c);
-    return make_float4(float(c * c - s * s), float(2.0 * c * s), float(c), float(s));
+// Points of the pointwise general rule, two by two: (cos phi, cos phi', sin phi, sin phi'); the last of an
+// odd number stands twice
+constexpr int kPointMax = 1024;  // points kept in shared memory, else computed where used
+__device__ __noinline__ inline float4 circle_points2(int k, int Q) {
+    const int k0 = 2 * k, k1 = min(2 * k + 1, Q - 1);
+    double s0, c0, s1, c1;
+    sincospi(double(k0) / double(Q), &s0, &c0);
+    sincospi(double(k1) / double(Q), &s1, &c1);
+    return make_float4(float(c0), float(c1), float(s0), float(s1));
 }
 __device__ __forceinline__ void point_table(int Q, float *tab) {
     if (Q > kPointMax) return;
-    for (int k = threadIdx.x; k < Q; k += blockDim.x) reinterpret_cast<float4 *>(tab)[k] = circle_point4(k, Q);
+    for (int k = threadIdx.x; 2 * k < Q; k += blockDim.x) reinterpret_cast<float4 *>(tab)[k] = circle_points2(k, Q);
 }
 
-// h of any medium, times 4 pi Q, point by point (FP32).  (zz) = m + u cos 2phi + v sin 2phi and its
-// derivative along T, S = sc cos phi + ss sin phi, are formed once per pair, so a circle point
-// costs 93 multiply-adds (from the 81-entry C: ~450) and
+// h of any medium, times 4 pi Q, point by point (FP32), two points a step in packed arithmetic.
+// (zz) comes from z itself, 36 multiply-adds, its derivative along T as S = sc cos phi + ss sin phi, and
 //     F_vp = (adj_vp (adj : S) / det - dadj_vp) / det
-// needs no matrix product.  Kept beside the moment form, which is 1.8 times cheaper at Q = 32,
-// because its FP32 rounding stays at that of the rule from the 81-entry C whatever the medium
-// (RMS of K over random separations, rule from C / this / moments: cubic A = 3.2, 1.2 / 1.1 /
-// 1.3e-7; A = 0.17, 7.6 / 7.6 / 10e-8; triclinic, 10.4 / 9.7 / 10.9e-8).
+// needs no matrix product: 66 instructions a point (132 multiply-adds; from the 81-entry C: ~450).
+// (zz) as m + u cos 2phi + v sin 2phi takes 24 multiply-adds less a point, but rounds three coefficients
+// into every point alike, which the sum over the points does not average out.  RMS error of the mixed
+// pass's K, rule from C / harmonics / this / moments, in 1e-7: turned cubic, A = 3.2, 3.9 / 4.7 / 3.4 /
+// 3.8, A = 0.17, 16.5 / 18 / 12 / 18; aligned, A = 0.48, 5.2 / 5.7 / 4.0 / 4.2; triclinic 2.8 / 3.0 / 2.3 /
+// 2.5.  6,101 segments in a turned crystal, whole pass: 3.22 ms with harmonics, 3.35 here; the near
+// field of 100,000 192 and 202 (88 in moment form, kept for the plain pairs beside the learned h).
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+// a b - c d
+__device__ __forceinline__ float2 det2(float2 a, float2 b, float2 c, float2 d) { return fma2(a, b, mul2(neg2(c), d)); }
 __device__ __forceinline__ void h_general_points(const NearMedium<float> &md, const float *tab, const float T[3],
                                                  float hs[18]) {
     float a[3], b[3];
     circle_axes<float>(T, a, b);
     constexpr int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
-    float m[6], u[6], v[6], sc[6], ss[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) m[i] = u[i] = v[i] = sc[i] = ss[i] = 0.f;
+    float sc[6], ss[6];
 #pragma unroll
     for (int x = 0; x < 6; ++x) {
         const int i = PV[x], l = PP[x];
-        const float p = a[i] * a[l], q = b[i] * b[l];
-        const float zm = 0.5f * (p + q), zu = 0.5f * (p - q), zv = 0.5f * (a[i] * b[l] + b[i] * a[l]);
-        const float zc = T[i] * a[l] + T[l] * a[i], zs = T[i] * b[l] + T[l] * b[i];
+        const float zc = i == l ? 2.f * T[i] * a[i] : T[i] * a[l] + T[l] * a[i];
+        const float zs = i == l ? 2.f * T[i] * b[i] : T[i] * b[l] + T[l] * b[i];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const float Z = md.Z[6 * k + x];
-            m[k] = fmaf(Z, zm, m[k]), u[k] = fmaf(Z, zu, u[k]), v[k] = fmaf(Z, zv, v[k]);
-            sc[k] = fmaf(Z, zc, sc[k]), ss[k] = fmaf(Z, zs, ss[k]);
+        for (int m = 0; m < 6; ++m) {
+            const float Z = md.Z[6 * m + x];
+            sc[m] = x == 0 ? Z * zc : fmaf(Z, zc, sc[m]);
+            ss[m] = x == 0 ? Z * zs : fmaf(Z, zs, ss[m]);
         }
     }
-    float A[6], B[6], G[6];
+    float2 A[6], B[6], G[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) A[i] = B[i] = G[i] = 0.f;
+    for (int i = 0; i < 6; ++i) A[i] = B[i] = G[i] = dup(0.f);
     const float4 *pt = reinterpret_cast<const float4 *>(tab);
-#pragma unroll 2
-    for (int k = 0; k < md.Q; ++k) {
-        const float4 t = md.Q <= kPointMax ? pt[k] : circle_point4(k, md.Q);
-        float M[6], S[6];
+#pragma unroll 1
+    for (int k = 0; 2 * k < md.Q; ++k) {
+        const float4 t = md.Q <= kPointMax ? pt[k] : circle_points2(k, md.Q);
+        const float2 c = make_float2(t.x, t.y), s = make_float2(t.z, t.w);
+        float2 z[3], M[6], S[6];
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            M[i] = fmaf(v[i], t.y, fmaf(u[i], t.x, m[i]));
-            S[i] = fmaf(ss[i], t.w, sc[i] * t.z);
+        for (int i = 0; i < 3; ++i) z[i] = fma2(c, dup(a[i]), mul2(s, dup(b[i])));
+#pragma unroll
+        for (int x = 0; x < 6; ++x) {
+            const int i = PV[x], l = PP[x];
+            const float2 zz = mul2(z[i], z[l]);
+#pragma unroll
+            for (int m = 0; m < 6; ++m) {
+                const float2 Z = md.Z2[6 * m + x];
+                M[m] = x == 0 ? mul2(Z, zz) : fma2(Z, zz, M[m]);
+            }
         }
-        const float adj[6] = {M[1] * M[2] - M[3] * M[3], M[0] * M[2] - M[4] * M[4], M[0] * M[1] - M[5] * M[5],
-                              M[5] * M[4] - M[0] * M[3], M[5] * M[3] - M[4] * M[1], M[4] * M[3] - M[5] * M[2]};
-        const float w = recip(M[0] * adj[0] + M[5] * adj[5] + M[4] * adj[4]);
-        const float S3 = 2.f * S[3], S4 = 2.f * S[4], S5 = 2.f * S[5];
-        const float da[6] = {S[1] * M[2] + M[1] * S[2] - M[3] * S3,
-                             S[0] * M[2] + M[0] * S[2] - M[4] * S4,
-                             S[0] * M[1] + M[0] * S[1] - M[5] * S5,
-                             S[5] * M[4] + M[5] * S[4] - S[0] * M[3] - M[0] * S[3],
-                             S[5] * M[3] + M[5] * S[3] - S[4] * M[1] - M[4] * S[1],
-                             S[4] * M[3] + M[4] * S[3] - S[5] * M[2] - M[5] * S[2]};
-        const float tau = w * (adj[0] * S[0] + adj[1] * S[1] + adj[2] * S[2] + adj[3] * S3 + adj[4] * S4 + adj[5] * S5);
-        const float cw = t.z * w, sw = t.w * w;
+#pragma unroll
+        for (int m = 0; m < 6; ++m) S[m] = fma2(s, dup(ss[m]), mul2(c, dup(sc[m])));
+        const float2 adj[6] = {det2(M[1], M[2], M[3], M[3]), det2(M[0], M[2], M[4], M[4]), det2(M[0], M[1], M[5], M[5]),
+                               det2(M[5], M[4], M[0], M[3]), det2(M[5], M[3], M[4], M[1]), det2(M[4], M[3], M[5], M[2])};
+        const float2 det = fma2(M[0], adj[0], fma2(M[5], adj[5], mul2(M[4], adj[4])));
+        float2 w = make_float2(recip(det.x), recip(det.y));
+        if (2 * k + 1 >= md.Q) w.y = 0.f;  // the point that stands twice
+        const float2 S3 = mul2(S[3], dup(2.f)), S4 = mul2(S[4], dup(2.f)), S5 = mul2(S[5], dup(2.f));
+        const float2 da[6] = {fma2(neg2(M[3]), S3, fma2(M[1], S[2], mul2(S[1], M[2]))),
+                              fma2(neg2(M[4]), S4, fma2(M[0], S[2], mul2(S[0], M[2]))),
+                              fma2(neg2(M[5]), S5, fma2(M[0], S[1], mul2(S[0], M[1]))),
+                              fma2(neg2(M[0]), S[3], fma2(neg2(S[0]), M[3], fma2(M[5], S[4], mul2(S[5], M[4])))),
+                              fma2(neg2(M[4]), S[1], fma2(neg2(S[4]), M[1], fma2(M[5], S[3], mul2(S[5], M[3])))),
+                              fma2(neg2(M[5]), S[2], fma2(neg2(S[5]), M[2], fma2(M[4], S[3], mul2(S[4], M[3]))))};
+        const float2 tau = mul2(w, fma2(adj[0], S[0], fma2(adj[1], S[1], fma2(adj[2], S[2],
+                                   fma2(adj[3], S3, fma2(adj[4], S4, mul2(adj[5], S5)))))));
+        const float2 cw = mul2(c, w), sw = mul2(s, w);
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
-            const float F = fmaf(adj[i], tau, -da[i]);
-            A[i] = fmaf(cw, F, A[i]);
-            B[i] = fmaf(sw, F, B[i]);
-            G[i] = fmaf(w, adj[i], G[i]);
+            const float2 F = fma2(adj[i], tau, neg2(da[i]));
+            A[i] = fma2(cw, F, A[i]);
+            B[i] = fma2(sw, F, B[i]);
+            G[i] = fma2(w, adj[i], G[i]);
         }
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) hs[3 * i + q] = a[q] * A[i] + b[q] * B[i] - T[q] * G[i];
+        for (int q = 0; q < 3; ++q)
+            hs[3 * i + q] = a[q] * (A[i].x + A[i].y) + b[q] * (B[i].x + B[i].y) - T[q] * (G[i].x + G[i].y);
 }
 
 // The contraction of Sec. 2, Eq. "kernel" with a point's strength q = b' x S, without the

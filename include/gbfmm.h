@@ -406,9 +406,11 @@ int fmm_mlp_train(gbfmm_ctx *ctx, int64_t n, const float *dirs, int epochs, int 
                   uint64_t seed, float *final_loss);
 
 /* Assess the network against the plain evaluator per angular bin (5 x 256
- * bins of direction, 64 sample directions each) and record which bins the
- * near field of GBFMM_H_MLP must evaluate with the plain rule: those whose
- * largest component error exceeds bin_tol x (RMS of h).  fallback_frac
+ * bins of direction) and record which bins the near field of GBFMM_H_MLP must
+ * evaluate with the plain rule: those whose largest component error exceeds
+ * bin_tol x (RMS of h), the error being the larger of the network's at 64
+ * directions of the bin and that of the bin's quadratic, which the near field
+ * reads, at these and at 25 more from edge to edge.  fallback_frac
  * (host, may be NULL): fraction of bins flagged.  Required before a
  * GBFMM_H_MLP evaluation.  Synchronises the stream.
  * Errors: INVALID_ARG (network not set), NO_MATERIAL, CUDA. */

@@ -311,8 +311,8 @@ class FMM:
         return loss.value
 
     def mlp_calibrate(self, bin_tol=2e-2):
-        """Flag the angular bins where the network's error exceeds bin_tol x RMS(h);
-        returns the flagged fraction."""
+        """Flag the angular bins where the error of the network, or of the quadratic that the
+        near field reads for it, exceeds bin_tol x RMS(h); returns the flagged fraction."""
         fr = ctypes.c_double()
         self._check(self._lib.fmm_mlp_calibrate(self._h, float(bin_tol), ctypes.byref(fr)), "fmm_mlp_calibrate")
         return fr.value

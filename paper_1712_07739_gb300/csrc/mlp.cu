@@ -383,20 +383,27 @@ __global__ void k_gather_rows(int n, int w, const int *__restrict__ idx, const f
 // the bin's coordinates (u, v) through the network's values at 8 x 8 directions, on the basis
 // 1, u, v, u^2 - m2, uv, v^2 - m2, which is orthogonal on that grid (m2 = mean of u^2); the 18
 // components symmetric in (v, p).  One block per bin, a thread per coefficient.  A
-// pair of the near field then costs 108 multiply-adds instead of 37,000 (a bin is 1/16 of a face
-// wide: the quadratic follows the network's values within its own BF16 noise).
+// pair of the near field then costs 108 multiply-adds instead of 37,000.  How far the quadratics are
+// from h depends on the medium as well as on the network (fitted to h itself they are 3e-4 of its RMS
+// off at a Zener ratio of 3.2, in the worst bin 3e-3; ten times that in the worst bin at 8):
+// fmm_mlp_calibrate judges them.
 constexpr int kBins = 5 * 256, kBinGrid = 8, kBinPer = kBinGrid * kBinGrid;
 __host__ __device__ inline float grid_coord(int i) { return float(2 * i + 1 - kBinGrid) / float(kBinGrid); }
 
-// the 8 x 8 directions of every angular bin (the near field's binning: dominant axis face +z, +x, -x,
-// +y, -y and a 16 x 16 grid of the other two components), [bin][64][3]
-__global__ void __launch_bounds__(kBinPer) k_bin_dirs(float *__restrict__ dirs) {
+constexpr int kBinEdge = 5, kBinEdgePer = kBinEdge * kBinEdge;
+__host__ __device__ inline float edge_coord(int i) { return float(2 * i) / float(kBinEdge - 1) - 1.f; }
+
+// directions of every angular bin (the near field's binning: dominant axis face +z, +x, -x, +y, -y and a
+// 16 x 16 grid of the other two components), [bin][m^2][3]: the 8 x 8 that the polynomials are fitted
+// at (m = kBinGrid), or 5 x 5 from edge to edge (m = kBinEdge), one thread each
+__global__ void k_bin_dirs(int m, float *__restrict__ dirs) {
     const int b = blockIdx.x, i = threadIdx.x, f = b / 256;
-    const float p = -1.f + (2.f * float((b / 16) % 16) + 1.f + grid_coord(i % kBinGrid)) / 16.f;
-    const float q = -1.f + (2.f * float(b % 16) + 1.f + grid_coord(i / kBinGrid)) / 16.f;
+    const float u = m == kBinGrid ? grid_coord(i % m) : edge_coord(i % m), v = m == kBinGrid ? grid_coord(i / m) : edge_coord(i / m);
+    const float p = -1.f + (2.f * float((b / 16) % 16) + 1.f + u) / 16.f;
+    const float q = -1.f + (2.f * float(b % 16) + 1.f + v) / 16.f;
     const float n = sqrtf(p * p + q * q + 1.f);
     const float x = f == 0 || f >= 3 ? p : f == 1 ? 1.f : -1.f, y = f == 0 ? q : f <= 2 ? p : f == 3 ? 1.f : -1.f;
-    float *d = dirs + (int64_t(b) * kBinPer + i) * 3;
+    float *d = dirs + (int64_t(b) * m * m + i) * 3;
     d[0] = x / n, d[1] = y / n, d[2] = (f == 0 ? 1.f : q) / n;
 }
 __global__ void k_bin_poly(const float *__restrict__ h, float m2, float *__restrict__ poly) {
@@ -405,14 +412,14 @@ __global__ void k_bin_poly(const float *__restrict__ h, float m2, float *__restr
     if (t >= 108) return;
     const int k = t / 6, c = t % 6, v = PV[k / 3], p = PP[k / 3], q = k % 3;
     const float *hb = h + int64_t(blockIdx.x) * kBinGrid * kBinGrid * 27;
-    float num = 0.f, den = 0.f;
+    double num = 0.0, den = 0.0;
     for (int i = 0; i < kBinGrid * kBinGrid; ++i) {
-        const float a = grid_coord(i % kBinGrid), b = grid_coord(i / kBinGrid);
-        const float phi = c == 0 ? 1.f : c == 1 ? a : c == 2 ? b : c == 3 ? a * a - m2 : c == 4 ? a * b : b * b - m2;
-        num += phi * 0.5f * (hb[27 * i + (v * 3 + p) * 3 + q] + hb[27 * i + (p * 3 + v) * 3 + q]);
+        const double a = grid_coord(i % kBinGrid), b = grid_coord(i / kBinGrid);
+        const double phi = c == 0 ? 1.0 : c == 1 ? a : c == 2 ? b : c == 3 ? a * a - m2 : c == 4 ? a * b : b * b - m2;
+        num += phi * 0.5 * (double(hb[27 * i + (v * 3 + p) * 3 + q]) + double(hb[27 * i + (p * 3 + v) * 3 + q]));
         den += phi * phi;
     }
-    poly[108 * blockIdx.x + t] = num / den;
+    poly[108 * blockIdx.x + t] = float(num / den);
 }
 
 }  // namespace
@@ -679,7 +686,7 @@ static int mlp_tabulate(gbfmm_ctx *ctx) {
     CK(cudaMalloc(&b.dirs, n * 3 * sizeof(float)));
     CK(cudaMalloc(&b.h, n * 27 * sizeof(float)));
     ctx->launches += 2;
-    k_bin_dirs<<<kBins, kBinPer, 0, ctx->stream>>>(b.dirs);
+    k_bin_dirs<<<kBins, kBinPer, 0, ctx->stream>>>(kBinGrid, b.dirs);
     if (int rc = mlp_forward(ctx, n, b.dirs, b.h)) return rc;
     k_bin_poly<<<kBins, 128, 0, ctx->stream>>>(b.h, mlp_poly_m2(), M.poly);
     CK(cudaGetLastError());
@@ -687,57 +694,82 @@ static int mlp_tabulate(gbfmm_ctx *ctx) {
     return GBFMM_OK;
 }
 
+// whether the context's near field reads the polynomials
+static bool mlp_near(const gbfmm_ctx *ctx) {
+    return ctx->opt.h_mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64;
+}
+
 // after the parameters changed: the polynomials, where the near field reads them
 static int mlp_changed(gbfmm_ctx *ctx) {
-    if (ctx->opt.h_mode == GBFMM_H_MLP && ctx->opt.precision != GBFMM_FP64)
+    if (mlp_near(ctx))
         if (int rc = mlp_tabulate(ctx)) return rc;
     ctx->mlp.trained = true;
     return GBFMM_OK;
 }
 
-// Assess the network per angular bin against the plain evaluator: 64 directions
-// per bin of the near-field kernel's binning (k_bin_dirs); a bin whose largest
-// component error exceeds bin_tol x (RMS of h over all samples) is flagged
-// and its pairs take the plain evaluator.
+// Assess per angular bin what the near field uses of the network against the plain evaluator: the
+// network's values at the bin's 64 fitted directions, and the bin's polynomial at these and at 25
+// more from edge to edge.  A bin whose largest component error of either kind exceeds bin_tol x (RMS
+// of h over the fitted directions) is flagged and its pairs take the plain evaluator.
 extern "C" int fmm_mlp_calibrate(gbfmm_ctx *ctx, double bin_tol, double *fallback_frac) {
     if (!ctx || !(bin_tol > 0.0)) return GBFMM_ERR_INVALID_ARG;
     if (!ctx->mlp.trained) return set_err(ctx, GBFMM_ERR_INVALID_ARG, "fmm_mlp_calibrate: train or set the network first");
-    const int nb = kBins, per = kBinPer;
-    constexpr int64_t n = int64_t(kBins) * kBinPer;
+    MlpState &M = ctx->mlp;
+    constexpr int64_t n = int64_t(kBins) * kBinPer, ne = int64_t(kBins) * kBinEdgePer;
     BinScratch b;
     CK(cudaMalloc(&b.dirs, n * 3 * sizeof(float)));
     CK(cudaMalloc(&b.y, n * 27 * sizeof(float)));
     CK(cudaMalloc(&b.h, n * 27 * sizeof(float)));
-    ++ctx->launches;
-    k_bin_dirs<<<kBins, kBinPer, 0, ctx->stream>>>(b.dirs);
-    int rc = fmm_mlp_labels(ctx, n, b.dirs, b.y);
-    if (rc) return rc;
-    rc = mlp_eval_device(ctx, n, b.dirs, b.h);
-    if (rc) return rc;
-    std::vector<float> hy(n * 27), hh(n * 27);
-    CK(cudaMemcpyAsync(hy.data(), b.y, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(hh.data(), b.h, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    if (!mlp_near(ctx))  // then they were not built with the network
+        if (int rc = mlp_tabulate(ctx)) return rc;
+    cudaStream_t st = ctx->stream;
+    std::vector<float> hy(n * 27), hh(n * 27), he(ne * 27), poly(size_t(kBins) * 108);
+    ctx->launches += 2;
+    k_bin_dirs<<<kBins, kBinPer, 0, st>>>(kBinGrid, b.dirs);
+    if (int rc = fmm_mlp_labels(ctx, n, b.dirs, b.y)) return rc;
+    if (int rc = mlp_eval_device(ctx, n, b.dirs, b.h)) return rc;
+    CK(cudaMemcpyAsync(hy.data(), b.y, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(hh.data(), b.h, n * 27 * sizeof(float), cudaMemcpyDeviceToHost, st));
+    k_bin_dirs<<<kBins, kBinEdgePer, 0, st>>>(kBinEdge, b.dirs);
+    if (int rc = fmm_mlp_labels(ctx, ne, b.dirs, b.y)) return rc;
+    CK(cudaMemcpyAsync(he.data(), b.y, ne * 27 * sizeof(float), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(poly.data(), M.poly, poly.size() * sizeof(float), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
     double ss = 0.0;
     for (float v : hy) ss += double(v) * v;
-    const double rms = std::sqrt(ss / double(hy.size()));
+    const double rms = std::sqrt(ss / double(hy.size())), m2 = mlp_poly_m2();
+    static const int PV[6] = {0, 1, 2, 1, 0, 0}, PP[6] = {0, 1, 2, 2, 2, 1};
     uint32_t mask[48] = {0};
     int flagged = 0;
-    for (int bin = 0; bin < nb; ++bin) {
+    for (int bin = 0; bin < kBins; ++bin) {
         double e = 0.0;
-        for (int i = 0; i < per * 27; ++i) {
-            const size_t k = size_t(bin) * per * 27 + i;
-            e = std::max(e, std::fabs(double(hh[k]) - double(hy[k])));
+        auto take = [&e](double d) {
+            if (!(d <= e)) e = std::isnan(d) ? INFINITY : d;
+        };
+        for (size_t k = size_t(bin) * kBinPer * 27; k < size_t(bin + 1) * kBinPer * 27; ++k)
+            take(std::fabs(double(hh[k]) - double(hy[k])));
+        for (int i = 0; i < kBinPer + kBinEdgePer; ++i) {
+            const bool fit = i < kBinPer;
+            const int g = fit ? i : i - kBinPer;
+            const double u = fit ? grid_coord(g % kBinGrid) : edge_coord(g % kBinEdge);
+            const double v = fit ? grid_coord(g / kBinGrid) : edge_coord(g / kBinEdge);
+            const float *y = fit ? &hy[(size_t(bin) * kBinPer + g) * 27] : &he[(size_t(bin) * kBinEdgePer + g) * 27];
+            const double phi[6] = {1.0, u, v, u * u - m2, u * v, v * v - m2};
+            for (int k = 0; k < 18; ++k) {
+                double h = 0.0;
+                for (int c = 0; c < 6; ++c) h += double(poly[size_t(bin) * 108 + 6 * k + c]) * phi[c];
+                take(std::fabs(h - double(y[(PV[k / 3] * 3 + PP[k / 3]) * 3 + k % 3])));
+            }
         }
         if (e > bin_tol * rms) {
             mask[bin >> 5] |= 1u << (bin & 31);
             ++flagged;
         }
     }
-    if (!ctx->mlp.d_binmask) CK(cudaMalloc(&ctx->mlp.d_binmask, sizeof(mask)));
-    CK(cudaMemcpy(ctx->mlp.d_binmask, mask, sizeof(mask), cudaMemcpyHostToDevice));
-    ctx->mlp.fallback_frac = double(flagged) / double(nb);
-    if (fallback_frac) *fallback_frac = ctx->mlp.fallback_frac;
+    if (!M.d_binmask) CK(cudaMalloc(&M.d_binmask, sizeof(mask)));
+    CK(cudaMemcpy(M.d_binmask, mask, sizeof(mask), cudaMemcpyHostToDevice));
+    M.fallback_frac = double(flagged) / double(kBins);
+    if (fallback_frac) *fallback_frac = M.fallback_frac;
     return GBFMM_OK;
 }
 

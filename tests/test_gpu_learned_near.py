@@ -177,7 +177,7 @@ def _restated(f, C, net, x, accepted, coef):
     return out, mag.max(1, keepdims=True), len(i)
 
 
-@pytest.mark.parametrize("part", [1.0])  # share of the bins that the network serves
+@pytest.mark.parametrize("part", [1.0, 0.5])  # share of the bins that the network serves (about)
 @pytest.mark.parametrize("free", [False, True])
 @pytest.mark.parametrize("medium", ["cubic", "turned"])
 @pytest.mark.parametrize("m", [1, 31, 32, 33, 63, 64, 65, 200])
@@ -187,7 +187,8 @@ def test_learned_pairs(m, medium, free, part):
     f = _context(C, net, seed=m)
     coef, e_net, e_poly = _tables(f)
     err = np.sort(np.maximum(e_net, e_poly))
-    k = min(int(part * 1280), 1279)
+    # the widest gap near the middle: no bin whose side FP32 could change
+    k = 513 + int(np.argmax(np.diff(err[512:769])))
     tol = 1e30 if part == 1.0 else 0.5 * (err[k - 1] + err[k])
     f.mlp_calibrate(tol)
     got = _stress(f, len(net[1]), x)
@@ -213,6 +214,26 @@ def test_learned_sum_beside_a_close_pair():
     f.close()
     assert np.abs(plain[2:4]).max() > 1e4 * mag[2:4].max()
     assert np.all(np.abs(got - plain - want) <= 5e-6 * mag + 1e-11 * np.abs(plain).max(1, keepdims=True))
+
+
+def test_calibration_judges_the_polynomials():
+    """A bin is flagged by the larger of two errors, the network's at 64 directions and its
+    polynomial's at these and at 25 more from edge to edge, both against the plain rule.  In a
+    crystal of Zener ratio 8 the two judge many bins differently at some tolerance."""
+    import paper_1712_07739_gb300 as gb
+
+    f = gb.FMM(p=3, levels=3, precision="mixed", h_mode="mlp", circle_q=32).set_material(
+        synth.cubic_voigt(1.684, 1.214, 1.88))
+    f.mlp_train(torch.tensor(synth.directions(300_000, seed=1), device="cuda"), epochs=15, batch=4096, lr=3e-3, seed=4)
+    _, e_net, e_poly = _tables(f)
+    both = np.maximum(e_net, e_poly)
+    tols = np.geomspace(np.quantile(both, 0.02), both.max(), 400)
+    gap = [(both > t).sum() - (e_net > t).sum() for t in tols]
+    tol = tols[int(np.argmax(gap))]
+    print(f"bins flagged at {tol:.3e}: by the network {(e_net > tol).sum()}, by either {(both > tol).sum()}")
+    assert max(gap) >= 8
+    near = np.sum(np.abs(both / tol - 1.0) < 1e-4)  # bins that FP32 could put on the other side
+    assert abs(f.mlp_calibrate(tol) * 1280 - (both > tol).sum()) <= near
 
 
 def test_force_call_after_new_network_under_capture():

@@ -67,9 +67,10 @@
 
 namespace {
 
+// geometry of the offsets, the same for every context of the process (which of them has a residual
+// operator is the context's: M2LParams::lo)
 struct OffsetEntry {
-    short top;      // operator index 0..315
-    short lo;       // index in the residual table, -1 when the offset has no split pass
+    short top;        // operator index 0..315
     signed char cls;  // source parity class
     signed char sx, sy, sz;
 };
@@ -98,6 +99,7 @@ struct M2LParams {
     int nblk;              // operators as A: 128-row blocks of operator rows (a CTA takes two)
     int o_lo, o_hi;        // this launch takes the entries o_lo .. o_hi - 1 of each class's offset list
     int accumulate;        // 0: the epilogue writes the local values, 1: it adds to them
+    short lo[316];         // residual operator of an offset, -1 without
 };
 
 // FP16 mode: power of two that brings a level's largest |W| into [2^12, 2^13)
@@ -263,7 +265,7 @@ constexpr int kMaxSeg = 8 * GB_TC_MAXLEV;
 
 // number of K-block iterations of one work item (same count on every warp);
 // split: the residual passes apply at this level
-__device__ __forceinline__ int passes_of(const OffsetEntry &e, int split) { return (split && e.lo >= 0) ? 3 : 1; }
+__device__ __forceinline__ int passes_of(const M2LParams &P, int o, int split) { return (split && P.lo[o] >= 0) ? 3 : 1; }
 
 // the stage a role works on and its phase: counted, not divided (a division by the run-time number
 // of stages costs more than the rest of a stage's bookkeeping)
@@ -435,10 +437,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int oi = P.o_lo; oi < P.o_hi && ok; ++oi) {
             if (!((s_active[oi / 32] >> (oi % 32)) & 1u)) continue;
             const OffsetEntry e = c_offs[cls][oi];
-            const int np = passes_of(e, split);
+            const int np = passes_of(P, e.top, split);
             for (int pass = 0; pass < np && ok; ++pass) {
                 const CUtensorMap *tb = (pass == 2) ? &P.tmTlo : &P.tmT;
-                const int tidx = (pass == 2) ? e.lo : e.top;
+                const int tidx = (pass == 2) ? P.lo[e.top] : e.top;
                 for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
                     const int s = rg.s;
                     if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (!((s_active[oi / 32] >> (oi % 32)) & 1u)) continue;
             const uint32_t tm = tiles_at<SWAP>(s_tact, oi);
             const OffsetEntry e = c_offs[cls][oi];
-            const int np = passes_of(e, split);
+            const int np = passes_of(P, e.top, split);
             for (int pass = 0; pass < np && ok; ++pass) {
                 for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
                     const int s = rg.s;
@@ -531,7 +533,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                 }
                 __syncwarp();
-                const int np = passes_of(e, split);
+                const int np = passes_of(P, e.top, split);
                 for (int pass = 0; pass < np && ok; ++pass) {
                     const uint8_t *src[TPC][4];
                     uint32_t size[TPC][4];
@@ -649,7 +651,6 @@ struct FewCount {
 };
 struct FewParams {
     M2LParams P;
-    short lo[316];  // residual operator of an offset, -1 without
     int groups;
     const uint32_t *masks;  // [tile][10]: offsets with a source, by k_few_mask
 };
@@ -825,10 +826,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         bool ok = true, drop = P.drop_first != 0;
         for (int oi = 0; oi < noff && ok; ++oi) {
             const int o = s_off[oi] & 511;
-            const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+            const int np = passes_of(P, o, P.split);
             for (int pass = 0; pass < np && ok; ++pass) {
                 const CUtensorMap *tb = pass == 2 ? &P.tmTlo : &P.tmT;
-                const int tidx = pass == 2 ? F.lo[o] : o;
+                const int tidx = pass == 2 ? P.lo[o] : o;
                 for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
                     const int s = rg.s;
                     if (!mbar_wait(empty0 + 8 * s, rg.ph ^ 1, status)) {
@@ -852,7 +853,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int oi = 0; oi < noff && ok; ++oi) {
             const int o = s_off[oi] & 511;
             const uint32_t tm = uint32_t(s_off[oi]) >> 9;
-            const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+            const int np = passes_of(P, o, P.split);
             for (int pass = 0; pass < np && ok; ++pass)
                 for (int kb = 0; kb < (pass == 0 ? P.kb : P.kb_res); ++kb, rg.next(stages)) {
                     const int s = rg.s;
@@ -896,7 +897,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                 }
                 __syncwarp();
-                const int np = P.split && F.lo[o] >= 0 ? 3 : 1;
+                const int np = passes_of(P, o, P.split);
                 for (int pass = 0; pass < np && ok; ++pass) {
                     const uint8_t *src[TPC][4];
                     uint32_t size[TPC][4];
@@ -1392,7 +1393,6 @@ int m2l_tc_setup(gbfmm_ctx *ctx) {
             if (!in) continue;
             OffsetEntry &e = ent[c][cnt++];
             e.top = short(i);
-            e.lo = short(lo_of[i]);
             int sc = 0;
             signed char sh[3];
             for (int d = 0; d < 3; ++d) {
@@ -1689,6 +1689,7 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
     prm.tmem_cols = T.tmem_cols;
     prm.split = T.split;
     prm.split_levels = split_levels;
+    for (int i = 0; i < 316; ++i) prm.lo[i] = T.lo_host[i];
     prm.drop_first = T.inject_drop;
     T.inject_drop = 0;
     const int stage_bytes = T.tpc * kTileA + (T.swap ? 2 * kTileA : T.ncta * 128);
@@ -1716,7 +1717,6 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
         fp.P = prm;
         fp.P.split = T.split && (split_levels & ((2 << few) - 4));
         fp.groups = T.groups;
-        for (int i = 0; i < 316; ++i) fp.lo[i] = T.lo_host[i];
         auto kern = T.tf32 ? k_m2l_few<true> : k_m2l_few<false>;
         if (int rc = fit((const void *)kern)) return rc;
         FewCount *cnt = reinterpret_cast<FewCount *>(T.few_list);

@@ -27,7 +27,6 @@ static void free_tree(gbfmm_ctx *ctx) {
     release(ctx->d_y);
     release(ctx->d_q);
     release(ctx->d_sid);
-    release(ctx->d_slen);
     release(ctx->d_pos);
     release(ctx->d_pleaf);
     release(ctx->d_sig);
@@ -35,7 +34,7 @@ static void free_tree(gbfmm_ctx *ctx) {
     release(ctx->d_q0);
     release(ctx->d_leaf_of);
     release(ctx->d_perm);
-    release(ctx->d_len0);
+    release(ctx->d_segv);
     release(ctx->d_W);
     release(ctx->d_S);
     release(ctx->d_Wf);
@@ -74,15 +73,15 @@ static int ensure_tree_buffers(gbfmm_ctx *ctx) {
     const int P3 = ctx->opt.p * ctx->opt.p * ctx->opt.p;
     const bool w64 = ctx->opt.precision != GBFMM_MIXED;  // FP64 multipole and local values
     {
-        GrowBuf b[11] = {{(void **)&ctx->d_y, N * 3 * sizeof(double)},  {(void **)&ctx->d_q, N * 9 * sizeof(double)},
-                         {(void **)&ctx->d_sid, N * sizeof(int64_t)},   {(void **)&ctx->d_slen, N * sizeof(double)},
+        GrowBuf b[10] = {{(void **)&ctx->d_y, N * 3 * sizeof(double)},  {(void **)&ctx->d_q, N * 9 * sizeof(double)},
+                         {(void **)&ctx->d_sid, N * sizeof(int64_t)},
                          {(void **)&ctx->d_pos, N * sizeof(int)},       {(void **)&ctx->d_pleaf, N * sizeof(int)},
                          {(void **)&ctx->d_sig, N * 6 * sizeof(double)}, {(void **)&ctx->d_y0, N * 3 * sizeof(double)},
                          {(void **)&ctx->d_q0, N * 9 * sizeof(double)}, {(void **)&ctx->d_leaf_of, N * sizeof(int)},
                          {(void **)&ctx->d_perm, N * sizeof(int)}};
-        if (int rc = grow_dev(ctx, ctx->cap_N, N, b, 11, "points")) return rc;
+        if (int rc = grow_dev(ctx, ctx->cap_N, N, b, 10, "points")) return rc;
     }
-    if (int rc = grow_dev(ctx, ctx->cap_segs, ns, {{(void **)&ctx->d_len0, ns * sizeof(double)}}, "segments"))
+    if (int rc = grow_dev(ctx, ctx->cap_segs, ns, {{(void **)&ctx->d_segv, ns * 6 * sizeof(double)}}, "segments"))
         return rc;
     {
         // occupancy scratch: sources and targets per cell (with the adaptive tree, one more
@@ -280,7 +279,7 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     v(c->L), v(c->N), v(c->n_segs), v(c->n_nodes), v(c->n_cells), v(c->n_leaves), v(c->t_cap);
     v(c->node_xyz), v(c->seg_nodes), v(c->burgers), v(c->stream);
     const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Asym_f, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
-                          c->d_slen, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf, c->d_scan,
+                          c->d_segv, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf, c->d_scan,
                           c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_t_pos, c->d_t_start,
                           c->d_t_x, c->d_t_sig, c->tc.Thi, c->tc.Tlo, c->tc.Whi, c->tc.Wlo, c->tc.d_status,
                           c->tc.d_flags, c->tc.d_pos, c->tc.d_list, c->tc.d_seg, c->tc.d_wmax, c->mlp.theta, c->mlp.theta_h,

@@ -108,7 +108,6 @@ struct gbfmm_ctx {
     double *d_y = nullptr;     // [N][3] sorted by leaf
     double *d_q = nullptr;     // [N][9]
     int64_t *d_sid = nullptr;  // [N] segment of each sorted point
-    double *d_slen = nullptr;  // [N] length of that segment
     int *d_pos = nullptr;      // [N] original point index -> sorted position
     int *d_pleaf = nullptr;    // [N] leaf of each sorted point
     int *d_leaf_start = nullptr;  // [n_leaves + 1]
@@ -116,7 +115,8 @@ struct gbfmm_ctx {
     int *d_tmp_i = nullptr;       // scratch ints, N + n_leaves + 1
     double *d_tmp_d = nullptr;    // scratch doubles
     // build scratch
-    double *d_y0 = nullptr, *d_q0 = nullptr, *d_len0 = nullptr, *d_part = nullptr;
+    double *d_y0 = nullptr, *d_q0 = nullptr, *d_part = nullptr;
+    double *d_segv = nullptr;     // [n_segs][6] line and Burgers vectors as built (the near field's)
     int *d_leaf_of = nullptr, *d_cnt = nullptr, *d_cursor = nullptr, *d_perm = nullptr, *d_bad = nullptr;
     // capacities (elements) of the buffers sized by N, segments, cells, leaves
     int64_t cap_N = 0, cap_segs = 0, cap_cells = 0, cap_leaves = 0;

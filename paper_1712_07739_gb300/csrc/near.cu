@@ -88,18 +88,16 @@ __device__ __forceinline__ void split_position(const double *y, const double c[3
 template <typename R>
 __global__ void k_near_records(int64_t N, int L, const TreeBox *__restrict__ box, const double *__restrict__ y,
                                const int *__restrict__ perm, const int *__restrict__ pleaf,
-                               const double *__restrict__ nodes, const int64_t *__restrict__ segs,
-                               const double *__restrict__ burgers, GaussWeights gw, double fac, void *__restrict__ rec) {
+                               const double *__restrict__ segv, GaussWeights gw, double fac, void *__restrict__ rec) {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= N) return;
     const int k = perm[i];
     const int64_t s = k / gw.n;
-    const int64_t n0 = segs[2 * s], n1 = segs[2 * s + 1];
     const double f = 0.5 * gw.w[k - int(s) * gw.n] * fac;
     double S[3], b[3];
     for (int d = 0; d < 3; ++d) {
-        S[d] = nodes[3 * n1 + d] - nodes[3 * n0 + d];
-        b[d] = f * burgers[3 * s + d];
+        S[d] = segv[6 * s + d];
+        b[d] = f * segv[6 * s + 3 + d];
     }
     if constexpr (sizeof(R) == 4) {
         float4 *r = static_cast<float4 *>(rec);
@@ -1061,12 +1059,10 @@ int near_prepare(gbfmm_ctx *ctx) {
     const double fac = near_factor(ctx->mat);
     if (ctx->opt.precision == GBFMM_FP64)
         k_near_records<double><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
-                                                                       ctx->d_pleaf, ctx->node_xyz, ctx->seg_nodes,
-                                                                       ctx->burgers, gw, fac, ctx->nw.rec);
+                                                                       ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->nw.rec);
     else
         k_near_records<float><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
-                                                                      ctx->d_pleaf, ctx->node_xyz, ctx->seg_nodes,
-                                                                      ctx->burgers, gw, fac, ctx->nw.rec);
+                                                                      ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->nw.rec);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }

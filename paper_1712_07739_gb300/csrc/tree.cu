@@ -26,7 +26,7 @@ struct GaussParams {
 
 __global__ void k_gauss_points(int64_t n_segs, const double *__restrict__ nodes, const int64_t *__restrict__ segs,
                                const double *__restrict__ b, GaussParams gp, double *__restrict__ y0,
-                               double *__restrict__ q0, double *__restrict__ len0, int *__restrict__ bad) {
+                               double *__restrict__ q0, double *__restrict__ segv, int *__restrict__ bad) {
     int64_t s = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (s >= n_segs) return;
     int64_t n0 = segs[2 * s], n1 = segs[2 * s + 1];
@@ -38,7 +38,7 @@ __global__ void k_gauss_points(int64_t n_segs, const double *__restrict__ nodes,
     }
     double len = sqrt(S[0] * S[0] + S[1] * S[1] + S[2] * S[2]);
     if (!(len > 0.0) || !isfinite(len)) atomicExch(bad, 1);
-    len0[s] = len;
+    for (int i = 0; i < 3; ++i) segv[6 * s + i] = S[i], segv[6 * s + 3 + i] = bb[i];
     for (int g = 0; g < gp.n; ++g) {
         int64_t k = s * gp.n + g;
         double f = 0.5 * (1.0 + gp.xi[g]);
@@ -225,10 +225,9 @@ __global__ void k_ref_children(int64_t nl, const int *__restrict__ start, const 
 }
 
 __global__ void k_gather_points(int64_t n, int n_g, const int *__restrict__ perm, const double *__restrict__ y0,
-                                const double *__restrict__ q0, const double *__restrict__ len0,
-                                const int *__restrict__ leaf_of, double *__restrict__ y, double *__restrict__ q,
-                                int64_t *__restrict__ sid, double *__restrict__ slen, int *__restrict__ pos,
-                                int *__restrict__ pleaf, const unsigned char *__restrict__ child_of,
+                                const double *__restrict__ q0, const int *__restrict__ leaf_of,
+                                double *__restrict__ y, double *__restrict__ q, int64_t *__restrict__ sid,
+                                int *__restrict__ pos, int *__restrict__ pleaf, const unsigned char *__restrict__ child_of,
                                 const int *__restrict__ ref_start, int *__restrict__ pfine) {
     int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= n) return;
@@ -241,7 +240,6 @@ __global__ void k_gather_points(int64_t n, int n_g, const int *__restrict__ perm
     for (int d = 0; d < 3; ++d) y[3 * i + d] = y0[3 * int64_t(k) + d];
     for (int d = 0; d < 9; ++d) q[9 * i + d] = q0[9 * int64_t(k) + d];
     sid[i] = k / n_g;
-    slen[i] = len0[k / n_g];
     pos[k] = int(i);
 }
 
@@ -370,14 +368,14 @@ int tree_build(gbfmm_ctx *ctx, bool validate) {
         ctx->gauss_w[i] = gp.w[i];
     }
     const int64_t nl = ctx->n_leaves;
-    double *y0 = ctx->d_y0, *q0 = ctx->d_q0, *len0 = ctx->d_len0, *part = ctx->d_part;
+    double *y0 = ctx->d_y0, *q0 = ctx->d_q0, *part = ctx->d_part;
     int *leaf_of = ctx->d_leaf_of, *cnt = ctx->d_cnt, *cursor = ctx->d_cursor, *perm = ctx->d_perm;
     int *bad = ctx->d_bad;
     const int nparts = int(std::min<int64_t>(kBoxParts, (N + 255) / 256));
     CK(cudaMemsetAsync(bad, 0, sizeof(int), st));
     ++ctx->launches;
     k_gauss_points<<<nblk(ctx->n_segs, 128), 128, 0, st>>>(ctx->n_segs, ctx->node_xyz, ctx->seg_nodes, ctx->burgers,
-                                                           gp, y0, q0, len0, bad);
+                                                           gp, y0, q0, ctx->d_segv, bad);
     ++ctx->launches;
     k_bbox_partial<<<nparts, 256, 0, st>>>(N, y0, part);
     ++ctx->launches;
@@ -404,8 +402,8 @@ int tree_build(gbfmm_ctx *ctx, bool validate) {
                                                       RF.ref_leaf, RF.child_start);
     }
     ++ctx->launches;
-    k_gather_points<<<nblk(N, 256), 256, 0, st>>>(N, ng, perm, y0, q0, len0, leaf_of, ctx->d_y, ctx->d_q,
-                                                  ctx->d_sid, ctx->d_slen, ctx->d_pos, ctx->d_pleaf,
+    k_gather_points<<<nblk(N, 256), 256, 0, st>>>(N, ng, perm, y0, q0, leaf_of, ctx->d_y, ctx->d_q,
+                                                  ctx->d_sid, ctx->d_pos, ctx->d_pleaf,
                                                   refine ? RF.child_of : nullptr, RF.ref_start,
                                                   refine ? RF.pfine : nullptr);
     CK(cudaGetLastError());

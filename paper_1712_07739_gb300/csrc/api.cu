@@ -192,6 +192,14 @@ extern "C" int fmm_create(gbfmm_ctx **out, const gbfmm_options *opt, void *strea
     return GBFMM_OK;
 }
 
+void free_scratch(PassScratch &w) {
+    NearWork &W = w.nw;
+    void *ps[] = {W.rec, W.trec, W.plan, W.lp, W.pitems, W.rows, W.pcnt, w.few_part};
+    for (void *q : ps)
+        if (q) cudaFree(q);
+    w = PassScratch{};
+}
+
 extern "C" void fmm_destroy(gbfmm_ctx *ctx) {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->stream);
@@ -210,12 +218,7 @@ extern "C" void fmm_destroy(gbfmm_ctx *ctx) {
     m2l_tc_free(ctx);
     m2l_fft_free(ctx);
     mlp_free(ctx);
-    {
-        NearWork &W = ctx->nw;
-        void *ps2[] = {W.rec, W.trec, W.plan, W.lp, W.pitems, W.rows, W.pcnt};
-        for (void *q : ps2)
-            if (q) cudaFree(q);
-    }
+    free_scratch(ctx->own_ws);
     if (ctx->timer.on)
         for (auto &e : ctx->timer.ev) cudaEventDestroy(e);
     delete ctx;
@@ -278,18 +281,19 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     mix(&c->opt, sizeof(c->opt));
     v(c->L), v(c->N), v(c->n_segs), v(c->n_nodes), v(c->n_cells), v(c->n_leaves), v(c->t_cap);
     v(c->node_xyz), v(c->seg_nodes), v(c->burgers), v(c->stream);
+    const PassScratch &w = c->ws();
     const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Asym_f, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
                           c->d_segv, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf, c->d_scan,
                           c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_t_pos, c->d_t_start,
                           c->d_t_x, c->d_t_sig, c->tc.Thi, c->tc.Tlo, c->tc.Whi, c->tc.Wlo, c->tc.d_status,
                           c->tc.d_flags, c->tc.d_pos, c->tc.d_list, c->tc.d_seg, c->tc.d_wmax, c->mlp.theta, c->mlp.theta_h,
                           c->mlp.scale, c->mlp.d_binmask, c->mlp.poly,
-                          c->nw.rec, c->nw.trec, c->nw.plan,
-                          c->nw.lp, c->nw.pitems, c->nw.rows, c->nw.pcnt, c->tc.Uh, c->tc.Ul, c->tc.Rh, c->tc.Rl,
+                          w.nw.rec, w.nw.trec, w.nw.plan,
+                          w.nw.lp, w.nw.pitems, w.nw.rows, w.nw.pcnt, c->tc.Uh, c->tc.Ul, c->tc.Rh, c->tc.Rl,
                           c->tc.Xh, c->tc.Xl, c->tc.d_scal, c->tc.d_bits, c->tc.Wc, c->tc.Sc, c->tc.blas_ws,
                           c->rf.child_of, c->rf.ref_start, c->rf.ref_leaf, c->rf.child_start, c->rf.pfine,
                           c->rf.W7, c->rf.S7, c->rf.Wc7, c->rf.Sc7, c->tc.d_pcnt, c->tc.d_pairs, c->tc.Gh,
-                          c->tc.Gl, c->tc.Yf, c->tc.few_list, c->tc.few_part};
+                          c->tc.Gl, c->tc.Yf, c->tc.few_list, w.few_part};
     mix(ptrs, sizeof(ptrs));
     v(c->mat.mode), v(c->mat.Q), v(c->mat.cubic), v(c->tc.n_work), v(c->tc.split), v(c->tc.tf32);
     mix(c->tc.wofs, sizeof(c->tc.wofs));

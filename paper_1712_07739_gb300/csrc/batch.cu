@@ -27,6 +27,7 @@ struct gbfmm_batch {
     cudaEvent_t in = nullptr, done = nullptr;  // caller -> cap and cap -> caller ordering
     std::vector<gbfmm_ctx *> ctx;
     std::vector<cudaStream_t> side;  // fan-out streams
+    std::vector<PassScratch> scratch;  // one for the slots of each side stream, whose passes follow one another
     std::vector<cudaEvent_t> ev;     // fork + one join per side stream
     std::vector<double *> out;       // force outputs recorded in the graph
     std::vector<uint64_t> layout;    // layout_hash of each context when the graph was recorded
@@ -96,6 +97,7 @@ extern "C" int fmm_batch_create(gbfmm_batch **out, const gbfmm_options *opt_in, 
     b->stream = (cudaStream_t)stream;
     const int ns = std::min(n, 8);
     b->side.resize(ns);
+    b->scratch.resize(ns);
     b->ev.resize(ns + 1);
     for (int i = 0; i < ns; ++i)
         if (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess) {
@@ -121,6 +123,7 @@ extern "C" int fmm_batch_create(gbfmm_batch **out, const gbfmm_options *opt_in, 
             delete b;
             return rc;
         }
+        c->shared_ws = &b->scratch[k % ns];
         b->ctx.push_back(c);
     }
     b->out.assign(n, nullptr);
@@ -138,6 +141,7 @@ extern "C" void fmm_batch_destroy(gbfmm_batch *b) {
     drop_graph(b);
     // borrowed material tables belong to context 0: free the others first
     for (size_t k = b->ctx.size(); k-- > 0;) fmm_destroy(b->ctx[k]);
+    for (auto &w : b->scratch) free_scratch(w);
     for (auto s : b->side) cudaStreamDestroy(s);
     for (auto e : b->ev) cudaEventDestroy(e);
     if (b->cap) cudaStreamDestroy(b->cap);
@@ -252,6 +256,8 @@ extern "C" int fmm_batch_build(gbfmm_batch *b, int k, int64_t n_nodes, const dou
     if (!b || k < 0 || k >= int(b->ctx.size())) return GBFMM_ERR_INVALID_ARG;
     if (!b->material) return berr(b, GBFMM_ERR_NO_MATERIAL, "fmm_batch_build: set the material first");
     gbfmm_ctx *c = b->ctx[k];
+    // a replay may still run, and the slots of a stream share their passes' scratch
+    if (cudaStreamSynchronize(b->cap) != cudaSuccess) return berr(b, GBFMM_ERR_CUDA, "fmm_batch_build: synchronise");
     drop_graph(b);
     auto build_at = [&](int L) {
         c->opt.levels = L;

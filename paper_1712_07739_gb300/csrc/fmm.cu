@@ -449,7 +449,7 @@ int mixed_pass(gbfmm_ctx *ctx, bool free_targets, int64_t n_t) {
     timer_mark(ctx);
     if (L >= 3) {
         int rc = m2l_tc_run(ctx, ctx->d_Wf, t64 ? ctx->d_W : nullptr, occ, tocc, ctx->d_Sf, t64 ? ctx->d_S : nullptr,
-                            fine);
+                            fine, n_t);
         if (rc) return rc;
     }
     timer_mark(ctx);

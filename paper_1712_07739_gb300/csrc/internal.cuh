@@ -65,6 +65,15 @@ struct NearWork {
     int64_t rec_cap = 0, trec_cap = 0, plan_cap = 0, item_cap = 0, row_cap = 0;
 };
 
+// What a pass only works in.  A context has its own; the contexts of a batch that run one after the
+// other on a stream share one (64 networks would hold 64 of up to 0.3 GB else).
+struct PassScratch {
+    NearWork nw;
+    float *few_part = nullptr;  // sums of the sections of the M2L of few cells (m2l_tc.cu)
+    int64_t few_cap = 0;
+};
+void free_scratch(PassScratch &w);  // api.cu
+
 struct Timer {
     cudaEvent_t ev[16];
     bool on = false;
@@ -94,7 +103,9 @@ struct gbfmm_ctx {
     FftPlan fft;
     // learned h
     MlpState mlp;
-    NearWork nw;
+    PassScratch own_ws, *shared_ws = nullptr;
+    PassScratch &ws() { return shared_ws ? *shared_ws : own_ws; }
+    const PassScratch &ws() const { return shared_ws ? *shared_ws : own_ws; }
     bool borrowed_material = false;  // medium tables belong to another context (a batch)
 
     // tree

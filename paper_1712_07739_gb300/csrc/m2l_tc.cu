@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const int q = warp % 4, trow = q * 32 + lane;
         for (int t = 0; t < tiles; ++t) {
             const int r = t * 128 + trow;
-            float *dst = part + ((int64_t(sec) * sets + set) * kFewRows + r) * Np + group * P.ncta;
+            float *dst = part + (int64_t(sec) * cells + set * kFewRows + r) * Np + group * P.ncta;
             for (int c0 = 16 * half; c0 < P.nsub; c0 += 32) {
                 float v[16];
                 for (int i = 0; i < 16; ++i) v[i] = 0.f;
@@ -957,7 +957,7 @@ __global__ void k_few_sum(const FewCount *__restrict__ cnt, const int *__restric
     const int64_t g = cell_base_d(level) + (int64_t((code >> 10) & 31) * n + ((code >> 5) & 31)) * n + (code & 31);
     float sc = float(double(n) / box->H) * float(double(n) / box->H);
     if (wmax) sc *= inv_op_scale / wscale_of(wmax[level]);
-    const int64_t step = int64_t(cnt->sets) * kFewRows * Np;
+    const int64_t step = int64_t(cnt->cells) * Np;
     for (int k = threadIdx.x; k < nvalid; k += blockDim.x) {
         const float *p = part + int64_t(cell) * Np + k;
         float hi = 0.f, lo = 0.f;
@@ -1553,6 +1553,24 @@ static int few_top_of(const gbfmm_ctx *ctx) {
     return std::min(ctx->L - 1, kFewTop);
 }
 
+// The sections' sums and the launch of k_m2l_few for n target points: every number of cells up to
+// what the levels hold and n points can occupy (p = 6, levels to 4: 169 MB; 600 points: 27 MB).
+static int few_alloc(gbfmm_ctx *ctx, int64_t n) {
+    TcPlan &T = ctx->tc;
+    const int chunks = std::max(1, ctx->opt.m2l_chunks);
+    int64_t cells = 0, rows = 0;
+    for (int l = 2; l <= T.few_top; ++l) cells += std::min(int64_t(1) << (3 * l), n);
+    T.few_work = 0;
+    for (int64_t k = 1; k <= (cells + kFewRows - 1) / kFewRows; ++k) {
+        const int64_t sec = few_sections(int(k), T.groups, chunks, ctx->sm_count);
+        rows = std::max(rows, sec * std::min(k * kFewRows, cells));
+        T.few_work = std::max<int>(T.few_work, int(k * sec * T.groups));
+    }
+    PassScratch &ws = ctx->ws();
+    return grow_dev(ctx, ws.few_cap, rows * T.Np, {{(void **)&ws.few_part, size_t(rows) * T.Np * sizeof(float)}},
+                    "M2L sections");
+}
+
 // Per-tree buffers: packed W (hi / lo), tensor maps, work list.
 int m2l_tc_prepare(gbfmm_ctx *ctx) {
     TcPlan &T = ctx->tc;
@@ -1566,22 +1584,10 @@ int m2l_tc_prepare(gbfmm_ctx *ctx) {
     if (int rc = grow_dev(ctx, T.w_cap, tot, {{&T.Whi, size_t(tot) * T.esz}, {&T.Wlo, size_t(tot) * T.esz}},
                           "packed multipole values"))
         return rc;
-    // levels 2 .. few_top go through k_m2l_few: its cell list, counts and the sections' sums, for
-    // every number of cell sets up to the levels' cells
+    // levels 2 .. few_top go through k_m2l_few: its cell list, counts and the sections' sums
     T.few_top = few_top_of(ctx);
     if (T.few_top >= 2) {
-        const int chunks = std::max(1, ctx->opt.m2l_chunks);
-        const int64_t cells = cell_base(T.few_top + 1) - cell_base(2), sets_max = (cells + kFewRows - 1) / kFewRows;
-        int64_t rows = 0;
-        T.few_work = 0;
-        for (int64_t k = 1; k <= sets_max; ++k) {
-            const int64_t sec = few_sections(int(k), T.groups, chunks, ctx->sm_count);
-            rows = std::max(rows, k * sec * kFewRows);
-            T.few_work = std::max<int>(T.few_work, int(k * sec * T.groups));
-        }
-        if (int rc = grow_dev(ctx, T.few_cap, rows * T.Np,
-                              {{(void **)&T.few_part, size_t(rows) * T.Np * sizeof(float)}}, "M2L sections"))
-            return rc;
+        if (int rc = few_alloc(ctx, ctx->N)) return rc;
         if (!T.few_list)
             CK(cudaMalloc(&T.few_list, 16 + (cell_base(kFewTop + 1) - cell_base(2)) * sizeof(int) +
                                            (kFewSetsMax * 3 * 10) * sizeof(uint32_t)));
@@ -1604,7 +1610,7 @@ int m2l_tc_prepare(gbfmm_ctx *ctx) {
 }
 
 int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *occ, const int *tocc, float *Sf,
-               double *S64, bool fine) {
+               double *S64, bool fine, int64_t n_targets) {
     TcPlan &T = ctx->tc;
     // fine: the adaptive tree's children (level ctx->L) take part through fine_m2l, after the
     // tensor-core M2L of levels 2 .. L-1
@@ -1713,6 +1719,8 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
     if (T.svd) CK(cudaMemsetAsync(T.Sc, 0, size_t(ctx->n_cells) * T.r1 * sizeof(float), st));
     const int few = T.few_top;
     if (few >= 2) {
+        if (int rc = few_alloc(ctx, n_targets)) return rc;  // (free targets may occupy more cells than the sources)
+        float *part = ctx->ws().few_part;
         FewParams fp;
         fp.P = prm;
         fp.P.split = T.split && (split_levels & ((2 << few) - 4));
@@ -1726,9 +1734,9 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
         k_few_list<<<1, 1024, 0, st>>>(few, T.groups, std::max(1, ctx->opt.m2l_chunks), ctx->sm_count, tocc, list, cnt);
         k_few_mask<<<dim3(unsigned((cell_base(few + 1) - cell_base(2) + 127) / 128), 10), 512, 0, st>>>(
             cnt, list, occ, const_cast<uint32_t *>(fp.masks));
-        kern<<<T.few_work, kTcThreads, smem, st>>>(fp, cnt, list, occ, T.few_part, T.Np, T.d_status, stages);
+        kern<<<T.few_work, kTcThreads, smem, st>>>(fp, cnt, list, occ, part, T.Np, T.d_status, stages);
         k_few_sum<<<unsigned(cell_base(few + 1) - cell_base(2)), 256, 0, st>>>(
-            cnt, list, T.few_part, T.Np, prm.nvalid, prm.wmax, prm.inv_op_scale, ctx->d_box, Sout, S64);
+            cnt, list, part, T.Np, prm.nvalid, prm.wmax, prm.inv_op_scale, ctx->d_box, Sout, S64);
         CK(cudaGetLastError());
         prm.drop_first = 0;
     }
@@ -1782,7 +1790,7 @@ void m2l_tc_free(gbfmm_ctx *ctx) {
     TcPlan &T = ctx->tc;
     svd_free(ctx, ctx->borrowed_material);
     void *ps[] = {T.Thi, T.Tlo, T.Whi, T.Wlo, T.d_status, T.d_flags, T.d_pos, T.d_list, T.d_seg, T.d_wmax,
-                  T.few_list, T.few_part};
+                  T.few_list};
     for (void *q : ps)
         if (q) cudaFree(q);
     T = TcPlan{};

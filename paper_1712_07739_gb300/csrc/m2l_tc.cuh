@@ -36,12 +36,9 @@ struct TcPlan {
     int4 *d_seg = nullptr;     // per (level, class): first list entry, count, first tile
     int64_t slot_cap = 0, n_slots = 0;
     int n_seg = 0;
-    // few cells (k_m2l_few): deepest level taken, CTAs of the largest launch, counts and cell list,
-    // the sections' sums
+    // few cells (k_m2l_few): deepest level taken, CTAs of the largest launch, counts and cell list
     int few_top = 1, few_work = 0;
     void *few_list = nullptr;
-    float *few_part = nullptr;
-    int64_t few_cap = 0;
     // SVD-compressed M2L (gbfmm_options.m2l_svd_tol > 0, m2l_svd.cu): the GEMM runs on
     // r2 source and r1 target coefficients per cell
     int svd = 0;
@@ -83,7 +80,7 @@ int m2l_tc_prepare(gbfmm_ctx *ctx);  // per tree
 // fine: the adaptive tree's children take part (compressed M2L: transforms of their values,
 // fine_m2l over their pairs, expansion into their local values)
 int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *occ, const int *tocc, float *Sf,
-               double *S64, bool fine = false);
+               double *S64, bool fine, int64_t n_targets);
 void m2l_tc_free(gbfmm_ctx *ctx);
 int m2l_tc_status(gbfmm_ctx *ctx, int *out);
 

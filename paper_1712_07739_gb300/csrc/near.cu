@@ -1028,7 +1028,7 @@ static int64_t items_cap(int64_t n, int64_t nl) { return n / 2 + std::min(n, nl)
 
 // buffers of the pair kernel for n targets (records of the targets only when they are free)
 static int pairs_alloc(gbfmm_ctx *ctx, int64_t n, bool free_targets) {
-    NearWork &W = ctx->nw;
+    NearWork &W = ctx->ws().nw;
     const bool f32 = ctx->opt.precision != GBFMM_FP64;
     const int64_t nl = ctx->n_leaves, rows = free_targets ? rows_free(n) : rows_sym(n), it = items_cap(n, nl);
     const size_t point = f32 ? 4 * sizeof(float4) : 5 * sizeof(double2), target = 2 * sizeof(float4);
@@ -1059,10 +1059,10 @@ int near_prepare(gbfmm_ctx *ctx) {
     const double fac = near_factor(ctx->mat);
     if (ctx->opt.precision == GBFMM_FP64)
         k_near_records<double><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
-                                                                       ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->nw.rec);
+                                                                       ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->ws().nw.rec);
     else
         k_near_records<float><<<nblk(N, 256), 256, 0, ctx->stream>>>(N, ctx->L, ctx->d_box, ctx->d_y, ctx->d_perm,
-                                                                      ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->nw.rec);
+                                                                      ctx->d_pleaf, ctx->d_segv, gw, fac, ctx->ws().nw.rec);
     CK(cudaGetLastError());
     return GBFMM_OK;
 }
@@ -1099,7 +1099,7 @@ static int launch_combine(gbfmm_ctx *ctx, const NearTree &tr, const int *tleaf, 
 template <typename R, bool SYM>
 static int run_pairs(gbfmm_ctx *ctx, const int *tstart, const double *xt, int64_t n_t, const int *tleaf, double *sig) {
     if (int rc = pairs_alloc(ctx, n_t, !SYM)) return rc;
-    NearWork &W = ctx->nw;
+    NearWork &W = ctx->ws().nw;
     cudaStream_t st = ctx->stream;
     const int64_t nl = ctx->n_leaves;
     // adaptive tree (nodal forces): split leaves, their children's ranges and local values

@@ -72,9 +72,10 @@ def near_pair_flops(precision, h_mode, q, cubic=False):
 
 
 def near_flops(wl, work):
-    """Algorithmic FLOP of the near field (+ L2P) of one pass and the kernel
-    that does it.  With the unit-circle h both passes evaluate h once per
-    unordered pair (h is odd) and contract it for both directions: per
+    """FLOP of the near field (+ L2P) of one pass by the pointwise rule and
+    108-entry source tensors, and the kernel that would do it (``near_work``
+    counts what the pair kernel does).  With the unit-circle h both passes
+    evaluate h once per unordered pair (h is odd) and contract it for both directions: per
     ordered pair half an h evaluation (cubic rule 193 Q + 77, general rule
     450 Q + 20) plus one contraction (229)."""
     p, q = wl["p"], wl.get("circle_q", 64)
@@ -701,7 +702,7 @@ def roofline_of(wl, work, m2l_ms, leaf_ms, m2l_fft, peaks, ranks=None):
     if leaf_ms >= m2l_ms:
         flops, kname = near_work(wl, work)
         achieved = flops / (leaf_ms / 1e3) / 1e12
-        nodal = near_flops(wl, work)[1] == "k_near_sym"  # the passes the captures below describe
+        nodal = wl["h_mode"] == "circle" and not fp64  # the passes the captures below describe
         dom, bound, peak, src = kname + " (L2P + near-field P2P)", "alu", alu_peak, peaks["source"]
         if nodal and wl.get("circle_q") == 16 and not wl.get("refine_points"):
             traffic = NEAR_SYM_DRAM_BYTES_PER_POINT * work["points"]

@@ -47,8 +47,8 @@ extern "C" {
 
 /* precision of the pass */
 #define GBFMM_FP64 0   /* every stage in FP64 */
-#define GBFMM_MIXED 1  /* FP32 P2M/M2M/L2L/L2P and near field (FP64 for close pairs),
-                          M2L on tcgen05 tensor cores (operand precision: m2l_split) */
+#define GBFMM_MIXED 1  /* FP32 P2M/M2M/L2L/L2P and near field (positions and sums of every pair
+                          carry two floats), M2L on tcgen05 tensor cores (operand precision: m2l_split) */
 #define GBFMM_MIXED_F64T 2  /* as GBFMM_MIXED with P2M, M2M, L2L and L2P in FP64, which removes the
                                rounding of those interpolations (the Lebesgue constants of
                                equispaced nodes amplify it at high orders) */

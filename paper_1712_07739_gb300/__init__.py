@@ -339,7 +339,7 @@ class FMM:
 
     def mlp_eval_noalloc(self, dirs, out):
         """Network h into a caller-provided tensor, with no device allocation
-        in the library (scratch is a static device array)."""
+        in the library (the activations stay in registers)."""
         dirs = self._f32(dirs)
         self._check(self._lib.fmm_mlp_eval_noalloc(self._h, dirs.shape[0], _ptr(dirs), _ptr(out)),
                     "fmm_mlp_eval_noalloc")

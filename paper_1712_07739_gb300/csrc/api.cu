@@ -207,11 +207,10 @@ extern "C" void fmm_destroy(gbfmm_ctx *ctx) {
     if (ctx->borrowed_material) {
         ctx->d_mat = nullptr;
         ctx->d_Asym = nullptr;
-        ctx->d_Asym_f = nullptr;
         ctx->d_Klat = nullptr;
         ctx->tc.Thi = ctx->tc.Tlo = nullptr;
     }
-    void *ps[] = {ctx->d_box, ctx->d_mat, ctx->d_Asym, ctx->d_Asym_f, ctx->d_Klat,
+    void *ps[] = {ctx->d_box, ctx->d_mat, ctx->d_Asym, ctx->d_Klat,
                   ctx->d_t_pos, ctx->d_t_leaf, ctx->d_t_x, ctx->d_t_sig, ctx->d_t_tmp};
     for (void *p : ps)
         if (p) cudaFree(p);
@@ -282,7 +281,7 @@ uint64_t layout_hash(const gbfmm_ctx *c) {
     v(c->L), v(c->N), v(c->n_segs), v(c->n_nodes), v(c->n_cells), v(c->n_leaves), v(c->t_cap);
     v(c->node_xyz), v(c->seg_nodes), v(c->burgers), v(c->stream);
     const PassScratch &w = c->ws();
-    const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Asym_f, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
+    const void *ptrs[] = {c->d_mat, c->d_Asym, c->d_Klat, c->d_box, c->d_y, c->d_q, c->d_sid,
                           c->d_segv, c->d_pos, c->d_pleaf, c->d_leaf_start, c->d_tmp_i, c->d_tmp_d, c->d_perm, c->d_t_leaf, c->d_scan,
                           c->d_W, c->d_S, c->d_Wf, c->d_Sf, c->d_sig, c->d_t_pos, c->d_t_start,
                           c->d_t_x, c->d_t_sig, c->tc.Thi, c->tc.Tlo, c->tc.Whi, c->tc.Wlo, c->tc.d_status,

@@ -93,7 +93,6 @@ struct gbfmm_ctx {
     DevMaterial *d_mat = nullptr;
     double Asym[6 * 9 * 18];   // A contracted over the (v,p) symmetry: [ab][wr][k]
     double *d_Asym = nullptr;
-    float *d_Asym_f = nullptr;
     int lat_n = 0;             // lattice points per dimension, 8 (p-1) + 1
     double *d_Klat = nullptr;  // [lat_n^3][54] kernel at unit-cell lattice differences
 

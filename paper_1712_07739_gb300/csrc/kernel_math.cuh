@@ -32,18 +32,6 @@ __device__ __forceinline__ void h_iso_sym(R hc, R ha, const R T[3], R hs[18]) {
     }
 }
 
-// sin and cos of pi k / Q in the precision of the caller (no FP64 on the FP32 path)
-template <typename R>
-__device__ __forceinline__ void circle_point(int k, int Q, R *s, R *c);
-template <>
-__device__ __forceinline__ void circle_point<double>(int k, int Q, double *s, double *c) {
-    sincospi(double(k) / double(Q), s, c);
-}
-template <>
-__device__ __forceinline__ void circle_point<float>(int k, int Q, float *s, float *c) {
-    sincospif(float(k) / float(Q), s, c);
-}
-
 // (a b)_jk = a_i C_ijkl b_l
 template <typename R, typename CT>
 __device__ __forceinline__ void cmat(const CT *C, const R a[3], const R b[3], R M[9]) {
@@ -83,7 +71,7 @@ __device__ __forceinline__ void h_circle_sym(const CT *C, int Q, const R Tin[3],
     for (int i = 0; i < 18; ++i) acc[i] = 0;
     for (int k = 0; k < Q; ++k) {
         R s, c;
-        circle_point<R>(k, Q, &s, &c);
+        sincospi(double(k) / double(Q), &s, &c);
         R z[3];
         for (int i = 0; i < 3; ++i) z[i] = c * e1[i] + s * e2[i];
         R M[9], ZT[9];
@@ -148,7 +136,7 @@ __device__ __forceinline__ void h_circle_cubic(R c12, R c44, R D, int Q, const R
     for (int i = 0; i < 18; ++i) acc[i] = 0;
     for (int k = 0; k < Q; ++k) {
         R sn, cs;
-        circle_point<R>(k, Q, &sn, &cs);
+        sincospi(double(k) / double(Q), &sn, &cs);
         R z[3];
         for (int i = 0; i < 3; ++i) z[i] = cs * e1[i] + sn * e2[i];
         // M = (zz) (symmetric; |z| = 1)

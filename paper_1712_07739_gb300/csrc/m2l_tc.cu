@@ -1632,7 +1632,7 @@ int m2l_tc_run(gbfmm_ctx *ctx, const float *Wf, const double *W64, const int *oc
         prm.wrow[l] = int(T.wofs[l] / T.Kp);
     }
     // blocks stride over the cells of a level, one row of blocks per level
-    const dim3 gw(unsigned(std::min<int64_t>(int64_t(1) << (3 * (L - 1)), 8 * 152)), unsigned(L - 2));
+    const dim3 gw(unsigned(std::min<int64_t>(int64_t(1) << (3 * (L - 1)), 8 * ctx->sm_count)), unsigned(L - 2));
     cudaStream_t st = ctx->stream;
     if (T.modal && !T.svd) {
         // node values -> Legendre moments (in place: nothing reads these W after the M2L)

@@ -100,14 +100,10 @@ int material_setup(gbfmm_ctx *ctx) {
                         ctx->Asym[(ab * 9 + w * 3 + r) * 18 + pr * 3 + q] = tot;
                     }
     }
-    float Af[6 * 9 * 18];
-    for (int i = 0; i < 6 * 9 * 18; ++i) Af[i] = float(ctx->Asym[i]);
     if (!ctx->d_mat) CK(cudaMalloc(&ctx->d_mat, sizeof(DevMaterial)));
     if (!ctx->d_Asym) CK(cudaMalloc(&ctx->d_Asym, sizeof(ctx->Asym)));
-    if (!ctx->d_Asym_f) CK(cudaMalloc(&ctx->d_Asym_f, sizeof(Af)));
     CK(cudaMemcpyAsync(ctx->d_mat, &ctx->mat, sizeof(DevMaterial), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_Asym, ctx->Asym, sizeof(ctx->Asym), cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->d_Asym_f, Af, sizeof(Af), cudaMemcpyHostToDevice, ctx->stream));
 
     int lat_n = 8 * (p - 1) + 1;
     int64_t total = int64_t(lat_n) * lat_n * lat_n;
@@ -137,7 +133,6 @@ int share_material(gbfmm_ctx *ctx, const gbfmm_ctx *src) {
     std::memcpy(ctx->Asym, src->Asym, sizeof(ctx->Asym));
     ctx->d_mat = src->d_mat;
     ctx->d_Asym = src->d_Asym;
-    ctx->d_Asym_f = src->d_Asym_f;
     ctx->d_Klat = src->d_Klat;
     ctx->lat_n = src->lat_n;
     TcPlan &T = ctx->tc;
@@ -200,7 +195,6 @@ extern "C" int fmm_set_material(gbfmm_ctx *ctx, const double *V) {
         // stop sharing: this context builds its own tables from here on
         ctx->d_mat = nullptr;
         ctx->d_Asym = nullptr;
-        ctx->d_Asym_f = nullptr;
         ctx->d_Klat = nullptr;
         ctx->lat_n = 0;
         ctx->tc.Thi = ctx->tc.Tlo = nullptr;

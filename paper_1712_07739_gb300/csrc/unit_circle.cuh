@@ -144,7 +144,7 @@ __device__ __forceinline__ void moments(const NearMedium<R> &m, const R *tab, co
     }
     if (m.np <= kMomMax) {
 #pragma unroll 1
-        for (int k = 0; k < m.np; ++k) moment_step(tab + kMomRow * k, det, dd, Th, Ps);  // UNR
+        for (int k = 0; k < m.np; ++k) moment_step(tab + kMomRow * k, det, dd, Th, Ps);
     } else {
         moments_long<R>(m.Q, m.np, det, dd, Th, Ps);
     }

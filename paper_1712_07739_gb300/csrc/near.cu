@@ -27,11 +27,11 @@
 // warp takes which item or on where the rows lie, so results repeat exactly.
 //
 // Bound: instruction issue and the FMA pipe (250,000-segment walls, cubic, Q = 16: issue slots 75 %
-// and FMA pipe 66 % busy, ~1,170 warp instructions per 32 pairs for both directions, DRAM 27
-// GB/s).  Time of the near field with L2P, one h by the pointwise rule, 108-entry source tensors and
-// one warp per leaf pair before: those walls 43 -> 21 ps a pair; 50,003 segments of loops
-// (Q = 32) 35.1 -> 9.9 ms; 6,101 segments in a turned crystal ~120 -> 5 ms; FP64, 3,001 segments
-// 620 -> 9 ms; 2,000 isotropic segments 125 -> 5 ms.
+// and FMA pipe 59 % busy, ~1,280 warp instructions per 32 pairs for both directions, DRAM 28
+// GB/s).  Near field with L2P: those walls 33.9 ms, 50,003 segments of loops (Q = 32) 8.8, 6,101 in a
+// turned crystal 3.0, 3,001 in FP64 12.1, 2,000 isotropic in FP64 2.7.  Whole calls, with one h by
+// the pointwise rule, 108-entry source tensors and one warp per leaf pair before: 83 -> 45 ms, 36 ->
+// 10.2, 80 to 90 -> 3.2, 490 to 580 -> 15.8, 66 to 146 -> 3.8 (uneven leaves made these vary).
 //
 // Precision of the FP32 form: positions are FP32 pairs (value + remainder) relative to the
 // leaf centre, so every separation is correct to its own rounding, also of close pairs; h and
@@ -834,10 +834,11 @@ __global__ void __launch_bounds__(near_warps<R>() * 32, near_blocks<R>())
 // Far field (L2P) plus the stress of the summed strain rows, LANES threads per point.  Eight lanes
 // share a point's 3 p basis values, take every eighth (y, z) row of the p^3 local values and every
 // eighth of its rows, and are added by a fixed tree: in the smallest calls one thread's chain is
-// the time (157 segments 64 -> 27 us, FP64 167 us).  One thread per point where there are enough
-// points to fill the GPU: the 32 points of a warp then mostly read the same local values (4M
-// points: 7.3 ms with eight lanes).
-constexpr int64_t kCombinePoints = 65536;  // up to this many points: eight lanes
+// the time.  One thread per point where there are enough points to fill the GPU: the 32 points of a
+// warp then mostly read the same local values.  One lane / eight, p = 5, us: 628 points 50 / 24, 8,000
+// 214 / 68, 24,000 87 / 81, 48,000 114 / 118, 64,000 98 / 138, 200,000 200 / 409, 4M 2,036 / 6,962; FP64
+// 628 points 103 / 34, 24,000 141 / 140, 48,000 234 / 232, 64,000 218 / 295.
+constexpr int64_t kCombinePoints = 40000;  // up to this many points: eight lanes
 
 template <int LANES, typename SR>
 __device__ __forceinline__ void l2p(int p, const NodeTab<SR> &nt, SR *basis, int g, const double c0[3], double ih,

@@ -117,12 +117,12 @@ def near_work(wl, work):
 
 # DRAM bytes per target point of one near-field launch (k_near_pairs, cubic rule, Q = 16), from
 # one ncu capture on the 250,000-segment slab network (dram__bytes_read.sum +
-# dram__bytes_write.sum = 0.161 + 0.760 GB for 1,000,000 points); valid for the
+# dram__bytes_write.sum = 0.154 + 0.761 GB for 1,000,000 points); valid for the
 # kernel version the capture was taken of
-NEAR_SYM_DRAM_BYTES_PER_POINT = (1.60587e8 + 7.60081e8) / 1.0e6
+NEAR_SYM_DRAM_BYTES_PER_POINT = (1.54447e8 + 7.60710e8) / 1.0e6
 # the same two counters for the headline's launch itself (1M segments, adaptive tree at
 # threshold 128; a one-pass capture of the full-size run)
-NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES = 1112050432 + 3203101952
+NEAR_SYM_ADAPTIVE_1M_DRAM_BYTES = 1121237248 + 3200880896
 
 
 def measured_alu_peaks():
@@ -162,8 +162,8 @@ WORKLOADS["c3"] = dict(
          "C44=0.754, order p=7 on Chebyshev nodes, adaptive octree: 7 levels with every leaf holding more than 128 "
          "Gauss points split once more (children of two split leaves that are not adjacent interact by an M2L one "
          "level down, adjacent ones directly), mixed precision (SVD-compressed M2L on the tensor cores: FP16 "
-         "operands, residual passes on the leading singular directions; FP32 near field with FP64 separations for "
-         "close pairs), unit-circle h (cubic form, Q=16 points on the half circle); the same step through the "
+         "operands, residual passes on the leading singular directions; FP32 near field with two-float "
+         "separations and sums), unit-circle h (cubic form, Q=16 points on the half circle); the same step through the "
          "plain FP64 pass (uniform 7-level tree) is timed in the same run",
     gen=lambda seed: synth.slab_loops(seed=2 + 1000 * seed), C=lambda: synth.cubic_voigt(),
     h_mode="circle", circle_q=16, p=7, levels=7, precision="mixed", refine_points=128, fp64_arm=True, **CHEB_M2L)
